@@ -1137,14 +1137,27 @@ struct NbList {
 };
 using NbList64 = NbList<double>;
 
-// Precision-form neighbour lists: pass 1 stores each accepted neighbour
-// j != s with its binary32 kernel value as {j, K bits} in slot k of s (entry
-// at k * stride + s); count[s] is the full number.  Pass 2 of a warp whose
-// lanes all fit their lists walks them instead of searching.
-struct NbList32 {
+// What pass 1 of the precision form keeps for pass 2, in planes of `stride`
+// entries (plane p of particle s at p * stride + s).
+// 3-d: neighbour lists.  Plane k holds s's k-th accepted neighbour j != s with
+// its binary32 kernel value, {j, K bits}; ex[s].w is the full number, and a
+// particle with more than `cap` searches in pass 2.
+// 1-d and 2-d: accept masks.  A word {base, bits} holds 32 consecutive
+// candidates of one neighbour row: bit k is set when candidate base + k is an
+// accepted neighbour j != s.  Plane w holds s's w-th word with a bit set, in
+// candidate order; ex[s].w is their number and the number of neighbours
+// (mask_word), or kMaskOver for a particle that needs more than `cap` words and
+// searches in pass 2.  With `pad` > 0 every row is filled up to `pad` words
+// with empty ones, so that a warp's lanes have the same row in the same plane.
+struct Nb32 {
     uint2* e;
-    int cap;           // 0: no list; a particle's count is in its record ex[s].w
+    int cap;           // planes (masks: at most 255); 0: nothing kept, pass 2 searches
+    int pad;           // words every row has at least (masks; see setup_grids)
 };
+constexpr uint32_t kMaskOver = 0xffffffffu;
+__device__ __forceinline__ uint32_t mask_word(uint32_t words, uint32_t neighbours, int cap) {
+    return words <= uint32_t(cap) && neighbours < (1u << 24) - 1u ? neighbours << 8 | words : kMaskOver;
+}
 
 // Phases A-C for the calling warp (every lane of the warp must call it; lanes
 // with valid = false walk nothing).  eval(owner_s, j, d2f) returns the pair
@@ -1411,62 +1424,221 @@ k_exchange_f64(int n, int64_t stride, const double* __restrict__ pos, const floa
     }
 }
 
+// The particle's record that pass 2 reads per neighbour, written whole by pass
+// 1: m = {m_hi, m_lo, r, list word (bits, see Nb32; of use to the particle
+// itself only)}, the mass's binary32 head/tail split and the row sum.  Below
+// 3-d it is preceded by a copy of the particle's rec, so that all of a
+// neighbour's 32 bytes (from which pass 2 also forms K again) are one sector
+// and one 32-byte load.
+template <int DIM>
+struct ExRec {
+    static constexpr int kVec = DIM == 3 ? 1 : 2;   // float4 per particle
+};
+struct PairRec {
+    float4 rec, m;
+};
+__device__ __forceinline__ PairRec load_pair_rec(const float4* __restrict__ ex, uint32_t j) {
+    PairRec q;
+    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(q.rec.x), "=f"(q.rec.y), "=f"(q.rec.z), "=f"(q.rec.w), "=f"(q.m.x), "=f"(q.m.y),
+          "=f"(q.m.z), "=f"(q.m.w)
+        : "l"(ex + 2 * size_t(j)));
+    return q;
+}
+__device__ __forceinline__ void store_pair_rec(float4* __restrict__ ex, uint32_t s, const float4& rec,
+                                               const float4& m) {
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(ex + 2 * size_t(s)),
+                 "f"(rec.x), "f"(rec.y), "f"(rec.z), "f"(rec.w), "f"(m.x), "f"(m.y), "f"(m.z), "f"(m.w)
+                 : "memory");
+}
+template <int DIM>
+__device__ __forceinline__ float4 load_ex(const float4* __restrict__ ex, uint32_t j) {
+    return __ldg(ex + size_t(ExRec<DIM>::kVec) * j + (ExRec<DIM>::kVec - 1));
+}
+
+// Pass 1 of a 1-d or 2-d particle that met candidates inside the narrow band
+// around the cutoff (about 1e-5 of all candidates): walks its windows again,
+// adds those the exact test accepts to the row sum and writes its mask words
+// with them.  Returns {rsum, rc, words (bits), neighbours (bits)}.  A real
+// call, so its registers do not weigh on the candidate loop.
+template <int DIM, class View>
+__device__ __noinline__ float4 band_accepts(uint32_t s, int64_t stride,
+                                            const double* __restrict__ pos,
+                                            const float4* __restrict__ rec,
+                                            const uint32_t* __restrict__ start, const View& v,
+                                            Nb32 nb, float rsum, float rc) {
+    const RealParams& P = v.of_sorted(s);
+    const PairParams& pp = P.pp;
+    const float4 me = rec[s];
+    uint32_t cnt = 0, nw = 0;
+    for_each_row<DIM>(0u, me, rec, start, P,
+                      [&](uint32_t j, uint32_t j3, float rx, float sy, float sz) {
+        // (no padding: pass 2 takes a particle's words as they come)
+        while (j < j3) {
+            const uint32_t base = j, end = min(j3, base + 32u);
+            uint32_t bits = 0;
+            for (; j < end; ++j) {
+                const float4 o = __ldg(rec + j);
+                const float dx = dx_f32(me, o, P.g.wf[0]);
+                if (dx > rx) {
+                    j3 = j;
+                    break;
+                }
+                const float d2f = d2_f32<DIM>(dx, me, o, sy, sz);
+                if (d2f > pp.band_hi) continue;
+                if (d2f >= pp.band_lo) {
+                    if (!exact_within<DIM>(pos, stride, s, j, pp.psi2)) continue;
+                    const float y = __fsub_rn(ex2_approx(-pp.a_log2e * d2f), rc);
+                    const float t = __fadd_rn(rsum, y);
+                    rc = __fsub_rn(__fsub_rn(t, rsum), y);
+                    rsum = t;
+                }
+                if (j != s) bits |= 1u << (j - base);
+            }
+            if (bits) {
+                cnt += uint32_t(__popc(bits));
+                if (nw < uint32_t(nb.cap)) nb.e[int64_t(nw) * stride + s] = make_uint2(base, bits);
+                ++nw;
+            }
+        }
+    });
+    return make_float4(rsum, rc, __uint_as_float(nw), __uint_as_float(cnt));
+}
+
 // Pass 1, precision form: binary32 kernel exp2(-a log2(e) d2f) with the
 // hardware ex2, compensated binary32 row sum, rounded to binary32; written
-// with the binary32 head/tail split of the mass as the particle's record
-// ex[s] = {m_hi, m_lo, r, list length (bits)} that pass 2 reads once per
-// neighbour (.w only for the particle itself);
-// with nb.cap > 0 also the neighbour lists of pass 2 (accepted j != s with
-// their K, in visiting order: the band's exact accepts come last).
-template <int DIM, class View, int BLOCK>
-__global__ void __launch_bounds__(BLOCK, (DIM == 3 ? 1536 : 2048) / BLOCK)
+// in the particle's record ex (ExRec); with nb.cap > 0 also what pass 2 needs
+// of the search (Nb32).  Bound by instruction issue and the candidate loads'
+// latency.  In 1-d and 2-d the accepted neighbours leave as mask words, one
+// 8-byte store a row next to the other lanes' stores: a {j, K} list entry per
+// neighbour was a partly written sector each, and those writes bounded the
+// pass (2-d, 4e6 particles with 5.7 neighbours each: 218 us with lists, 170
+// with masks; 1e7 with 57 each: 6.5 and 1.5 ms).  In 3-d (3.6 neighbours over
+// nine rows) the list is the shorter of the two.
+template <int DIM, class View>
+__global__ void __launch_bounds__(kBlock, (DIM == 3 ? 1536 : 2048) / kBlock)
 k_rowsum_f32(int n, int64_t stride, const double* __restrict__ pos, const float4* __restrict__ rec,
              const uint32_t* __restrict__ cell, const uint32_t* __restrict__ start,
              const __grid_constant__ View v, const double* __restrict__ mass,
              float4* __restrict__ ex, unsigned long long* __restrict__ pair_counter,
-             const uint32_t* __restrict__ ghost_id, NbList32 nb) {
+             const uint32_t* __restrict__ ghost_id, Nb32 nb) {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     uint32_t cnt = 0;
     if (s < n) {
         const RealParams& P = v.of_sorted(uint32_t(s));
         float rsum = 0.0f, rc = 0.0f;
-        uint32_t listed = 0;
-        if (P.transfer) {
+        uint32_t list_word = 0;
+        // compensated (Kahan) step for positive terms: rsum - rc carries the
+        // sum; kept only for accepted pairs
+        auto add = [&](float K, bool accept) {
+            const float y = __fsub_rn(K, rc);
+            const float t = __fadd_rn(rsum, y);
+            const float cn = __fsub_rn(__fsub_rn(t, rsum), y);
+            rsum = accept ? t : rsum;
+            rc = accept ? cn : rc;
+        };
+        if (!P.transfer) {
+            rsum = 1.0f;
+        } else if constexpr (DIM == 3) {
             const float na = -P.pp.a_log2e;
             const uint32_t cap = uint32_t(nb.cap);
-            uint2* lp = nb.e + s;          // slot `listed` of s
-            scan_neighbours<DIM, true>(uint32_t(s), cell_arg<DIM>(cell, s), stride, rec, pos, start, P,
+            uint2* lp = nb.e + s;          // slot `cnt` of s
+            scan_neighbours<DIM, true>(uint32_t(s), cell[s], stride, rec, pos, start, P,
                                  [&](uint32_t j, float d2f, bool accept) {
-                                     // compensated (Kahan) step for positive terms:
-                                     // rsum - rc carries the sum; kept only for
-                                     // accepted pairs
                                      const float K = ex2_approx(na * d2f);
-                                     const float y = __fsub_rn(K, rc);
-                                     const float t = __fadd_rn(rsum, y);
-                                     const float cn = __fsub_rn(__fsub_rn(t, rsum), y);
-                                     rsum = accept ? t : rsum;
-                                     rc = accept ? cn : rc;
+                                     add(K, accept);
                                      const bool keep = accept && j != uint32_t(s);
-                                     if (keep && listed < cap) *lp = make_uint2(j, __float_as_uint(K));
+                                     if (keep && cnt < cap) *lp = make_uint2(j, __float_as_uint(K));
                                      if (keep) lp += stride;
-                                     listed += keep ? 1u : 0u;
+                                     cnt += keep ? 1u : 0u;
                                  });
-            cnt = listed;   // the accepted pairs but the self pair
+            list_word = cnt;
         } else {
-            rsum = 1.0f;
+            const PairParams& pp = P.pp;
+            const Grid& g = P.g;
+            const float4 me = rec[s];
+            const float na = -pp.a_log2e, wx = g.wf[0], eps = pp.trim_eps;
+            const int R = g.reach, cx = int(me.w), cy = DIM == 2 ? int(me.z) : 0;
+            const int xlo = max(cx - R, 0), xhi = min(cx + R, g.n[0] - 1);
+            uint2* wp = nb.e + s;          // next mask word
+            uint32_t nw = 0;
+            bool band = false;
+            // rows in a fixed order for the whole warp: an empty window where
+            // the row is outside the grid or beyond the cutoff (for_each_row
+            // has the windows' derivation)
+#pragma unroll 1
+            for (int dy = DIM == 2 ? -R : 0; dy <= (DIM == 2 ? R : 0); ++dy) {
+                const float sy = DIM == 2 ? float(dy) * g.wf[1] : 0.0f;
+                const float gy = DIM == 2 ? row_gap(dy, me.y, g.wf[1], eps) : 0.0f;
+                const float r2 = __fsub_rn(pp.reach2, __fmul_rn(gy, gy));
+                const bool in_grid = DIM == 1 || (cy + dy >= 0 && cy + dy < g.n[1]);
+                uint32_t j = 0, j3 = 0;
+                float rx = 0.0f;
+                if (in_grid && r2 >= 0.0f) {
+                    rx = __fadd_rn(sqrt_approx(r2), eps);
+                    const uint32_t rowc =
+                        P.cell_base + uint32_t(DIM == 2 ? cy + dy : 0) * uint32_t(g.n[0]);
+                    if (check(rowc + uint32_t(xhi) + 1u - P.cell_base <=
+                                  uint32_t(g.n[0]) * uint32_t(g.n[1]) * uint32_t(g.n[2]), kChkRow)) {
+                        j = __ldg(start + rowc + xlo);
+                        j3 = __ldg(start + rowc + xhi + 1);
+                        uint32_t hi = j3;
+                        while (j < hi) {
+                            const uint32_t mid = (j + hi) >> 1;
+                            if (dx_f32(me, __ldg(rec + mid), wx) < -rx) j = mid + 1;
+                            else hi = mid;
+                        }
+                    }
+                }
+                const uint32_t padded = nw + uint32_t(nb.pad);
+                while (j < j3) {
+                    const uint32_t base = j, end = min(j3, base + 32u);
+                    uint32_t bits = 0, bit = 1;
+                    for (; j < end; ++j, bit <<= 1) {
+                        const float4 o = __ldg(rec + j);
+                        const float dx = dx_f32(me, o, wx);
+                        if (dx > rx) {
+                            j3 = j;
+                            break;
+                        }
+                        const float d2f = d2_f32<DIM>(dx, me, o, sy, 0.0f);
+                        band |= (d2f >= pp.band_lo) & (d2f <= pp.band_hi);
+                        const bool accept = d2f < pp.band_lo;
+                        add(ex2_approx(na * d2f), accept);
+                        bits |= accept ? bit : 0u;
+                    }
+                    // the self pair gives the row sum's self term only
+                    if (uint32_t(s) - base < 32u) bits &= ~(1u << (uint32_t(s) - base));
+                    if (bits) {
+                        cnt += uint32_t(__popc(bits));
+                        if (nw < uint32_t(nb.cap)) *wp = make_uint2(base, bits);
+                        wp += stride;
+                        ++nw;
+                    }
+                }
+                for (; nw < padded; ++nw, wp += stride)
+                    if (nw < uint32_t(nb.cap)) *wp = make_uint2(0u, 0u);
+            }
+            if (band) {
+                const float4 b = band_accepts<DIM>(uint32_t(s), stride, pos, rec, start, v, nb, rsum, rc);
+                rsum = b.x;
+                rc = b.y;
+                nw = __float_as_uint(b.z);
+                cnt = __float_as_uint(b.w);
+            }
+            list_word = mask_word(nw, cnt, nb.cap);
         }
         float mhi, mlo;
         split_double(mass[s], &mhi, &mlo);
-        ex[s] = make_float4(mhi, mlo, __fsub_rn(rsum, rc), __uint_as_float(listed));
+        const float4 m = make_float4(mhi, mlo, __fsub_rn(rsum, rc), __uint_as_float(list_word));
+        if constexpr (DIM == 3) ex[s] = m;
+        else store_pair_rec(ex, uint32_t(s), rec[s], m);
         // with ghost_id (a tile), pairs are counted for the tile's own particles only
         if (ghost_id && (ghost_id[s] & kGhostBit)) cnt = 0;
     }
     add_pair_count(cnt, pair_counter);
 }
 
-// Pass 2, precision form: W = 2K / (r_s + r_j) in binary32 (symmetric bit for
-// bit), mass difference from the binary32 head/tail split (exactly
-// antisymmetric), flux accumulated with compensation, update in binary64.
 // The flux sum of pass 2, precision form: W = 2 beta K / (r_s + r_j) in
 // binary32 (symmetric bit for bit), the mass difference from the binary32
 // head/tail split (exactly antisymmetric), compensated accumulation, and the
@@ -1495,10 +1667,10 @@ struct FluxSum {
     }
 };
 
-// Pass 2 of one particle by search, as pass 1 visited its candidates (the
-// band's exact accepts last), for a particle whose list overflowed or when
-// there are no lists.  A real call, so its registers do not weigh on the
-// list loop.
+// Pass 2 of one particle by search, in the order in which its list or masks
+// hold its neighbours (3-d: the band's exact accepts last), for a particle
+// they do not cover or when there are none.  A real call, so its registers do
+// not weigh on the list loop.
 template <int DIM, class View>
 __device__ __noinline__ float2 search_flux(uint32_t s, int64_t stride,
                                            const double* __restrict__ pos,
@@ -1510,9 +1682,9 @@ __device__ __noinline__ float2 search_flux(uint32_t s, int64_t stride,
     const RealParams& P = v.of_sorted(s);
     const float na = -P.pp.a_log2e;
     FluxSum g{rs, two_beta, ms};
-    scan_neighbours<DIM, true>(s, cell_arg<DIM>(cell, s), stride, rec, pos, start, P,
+    scan_neighbours<DIM, DIM == 3>(s, cell_arg<DIM>(cell, s), stride, rec, pos, start, P,
                          [&](uint32_t j, float d2f, bool accept) {
-                             g.add(__ldg(ex + j), ex2_approx(na * d2f), accept);
+                             g.add(load_ex<DIM>(ex, j), ex2_approx(na * d2f), accept);
                          });
     return make_float2(g.acc, g.comp);
 }
@@ -1601,9 +1773,9 @@ __device__ __noinline__ float4 search_flux2(uint32_t s, int64_t stride,
     const RealParams& P = v.of_sorted(s);
     const float na = -P.pp.a_log2e;
     FluxSum a{rs, two_beta, ms}, b{rs, two_beta, msb};
-    scan_neighbours<DIM, true>(s, cell_arg<DIM>(cell, s), stride, rec, pos, start, P,
+    scan_neighbours<DIM, DIM == 3>(s, cell_arg<DIM>(cell, s), stride, rec, pos, start, P,
                          [&](uint32_t j, float d2f, bool accept) {
-                             const float4 xj = __ldg(ex + j);
+                             const float4 xj = load_ex<DIM>(ex, j);
                              const float W = a.weight(xj, ex2_approx(na * d2f));
                              a.add_w(make_float2(xj.x, xj.y), W, accept);
                              b.add_w(__ldg(exb + j), W, accept);
@@ -1611,16 +1783,87 @@ __device__ __noinline__ float4 search_flux2(uint32_t s, int64_t stride,
     return make_float4(a.acc, a.comp, b.acc, b.comp);
 }
 
-// Pass 2, precision form: each particle walks its neighbour list (the
-// accepted neighbours only, with pass 1's K), two entries at a time so two
-// gathers are in flight, or searches when it has none (no lists, or an
-// overflowing one).  Both add the same terms in the same order.
-template <int DIM, class View, int BLOCK, bool TWO = false, int WALK = 0>
-__global__ void __launch_bounds__(BLOCK, 2048 / BLOCK)
+// The 32-byte records of neighbours j0 and, with `two`, j1 (both gathers in
+// flight), their kernel formed by pass 1's operations from the same values,
+// and their fluxes.
+// WIDE: one 32-byte load a record (not in real calls: ptxas 13.0 crashes on
+// it there), otherwise two of 16 bytes.
+template <int DIM, bool TWO, bool WIDE>
+struct PairFlux {
+    const float4* ex;
+    const float2* exb;
+    float4 me;
+    float na, wx, wy;
+    __device__ __forceinline__ float kernel(const float4& o) const {
+        const float sy = DIM == 2 ? __fmul_rn(__fsub_rn(o.z, me.z), wy) : 0.0f;
+        return ex2_approx(na * d2_f32<DIM>(dx_f32(me, o, wx), me, o, sy, 0.0f));
+    }
+    __device__ __forceinline__ PairRec load(uint32_t j) const {
+        if constexpr (WIDE) return load_pair_rec(ex, j);
+        else return PairRec{__ldg(ex + 2 * size_t(j)), __ldg(ex + 2 * size_t(j) + 1)};
+    }
+    __device__ __forceinline__ void add(FluxSum& f, FluxSum& g, uint32_t j0, uint32_t j1,
+                                        bool two) const {
+        const PairRec q0 = load(j0), q1 = load(j1);
+        if constexpr (TWO) {
+            const float2 b0 = __ldg(exb + j0), b1 = __ldg(exb + j1);
+            const float w0 = f.weight(q0.m, kernel(q0.rec)), w1 = f.weight(q1.m, kernel(q1.rec));
+            f.add_w(make_float2(q0.m.x, q0.m.y), w0);
+            g.add_w(b0, w0);
+            f.add_w(make_float2(q1.m.x, q1.m.y), w1, two);
+            g.add_w(b1, w1, two);
+        } else {
+            f.add(q0.m, kernel(q0.rec));
+            f.add(q1.m, kernel(q1.rec), two);
+        }
+    }
+};
+
+// Pass 2 of a particle with more than three mask words (long windows), word
+// by word, the next word loaded ahead: {acc_A, comp_A, acc_B, comp_B}.  A
+// real call, so its registers do not weigh on the short particles' loop.
+template <int DIM, bool TWO>
+__device__ __noinline__ float4 words_flux(const uint2* __restrict__ e, int64_t stride,
+                                          uint32_t words, const float4* __restrict__ ex,
+                                          const float2* __restrict__ exb, float4 me, float na,
+                                          float wx, float wy, float rs, float two_beta, float2 ms,
+                                          float2 msb) {
+    const PairFlux<DIM, TWO, false> pf{ex, exb, me, na, wx, wy};
+    FluxSum f{rs, two_beta, ms}, g{rs, two_beta, msb};
+    uint2 ahead = __ldg(e);
+    for (uint32_t w = 1; w <= words; ++w) {
+        const uint32_t base = ahead.x;
+        uint32_t bits = ahead.y;
+        if (w < words) ahead = __ldg(e += stride);
+        while (bits) {
+            const uint32_t j0 = base + uint32_t(__ffs(int(bits)) - 1);
+            bits &= bits - 1u;
+            const bool two = bits != 0u;
+            const uint32_t j1 = two ? base + uint32_t(__ffs(int(bits)) - 1) : j0;
+            bits &= bits - 1u;
+            pf.add(f, g, j0, j1, two);
+        }
+    }
+    return make_float4(f.acc, f.comp, g.acc, g.comp);
+}
+
+// Pass 2, precision form: each particle walks the neighbours that pass 1 kept
+// (3-d: its list, with pass 1's K; 1-d and 2-d: its mask words, with K formed
+// again from the two records as pass 1 formed it), two at a time so two
+// gathers are in flight, or searches when it has none or they do not cover
+// it.  Both add the same terms in the same order.  Bound by the gathers'
+// latency.  Masks in place of lists move 24 instead of 45 bytes a particle for
+// eight more operations a neighbour: 104 us at 4e6 particles in 2-d (100 with
+// lists), 1.5 ms at 1e7 with 57 neighbours (2.0).  Registers: 32 keep all 2048
+// threads of an SM (four more would cost 4 us); both species, or a batch's
+// view, need 40 (62 and 58 us at 32 and 40 for the reaction at 1e6).
+// The bounds hold for blocks of 128 too (the tuning's other block size).
+template <int DIM, class View, bool TWO = false, int WALK = 0>
+__global__ void __launch_bounds__(kBlock, (TWO || View::kBatch ? 1536 : 2048) / kBlock)
 k_exchange_f32(int n, int64_t stride, const double* __restrict__ pos, const float4* __restrict__ rec,
                const uint32_t* __restrict__ cell, const uint32_t* __restrict__ start,
                const __grid_constant__ View v, const float4* __restrict__ ex,
-               const double* __restrict__ mass, double* __restrict__ mass_out, NbList32 nb,
+               const double* __restrict__ mass, double* __restrict__ mass_out, Nb32 nb,
                const float2* __restrict__ exb = nullptr, const double* __restrict__ mass_b = nullptr,
                double* __restrict__ mass_b_out = nullptr, double kp = 0.0, double dt = 0.0,
                float kpdt_f = 0.0f, const WalkAhead wa = WalkAhead{}) {
@@ -1639,46 +1882,87 @@ k_exchange_f32(int n, int64_t stride, const double* __restrict__ pos, const floa
         if constexpr (WALK > 0) walk_ahead<DIM, WALK>(P, s, stride, pos, wa);
         return;
     }
-    const float4 xs = ex[s];
+    const float4 xs = load_ex<DIM>(ex, uint32_t(s));
     FluxSum f{xs.z, float(2.0 * P.pp.beta), make_float2(xs.x, xs.y)};   // beta folded into W
     FluxSum g{xs.z, f.two_beta, TWO ? __ldg(exb + s) : make_float2(0.0f, 0.0f)};
-    const uint32_t listed = nb.cap > 0 ? __float_as_uint(xs.w) : 0xffffffffu;
-    if (listed <= uint32_t(nb.cap)) {
-        const uint2* e = nb.e + s;
-        uint32_t k = 0;
-        if constexpr (TWO) {
-            for (; k + 2 <= listed; k += 2, e += 2 * stride) {
-                const uint2 q0 = __ldg(e), q1 = __ldg(e + stride);
-                const float4 x0 = __ldg(ex + q0.x), x1 = __ldg(ex + q1.x);
-                const float2 b0 = __ldg(exb + q0.x), b1 = __ldg(exb + q1.x);
-                const float w0 = f.weight(x0, __uint_as_float(q0.y));
-                f.add_w(make_float2(x0.x, x0.y), w0);
-                g.add_w(b0, w0);
-                const float w1 = f.weight(x1, __uint_as_float(q1.y));
-                f.add_w(make_float2(x1.x, x1.y), w1);
-                g.add_w(b1, w1);
-            }
-            if (k < listed) {
-                const uint2 q = __ldg(e);
-                const float4 x = __ldg(ex + q.x);
-                const float w = f.weight(x, __uint_as_float(q.y));
-                f.add_w(make_float2(x.x, x.y), w);
-                g.add_w(__ldg(exb + q.x), w);
+    const uint32_t listed = __float_as_uint(xs.w);   // see Nb32
+    if (nb.cap > 0 && (DIM == 3 ? listed <= uint32_t(nb.cap) : listed != kMaskOver)) {
+        if constexpr (DIM < 3) {
+            const PairFlux<DIM, TWO, true> pf{ex, exb, __ldg(ex + 2 * size_t(s)), -P.pp.a_log2e,
+                                              P.g.wf[0], P.g.wf[1]};
+            const uint2* e = nb.e + s;
+            const uint32_t words = listed & 255u;
+            if (words <= 3u) {
+                // up to three words (a row each, at the densities where a row's
+                // window stays below 32 candidates): one stream of neighbours
+                // over them, so a warp runs as long as its longest particle's
+                // count and not its rows'
+                const uint2 none = make_uint2(0u, 0u);
+                uint2 w0 = words > 0u ? __ldg(e) : none;
+                uint2 w1 = words > 1u ? __ldg(e + stride) : none;
+                const uint2 w2 = words > 2u ? __ldg(e + 2 * stride) : none;
+                auto next = [&]() {
+                    const bool shift = w0.y == 0u;
+                    w0 = shift ? w1 : w0;
+                    w1 = shift ? w2 : w1;
+                    const uint32_t j = w0.x + uint32_t(__ffs(int(w0.y)) - 1);
+                    w0.y &= w0.y - 1u;
+                    return j;
+                };
+                uint32_t left = listed >> 8;
+                for (; left >= 2u; left -= 2u) {
+                    const uint32_t j0 = next();
+                    pf.add(f, g, j0, next(), true);
+                }
+                if (left) {
+                    const uint32_t j = next();
+                    pf.add(f, g, j, j, false);
+                }
+            } else {
+                const float4 sum = words_flux<DIM, TWO>(e, stride, words, ex, exb, pf.me, pf.na, pf.wx,
+                                                        pf.wy, f.rs, f.two_beta, f.ms, g.ms);
+                f.acc = sum.x;
+                f.comp = sum.y;
+                g.acc = sum.z;
+                g.comp = sum.w;
             }
         } else {
-            // two entries per iteration, the next two list entries loaded
-            // while this pair's neighbour records are in flight
-            uint2 p0 = listed > 0u ? __ldg(e) : make_uint2(uint32_t(s), 0u);
-            uint2 p1 = listed > 1u ? __ldg(e + stride) : p0;
-            for (; k + 2 <= listed; k += 2, e += 2 * stride) {
-                const uint2 q0 = p0, q1 = p1;
-                const float4 x0 = __ldg(ex + q0.x), x1 = __ldg(ex + q1.x);
-                p0 = k + 2 < listed ? __ldg(e + 2 * stride) : q0;
-                p1 = k + 3 < listed ? __ldg(e + 3 * stride) : q1;
-                f.add(x0, __uint_as_float(q0.y));
-                f.add(x1, __uint_as_float(q1.y));
+            const uint2* e = nb.e + s;
+            uint32_t k = 0;
+            if constexpr (TWO) {
+                for (; k + 2 <= listed; k += 2, e += 2 * stride) {
+                    const uint2 q0 = __ldg(e), q1 = __ldg(e + stride);
+                    const float4 x0 = __ldg(ex + q0.x), x1 = __ldg(ex + q1.x);
+                    const float2 b0 = __ldg(exb + q0.x), b1 = __ldg(exb + q1.x);
+                    const float w0 = f.weight(x0, __uint_as_float(q0.y));
+                    f.add_w(make_float2(x0.x, x0.y), w0);
+                    g.add_w(b0, w0);
+                    const float w1 = f.weight(x1, __uint_as_float(q1.y));
+                    f.add_w(make_float2(x1.x, x1.y), w1);
+                    g.add_w(b1, w1);
+                }
+                if (k < listed) {
+                    const uint2 q = __ldg(e);
+                    const float4 x = __ldg(ex + q.x);
+                    const float w = f.weight(x, __uint_as_float(q.y));
+                    f.add_w(make_float2(x.x, x.y), w);
+                    g.add_w(__ldg(exb + q.x), w);
+                }
+            } else {
+                // two entries per iteration, the next two list entries loaded
+                // while this pair's neighbour records are in flight
+                uint2 p0 = listed > 0u ? __ldg(e) : make_uint2(uint32_t(s), 0u);
+                uint2 p1 = listed > 1u ? __ldg(e + stride) : p0;
+                for (; k + 2 <= listed; k += 2, e += 2 * stride) {
+                    const uint2 q0 = p0, q1 = p1;
+                    const float4 x0 = __ldg(ex + q0.x), x1 = __ldg(ex + q1.x);
+                    p0 = k + 2 < listed ? __ldg(e + 2 * stride) : q0;
+                    p1 = k + 3 < listed ? __ldg(e + 3 * stride) : q1;
+                    f.add(x0, __uint_as_float(q0.y));
+                    f.add(x1, __uint_as_float(q1.y));
+                }
+                if (k < listed) f.add(__ldg(ex + p0.x), __uint_as_float(p0.y));   // p0 = entry k
             }
-            if (k < listed) f.add(__ldg(ex + p0.x), __uint_as_float(p0.y));   // p0 = entry k
         }
     } else if constexpr (TWO) {
         const float4 sum = search_flux2<DIM>(uint32_t(s), stride, pos, rec, cell, start, v, ex, exb,

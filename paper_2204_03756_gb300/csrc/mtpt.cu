@@ -234,8 +234,8 @@ struct mtpt_handle {
     DevBuf<uint32_t> nb_j, nb_count;      // binary64 form neighbour lists
     DevBuf<double> nb_k;
     int nb_cap = 0;
-    DevBuf<uint2> nb32_e;                 // precision form neighbour lists {j, K}
-    int nb32_cap = 0;
+    DevBuf<uint2> nb32_e;                 // precision form: what pass 2 reads of pass 1's search (Nb32)
+    int nb32_cap = 0, nb32_pad = 0;       // its planes; mask words every row is filled up to
     DevBuf<uint32_t> adj_nb_j, adj_nb_count;     // adjoint (K, dK) lists
     DevBuf<double2> adj_nb_k;
     int adj_cap = 0;
@@ -592,10 +592,11 @@ int setup_grids(mtpt_handle* h) {
         h->any_advect |= h->params[k].advect != 0;
     }
     if (cell_base > int64_t(0xffffffffLL) - kScanTile) return MTPT_ERR_INVALID_ARG;
-    // binary64 neighbour-list slots: the expected neighbour count of the
-    // densest realisation (density x volume of the cutoff ball) plus four
-    // standard deviations of its Poisson spread plus 4, within [8, 64]
-    double expect = 0.0;
+    // neighbour-list slots: the expected neighbour count of the densest
+    // realisation (density x volume of the cutoff ball) plus four standard
+    // deviations of its Poisson spread plus 4, within [8, 64]; `window`: the
+    // expected candidates of one neighbour row (density x 2 psi x row height)
+    double expect = 0.0, window = 0.0;
     for (int k = 0; k < h->nreal; ++k) {
         const mtpt_params& p = h->reals[k].prm;
         double vol = 1.0;
@@ -603,11 +604,28 @@ int setup_grids(mtpt_handle* h) {
         const double ball = p.dim == 1 ? 2.0 : (p.dim == 2 ? M_PI : 4.0 * M_PI / 3.0);
         const double nk = double(h->reals[k].tiled ? h->reals[k].n_global : h->reals[k].n);
         expect = std::max(expect, nk / vol * ball * std::pow(h->reals[k].psi, double(p.dim)));
+        window = std::max(window, nk / vol * 2.0 * h->reals[k].psi *
+                                      (p.dim == 2 ? h->params[k].g.w[1] : 1.0));
     }
     const int list_cap =
         int(std::min(64.0, std::max(8.0, std::ceil(expect + 4.0 * std::sqrt(expect) + 4.0))));
     h->nb_cap = h->precision == MTPT_FP64 ? list_cap : 0;
-    h->nb32_cap = h->precision == MTPT_FP32W ? list_cap : 0;
+    // the precision form keeps lists in 3-d and mask words per row below it
+    // (32 candidates a word; five standard deviations, at most 8 words); rows
+    // that often need a second word are padded to the same number of words
+    // (pass 2 at density 10: 1.6 instead of 2.2 ms for 1e7 particles; at
+    // windows that seldom do, the padding only lengthens pass 2: 1.46 instead
+    // of 1.20 ms for the 512-realisation ensemble)
+    h->nb32_cap = h->nb32_pad = 0;
+    if (h->precision == MTPT_FP32W && h->dim == 3) {
+        h->nb32_cap = list_cap;
+    } else if (h->precision == MTPT_FP32W) {
+        const double longest = window + 5.0 * std::sqrt(window) + 4.0;
+        const int rows = h->dim == 2 ? 2 * h->params[0].g.reach + 1 : 1;
+        h->nb32_cap = rows * int(std::min(8.0, std::ceil(longest / 32.0)));
+        const double usual = window + 2.0 * std::sqrt(window);
+        if (rows > 1 && usual > 32.0) h->nb32_pad = int(std::min(8.0, std::ceil(usual / 32.0)));
+    }
     h->adj_cap = list_cap;
     h->n_cells = cell_base;
     h->n_corners = corner_base;
@@ -638,6 +656,9 @@ int build_corners(mtpt_handle* h, const RealParams* params_dev, const int* first
 // Payload-record chunks per particle of the record sort, tangents included
 // (the adjoint's), so one allocation serves every record sort.
 int64_t sort_rec_chunks(int dim) { return (2 + 2 * dim + 1) / 2; }
+
+// float4 per particle of the precision form's pair records (ExRec).
+int ex_vec(int dim) { return dim == 3 ? ExRec<3>::kVec : ExRec<2>::kVec; }
 
 // State and per-step buffers for n particles, grown all or nothing (a failed
 // growth leaves the handle's state and buffers as they were).  A growth
@@ -671,7 +692,7 @@ int ensure_capacity(mtpt_handle* h, int64_t n, int64_t keep = 0) {
         g.want(h->cell, size_t(cap));
         g.want(h->rec, size_t(cap));
         if (h->precision == MTPT_FP64) g.want(h->r64, size_t(cap));
-        else g.want(h->ex, size_t(cap));
+        else g.want(h->ex, size_t(ex_vec(d)) * size_t(cap));
     }
     if (!h->batch) g.want(h->sortrec, size_t(sort_rec_chunks(d)) * size_t(std::max(cap, h->cap)));
     g.want(h->status, 1);
@@ -743,9 +764,7 @@ int ensure_cells(mtpt_handle* h) {
         g.want(h->nb_k, slots);
         g.want(h->nb_count, size_t(h->cap));
     }
-    if (h->nb32_cap > 0) {
-        g.want(h->nb32_e, size_t(h->nb32_cap) * size_t(h->cap));
-    }
+    if (h->nb32_cap > 0) g.want(h->nb32_e, size_t(h->nb32_cap) * size_t(h->cap));
     if (g.grows()) drop_graph(h);
     MTPT_TRY(g.commit());
     // the scan's words for this grid's tiles
@@ -904,77 +923,59 @@ void reaction_rate(const mtpt_handle* h, double* kp, double* dt) {
     *dt = p.dt;
 }
 
-template <int DIM, class View, int BLOCK>
-int launch_pairs_f32(mtpt_handle* h, int n, int64_t stride, const double* pos_s, const View& vs,
-                     int o, int c, bool walk_ahead) {
-    const int blocks = int((n + BLOCK - 1) / BLOCK);
-    const NbList32 nb{h->nb32_e.p, h->nb32_e.p ? h->nb32_cap : 0};
-    {
-        MTPT_TIMED(h, "rowsum_f32");
-        k_rowsum_f32<DIM, View, BLOCK><<<blocks, BLOCK, 0, h->stream>>>(
-            n, stride, pos_s, h->rec.p, h->cell.p, h->start.p, vs, h->mass[o].p, h->ex.p,
-            h->pair_counter.p,
-            h->ntiles > 0 ? h->id[o].p : nullptr, nb);
-    }
-    if (h->reactive) {
-        // species B's split, then one pass 2 for both species and the reaction
-        // (a reaction runs on a plain handle only: batches refuse it)
-        k_split_mass<<<grid_for(n), kBlock, 0, h->stream>>>(n, h->massb[o].p, h->exb.p);
-        double kp, dt;
-        reaction_rate(h, &kp, &dt);
-        if constexpr (!View::kBatch) {
-            if (walk_ahead) {
-                // and the next step's walk into buffer c (see WalkAhead)
-                const WalkAhead wa{h->id[o].p, h->pos[c].p, h->id[c].p, h->key.p, h->count.p,
-                                   h->status.p, h->step_dev.p};
-                MTPT_TIMED(h, "exchange_walk_f32");
-                if (h->any_advect)
-                    k_exchange_f32<DIM, View, BLOCK, true, 2><<<blocks, BLOCK, 0, h->stream>>>(
-                        n, stride, pos_s, h->rec.p, h->cell.p, h->start.p, vs, h->ex.p,
-                        h->mass[o].p, h->mass[c].p, nb, h->exb.p, h->massb[o].p, h->massb[c].p,
-                        kp, dt, float(kp * dt), wa);
-                else
-                    k_exchange_f32<DIM, View, BLOCK, true, 1><<<blocks, BLOCK, 0, h->stream>>>(
-                        n, stride, pos_s, h->rec.p, h->cell.p, h->start.p, vs, h->ex.p,
-                        h->mass[o].p, h->mass[c].p, nb, h->exb.p, h->massb[o].p, h->massb[c].p,
-                        kp, dt, float(kp * dt), wa);
-                MTPT_CUDA_TRY(cudaGetLastError());
-                return MTPT_OK;
-            }
-        }
-        MTPT_TIMED(h, "exchange_f32");
-        k_exchange_f32<DIM, View, BLOCK, true><<<blocks, BLOCK, 0, h->stream>>>(
-            n, stride, pos_s, h->rec.p, h->cell.p, h->start.p, vs, h->ex.p, h->mass[o].p,
-            h->mass[c].p, nb, h->exb.p, h->massb[o].p, h->massb[c].p, kp, dt, float(kp * dt));
-        MTPT_CUDA_TRY(cudaGetLastError());
-        return MTPT_OK;
-    }
-    if (walk_ahead) {
-        // pass 2 plus the next step's walk into buffer c (see WalkAhead)
-        WalkAhead wa{h->id[o].p, h->pos[c].p, h->id[c].p, h->key.p, h->count.p,
-                     h->status.p, h->step_dev.p};
-        if (View::kBatch) {
-            wa.rid_in = h->rid[o].p;
-            wa.rid_next = h->rid[c].p;
-        }
-        MTPT_TIMED(h, "exchange_walk_f32");
-        if (h->any_advect)
-            k_exchange_f32<DIM, View, BLOCK, false, 2><<<blocks, BLOCK, 0, h->stream>>>(
-                n, stride, pos_s, h->rec.p, h->cell.p, h->start.p, vs, h->ex.p, h->mass[o].p,
-                h->mass[c].p, nb, nullptr, nullptr, nullptr, 0.0, 0.0, 0.0f, wa);
-        else
-            k_exchange_f32<DIM, View, BLOCK, false, 1><<<blocks, BLOCK, 0, h->stream>>>(
-                n, stride, pos_s, h->rec.p, h->cell.p, h->start.p, vs, h->ex.p, h->mass[o].p,
-                h->mass[c].p, nb, nullptr, nullptr, nullptr, 0.0, 0.0, 0.0f, wa);
-        MTPT_CUDA_TRY(cudaGetLastError());
-        return MTPT_OK;
-    }
-    MTPT_TIMED(h, "exchange_f32");
-    k_exchange_f32<DIM, View, BLOCK><<<blocks, BLOCK, 0, h->stream>>>(
-        n, stride, pos_s, h->rec.p, h->cell.p, h->start.p, vs, h->ex.p, h->mass[o].p,
-        h->mass[c].p, nb);
+// Pass 2 of the precision form: plain (walk 0), or with the next step's walk
+// into buffer c (1; 2 with advection: see WalkAhead); TWO: both species and
+// the reaction (plain handles only).
+template <int DIM, class View, bool TWO, int WALK>
+int launch_exchange_f32(mtpt_handle* h, const View& vs, int o, int c, const Nb32& nb,
+                        const WalkAhead& wa) {
+    double kp = 0.0, dt = 0.0;
+    if (TWO) reaction_rate(h, &kp, &dt);
+    MTPT_TIMED(h, WALK ? "exchange_walk_f32" : "exchange_f32");
+    const int n = int(h->n), block = h->pair_block;
+    k_exchange_f32<DIM, View, TWO, WALK><<<(n + block - 1) / block, block, 0, h->stream>>>(
+        n, h->cap, h->pos[o].p, h->rec.p, h->cell.p, h->start.p, vs, h->ex.p, h->mass[o].p,
+        h->mass[c].p, nb, TWO ? h->exb.p : nullptr, TWO ? h->massb[o].p : nullptr,
+        TWO ? h->massb[c].p : nullptr, kp, dt, float(kp * dt), wa);
     MTPT_CUDA_TRY(cudaGetLastError());
     return MTPT_OK;
+}
+
+template <int DIM, class View, bool TWO>
+int launch_exchange_f32(mtpt_handle* h, const View& vs, int o, int c, const Nb32& nb,
+                        bool walk_ahead) {
+    WalkAhead wa{};
+    if (!walk_ahead) return launch_exchange_f32<DIM, View, TWO, 0>(h, vs, o, c, nb, wa);
+    wa = {h->id[o].p, h->pos[c].p, h->id[c].p, h->key.p, h->count.p, h->status.p, h->step_dev.p};
+    if (View::kBatch) {
+        wa.rid_in = h->rid[o].p;
+        wa.rid_next = h->rid[c].p;
+    }
+    if (h->any_advect) return launch_exchange_f32<DIM, View, TWO, 2>(h, vs, o, c, nb, wa);
+    return launch_exchange_f32<DIM, View, TWO, 1>(h, vs, o, c, nb, wa);
+}
+
+template <int DIM, class View>
+int launch_pairs_f32(mtpt_handle* h, const View& vs, int o, int c, bool walk_ahead) {
+    const int n = int(h->n), block = h->pair_block;
+    const Nb32 nb{h->nb32_e.p, h->nb32_e.p ? h->nb32_cap : 0, h->nb32_pad};
+    {
+        MTPT_TIMED(h, "rowsum_f32");
+        k_rowsum_f32<DIM, View><<<(n + block - 1) / block, block, 0, h->stream>>>(
+            n, h->cap, h->pos[o].p, h->rec.p, h->cell.p, h->start.p, vs, h->mass[o].p, h->ex.p,
+            h->pair_counter.p, h->ntiles > 0 ? h->id[o].p : nullptr, nb);
+        MTPT_CUDA_TRY(cudaGetLastError());
+    }
+    if constexpr (!View::kBatch) {
+        if (h->reactive) {
+            // species B's split, then one pass 2 for both species and the
+            // reaction (batches refuse it)
+            k_split_mass<<<grid_for(n), kBlock, 0, h->stream>>>(n, h->massb[o].p, h->exb.p);
+            MTPT_CUDA_TRY(cudaGetLastError());
+            return launch_exchange_f32<DIM, View, true>(h, vs, o, c, nb, walk_ahead);
+        }
+    }
+    return launch_exchange_f32<DIM, View, false>(h, vs, o, c, nb, walk_ahead);
 }
 
 // Species B of a binary64 reaction run: its transfer with the weights of
@@ -1104,11 +1105,7 @@ int launch_step(mtpt_handle* h, int flags, bool walk_ahead) {
                 h->mass[o].p, h->mass[c].p, nb64);
         }
     } else {
-        if (h->pair_block == 128) {
-            MTPT_TRY((launch_pairs_f32<DIM, View, 128>(h, n, stride, pos_s, vs, o, c, walk_ahead)));
-        } else {
-            MTPT_TRY((launch_pairs_f32<DIM, View, 256>(h, n, stride, pos_s, vs, o, c, walk_ahead)));
-        }
+        MTPT_TRY((launch_pairs_f32<DIM, View>(h, vs, o, c, walk_ahead)));
     }
     MTPT_CUDA_TRY(cudaGetLastError());
     h->have_row_sums = true;
@@ -1297,7 +1294,8 @@ struct HostSnapshot {
     std::vector<RealHost> reals;
     std::vector<RealParams> params;
     int64_t n = 0, n_cells = 0, n_cells_pad = 0;
-    int n_corners = 0, nb_cap = 0, nb32_cap = 0, adj_cap = 0, cur = 0, pair_block = 256;
+    int n_corners = 0, nb_cap = 0, nb32_cap = 0, nb32_pad = 0, adj_cap = 0, cur = 0;
+    int pair_block = 256;
     bool any_transfer = false, any_walk = false, any_advect = false, fresh = false;
     bool have_row_sums = false, have_particles = false, adj_ready = false;
     uint64_t step = 0;
@@ -1311,7 +1309,7 @@ struct HostSnapshot {
             return false;
         }
         n = h->n; n_cells = h->n_cells; n_cells_pad = h->n_cells_pad;
-        n_corners = h->n_corners; nb_cap = h->nb_cap; nb32_cap = h->nb32_cap;
+        n_corners = h->n_corners; nb_cap = h->nb_cap; nb32_cap = h->nb32_cap; nb32_pad = h->nb32_pad;
         adj_cap = h->adj_cap; cur = h->cur; pair_block = h->pair_block;
         any_transfer = h->any_transfer; any_walk = h->any_walk; any_advect = h->any_advect;
         fresh = h->fresh; have_row_sums = h->have_row_sums; have_particles = h->have_particles;
@@ -1322,7 +1320,7 @@ struct HostSnapshot {
         std::copy(reals.begin(), reals.end(), h->reals);
         std::copy(params.begin(), params.end(), h->params);
         h->n = n; h->n_cells = n_cells; h->n_cells_pad = n_cells_pad;
-        h->n_corners = n_corners; h->nb_cap = nb_cap; h->nb32_cap = nb32_cap;
+        h->n_corners = n_corners; h->nb_cap = nb_cap; h->nb32_cap = nb32_cap; h->nb32_pad = nb32_pad;
         h->adj_cap = adj_cap; h->cur = cur; h->pair_block = pair_block;
         h->any_transfer = any_transfer; h->any_walk = any_walk; h->any_advect = any_advect;
         h->fresh = fresh; h->have_row_sums = have_row_sums; h->have_particles = have_particles;
@@ -2099,9 +2097,11 @@ int mtpt_get_row_sums(mtpt_handle* h, double* out) {
             if (h->batch) MTPT_TRY((launch_row_sums_out<BatchView, double>(h, h->r64.p, 1)));
             else MTPT_TRY((launch_row_sums_out<SingleView, double>(h, h->r64.p, 1)));
         } else {
-            const float* r = reinterpret_cast<const float*>(h->ex.p) + 2;   // ex[s].z
-            if (h->batch) MTPT_TRY((launch_row_sums_out<BatchView, float>(h, r, 4)));
-            else MTPT_TRY((launch_row_sums_out<SingleView, float>(h, r, 4)));
+            // r: .z of the record's last float4
+            const int step = 4 * ex_vec(h->dim);
+            const float* r = reinterpret_cast<const float*>(h->ex.p) + step - 2;
+            if (h->batch) MTPT_TRY((launch_row_sums_out<BatchView, float>(h, r, step)));
+            else MTPT_TRY((launch_row_sums_out<SingleView, float>(h, r, step)));
         }
     }
     return copy_out_host(h, 1, out);
@@ -2817,9 +2817,9 @@ struct NoallocHead {
 constexpr size_t kNoallocHeadBytes = (sizeof(NoallocHead) + 255) & ~size_t(255);
 
 // Worst case of the per-call pieces carved after the head, at n =
-// MTPT_NOALLOC_MAX_PARTICLES: 3-d binary32 form, 108 bytes per particle
-// (mass copy 8, sorted positions 24 and mass 8, two id arrays 8, key 4,
-// permutation 4, sort key 16, cell 4, rec 16, mass split and row sum 16); the
+// MTPT_NOALLOC_MAX_PARTICLES: 2-d binary32 form, 116 bytes per particle
+// (mass copy 8, sorted positions 16 and mass 8, two id arrays 8, key 4,
+// permutation 4, sort key 16, cell 4, rec 16, pair record 32; 3-d 108); the
 // cell grid capped at 4 n + 64 cells (setup_grid), so count and start hold at
 // most that many plus one cells padded to a scan tile, and the corner tables
 // at most the sum of the per-axis cell counts (<= their product + 2); each
@@ -2827,7 +2827,7 @@ constexpr size_t kNoallocHeadBytes = (sizeof(NoallocHead) + 255) & ~size_t(255);
 constexpr size_t kNoallocMaxCells = 4 * size_t(MTPT_NOALLOC_MAX_PARTICLES) + 64;
 constexpr size_t kNoallocMaxCellsPad = (kNoallocMaxCells + 1 + kScanTile - 1) / kScanTile * kScanTile;
 constexpr size_t kNoallocWorstBytes =
-    kNoallocHeadBytes + 108 * size_t(MTPT_NOALLOC_MAX_PARTICLES) +
+    kNoallocHeadBytes + 116 * size_t(MTPT_NOALLOC_MAX_PARTICLES) +
     2 * sizeof(uint32_t) * kNoallocMaxCellsPad +
     sizeof(unsigned long long) * (kNoallocMaxCellsPad / kScanTile + 1) +
     sizeof(float2) * (kNoallocMaxCells + 2) + 16 * 256;
@@ -2915,8 +2915,6 @@ extern "C" int mtpt_step_noalloc(const mtpt_params* params, int64_t n, uint64_t 
     h.reals[0].n = n;
     h.params[0].id_offset = 0;
     MTPT_TRY(setup_grids(&h));
-    h.nb_cap = 0;                        // no neighbour lists: pass 2 searches
-    h.nb32_cap = 0;
     const int d = h.dim;
     const size_t cells_pad = size_t(h.n_cells_pad);
 
@@ -2939,13 +2937,26 @@ extern "C" int mtpt_step_noalloc(const mtpt_params* params, int64_t n, uint64_t 
     if (h.precision == MTPT_FP64) {
         h.r64.p = cv.take<double>(size_t(n));
     } else {
-        h.ex.p = cv.take<float4>(size_t(n));
+        h.ex.p = cv.take<float4>(size_t(ex_vec(d)) * size_t(n));
     }
     h.corners.p = cv.take<float2>(size_t(std::max(h.n_corners, 1)));
     h.count.p = cv.take<uint32_t>(cells_pad);
     h.start.p = cv.take<uint32_t>(cells_pad);
     h.scan_state.p = cv.take<unsigned long long>(cells_pad / kScanTile + 1);   // + the ticket
     if (cv.overflow) return MTPT_ERR_TOO_LARGE;
+    // neighbour lists or masks in what is left, where they fit whole (the same
+    // sums either way: without them pass 2 searches, which took 73 instead of
+    // 68 us for the call at 20,011 particles in 2-d, precision form)
+    const size_t list_bytes = size_t(n) * (size_t(h.nb_cap) * 12 + 4 + size_t(h.nb32_cap) * 8);
+    if (cv.used + 4 * 256 + list_bytes > size_t(MTPT_NOALLOC_SCRATCH_BYTES)) {
+        h.nb_cap = h.nb32_cap = h.nb32_pad = 0;
+    } else if (h.nb_cap > 0) {
+        h.nb_k.p = cv.take<double>(size_t(h.nb_cap) * size_t(n));
+        h.nb_j.p = cv.take<uint32_t>(size_t(h.nb_cap) * size_t(n));
+        h.nb_count.p = cv.take<uint32_t>(size_t(n));
+    } else if (h.nb32_cap > 0) {
+        h.nb32_e.p = cv.take<uint2>(size_t(h.nb32_cap) * size_t(n));
+    }
 
     // The handle's buffer pairs: index 0 is the caller's state (positions are
     // walked in place; masses are read from a scratch copy), index 1 the
