@@ -1,77 +1,248 @@
-// expneg.cuh -- K = exp(-a d2) in binary64 for the pair kernel (Eq. 4 with
-// a = 1 / (2 h^2)).
+// expneg.cuh -- the binary64 pair terms of Eq. 4 in 64-bit integer arithmetic:
+// K = exp(-a d2) with a = 1 / (2 h^2), and the weight 2 K / (r_i + r_j).
 //
-// Table-driven method of P. T. P. Tang, "Table-driven implementation of the
+// GB300's binary64 unit takes a warp instruction per 16 clocks an SM, in which
+// the SM issues 64 others, so a 64 x 64-bit product from 32-bit multiply-adds
+// (about ten instructions) costs a sixth of a binary64 operation, and carries
+// more digits.
+//
+// Positions come as fixed-point images X = round(x 2^S) mod 2^64 (x_image),
+// with S such that the cutoff psi is in (2^61, 2^62]: the difference of two
+// neighbours' images, as int64, is their distance along the axis to 2^-61 psi,
+// wherever the box lies (the upper bits, equal up to a borrow, drop out).
+//
+// The exponential follows P. T. P. Tang, "Table-driven implementation of the
 // exponential function in IEEE floating-point arithmetic", ACM TOMS 15(2),
-// 1989, arranged so that only the parts that set the accuracy use binary64
-// (GB300 runs binary64 at about 1/70 of the binary32 rate):
-//
-//   t = a d2 = k ln2/256 + a r,   k = round(t 256 / ln 2),
-//   exp(-t) = 2^-(k >> 8) * 2^(-(k & 255)/256) * exp(-a r).
-//
-// * k comes from the binary32 head of d2 (bit truncation, no binary64
-//   instruction) times a 256 / ln 2 in binary32: it is within 0.53 of
-//   t 256 / ln 2 for t <= 400, so |a r| <= 0.53 ln2 / 256 < 1.44e-3.  Any k
-//   gives a correct reduction; only the bound on r depends on it.
-// * r = d2 - k c with c = ln 2 / (256 a) held as c_hi + c_lo, c_hi with 32
-//   significant bits so k c_hi is exact for k < 2^21; two fma.
-// * exp(-a r) is its Taylor series through (a r)^4 with a folded into the
-//   coefficients p_m = (-a)^m / m! (four fma on r; the first omitted term is
-//   below 5e-17 relative), so no binary64 multiply forms a r or t.
-// * 2^(-j/256) is a 256-entry host table; 2^-(k >> 8) goes into the exponent
-//   field with an integer subtraction.
-//
-// Cost: 7 binary64 operations (2 + 4 fma, 1 mul) and integer/binary32 work.
-// Valid for 0 <= a d2 <= 400.1 (lambda <= 20 with the band margin: the
-// result stays normal) and a <= 5e34: the binary32 scale and p_4 stay finite,
-// and a d2 whose head underflows binary32 (d2 < 2^-126, so k = 0) has
-// a d2 < 6e-4, inside the polynomial's range.  The host rejects parameters
-// outside.  Error: within 1.5 ulp of exp(-a d2) for the binary64 a and d2.
+// 1989, with every step a fixed-point one:
+//   T = a d2 256 log2(e) = k + f, k an integer, 0 <= f < 1,
+//   exp(-a d2) = 2^-(k >> 8) * 2^(-(k & 255) / 256) * exp(-c f), c = ln 2 / 256,
+// the table's 2^(-j / 256) to 63 bits, and exp(-c f) its Taylor series through
+// (c f)^5 (the first omitted term is below 2^-60).  K = m 2^-62 2^-q with the
+// error of m below 2^-55 relative (a tenth of a binary64 unit), against 1.5
+// units with binary64 operations.  Valid for a d2 <= 400.1 (lambda <= 20 with
+// the band margin); the host bounds lambda.
 #pragma once
+#include <cmath>
 #include <cstdint>
+
+#if defined(__CUDACC__)
+#define MTPT_HD __host__ __device__ __forceinline__
+#else
+#define MTPT_HD inline
+#endif
 
 namespace mtpt {
 
 constexpr int kExpTable = 256;
 
-struct ExpNegConsts {
-    float k_scale;      // a * 256 / ln 2 in binary32
-    double c_hi, c_lo;  // ln 2 / (256 a) = c_hi + c_lo
-    double p1, p2, p3, p4;   // (-a)^m / m!
+// Constants of one realisation's kernel (kernel_consts).
+struct KernelConsts {
+    int x_shift;        // S
+    int f_bits;         // fraction bits of T, in [33, 60]
+    uint64_t a_fix;     // T = high 64 bits of d2h a_fix, d2h = d2 2^(2 S - 64)
 };
 
-// Head of a binary64 x >= 0 with x < 2^128 as binary32, truncated (integer
-// operations only); 0 below 2^-126.
-__device__ __forceinline__ float head_f32(double x) {
-    const uint32_t whi = uint32_t(__double2hiint(x));
-    const uint32_t wlo = uint32_t(__double2loint(x));
-    const int e = int(whi >> 20);
-    const uint32_t bits = (uint32_t(e - 896) << 23) | ((whi & 0xfffffu) << 3) | (wlo >> 29);
-    return e < 897 ? 0.0f : __uint_as_float(bits);
+// Leading zeros of v != 0.
+MTPT_HD int clz64(uint64_t v) {
+#if defined(__CUDA_ARCH__)
+    return __clzll((long long)v);
+#else
+    return __builtin_clzll(v);
+#endif
+}
+MTPT_HD uint64_t bits_of(double x) {
+#if defined(__CUDA_ARCH__)
+    return uint64_t(__double_as_longlong(x));
+#else
+    uint64_t b;
+    __builtin_memcpy(&b, &x, 8);
+    return b;
+#endif
+}
+MTPT_HD double double_of(uint64_t b) {
+#if defined(__CUDA_ARCH__)
+    return __longlong_as_double((long long)b);
+#else
+    double x;
+    __builtin_memcpy(&x, &b, 8);
+    return x;
+#endif
 }
 
-// Exact binary64 image of 0 <= k < 2^31 from integer operations.
-__device__ __forceinline__ double small_uint_to_f64(uint32_t k) {
-    const int m = 31 - __clz(int(k | 1u));
-    const uint64_t mant = (uint64_t(k) << (52 - m)) & 0xfffffffffffffull;
-    const double v = __longlong_as_double((long long)((uint64_t(1023 + m) << 52) | mant));
-    return k == 0u ? 0.0 : v;
+// 32 x 32 -> 64-bit product, and the high 64 bits of 64 x 64 without the low
+// words' product (at most 3 below the exact ones).
+MTPT_HD uint64_t mul_wide(uint32_t a, uint32_t b) { return uint64_t(a) * b; }
+MTPT_HD uint64_t mul_hi(uint64_t a, uint64_t b) {
+    const uint32_t ah = uint32_t(a >> 32), al = uint32_t(a), bh = uint32_t(b >> 32), bl = uint32_t(b);
+    return mul_wide(ah, bh) + (mul_wide(ah, bl) >> 32) + (mul_wide(al, bh) >> 32);
+}
+MTPT_HD uint64_t square_hi(uint64_t a) {
+    const uint32_t ah = uint32_t(a >> 32), al = uint32_t(a);
+    return mul_wide(ah, ah) + (mul_wide(ah, al) >> 31);
+}
+MTPT_HD uint32_t mul_hi32(uint32_t a, uint32_t b) { return uint32_t(mul_wide(a, b) >> 32); }
+
+// The binary64 value w 2^(e - 63) of a 64-bit mantissa with its top bit set,
+// rounded to nearest (a carry runs into the exponent field), for a normal
+// result.
+MTPT_HD double from_mantissa(uint64_t w, int e) {
+    return double_of((uint64_t(e + 1022) << 52) + (w >> 11) + ((w >> 10) & 1u));
 }
 
-__device__ __forceinline__ double gauss_exp(double d2, const double* __restrict__ table,
-                                            const ExpNegConsts& c) {
-    const float yk = __fmaf_rn(head_f32(d2), c.k_scale, 12582912.0f);   // + 1.5 * 2^23
-    const uint32_t k = uint32_t(__float_as_int(yk) - 0x4b400000);
-    const double kd = small_uint_to_f64(k);
-    double r = __fma_rn(-kd, c.c_hi, d2);
-    r = __fma_rn(-kd, c.c_lo, r);
-    double p = __fma_rn(c.p4, r, c.p3);
-    p = __fma_rn(p, r, c.p2);
-    p = __fma_rn(p, r, c.p1);
-    p = __fma_rn(p, r, 1.0);
-    const double v = __dmul_rn(table[k & (kExpTable - 1)], p);
-    const long long scaled = __double_as_longlong(v) - (static_cast<long long>(k >> 8) << 52);
-    return __longlong_as_double(scaled);
+// X = round(x 2^S) mod 2^64 (0 for subnormals, infinities and NaN, which no
+// accepted pair has beyond its own zero).
+MTPT_HD uint64_t x_image(double x, int shift) {
+    const uint64_t b = bits_of(x);
+    const int e = int(b >> 52) & 0x7ff;
+    const int s = e - 1075 + shift;
+    const uint64_t m = (b & 0xfffffffffffffull) | 0x10000000000000ull;
+    uint64_t v;
+    if (s >= 0) v = s < 64 ? m << s : 0u;
+    else v = s > -55 ? (m + (1ull << (-s - 1))) >> -s : 0u;
+    if (e == 0 || e == 0x7ff) v = 0u;
+    return (b >> 63) ? 0u - v : v;
+}
+
+// |dx|^2 of one axis, in units of 2^(64 - 2 S).
+MTPT_HD uint64_t axis_square(uint64_t xi, uint64_t xj) {
+    const uint64_t d = xi - xj;
+    return square_hi((d >> 63) ? 0u - d : d);
+}
+
+// K = m 2^-62 2^-q, m in (2^60, 2^62].
+struct FixedK {
+    uint64_t m;
+    uint32_t q;
+    // K in units of 2^-62 (the row sums'), and as a binary64 value
+    MTPT_HD uint64_t unit() const { return q < 64u ? m >> q : 0u; }
+    MTPT_HD double value() const {
+        const int z = clz64(m);
+        return from_mantissa(m << z, 1 - z - int(q));
+    }
+};
+
+MTPT_HD FixedK gauss_fixed(uint64_t d2h, const uint64_t* __restrict__ table, const KernelConsts& c) {
+    const uint64_t t = mul_hi(d2h, c.a_fix);
+    const uint32_t k = uint32_t(t >> 32) >> (c.f_bits - 32);
+    const uint64_t f = t << (64 - c.f_bits);
+    const uint32_t fh = uint32_t(f >> 32);
+    // exp(-c f) = 1 - f (c1 - f (c2 - f (c3 - f (c4 - f c5)))), c_m = c^m / m!;
+    // c3..c5 in units of 2^-60, c1 and c2 of 2^-64
+    uint32_t p = 0x276557u - mul_hi32(fh, 0x576u);
+    p = 0xe35846b8u - mul_hi32(fh, p);
+    const uint64_t p2 = 0x3d7f7bff058bull - (mul_wide(fh, p) >> 28);
+    const uint64_t p1 = 0xb17217f7d1cf7aull - mul_hi(f, p2);
+    const uint64_t e = (1ull << 63) - (mul_hi(f, p1) >> 1);   // in units of 2^-63
+    return {mul_hi(table[k & (kExpTable - 1)], e), k >> 8};
+}
+
+// 2 K / (ra + rb) for a positive normal K and 1 <= ra, rb < 2^60: the quotient
+// of the 64-bit mantissas from a binary32 reciprocal seed, one Newton-Raphson
+// step in 32 bits and one residual correction of the quotient in 64 (error
+// below 2^-54), then rounded to binary64.
+MTPT_HD double weight_fixed(double K, double ra, double rb) {
+    const uint64_t kb = bits_of(K), ab = bits_of(ra), bb = bits_of(rb);
+    const uint64_t frac = 0xfffffffffffffull, one = 0x10000000000000ull;
+    const int ek = int(kb >> 52), ea = int(ab >> 52), eb = int(bb >> 52);
+    const int e = ea > eb ? ea : eb;
+    const uint64_t mk = ((kb & frac) | one) << 10;                      // [2^62, 2^63)
+    const uint64_t d = ((((ab & frac) | one) << 10) >> (e - ea)) +
+                       ((((bb & frac) | one) << 10) >> (e - eb));       // [2^62, 2^64)
+    const uint32_t dh = uint32_t(d >> 32), dl = uint32_t(d);
+    // y = 2^93 / d, in [2^29, 2^31]
+#if defined(__CUDA_ARCH__)
+    float s;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(s) : "f"(__uint2float_rn(dh)));
+    uint32_t y = __float2uint_rz(s * 2305843009213693952.0f);           // 2^61
+#else
+    uint32_t y = uint32_t(2305843009213693952.0f / float(dh));
+#endif
+    const int64_t e0 = int64_t((1ull << 61) - mul_wide(dh, y));         // |e0| < 2^40
+    y += uint32_t((int64_t(int32_t(e0 >> 19)) * int64_t(y)) >> 42);
+    const int64_t e1 = int64_t((1ull << 61) - mul_wide(dh, y) - (mul_wide(dl, y) >> 32));   // < 2^34
+    const uint64_t q0 = mul_wide(uint32_t(mk >> 32), y) + (mul_wide(uint32_t(mk), y) >> 32);
+    const uint64_t q = q0 + uint64_t((int64_t(int32_t(e1 >> 3)) * int64_t(q0 >> 31)) >> 27);
+    const int z = clz64(q);
+    // q = mk / d 2^61, so the weight is q 2^(ek - 1083 - (e - 1023))
+    return from_mantissa(q << z, ek - 1020 - (e - 1023) - z);
+}
+
+// Row sum 1 + sum K in units of 2^-62, exact in 96 bits.
+struct RowSum {
+    uint64_t lo = 1ull << 62;
+    uint32_t hi = 0;
+    MTPT_HD void add(uint64_t unit) {
+        lo += unit;
+        hi += lo < unit ? 1u : 0u;
+    }
+    MTPT_HD double value() const {
+        uint64_t w = lo;
+        int top = 63;               // bit that w's top bit stands for
+        if (hi) {
+            const int z = clz64(hi) - 32;
+            w = (uint64_t(hi) << (32 + z)) | (lo >> (32 - z));
+            top = 95 - z;
+        } else {
+            const int z = clz64(lo);
+            w <<= z;
+            top -= z;
+        }
+        return from_mantissa(w, top - 62);
+    }
+};
+
+// --- host: constants, in integers so that every machine gets the same ones ------
+
+// The kernel's constants for a = 1 / (2 h^2) and cutoff psi.
+inline KernelConsts kernel_consts(double a, double psi) {
+    KernelConsts c{0, 60, 0};
+    if (!(a > 0.0) || !(psi > 0.0)) return c;
+    int e = 0;
+    std::frexp(psi * (1.0 + 0x1p-20), &e);       // psi (1 + slack) < 2^e
+    c.x_shift = 62 - e;
+    // a 256 log2(e) 2^(f + 128 - 2 S), with the largest f <= 60 that keeps it
+    // below 2^64; log2(e) in units of 2^-63
+    int ea = 0;
+    const uint64_t am = uint64_t(std::ldexp(std::frexp(a, &ea), 53));
+    const unsigned __int128 prod = (unsigned __int128)am * 0xb8aa3b295c17f0bcull;
+    const int top = (prod >> 116) ? 117 : 116;   // its bits
+    const int drop = top - 64;
+    const uint64_t fix = uint64_t(prod >> drop);
+    // prod 2^(ea - 53 - 63 + 8 + f + 128 - 2 S) = fix 2^0
+    c.f_bits = -drop - (ea - 53 - 63 + 8 + 128 - 2 * c.x_shift);
+    c.a_fix = fix;
+    if (c.f_bits > 60) {
+        const int more = c.f_bits - 60;
+        c.a_fix = more < 64 ? fix >> more : 0u;
+        c.f_bits = 60;
+    }
+    return c;
+}
+
+// 2^(-j / 256) in units of 2^-63, j in [0, 256): products of the eight square
+// roots 2^(-1/2), 2^(-1/4), ..., each the integer root of the one before.
+inline void fill_exp_table(uint64_t* table) {
+    uint64_t root[8];
+    unsigned __int128 v = (unsigned __int128)1 << 127;   // 1/2 in units of 2^-128
+    for (int k = 0; k < 8; ++k) {
+        uint64_t r = 0;
+        for (int b = 63; b >= 0; --b) {
+            const uint64_t t = r | (1ull << b);
+            if ((unsigned __int128)t * t <= v) r = t;
+        }
+        root[k] = r;                                     // 2^(-1 / 2^(k + 1)), 2^-64
+        v = (unsigned __int128)r << 64;
+    }
+    for (int j = 0; j < kExpTable; ++j) {
+        // the product of the roots of j's bits, with 127 fraction bits
+        unsigned __int128 p = (unsigned __int128)1 << 127;
+        for (int k = 0; k < 8; ++k) {
+            if (!((j >> (7 - k)) & 1)) continue;
+            const uint64_t ph = uint64_t(p >> 64), pl = uint64_t(p);
+            p = (unsigned __int128)ph * root[k] + (((unsigned __int128)pl * root[k]) >> 64);
+        }
+        table[j] = uint64_t((p + ((unsigned __int128)1 << 63)) >> 64);
+    }
 }
 
 }  // namespace mtpt

@@ -93,7 +93,7 @@ struct PairParams {
     double a;          // 1 / (2 h^2)
     float a_log2e;     // a * log2(e) in binary32 (precision form)
     double beta;
-    ExpNegConsts ec;
+    KernelConsts kc;   // of the binary64 form's fixed-point kernel
 };
 
 // Everything one realisation's kernels need.  A single run passes one by
@@ -182,6 +182,16 @@ __device__ __forceinline__ double f32_to_f64(float f) {
     if (e == 0u || e == 255u) return double(f);
     const uint32_t m = mag & 0x7fffffu;
     return __hiloint2double(int(sign | ((e + 896u) << 20) | (m >> 3)), int(m << 29));
+}
+
+// Head of a binary64 x >= 0 with x < 2^128 as binary32, truncated (integer
+// operations only); 0 below 2^-126.
+__device__ __forceinline__ float head_f32(double x) {
+    const uint32_t whi = uint32_t(__double2hiint(x));
+    const uint32_t wlo = uint32_t(__double2loint(x));
+    const int e = int(whi >> 20);
+    const uint32_t bits = (uint32_t(e - 896) << 23) | ((whi & 0xfffffu) << 3) | (wlo >> 29);
+    return e < 897 ? 0.0f : __uint_as_float(bits);
 }
 
 // num / den for num >= 0 and 1 <= den < 2^127 with binary64 fma only: a
@@ -665,7 +675,7 @@ k_gather(int n, int64_t stride, const uint32_t* __restrict__ perm,
          const float2* __restrict__ corners, uint32_t* __restrict__ rid_out,
          const __grid_constant__ View v, const double* __restrict__ tan_in = nullptr,
          double* __restrict__ tan_out = nullptr, const double* __restrict__ mass_b_in = nullptr,
-         double* __restrict__ mass_b_out = nullptr) {
+         double* __restrict__ mass_b_out = nullptr, uint64_t* __restrict__ image_out = nullptr) {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     const uint32_t src = perm[s];
@@ -706,6 +716,7 @@ k_gather(int n, int64_t stride, const uint32_t* __restrict__ perm,
         const double x = xa[a];
         pos_out[a * stride + dst] = x;
         if constexpr (TANGENT) tan_out[a * stride + dst] = tan_in[a * stride + src];
+        if (image_out) image_out[a * stride + dst] = x_image(x, P.pp.kc.x_shift);
         if (P.transfer) {
             float xh, xlo;
             split_double(x, &xh, &xlo);
@@ -772,7 +783,8 @@ k_gather_rec(int n, int64_t stride, const double2* __restrict__ recs,
              double* __restrict__ pos_out, double* __restrict__ mass_out,
              uint32_t* __restrict__ cell_out, float4* __restrict__ rec_out,
              const float2* __restrict__ corners,
-             const __grid_constant__ SingleView v, double* __restrict__ tan_out) {
+             const __grid_constant__ SingleView v, double* __restrict__ tan_out,
+             uint64_t* __restrict__ image_out) {
     using R = SortRec<DIM, TANGENT>;
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
@@ -813,6 +825,7 @@ k_gather_rec(int n, int64_t stride, const double2* __restrict__ recs,
         const double x = lane[a == 0 ? 0 : 1 + a];
         pos_out[a * stride + dst] = x;
         if constexpr (TANGENT) tan_out[a * stride + dst] = lane[R::kTan + a];
+        if (image_out) image_out[a * stride + dst] = x_image(x, P.pp.kc.x_shift);
         if (P.transfer) {
             float xh, xlo;
             split_double(x, &xh, &xlo);
@@ -853,19 +866,17 @@ __device__ __forceinline__ double exact_d2(const double* __restrict__ pos, int64
     return d2;
 }
 
-// Squared distance for the kernel value (not for the pair test): one fma per
-// axis after the first.  Symmetric in (i, j) bit for bit (the differences
-// only change sign), and within 2 ulp of the exact square sum.
+// Kernel value of an accepted pair from the particles' fixed-point images (see
+// expneg.cuh).  Symmetric in (i, j) bit for bit.
 template <int DIM>
-__device__ __forceinline__ double kernel_d2(const double* __restrict__ pos, int64_t stride,
-                                            uint32_t i, uint32_t j) {
-    double d2 = 0.0;
+__device__ __forceinline__ FixedK pair_kernel(const uint64_t* __restrict__ image, int64_t stride,
+                                              uint32_t i, uint32_t j, const uint64_t* table,
+                                              const KernelConsts& kc) {
+    uint64_t d2h = 0;
 #pragma unroll
-    for (int a = 0; a < DIM; ++a) {
-        const double d = __dsub_rn(__ldg(pos + a * stride + i), __ldg(pos + a * stride + j));
-        d2 = (a == 0) ? __dmul_rn(d, d) : __fma_rn(d, d, d2);
-    }
-    return d2;
+    for (int a = 0; a < DIM; ++a)
+        d2h += axis_square(__ldg(image + a * stride + i), __ldg(image + a * stride + j));
+    return gauss_fixed(d2h, table, kc);
 }
 
 // Hardware square root approximation (relative error far below the
@@ -1109,13 +1120,11 @@ __device__ __forceinline__ uint32_t warp_exclusive_scan(uint32_t v, uint32_t* to
     return inc - v;
 }
 
-// Shared state of one block's warps.  V: type of the pair terms; D2: keep the
-// binary32 d2 of each entry (binary32 passes).
-template <int NW, class V, bool D2, int SEG = kSeg>
+// Shared state of one block's warps.  V: type of the pair terms.
+template <int NW, class V, int SEG = kSeg>
 struct SegShared {
     static constexpr int kCap = SEG;   // entries per lane
     uint32_t j[NW][SEG][32];           // lane-owned segments, entry k of lane l at [k][l]
-    float d2[NW][D2 ? SEG : 1][32];
     V v[NW][SEG * 32];                 // phase-B results, lane-major
     uint8_t owner[NW][SEG * 32];       // lane of each lane-major entry
     uint32_t off[NW][32];              // first lane-major entry of each lane
@@ -1160,18 +1169,18 @@ __device__ __forceinline__ uint32_t mask_word(uint32_t words, uint32_t neighbour
 }
 
 // Phases A-C for the calling warp (every lane of the warp must call it; lanes
-// with valid = false walk nothing).  eval(owner_s, j, d2f) returns the pair
-// term (d2f is 0 unless D2); add(term) is called by each lane for its own
-// entries in order.  Returns the lane's number of accepted neighbours j != s.
-template <int DIM, int NW, class V, bool D2, int SEG, class Eval, class Add>
+// with valid = false walk nothing).  eval(owner_s, j, keep) returns the pair
+// term and sets keep to what the list stores; add(term) is called by each lane
+// for its own entries in order.  Returns the lane's number of accepted
+// neighbours j != s.
+template <int DIM, int NW, class V, int SEG, class VL, class Eval, class Add>
 __device__ __forceinline__ uint32_t seg_pairs(bool valid, uint32_t s, int64_t stride,
                                               const float4* __restrict__ rec,
                                               const double* __restrict__ pos,
                                               const uint32_t* __restrict__ cell,
                                               const uint32_t* __restrict__ start,
-                                              const RealParams& P, SegShared<NW, V, D2, SEG>& S,
-                                              Eval&& eval, Add&& add,
-                                              NbList<V> store = NbList<V>{}) {
+                                              const RealParams& P, SegShared<NW, V, SEG>& S,
+                                              Eval&& eval, Add&& add, const NbList<VL>& store) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t warp_s0 = s - uint32_t(lane);
     uint32_t cnt = 0, done = 0;
@@ -1187,14 +1196,14 @@ __device__ __forceinline__ uint32_t seg_pairs(bool valid, uint32_t s, int64_t st
             const uint32_t o = S.owner[warp][e];
             const uint32_t k = e - S.off[warp][o];
             const uint32_t j = S.j[warp][k][o];
-            const V val = eval(warp_s0 + o, j, D2 ? S.d2[warp][D2 ? k : 0][o] : 0.0f);
-            S.v[warp][e] = val;
+            VL keep;
+            S.v[warp][e] = eval(warp_s0 + o, j, keep);
             if (store.cap > 0) {
                 const uint32_t slot = S.base[warp][o] + k;
                 if (slot < uint32_t(store.cap)) {
                     const int64_t at = int64_t(slot) * stride + (warp_s0 + o);
                     store.j[at] = j;
-                    store.k[at] = val;
+                    store.k[at] = keep;
                 }
             }
         }
@@ -1263,7 +1272,6 @@ __device__ __forceinline__ uint32_t seg_pairs(bool valid, uint32_t s, int64_t st
                         accept = exact_within<DIM>(pos, stride, s, j, pp.psi2);
                     if (accept && j != s) {
                         S.j[warp][cnt][lane] = j;
-                        if (D2) S.d2[warp][D2 ? cnt : 0][lane] = d2f;
                         ++cnt;
                     }
                     ++j;
@@ -1281,7 +1289,7 @@ __device__ __forceinline__ uint32_t seg_pairs(bool valid, uint32_t s, int64_t st
 template <int NW, class V, int SEG, class VL, class Eval, class Add>
 __device__ __forceinline__ void dense_listed(bool valid, uint32_t s, int64_t stride,
                                              uint32_t cnt, const NbList<VL>& nb,
-                                             SegShared<NW, V, false, SEG>& S, Eval&& eval,
+                                             SegShared<NW, V, SEG>& S, Eval&& eval,
                                              Add&& add) {
     constexpr uint32_t kChunk = SEG * 32;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1314,30 +1322,35 @@ __device__ __forceinline__ void dense_listed(bool valid, uint32_t s, int64_t str
 
 // Pass 1, binary64 form: r_s = 1 + sum_{j != s} exp(-a d2_sj) (the kernel
 // without its constant factor, which cancels in W; the self term is 1), and
-// the ordered pair count.
+// the ordered pair count.  The kernel values and their sum are fixed-point
+// (expneg.cuh): no binary64 instruction, and the sum is exact whatever its
+// order.  With binary64 operations the pass was bound by that unit (86 % busy):
+// 732 us at 4e6 particles in 2-d with 5.7 neighbours each, 420 now.
 template <int DIM, class View>
 __global__ void __launch_bounds__(kBlock)
-k_rowsum_f64(int n, int64_t stride, const double* __restrict__ pos, const float4* __restrict__ rec,
+k_rowsum_f64(int n, int64_t stride, const double* __restrict__ pos,
+             const uint64_t* __restrict__ image, const float4* __restrict__ rec,
              const uint32_t* __restrict__ cell, const uint32_t* __restrict__ start,
-             const double* __restrict__ exp_table, const __grid_constant__ View v,
+             const uint64_t* __restrict__ exp_table, const __grid_constant__ View v,
              double* __restrict__ r_out, unsigned long long* __restrict__ pair_counter,
              NbList64 nb, const uint32_t* __restrict__ ghost_id) {
-    __shared__ double table[kExpTable];
-    __shared__ SegShared<kWarpsPerBlock, double, false> seg;
+    __shared__ uint64_t table[kExpTable];
+    __shared__ SegShared<kWarpsPerBlock, uint64_t> seg;
     for (int t = threadIdx.x; t < kExpTable; t += blockDim.x) table[t] = exp_table[t];
     __syncthreads();
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     const RealParams& P = v.of_sorted(uint32_t(s < n ? s : 0));
     const bool valid = s < n && P.transfer;
-    double r = 1.0;
+    RowSum r;
     const uint32_t cnt = seg_pairs<DIM>(
         valid, uint32_t(s), stride, rec, pos, cell, start, P, seg,
-        [&](uint32_t so, uint32_t j, float) {
-            const RealParams& Po = v.of_sorted(so);
-            return gauss_exp(kernel_d2<DIM>(pos, stride, so, j), table, Po.pp.ec);
+        [&](uint32_t so, uint32_t j, double& K) {
+            const FixedK f = pair_kernel<DIM>(image, stride, so, j, table, v.of_sorted(so).pp.kc);
+            K = f.value();
+            return f.unit();
         },
-        [&](double K) { r = __dadd_rn(r, K); }, nb);
-    if (s < n) r_out[s] = r;
+        [&](uint64_t unit) { r.add(unit); }, nb);
+    if (s < n) r_out[s] = r.value();
     if (nb.cap > 0 && s < n) nb.count[s] = valid ? cnt : 0u;
     // with ghost_id (a tile), pairs are counted for the tile's own particles only
     const bool counted = valid && !(ghost_id && (ghost_id[s] & kGhostBit));
@@ -1381,15 +1394,18 @@ __device__ __forceinline__ void walk_ahead(const RealParams& P, int s, int64_t s
 }
 
 // Pass 2, binary64 form: M'_s = M_s + beta sum_j (M_j - M_s) 2 K_sj / (r_s + r_j).
+// The weight is formed in integers (expneg.cuh), which leaves the binary64
+// unit three operations a pair of nine: 543 -> 330 us (4e6 particles, 2-d).
 template <int DIM, class View, int WALK = 0>
 __global__ void __launch_bounds__(kBlock)
-k_exchange_f64(int n, int64_t stride, const double* __restrict__ pos, const float4* __restrict__ rec,
+k_exchange_f64(int n, int64_t stride, const double* __restrict__ pos,
+               const uint64_t* __restrict__ image, const float4* __restrict__ rec,
                const uint32_t* __restrict__ cell, const uint32_t* __restrict__ start,
-               const double* __restrict__ exp_table, const __grid_constant__ View v,
+               const uint64_t* __restrict__ exp_table, const __grid_constant__ View v,
                const double* __restrict__ r, const double* __restrict__ mass,
                double* __restrict__ mass_out, NbList64 nb, const WalkAhead wa = WalkAhead{}) {
-    __shared__ double table[kExpTable];
-    __shared__ SegShared<kWarpsPerBlock, double, false> seg;
+    __shared__ uint64_t table[kExpTable];
+    __shared__ SegShared<kWarpsPerBlock, double> seg;
     for (int t = threadIdx.x; t < kExpTable; t += blockDim.x) table[t] = exp_table[t];
     __syncthreads();
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1397,10 +1413,7 @@ k_exchange_f64(int n, int64_t stride, const double* __restrict__ pos, const floa
     const bool valid = s < n && P.transfer;
     double acc = 0.0;
     auto flux = [&](uint32_t so, uint32_t j, double K) {
-        // 2K by an exponent increment (K is a positive normal), so
-        // W = 2K / (r_s + r_j) rounds once
-        const double K2 = __longlong_as_double(__double_as_longlong(K) + (1LL << 52));
-        const double W = quot_pos(K2, __dadd_rn(__ldg(r + so), __ldg(r + j)));
+        const double W = weight_fixed(K, __ldg(r + so), __ldg(r + j));
         return __dmul_rn(__dsub_rn(__ldg(mass + j), __ldg(mass + so)), W);
     };
     const uint32_t listed = (nb.cap > 0 && valid) ? nb.count[s] : 0u;
@@ -1411,12 +1424,11 @@ k_exchange_f64(int n, int64_t stride, const double* __restrict__ pos, const floa
     } else {
         seg_pairs<DIM>(
             valid, uint32_t(s), stride, rec, pos, cell, start, P, seg,
-            [&](uint32_t so, uint32_t j, float) {
-                const RealParams& Po = v.of_sorted(so);
-                const double K = gauss_exp(kernel_d2<DIM>(pos, stride, so, j), table, Po.pp.ec);
+            [&](uint32_t so, uint32_t j, double& K) {
+                K = pair_kernel<DIM>(image, stride, so, j, table, v.of_sorted(so).pp.kc).value();
                 return flux(so, j, K);
             },
-            [&](double f) { acc = __dadd_rn(acc, f); });
+            [&](double f) { acc = __dadd_rn(acc, f); }, NbList64{});
     }
     if (s < n) mass_out[s] = valid ? __dadd_rn(mass[s], __dmul_rn(P.pp.beta, acc)) : mass[s];
     if constexpr (WALK > 0) {
@@ -2027,18 +2039,19 @@ k_emit_pairs(int n, int64_t stride, const double* __restrict__ pos, const float4
 // ---------------------------------------------------------------------------
 template <int DIM>
 __device__ __forceinline__ void pair_terms(const double* __restrict__ pos,
+                                           const uint64_t* __restrict__ image,
                                            const double* __restrict__ tan, int64_t stride,
                                            uint32_t s, uint32_t j, const RealParams& P,
-                                           const double* table, double* K, double* dK) {
+                                           const uint64_t* table, double* K, double* dK) {
     double d2 = 0.0, dot = 0.0;
 #pragma unroll
     for (int a = 0; a < DIM; ++a) {
         const double d = __dsub_rn(__ldg(pos + a * stride + s), __ldg(pos + a * stride + j));
         const double dt = __dsub_rn(__ldg(tan + a * stride + s), __ldg(tan + a * stride + j));
-        d2 = (a == 0) ? __dmul_rn(d, d) : __fma_rn(d, d, d2);   // as kernel_d2
+        d2 = (a == 0) ? __dmul_rn(d, d) : __fma_rn(d, d, d2);
         dot = __fma_rn(d, dt, dot);
     }
-    *K = gauss_exp(d2, table, P.pp.ec);
+    *K = pair_kernel<DIM>(image, stride, s, j, table, P.pp.kc).value();
     *dK = __dmul_rn(*K, __dmul_rn(__fma_rn(d2, P.inv_2D, -dot), P.inv_h2));
 }
 
@@ -2049,13 +2062,14 @@ constexpr int kAdjSeg = 8;
 // Pass A: r_s = sum_j K_sj (self included) and dr_s = sum_j dK_sj / dD.
 template <int DIM, class View>
 __global__ void __launch_bounds__(kBlock)
-k_adj_rowsum(int n, int64_t stride, const double* __restrict__ pos, const double* __restrict__ tan,
+k_adj_rowsum(int n, int64_t stride, const double* __restrict__ pos,
+             const uint64_t* __restrict__ image, const double* __restrict__ tan,
              const float4* __restrict__ rec, const uint32_t* __restrict__ cell,
-             const uint32_t* __restrict__ start, const double* __restrict__ exp_table,
+             const uint32_t* __restrict__ start, const uint64_t* __restrict__ exp_table,
              const __grid_constant__ View v, double* __restrict__ r_out,
              double* __restrict__ dr_out, NbList<double2> nb) {
-    __shared__ double table[kExpTable];
-    __shared__ SegShared<kWarpsPerBlock, double2, false, kAdjSeg> seg;
+    __shared__ uint64_t table[kExpTable];
+    __shared__ SegShared<kWarpsPerBlock, double2, kAdjSeg> seg;
     for (int t = threadIdx.x; t < kExpTable; t += blockDim.x) table[t] = exp_table[t];
     __syncthreads();
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
@@ -2064,10 +2078,9 @@ k_adj_rowsum(int n, int64_t stride, const double* __restrict__ pos, const double
     double r = 1.0, dr = 0.0;
     const uint32_t cnt = seg_pairs<DIM>(
         valid, uint32_t(s), stride, rec, pos, cell, start, P, seg,
-        [&](uint32_t so, uint32_t j, float) {
-            double K, dK;
-            pair_terms<DIM>(pos, tan, stride, so, j, v.of_sorted(so), table, &K, &dK);
-            return make_double2(K, dK);
+        [&](uint32_t so, uint32_t j, double2& keep) {
+            pair_terms<DIM>(pos, image, tan, stride, so, j, v.of_sorted(so), table, &keep.x, &keep.y);
+            return keep;
         },
         [&](double2 t) {
             r = __dadd_rn(r, t.x);
@@ -2086,14 +2099,14 @@ k_adj_rowsum(int n, int64_t stride, const double* __restrict__ pos, const double
 template <int DIM, class View>
 __global__ void __launch_bounds__(kBlock)
 k_adj_exchange(int n, int64_t stride, const double* __restrict__ pos,
-               const double* __restrict__ tan, const float4* __restrict__ rec,
+               const uint64_t* __restrict__ image, const double* __restrict__ tan, const float4* __restrict__ rec,
                const uint32_t* __restrict__ cell, const uint32_t* __restrict__ start,
-               const double* __restrict__ exp_table, const __grid_constant__ View v,
+               const uint64_t* __restrict__ exp_table, const __grid_constant__ View v,
                const double* __restrict__ r, const double* __restrict__ dr,
                const double* __restrict__ mass, const double* __restrict__ lam,
                double* __restrict__ lam_out, double* __restrict__ gD, NbList<double2> nb) {
-    __shared__ double table[kExpTable];
-    __shared__ SegShared<kWarpsPerBlock, double2, false, kAdjSeg> seg;
+    __shared__ uint64_t table[kExpTable];
+    __shared__ SegShared<kWarpsPerBlock, double2, kAdjSeg> seg;
     for (int t = threadIdx.x; t < kExpTable; t += blockDim.x) table[t] = exp_table[t];
     __syncthreads();
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
@@ -2122,12 +2135,12 @@ k_adj_exchange(int n, int64_t stride, const double* __restrict__ pos,
     } else {
         seg_pairs<DIM>(
             valid, uint32_t(s), stride, rec, pos, cell, start, P, seg,
-            [&](uint32_t so, uint32_t j, float) {
-                double K, dK;
-                pair_terms<DIM>(pos, tan, stride, so, j, v.of_sorted(so), table, &K, &dK);
-                return terms(so, j, K, dK);
+            [&](uint32_t so, uint32_t j, double2& keep) {
+                pair_terms<DIM>(pos, image, tan, stride, so, j, v.of_sorted(so), table, &keep.x,
+                                &keep.y);
+                return terms(so, j, keep.x, keep.y);
             },
-            add);
+            add, NbList<double2>{});
     }
     if (s < n) {
         const double ls = lam[s];

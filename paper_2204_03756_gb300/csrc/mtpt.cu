@@ -243,7 +243,8 @@ struct mtpt_handle {
     // staging copy of host-loaded input and its check tables
     DevBuf<double> stage, chk_box;
     DevBuf<uint32_t> chk_first, chk_flag;
-    DevBuf<double> exp_table;
+    DevBuf<uint64_t> exp_table;
+    DevBuf<uint64_t> image;           // fixed-point images of the positions (expneg.cuh), cell order
     // pipelined host I/O: two staging slots each way, per-slot check flags,
     // copy streams and the events that order them against `stream`
     DevBuf<double> in_slot[2], out_slot[2];
@@ -266,6 +267,7 @@ struct mtpt_handle {
     int64_t adj_steps = 0, adj_every = 0, adj_nck = 0;
     uint64_t adj_step0 = 0;
     bool adj_ready = false;
+    bool adjoint_sweep = false;       // the sorts feed the adjoint's pair passes
     DevBuf<double> dr64, lam_in, lam_s, lam_new, gD, partial, acc;
     // captured two-step graph (valid for `graph_cur`, `graph_flags` and the
     // mass buffer pair as it was: every step swaps the pair, so between loads
@@ -376,8 +378,8 @@ int validate_params(const mtpt_params* p) {
     if (!(p->beta > 0.0) || !std::isfinite(p->beta)) return MTPT_ERR_INVALID_ARG;
     if (!(p->lambda > 0.0 && p->lambda <= 20.0)) return MTPT_ERR_INVALID_ARG;
     // kernel variance h^2 = 2 (1 - kappa) D dt / beta: 0 (no transfer) or at
-    // least 1e-35, so a = 1 / (2 h^2) <= 5e34 stays within the range of the
-    // binary64 kernel exponential
+    // least 1e-35, so a = 1 / (2 h^2) <= 5e34 stays within binary32's range
+    // (the precision form's scale)
     const double h2 = 2.0 * (1.0 - p->kappa) * p->D * p->dt / p->beta;
     if (h2 > 0.0 && h2 < 1e-35) return MTPT_ERR_INVALID_ARG;
     for (int a = 0; a < p->dim; ++a) {
@@ -555,23 +557,7 @@ int setup_grid(RealHost& R, RealParams& P, int64_t cell_base, int corner_base, d
     pp.a = R.h2 > 0.0 ? 1.0 / (2.0 * R.h2) : 0.0;
     pp.a_log2e = float(pp.a * 1.4426950408889634);
     pp.beta = p.beta;
-    // Constants of the binary64 kernel exponential exp(-a d2) (reduction step
-    // c = ln 2 / (256 a), c_hi with 32 significant bits; Taylor coefficients
-    // (-a)^m / m!), formed in long double.
-    pp.ec = ExpNegConsts{};
-    if (pp.a > 0.0) {
-        const long double ln2 = std::log(2.0L), a = pp.a;
-        const long double c = ln2 / (256.0L * a);
-        int e = 0;
-        const double m = std::frexp(double(c), &e);
-        pp.ec.c_hi = std::ldexp(std::nearbyint(std::ldexp(m, 32)), e - 32);
-        pp.ec.c_lo = double(c - (long double)pp.ec.c_hi);
-        pp.ec.k_scale = float(256.0L * a / ln2);
-        pp.ec.p1 = double(-a);
-        pp.ec.p2 = double(a * a / 2.0L);
-        pp.ec.p3 = double(-a * a * a / 6.0L);
-        pp.ec.p4 = double(a * a * a * a / 24.0L);
-    }
+    pp.kc = kernel_consts(pp.a, R.psi);
     return MTPT_OK;
 }
 
@@ -633,13 +619,10 @@ int setup_grids(mtpt_handle* h) {
     return MTPT_OK;
 }
 
-double* exp_table_host() {
-    static double table[kExpTable];
+uint64_t* exp_table_host() {
+    static uint64_t table[kExpTable];
     static std::once_flag once;
-    std::call_once(once, []() {
-        for (int j = 0; j < kExpTable; ++j)
-            table[j] = double(exp2l(-static_cast<long double>(j) / static_cast<long double>(kExpTable)));
-    });
+    std::call_once(once, []() { fill_exp_table(table); });
     return table;
 }
 
@@ -691,8 +674,12 @@ int ensure_capacity(mtpt_handle* h, int64_t n, int64_t keep = 0) {
         g.want(h->sortkey, size_t(cap));
         g.want(h->cell, size_t(cap));
         g.want(h->rec, size_t(cap));
-        if (h->precision == MTPT_FP64) g.want(h->r64, size_t(cap));
-        else g.want(h->ex, size_t(ex_vec(d)) * size_t(cap));
+        if (h->precision == MTPT_FP64) {
+            g.want(h->r64, size_t(cap));
+            g.want(h->image, size_t(d) * size_t(cap));
+        } else {
+            g.want(h->ex, size_t(ex_vec(d)) * size_t(cap));
+        }
     }
     if (!h->batch) g.want(h->sortrec, size_t(sort_rec_chunks(d)) * size_t(std::max(cap, h->cap)));
     g.want(h->status, 1);
@@ -846,6 +833,12 @@ BatchView make_view<BatchView>(const mtpt_handle* h, int input_buf, int sorted_b
     return v;
 }
 
+// Where the gather writes the positions' fixed-point images: the passes that
+// form K in binary64 read them (the binary64 form, the adjoint sweep).
+uint64_t* image_buf(const mtpt_handle* h) {
+    return h->precision == MTPT_FP64 || h->adjoint_sweep ? h->image.p : nullptr;
+}
+
 // Counting-sort scatter of buffer c's particles into slots (index and sort
 // key), then the gather into buffer o in cell order (tangents too when on).
 template <int DIM, class View, bool TANGENT>
@@ -867,7 +860,8 @@ int launch_sort_t(mtpt_handle* h, int c, int o, const View& vin) {
     k_gather<DIM, View, TANGENT><<<blocks, kBlock, 0, h->stream>>>(
         n, stride, h->perm.p, h->sortkey.p, h->start.p, h->pos[c].p, h->mass[c].p, h->id[o].p,
         h->pos[o].p, h->mass[o].p, h->cell.p, h->rec.p, h->corners.p, rid_out, vin, tan_in,
-        tan_out, h->reactive ? h->massb[c].p : nullptr, h->reactive ? h->massb[o].p : nullptr);
+        tan_out, h->reactive ? h->massb[c].p : nullptr, h->reactive ? h->massb[o].p : nullptr,
+        image_buf(h));
     MTPT_CUDA_TRY(cudaGetLastError());
     return MTPT_OK;
 }
@@ -891,7 +885,7 @@ int launch_sort_rec(mtpt_handle* h, int c, int o, const SingleView& vin) {
     double* tan_out = TANGENT ? h->tan[o].p : nullptr;
     k_gather_rec<DIM, TANGENT><<<blocks, kBlock, 0, h->stream>>>(
         n, stride, h->sortrec.p, h->start.p, h->id[o].p, h->pos[o].p, h->mass[o].p, h->cell.p,
-        h->rec.p, h->corners.p, vin, tan_out);
+        h->rec.p, h->corners.p, vin, tan_out, image_buf(h));
     MTPT_CUDA_TRY(cudaGetLastError());
     return MTPT_OK;
 }
@@ -992,7 +986,7 @@ int launch_species_b(mtpt_handle* h, int n, int64_t stride, const double* pos_s,
     {
         MTPT_TIMED(h, "exchange_f64");
         k_exchange_f64<DIM, View><<<blocks, kBlock, 0, st>>>(
-            n, stride, pos_s, h->rec.p, h->cell.p, h->start.p, h->exp_table.p, vs, h->r64.p,
+            n, stride, pos_s, h->image.p, h->rec.p, h->cell.p, h->start.p, h->exp_table.p, vs, h->r64.p,
             h->massb[o].p, h->massb[c].p, NbList64{h->nb_j.p, h->nb_k.p, h->nb_count.p, h->nb_cap});
     }
     MTPT_CUDA_TRY(cudaGetLastError());
@@ -1076,7 +1070,7 @@ int launch_step(mtpt_handle* h, int flags, bool walk_ahead) {
         {
             MTPT_TIMED(h, "rowsum_f64");
             k_rowsum_f64<DIM, View><<<blocks, kBlock, 0, st>>>(
-                n, stride, pos_s, h->rec.p, h->cell.p, h->start.p, h->exp_table.p, vs, h->r64.p,
+                n, stride, pos_s, h->image.p, h->rec.p, h->cell.p, h->start.p, h->exp_table.p, vs, h->r64.p,
                 h->pair_counter.p, NbList64{h->nb_j.p, h->nb_k.p, h->nb_count.p, h->nb_cap},
                 h->ntiles > 0 ? h->id[o].p : nullptr);
         }
@@ -1092,16 +1086,16 @@ int launch_step(mtpt_handle* h, int flags, bool walk_ahead) {
             MTPT_TIMED(h, "exchange_walk_f64");
             if (h->any_advect)
                 k_exchange_f64<DIM, View, 2><<<blocks, kBlock, 0, st>>>(
-                    n, stride, pos_s, h->rec.p, h->cell.p, h->start.p, h->exp_table.p, vs,
+                    n, stride, pos_s, h->image.p, h->rec.p, h->cell.p, h->start.p, h->exp_table.p, vs,
                     h->r64.p, h->mass[o].p, h->mass[c].p, nb64, wa);
             else
                 k_exchange_f64<DIM, View, 1><<<blocks, kBlock, 0, st>>>(
-                    n, stride, pos_s, h->rec.p, h->cell.p, h->start.p, h->exp_table.p, vs,
+                    n, stride, pos_s, h->image.p, h->rec.p, h->cell.p, h->start.p, h->exp_table.p, vs,
                     h->r64.p, h->mass[o].p, h->mass[c].p, nb64, wa);
         } else {
             MTPT_TIMED(h, "exchange_f64");
             k_exchange_f64<DIM, View><<<blocks, kBlock, 0, st>>>(
-                n, stride, pos_s, h->rec.p, h->cell.p, h->start.p, h->exp_table.p, vs, h->r64.p,
+                n, stride, pos_s, h->image.p, h->rec.p, h->cell.p, h->start.p, h->exp_table.p, vs, h->r64.p,
                 h->mass[o].p, h->mass[c].p, nb64);
         }
     } else {
@@ -1381,7 +1375,7 @@ int load_particles_body(mtpt_handle* h, const int64_t* counts, const double* pos
     drop_graph(h);
     if (!h->exp_table.p) {
         MTPT_TRY(h->exp_table.ensure(kExpTable));
-        MTPT_CUDA_TRY(cudaMemcpyAsync(h->exp_table.p, exp_table_host(), kExpTable * sizeof(double),
+        MTPT_CUDA_TRY(cudaMemcpyAsync(h->exp_table.p, exp_table_host(), kExpTable * sizeof(uint64_t),
                                       cudaMemcpyHostToDevice, h->stream));
     }
     MTPT_TRY(upload_tables(h));
@@ -1762,15 +1756,18 @@ int launch_adjoint_step(mtpt_handle* h) {
             n, stride, h->pos[c].p, h->id[c].p, h->step_dev.p, h->any_walk ? 1 : 0, 1, v,
             h->key.p, h->count.p, h->status.p, h->tan[c].p);
     MTPT_TRY(launch_scan(h, st, true));
-    MTPT_TRY((launch_sort<DIM, SingleView>(h, c, o, v)));
+    h->adjoint_sweep = true;
+    const int sorted = launch_sort<DIM, SingleView>(h, c, o, v);
+    h->adjoint_sweep = false;
+    MTPT_TRY(sorted);
     k_take_by_id<<<blocks, kBlock, 0, st>>>(n, h->id[o].p, h->lam_in.p, h->lam_s.p);
     const NbList<double2> adj_nb{h->adj_nb_j.p, h->adj_nb_k.p, h->adj_nb_count.p,
                                  h->adj_nb_k.p ? h->adj_cap : 0};
     k_adj_rowsum<DIM, SingleView><<<blocks, kBlock, 0, st>>>(
-        n, stride, h->pos[o].p, h->tan[o].p, h->rec.p, h->cell.p, h->start.p, h->exp_table.p, v,
+        n, stride, h->pos[o].p, h->image.p, h->tan[o].p, h->rec.p, h->cell.p, h->start.p, h->exp_table.p, v,
         h->r64.p, h->dr64.p, adj_nb);
     k_adj_exchange<DIM, SingleView><<<blocks, kBlock, 0, st>>>(
-        n, stride, h->pos[o].p, h->tan[o].p, h->rec.p, h->cell.p, h->start.p, h->exp_table.p, v,
+        n, stride, h->pos[o].p, h->image.p, h->tan[o].p, h->rec.p, h->cell.p, h->start.p, h->exp_table.p, v,
         h->r64.p, h->dr64.p, h->mass[o].p, h->lam_s.p, h->lam_new.p, h->gD.p, adj_nb);
     k_put_by_id<<<blocks, kBlock, 0, st>>>(n, h->id[o].p, h->lam_new.p, h->lam_in.p);
     const int nparts = (n + kReduceThreads - 1) / kReduceThreads;
@@ -1808,6 +1805,7 @@ int mtpt_adjoint_forward(mtpt_handle* h, int64_t nsteps, int64_t checkpoint_ever
     for (auto* b : {&h->dr64, &h->lam_in, &h->lam_s, &h->lam_new, &h->gD})
         MTPT_TRY(b->ensure(cap));
     MTPT_TRY(h->r64.ensure(cap));
+    MTPT_TRY(h->image.ensure(size_t(h->dim) * cap));
     if (h->adj_cap > 0) {
         MTPT_TRY(h->adj_nb_j.ensure(size_t(h->adj_cap) * cap));
         MTPT_TRY(h->adj_nb_k.ensure(size_t(h->adj_cap) * cap));
@@ -1919,7 +1917,7 @@ int mtpt_destroy(mtpt_handle* h) {
     h->start.release(); h->scan_state.release(); h->rec.release(); h->corners.release();
     h->corner_first.release(); h->id_first.release(); h->params_dev.release();
     h->r64.release(); h->ex.release(); h->out_tmp.release();
-    h->exp_table.release();
+    h->exp_table.release(); h->image.release();
     h->stage.release(); h->chk_box.release(); h->chk_first.release(); h->chk_flag.release();
     h->status.release(); h->pair_counter.release(); h->step_dev.release();
     h->emit_counter.release(); h->emit_i.release(); h->emit_j.release();
@@ -2407,7 +2405,7 @@ int tile_install_t(mtpt_handle* h, int64_t n_keep, const double* keep, int64_t n
         if (!h->exp_table.p) {
             MTPT_TRY(h->exp_table.ensure(kExpTable));
             MTPT_CUDA_TRY(cudaMemcpyAsync(h->exp_table.p, exp_table_host(),
-                                          kExpTable * sizeof(double), cudaMemcpyHostToDevice,
+                                          kExpTable * sizeof(uint64_t), cudaMemcpyHostToDevice,
                                           h->stream));
         }
         MTPT_TRY(upload_tables(h));
@@ -2807,7 +2805,7 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[MTPT_NOALLOC_SC
 // exponential's table (written once per device at set-up) and the per-call
 // words that the init kernel writes.
 struct NoallocHead {
-    double exp_table[kExpTable];
+    uint64_t exp_table[kExpTable];
     RealParams params;
     int corner_first[2];
     uint32_t status;
@@ -2817,9 +2815,9 @@ struct NoallocHead {
 constexpr size_t kNoallocHeadBytes = (sizeof(NoallocHead) + 255) & ~size_t(255);
 
 // Worst case of the per-call pieces carved after the head, at n =
-// MTPT_NOALLOC_MAX_PARTICLES: 2-d binary32 form, 116 bytes per particle
-// (mass copy 8, sorted positions 16 and mass 8, two id arrays 8, key 4,
-// permutation 4, sort key 16, cell 4, rec 16, pair record 32; 3-d 108); the
+// MTPT_NOALLOC_MAX_PARTICLES: 3-d binary64 form, 124 bytes per particle (mass
+// copy 8, sorted positions 24 and mass 8, two id arrays 8, key 4, permutation
+// 4, sort key 16, cell 4, rec 16, row sum 8, images 24); the
 // cell grid capped at 4 n + 64 cells (setup_grid), so count and start hold at
 // most that many plus one cells padded to a scan tile, and the corner tables
 // at most the sum of the per-axis cell counts (<= their product + 2); each
@@ -2827,7 +2825,7 @@ constexpr size_t kNoallocHeadBytes = (sizeof(NoallocHead) + 255) & ~size_t(255);
 constexpr size_t kNoallocMaxCells = 4 * size_t(MTPT_NOALLOC_MAX_PARTICLES) + 64;
 constexpr size_t kNoallocMaxCellsPad = (kNoallocMaxCells + 1 + kScanTile - 1) / kScanTile * kScanTile;
 constexpr size_t kNoallocWorstBytes =
-    kNoallocHeadBytes + 116 * size_t(MTPT_NOALLOC_MAX_PARTICLES) +
+    kNoallocHeadBytes + 124 * size_t(MTPT_NOALLOC_MAX_PARTICLES) +
     2 * sizeof(uint32_t) * kNoallocMaxCellsPad +
     sizeof(unsigned long long) * (kNoallocMaxCellsPad / kScanTile + 1) +
     sizeof(float2) * (kNoallocMaxCells + 2) + 16 * 256;
@@ -2852,7 +2850,7 @@ int noalloc_scratch(void** out) {
         cudaError_t e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
         if (e == cudaSuccess)
             e = cudaMemcpy(static_cast<NoallocHead*>(p)->exp_table, exp_table_host(),
-                           kExpTable * sizeof(double), cudaMemcpyHostToDevice);
+                           kExpTable * sizeof(uint64_t), cudaMemcpyHostToDevice);
         if (e != cudaSuccess) (void)cudaGetLastError();
         g_noalloc_err[dev] = e;
         g_noalloc_addr[dev] = (e == cudaSuccess) ? p : nullptr;
@@ -2936,6 +2934,7 @@ extern "C" int mtpt_step_noalloc(const mtpt_params* params, int64_t n, uint64_t 
     h.rec.p = cv.take<float4>(size_t(n));
     if (h.precision == MTPT_FP64) {
         h.r64.p = cv.take<double>(size_t(n));
+        h.image.p = cv.take<uint64_t>(size_t(d) * size_t(n));
     } else {
         h.ex.p = cv.take<float4>(size_t(ex_vec(d)) * size_t(n));
     }

@@ -1,0 +1,103 @@
+"""The binary64 form's fixed-point pair terms (csrc/expneg.cuh), compiled for the
+host (the device code is the same source): the kernel exp(-d^2 / (2 h^2)) from
+position images, the weight 2K / (r_i + r_j) and the 96-bit row sum, against
+50-digit decimal arithmetic."""
+import ctypes
+import os
+import subprocess
+from decimal import Decimal, getcontext
+
+import numpy as np
+import pytest
+
+from paper_2204_03756_gb300 import build
+
+SRC = """
+#include "expneg.cuh"
+using namespace mtpt;
+extern "C" {
+double kernel(int dim, const double* x, const double* y, double a, double psi) {
+    uint64_t table[kExpTable];
+    fill_exp_table(table);
+    const KernelConsts c = kernel_consts(a, psi);
+    uint64_t d2h = 0;
+    for (int k = 0; k < dim; ++k) d2h += axis_square(x_image(x[k], c.x_shift), x_image(y[k], c.x_shift));
+    return gauss_fixed(d2h, table, c).value();
+}
+double weight(double K, double ra, double rb) { return weight_fixed(K, ra, rb); }
+double row_sum(int n, const unsigned long long* unit) {
+    RowSum r;
+    for (int k = 0; k < n; ++k) r.add(unit[k]);
+    return r.value();
+}
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    d = tmp_path_factory.mktemp("terms")
+    src, out = d / "terms.cpp", d / "terms.so"
+    src.write_text(SRC)
+    subprocess.run(["g++", "-O2", "-std=gnu++17", "-shared", "-fPIC", "-I", build.SRC_DIR,
+                    "-o", str(out), str(src)], check=True)
+    so = ctypes.CDLL(os.fspath(out))
+    dp = ctypes.POINTER(ctypes.c_double)
+    so.kernel.argtypes = [ctypes.c_int, dp, dp, ctypes.c_double, ctypes.c_double]
+    so.weight.argtypes = [ctypes.c_double] * 3
+    so.row_sum.argtypes = [ctypes.c_int, ctypes.POINTER(ctypes.c_ulonglong)]
+    so.kernel.restype = so.weight.restype = so.row_sum.restype = ctypes.c_double
+    getcontext().prec = 50
+    return so
+
+
+def _ptr(a):
+    return a.ctypes.data_as(ctypes.POINTER(ctypes.c_double))
+
+
+@pytest.mark.parametrize("lam,h2,side", [(3.0, 0.1, 100.0), (3.0, 0.1, 2000.0), (3.0, 1e-30, 1e-9),
+                                         (3.0, 7.0, 1e15), (0.001, 0.1, 10.0), (20.0, 0.05, 126.0)])
+@pytest.mark.parametrize("dim", [1, 2, 3])
+def test_kernel_against_decimal(lib, lam, h2, side, dim):
+    rng = np.random.default_rng(dim)
+    psi, a = lam * np.sqrt(2.0 * h2), 1.0 / (2.0 * h2)
+    # |T's error| <= 3 + 6 d units of 2^-60 (psi^2) in d2 and the constant's
+    # 2^-63: a relative error of K of lam^2 (3 + 6 d) 2^-60 at most, plus the
+    # rounding of T (4 units of at most lam^2 2^-57) and of K itself (2^-53)
+    bound = 2.0 ** -53 + lam ** 2 * ((3 + 6 * dim) * 2.0 ** -60 + 4 * 2.0 ** -57) + 2.0 ** -58
+    for it in range(300):
+        x = rng.uniform(-side, side, dim) * (1e-3 if it % 3 == 0 else 1.0)
+        y = x + rng.uniform(-1.0, 1.0, dim) * psi / np.sqrt(dim) * (it % 7 != 0)
+        d2 = sum((Decimal(float(u)) - Decimal(float(v))) ** 2 for u, v in zip(x, y))
+        if d2 > Decimal(psi) ** 2:
+            continue
+        want = (-Decimal(a) * d2).exp()
+        got = lib.kernel(dim, _ptr(x), _ptr(y), a, psi)
+        assert lib.kernel(dim, _ptr(y), _ptr(x), a, psi) == got
+        assert abs(Decimal(got) - want) <= Decimal(bound) * want
+        if d2 == 0:
+            assert got == 1.0
+
+
+def test_weight_against_decimal(lib):
+    rng = np.random.default_rng(4)
+    for it in range(4000):
+        K = float(np.exp(-rng.uniform(0.0, 9.0 if it % 2 else 400.0)))
+        ra = 1.0 + (rng.uniform(0.0, 60.0) if it % 5 else 0.0)
+        rb = 1.0 + rng.uniform(0.0, 2.0 ** 30 if it % 3 == 0 else 2.0)
+        want = 2 * Decimal(K) / (Decimal(ra) + Decimal(rb))
+        got = lib.weight(K, ra, rb)
+        assert got == lib.weight(K, rb, ra)
+        assert abs(Decimal(got) - want) <= Decimal(2.0 ** -53 + 2.0 ** -54) * want
+    assert lib.weight(1.0, 1.0, 1.0) == 1.0
+
+
+@pytest.mark.parametrize("n", [0, 1, 2, 3, 4, 7, 8, 63, 64, 1000, 5000])
+def test_row_sum_is_exact(lib, n):
+    rng = np.random.default_rng(n)
+    unit = rng.integers(0, 2 ** 62, n, dtype=np.uint64, endpoint=True)
+    if n > 2:
+        unit[:2] = 2 ** 62
+    want = Decimal(1) + sum((Decimal(int(u)) for u in unit), Decimal(0)) / Decimal(2) ** 62
+    got = lib.row_sum(n, unit.ctypes.data_as(ctypes.POINTER(ctypes.c_ulonglong)))
+    assert abs(Decimal(got) - want) <= Decimal(2.0 ** -53) * want
