@@ -1,10 +1,11 @@
 // expneg.cuh -- the binary64 pair terms of Eq. 4 in 64-bit integer arithmetic:
-// K = exp(-a d2) with a = 1 / (2 h^2), and the weight 2 K / (r_i + r_j).
+// K = exp(-a d2) with a = 1 / (2 h^2), the row sum of K, the weight
+// 2 K / (r_i + r_j) and the sum of the fluxes.
 //
-// GB300's binary64 unit takes a warp instruction per 16 clocks an SM, in which
-// the SM issues 64 others, so a 64 x 64-bit product from 32-bit multiply-adds
-// (about ten instructions) costs a sixth of a binary64 operation, and carries
-// more digits.
+// GB300's binary64 unit takes a warp instruction per 16 to 20 clocks an SM, in
+// which the SM issues 64 others, so a 64 x 64-bit product from 32-bit
+// multiply-adds (about ten instructions) costs a sixth of a binary64
+// operation, and carries more digits.
 //
 // Positions come as fixed-point images X = round(x 2^S) mod 2^64 (x_image),
 // with S such that the cutoff psi is in (2^61, 2^62]: the difference of two
@@ -13,14 +14,16 @@
 //
 // The exponential follows P. T. P. Tang, "Table-driven implementation of the
 // exponential function in IEEE floating-point arithmetic", ACM TOMS 15(2),
-// 1989, with every step a fixed-point one:
+// 1989, in fixed point but for its last multiplication:
 //   T = a d2 256 log2(e) = k + f, k an integer, 0 <= f < 1,
 //   exp(-a d2) = 2^-(k >> 8) * 2^(-(k & 255) / 256) * exp(-c f), c = ln 2 / 256,
-// the table's 2^(-j / 256) to 63 bits, and exp(-c f) its Taylor series through
-// (c f)^5 (the first omitted term is below 2^-60).  K = m 2^-62 2^-q with the
-// error of m below 2^-55 relative (a tenth of a binary64 unit), against 1.5
-// units with binary64 operations.  Valid for a d2 <= 400.1 (lambda <= 20 with
-// the band margin); the host bounds lambda.
+// exp(-c f) its Taylor series through (c f)^5 (the first omitted term is below
+// 2^-60).  That multiplication by the table's 2^(-j / 256) is a binary64 one:
+// it rounds and normalises K, which took 29 integer instructions, and the
+// binary64 unit has the time (one operation a pair).  The error of K is three
+// roundings (2^-53 each) and T's; with binary64 operations throughout it was 14
+// such units at lambda = 3, from the rounding of d2.  Valid for a d2 <= 400.1
+// (lambda <= 20 with the band margin); the host bounds lambda.
 #pragma once
 #include <cmath>
 #include <cstdint>
@@ -109,19 +112,8 @@ MTPT_HD uint64_t axis_square(uint64_t xi, uint64_t xj) {
     return square_hi((d >> 63) ? 0u - d : d);
 }
 
-// K = m 2^-62 2^-q, m in (2^60, 2^62].
-struct FixedK {
-    uint64_t m;
-    uint32_t q;
-    // K in units of 2^-62 (the row sums'), and as a binary64 value
-    MTPT_HD uint64_t unit() const { return q < 64u ? m >> q : 0u; }
-    MTPT_HD double value() const {
-        const int z = clz64(m);
-        return from_mantissa(m << z, 1 - z - int(q));
-    }
-};
-
-MTPT_HD FixedK gauss_fixed(uint64_t d2h, const uint64_t* __restrict__ table, const KernelConsts& c) {
+// exp(-a d2) from d2h = d2 2^(2 S - 64).
+MTPT_HD double gauss_fixed(uint64_t d2h, const double* __restrict__ table, const KernelConsts& c) {
     const uint64_t t = mul_hi(d2h, c.a_fix);
     const uint32_t k = uint32_t(t >> 32) >> (c.f_bits - 32);
     const uint64_t f = t << (64 - c.f_bits);
@@ -132,15 +124,30 @@ MTPT_HD FixedK gauss_fixed(uint64_t d2h, const uint64_t* __restrict__ table, con
     p = 0xe35846b8u - mul_hi32(fh, p);
     const uint64_t p2 = 0x3d7f7bff058bull - (mul_wide(fh, p) >> 28);
     const uint64_t p1 = 0xb17217f7d1cf7aull - mul_hi(f, p2);
-    const uint64_t e = (1ull << 63) - (mul_hi(f, p1) >> 1);   // in units of 2^-63
-    return {mul_hi(table[k & (kExpTable - 1)], e), k >> 8};
+    // 1 - f p1 in (0.997, 1] as a binary64 value: below 1, 52 bits under the
+    // leading one of 2^-1; at 1 the sum carries into the exponent
+    const uint64_t below = mul_hi(f, p1) >> 11;
+    const double e = double_of(0x3ff0000000000000ull - below);
+    const double v = table[k & (kExpTable - 1)] * e;
+    return double_of(bits_of(v) - (uint64_t(k >> 8) << 52));
 }
 
-// 2 K / (ra + rb) for a positive normal K and 1 <= ra, rb < 2^60: the quotient
-// of the 64-bit mantissas from a binary32 reciprocal seed, one Newton-Raphson
-// step in 32 bits and one residual correction of the quotient in 64 (error
-// below 2^-54), then rounded to binary64.
-MTPT_HD double weight_fixed(double K, double ra, double rb) {
+// K <= 1 in units of 2^-62 (the row sums').
+MTPT_HD uint64_t unit_of(double K) {
+    const uint64_t b = bits_of(K);
+    const uint32_t n = 1023u - uint32_t(b >> 52);
+    return (((b & 0xfffffffffffffull) | 0x10000000000000ull) << 10) >> (n < 63u ? n : 63u);
+}
+
+// The weight 2 K / (ra + rb) for a positive normal K and 1 <= ra, rb < 2^60, as
+// q 2^x, q in [2^59, 2^62): the quotient of the 64-bit mantissas from a
+// binary32 reciprocal seed, one Newton-Raphson step in 32 bits and one
+// residual correction of the quotient in 64 (relative error below 2^-54).
+struct FixedWeight {
+    uint64_t q;
+    int x;
+};
+MTPT_HD FixedWeight weight_fixed(double K, double ra, double rb) {
     const uint64_t kb = bits_of(K), ab = bits_of(ra), bb = bits_of(rb);
     const uint64_t frac = 0xfffffffffffffull, one = 0x10000000000000ull;
     const int ek = int(kb >> 52), ea = int(ab >> 52), eb = int(bb >> 52);
@@ -162,10 +169,54 @@ MTPT_HD double weight_fixed(double K, double ra, double rb) {
     const int64_t e1 = int64_t((1ull << 61) - mul_wide(dh, y) - (mul_wide(dl, y) >> 32));   // < 2^34
     const uint64_t q0 = mul_wide(uint32_t(mk >> 32), y) + (mul_wide(uint32_t(mk), y) >> 32);
     const uint64_t q = q0 + uint64_t((int64_t(int32_t(e1 >> 3)) * int64_t(q0 >> 31)) >> 27);
-    const int z = clz64(q);
-    // q = mk / d 2^61, so the weight is q 2^(ek - 1083 - (e - 1023))
-    return from_mantissa(q << z, ek - 1020 - (e - 1023) - z);
+    // q = mk / d 2^61; K = mk 2^(ek - 1085), ra + rb = d 2^(e - 1085)
+    return {q, ek - e - 60};
 }
+
+// A particle's flux sum, sum W dm over its neighbours with dm a difference of
+// masses: 64-bit integers against the largest exponent so far (each term keeps
+// 54 bits or more, and the sum five bits above the terms, or more when it
+// needs them).  A term changes sign exactly when dm does.  Differences that
+// are not finite make the sum what binary64 additions would.
+struct FluxSum64 {
+    int64_t acc = 0;
+    int x = -100000;             // the sum is acc 2^x
+    double special = 0.0;
+    MTPT_HD void add(double dm, const FixedWeight& w) {
+        const uint64_t b = bits_of(dm);
+        const int e = int(b >> 52) & 0x7ff;
+        if (e == 0x7ff) {
+            special += dm;
+            return;
+        }
+        const uint64_t m = (b & 0xfffffffffffffull) | (e ? 0x10000000000000ull : 0u);
+        // dm = m 2^(e - 1075), subnormals with e = 1
+        int64_t g = int64_t(mul_hi(m << 10, w.q) >> 3);                 // below 2^58
+        int y = (e ? e : 1) - 1075 - 10 + 64 + 3 + w.x;
+        g = (b >> 63) ? -g : g;
+        const int up = y - x;
+        if (up > 0) {
+            acc >>= up < 63 ? up : 63;
+            x = y;
+        } else {
+            g >>= up > -63 ? -up : 63;
+        }
+        acc += g;
+        if (uint64_t(acc + (1ll << 61)) >> 62) {                        // |acc| >= 2^61
+            acc >>= 4;
+            x += 4;
+        }
+    }
+    MTPT_HD double value() const {
+        if (!(special == 0.0)) return special;
+        if (acc == 0) return 0.0;
+        const uint64_t mag = acc < 0 ? 0u - uint64_t(acc) : uint64_t(acc);
+        const int z = clz64(mag), e = 63 - z + x;
+        const double v = (e > -1000 && e < 1000) ? from_mantissa(mag << z, e)
+                                                 : scalbn(from_mantissa(mag << z, 0), e);
+        return acc < 0 ? -v : v;
+    }
+};
 
 // Row sum 1 + sum K in units of 2^-62, exact in 96 bits.
 struct RowSum {
@@ -219,9 +270,9 @@ inline KernelConsts kernel_consts(double a, double psi) {
     return c;
 }
 
-// 2^(-j / 256) in units of 2^-63, j in [0, 256): products of the eight square
+// 2^(-j / 256), j in [0, 256), from 63-bit integers: products of the eight square
 // roots 2^(-1/2), 2^(-1/4), ..., each the integer root of the one before.
-inline void fill_exp_table(uint64_t* table) {
+inline void fill_exp_table(double* table) {
     uint64_t root[8];
     unsigned __int128 v = (unsigned __int128)1 << 127;   // 1/2 in units of 2^-128
     for (int k = 0; k < 8; ++k) {
@@ -241,7 +292,7 @@ inline void fill_exp_table(uint64_t* table) {
             const uint64_t ph = uint64_t(p >> 64), pl = uint64_t(p);
             p = (unsigned __int128)ph * root[k] + (((unsigned __int128)pl * root[k]) >> 64);
         }
-        table[j] = uint64_t((p + ((unsigned __int128)1 << 63)) >> 64);
+        table[j] = std::ldexp(double(uint64_t((p + ((unsigned __int128)1 << 63)) >> 64)), -63);
     }
 }
 

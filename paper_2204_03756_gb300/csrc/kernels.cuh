@@ -45,7 +45,7 @@ enum : uint32_t {
     kChkSlot = 2u,       // scatter: counting-sort slot inside [0, n)
     kChkGather = 4u,     // gather: source and in-cell rank inside the cell's range
     kChkRow = 8u,        // pair search: neighbour row inside the realisation's cells
-    kChkSegment = 16u,   // segment engine: entries within the segments' capacity
+    kChkSegment = 16u,   // dense pair passes: a particle's words hold all its neighbours
     kChkOutput = 32u,    // outputs: particle id inside [0, n)
 };
 #ifdef MTPT_CHECKED
@@ -869,8 +869,8 @@ __device__ __forceinline__ double exact_d2(const double* __restrict__ pos, int64
 // Kernel value of an accepted pair from the particles' fixed-point images (see
 // expneg.cuh).  Symmetric in (i, j) bit for bit.
 template <int DIM>
-__device__ __forceinline__ FixedK pair_kernel(const uint64_t* __restrict__ image, int64_t stride,
-                                              uint32_t i, uint32_t j, const uint64_t* table,
+__device__ __forceinline__ double pair_kernel(const uint64_t* __restrict__ image, int64_t stride,
+                                              uint32_t i, uint32_t j, const double* table,
                                               const KernelConsts& kc) {
     uint64_t d2h = 0;
 #pragma unroll
@@ -935,7 +935,7 @@ __device__ __forceinline__ float row_gap(int d, float off, float w, float eps) {
 // neighbour, so the accepted set is the exact binary64 one as before.
 // row(j0, j3, rx, sy, sz) is called for every row that can hold a neighbour.
 template <int DIM, class Row>
-__device__ __forceinline__ void for_each_row(uint32_t cell, const float4& me,
+__device__ __forceinline__ void for_each_row(uint32_t cell, const float4 me,
                                              const float4* __restrict__ rec,
                                              const uint32_t* __restrict__ start,
                                              const RealParams& P, Row&& row) {
@@ -1087,26 +1087,190 @@ __device__ __forceinline__ void add_pair_count(uint32_t cnt, unsigned long long*
 }
 
 // ---------------------------------------------------------------------------
-// Binary64 pair passes.  A thread per particle walks its candidate windows,
-// whose lengths differ from lane to lane, so work done inside that loop runs
-// at a fraction of the warp's lanes, and GB300's binary64 unit charges a warp
-// instruction the same whether 32 lanes or 3 are active.  These passes
-// therefore split the work per warp:
-//  (A) each lane walks its windows once with the binary32 prefilter and
-//      appends every accepted neighbour j != s (and its binary32 d2) to its
-//      own kSeg-entry segment in shared memory;
-//  (B) when a lane's segment is full (checked at window ends) or the walk is
-//      over, the warp evaluates the pair terms of all segments with all 32
-//      lanes, one entry per lane, in lane-major order;
-//  (C) each lane then adds its own results in the order it found them.
-// Every sum therefore runs in candidate order and repeats bit for bit, the
-// divergent loop holds only the prefilter, and the binary64 arithmetic runs
-// at full width.  (The binary32 passes below keep the pair arithmetic inside
-// the candidate loop: there the segment traffic costs more than the
-// divergence it removes, measured at 1.5x their time.)
+// What pass 1 keeps of its search for pass 2: accept masks.  A word {base,
+// bits} holds 32 consecutive candidates of one neighbour row: bit k is set when
+// candidate base + k is an accepted neighbour j != s.  Plane w (entry w * stride
+// + s) holds s's w-th word with a bit set, in candidate order; a particle's
+// list word is their number and the number of neighbours (mask_word), or
+// kMaskOver for a particle that needs more than `cap` words: it searches again.
+// With `pad` > 0 every row is filled up to `pad` words with empty ones, so
+// that a warp's lanes have the same row in the same plane.
+// (The precision form's 3-d runs keep lists in the same planes: plane k holds
+// s's k-th accepted neighbour with its binary32 kernel value, {j, K bits}; the
+// list word is the full number, and a particle with more than `cap` searches.)
 // ---------------------------------------------------------------------------
-constexpr int kSeg = 12;                   // segment entries per lane
+struct NbPlanes {
+    uint2* e;
+    int cap;           // planes (masks: at most 255); 0: nothing kept
+    int pad;           // words every row has at least (masks; see setup_grids)
+};
+constexpr uint32_t kMaskOver = 0xffffffffu;
+__device__ __forceinline__ uint32_t mask_word(uint32_t words, uint32_t neighbours, int cap) {
+    return words <= uint32_t(cap) && neighbours < (1u << 24) - 1u ? neighbours << 8 | words : kMaskOver;
+}
+
+// The search of one particle: its windows row by row, the accepted candidates
+// (those below the narrow band around the cutoff; `band` reports candidates
+// inside it) into mask words at e (its first plane's entry).  cand(d2f,
+// accept) is called for every candidate, the self pair included.  Returns the
+// words written or wanted; cnt receives the accepted neighbours j != s.
+template <int DIM, class Cand>
+__device__ __forceinline__ uint32_t search_words(uint32_t s, uint32_t cell, const float4 me,
+                                                 int64_t stride, const float4* __restrict__ rec,
+                                                 const uint32_t* __restrict__ start,
+                                                 const RealParams& P, const NbPlanes& nb,
+                                                 uint32_t& cnt, bool& band, Cand&& cand) {
+    const PairParams& pp = P.pp;
+    const Grid& g = P.g;
+    int c[3];
+    cell_coords_rec<DIM>(cell, me, P, c);
+    const float wx = g.wf[0], eps = pp.trim_eps;
+    const int R = g.reach, xlo = max(c[0] - R, 0), xhi = min(c[0] + R, g.n[0] - 1);
+    uint2* wp = nb.e + s;          // next mask word
+    uint32_t nw = 0;
+    cnt = 0;
+    band = false;
+    // one row's window and candidates: an empty window where the row is outside
+    // the grid or beyond the cutoff (for_each_row has the windows' derivation)
+    auto row = [&](int dy, int dz) {
+        const float sy = DIM >= 2 ? float(dy) * g.wf[1] : 0.0f;
+        const float sz = DIM == 3 ? float(dz) * g.wf[2] : 0.0f;
+        const float gy = DIM >= 2 ? row_gap(dy, me.y, g.wf[1], eps) : 0.0f;
+        const float gz = DIM == 3 ? row_gap(dz, me.z, g.wf[2], eps) : 0.0f;
+        const float r2 = __fsub_rn(pp.reach2, __fmaf_rn(gy, gy, __fmul_rn(gz, gz)));
+        const bool in_grid = (DIM < 2 || (c[1] + dy >= 0 && c[1] + dy < g.n[1])) &&
+                             (DIM < 3 || (c[2] + dz >= 0 && c[2] + dz < g.n[2]));
+        uint32_t j = 0, j3 = 0;
+        float rx = 0.0f;
+        if (in_grid && r2 >= 0.0f) {
+            rx = __fadd_rn(sqrt_approx(r2), eps);
+            const uint32_t rowc = P.cell_base + (uint32_t(c[2] + dz) * uint32_t(g.n[1]) +
+                                                 uint32_t(c[1] + dy)) * uint32_t(g.n[0]);
+            if (check(rowc + uint32_t(xhi) + 1u - P.cell_base <=
+                          uint32_t(g.n[0]) * uint32_t(g.n[1]) * uint32_t(g.n[2]), kChkRow)) {
+                j = __ldg(start + rowc + xlo);
+                j3 = __ldg(start + rowc + xhi + 1);
+                uint32_t hi = j3;
+                while (j < hi) {
+                    const uint32_t mid = (j + hi) >> 1;
+                    if (dx_f32(me, __ldg(rec + mid), wx) < -rx) j = mid + 1;
+                    else hi = mid;
+                }
+            }
+        }
+        const uint32_t padded = nw + uint32_t(nb.pad);
+        while (j < j3) {
+            const uint32_t base = j, end = min(j3, base + 32u);
+            uint32_t bits = 0, bit = 1;
+            for (; j < end; ++j, bit <<= 1) {
+                const float4 o = __ldg(rec + j);
+                const float dx = dx_f32(me, o, wx);
+                if (dx > rx) {
+                    j3 = j;
+                    break;
+                }
+                const float d2f = d2_f32<DIM>(dx, me, o, sy, sz);
+                band |= (d2f >= pp.band_lo) & (d2f <= pp.band_hi);
+                const bool accept = d2f < pp.band_lo;
+                cand(d2f, accept);
+                bits |= accept ? bit : 0u;
+            }
+            if (s - base < 32u) bits &= ~(1u << (s - base));   // the self pair is no neighbour
+            if (bits) {
+                cnt += uint32_t(__popc(bits));
+                if (nw < uint32_t(nb.cap)) *wp = make_uint2(base, bits);
+                wp += stride;
+                ++nw;
+            }
+        }
+        for (; nw < padded; ++nw, wp += stride)
+            if (nw < uint32_t(nb.cap)) *wp = make_uint2(0u, 0u);
+    };
+    // rows in a fixed order for the whole warp
+    if constexpr (DIM == 1) {
+        row(0, 0);
+    } else if constexpr (DIM == 2) {
+#pragma unroll 1
+        for (int dy = -R; dy <= R; ++dy) row(dy, 0);
+    } else {
+#pragma unroll 1
+        for (int dz = -R; dz <= R; ++dz)
+#pragma unroll 1
+            for (int dy = -R; dy <= R; ++dy) row(dy, dz);
+    }
+    return nw;
+}
+
+// The mask words of a particle that met candidates inside the band (about 1e-5
+// of all candidates): walks its windows again with the exact test and writes
+// all its words anew (without padding).  SUM (the precision form's pass 1):
+// also adds the kernel values of those it accepts to the row sum {rsum, rc}.
+// Returns {rsum, rc, words (bits), neighbours (bits)}.  A real call, so its
+// registers do not weigh on the candidate loop.
+template <int DIM, bool SUM, class View>
+__device__ __noinline__ float4 band_words(uint32_t s, const uint32_t* __restrict__ cell, int64_t stride,
+                                          const double* __restrict__ pos,
+                                          const float4* __restrict__ rec,
+                                          const uint32_t* __restrict__ start, const View& v,
+                                          const NbPlanes& nb, float rsum, float rc) {
+    const RealParams& P = v.of_sorted(s);
+    const PairParams& pp = P.pp;
+    const float4 me = rec[s];
+    uint32_t cnt = 0, nw = 0;
+    for_each_row<DIM>(cell_arg<DIM>(cell, s), me, rec, start, P,
+                      [&](uint32_t j, uint32_t j3, float rx, float sy, float sz) {
+        while (j < j3) {
+            const uint32_t base = j, end = min(j3, base + 32u);
+            uint32_t bits = 0;
+            for (; j < end; ++j) {
+                const float4 o = __ldg(rec + j);
+                const float dx = dx_f32(me, o, P.g.wf[0]);
+                if (dx > rx) {
+                    j3 = j;
+                    break;
+                }
+                const float d2f = d2_f32<DIM>(dx, me, o, sy, sz);
+                if (d2f > pp.band_hi) continue;
+                if (d2f >= pp.band_lo) {
+                    if (!exact_within<DIM>(pos, stride, s, j, pp.psi2)) continue;
+                    if constexpr (SUM) {
+                        const float y = __fsub_rn(ex2_approx(-pp.a_log2e * d2f), rc);
+                        const float t = __fadd_rn(rsum, y);
+                        rc = __fsub_rn(__fsub_rn(t, rsum), y);
+                        rsum = t;
+                    }
+                }
+                if (j != s) bits |= 1u << (j - base);
+            }
+            if (bits) {
+                cnt += uint32_t(__popc(bits));
+                if (nw < uint32_t(nb.cap)) nb.e[int64_t(nw) * stride + s] = make_uint2(base, bits);
+                ++nw;
+            }
+        }
+    });
+    return make_float4(rsum, rc, __uint_as_float(nw), __uint_as_float(cnt));
+}
+
+// ---------------------------------------------------------------------------
+// Binary64 pair passes.  The binary64 form's two passes are a thread per
+// particle throughout: its pair terms are integer arithmetic (expneg.cuh), and
+// a warp that takes its particles' k-th neighbours together stores and reads
+// their kernel values in whole rows.  (Evaluating the warp's neighbours one a
+// lane, as below, saves the lanes idle in the longest particle's tail but
+// spends as many instructions on handing them out: pass 1 took 405 us that way
+// instead of 381, pass 2 with the walk 389 instead of 322, 4e6 particles in
+// 2-d.)
+// The adjoint's pair terms are mostly binary64 operations, which cost the same
+// however many lanes are active, so there a warp works in two parts: each lane
+// searches its particle and leaves mask words; then the warp takes the words'
+// neighbours in lane-major order, kChunk at a time: the lanes write out their
+// neighbours' indexes (shared memory), all 32 evaluate one each until the chunk
+// is done, and each lane adds its own results in candidate order.
+// Either way every sum runs in candidate order and repeats bit for bit.
+// ---------------------------------------------------------------------------
 constexpr int kWarpsPerBlock = kBlock / 32;
+constexpr int kChunk = 128;                // neighbours of a warp evaluated at a time
 
 __device__ __forceinline__ uint32_t warp_exclusive_scan(uint32_t v, uint32_t* total) {
     const int lane = threadIdx.x & 31;
@@ -1121,203 +1285,126 @@ __device__ __forceinline__ uint32_t warp_exclusive_scan(uint32_t v, uint32_t* to
 }
 
 // Shared state of one block's warps.  V: type of the pair terms.
-template <int NW, class V, int SEG = kSeg>
-struct SegShared {
-    static constexpr int kCap = SEG;   // entries per lane
-    uint32_t j[NW][SEG][32];           // lane-owned segments, entry k of lane l at [k][l]
-    V v[NW][SEG * 32];                 // phase-B results, lane-major
-    uint8_t owner[NW][SEG * 32];       // lane of each lane-major entry
-    uint32_t off[NW][32];              // first lane-major entry of each lane
-    uint32_t base[NW][32];             // entries each lane had before this flush
-};
-
-// Neighbour lists: pass 1 stores each accepted neighbour j != s and its pair
-// value (the binary64 K_sj, or (K_sj, dK_sj/dD) in the adjoint) in slot k of
-// s (entry at k * stride + s), up to `cap` slots; count[s] is the full
-// number.  Pass 2 of a warp whose lanes all fit their lists reads them
-// instead of searching and re-evaluating exp; otherwise the warp searches.
-// Both paths visit the same pairs in the same order with the same values.
 template <class V>
-struct NbList {
-    uint32_t* j;
-    V* k;
-    uint32_t* count;
-    int cap;           // 0: no list
+struct ChunkShared {
+    V v[kWarpsPerBlock][kChunk];               // pair terms
+    uint32_t j[kWarpsPerBlock][kChunk];        // neighbour indexes
+    uint8_t owner[kWarpsPerBlock][kChunk];     // lane of each
 };
-using NbList64 = NbList<double>;
 
-// What pass 1 of the precision form keeps for pass 2, in planes of `stride`
-// entries (plane p of particle s at p * stride + s).
-// 3-d: neighbour lists.  Plane k holds s's k-th accepted neighbour j != s with
-// its binary32 kernel value, {j, K bits}; ex[s].w is the full number, and a
-// particle with more than `cap` searches in pass 2.
-// 1-d and 2-d: accept masks.  A word {base, bits} holds 32 consecutive
-// candidates of one neighbour row: bit k is set when candidate base + k is an
-// accepted neighbour j != s.  Plane w holds s's w-th word with a bit set, in
-// candidate order; ex[s].w is their number and the number of neighbours
-// (mask_word), or kMaskOver for a particle that needs more than `cap` words and
-// searches in pass 2.  With `pad` > 0 every row is filled up to `pad` words
-// with empty ones, so that a warp's lanes have the same row in the same plane.
-struct Nb32 {
-    uint2* e;
-    int cap;           // planes (masks: at most 255); 0: nothing kept, pass 2 searches
-    int pad;           // words every row has at least (masks; see setup_grids)
+// Kernel values that pass 1 of the binary64 form leaves for pass 2: plane k
+// holds s's k-th neighbour's, k < cap - 1 (pass 2 evaluates the others again).
+struct PairValues {
+    double* v;
+    int cap;           // 0: none kept
 };
-constexpr uint32_t kMaskOver = 0xffffffffu;
-__device__ __forceinline__ uint32_t mask_word(uint32_t words, uint32_t neighbours, int cap) {
-    return words <= uint32_t(cap) && neighbours < (1u << 24) - 1u ? neighbours << 8 | words : kMaskOver;
-}
 
-// Phases A-C for the calling warp (every lane of the warp must call it; lanes
-// with valid = false walk nothing).  eval(owner_s, j, keep) returns the pair
-// term and sets keep to what the list stores; add(term) is called by each lane
-// for its own entries in order.  Returns the lane's number of accepted
-// neighbours j != s.
-template <int DIM, int NW, class V, int SEG, class VL, class Eval, class Add>
-__device__ __forceinline__ uint32_t seg_pairs(bool valid, uint32_t s, int64_t stride,
-                                              const float4* __restrict__ rec,
-                                              const double* __restrict__ pos,
-                                              const uint32_t* __restrict__ cell,
-                                              const uint32_t* __restrict__ start,
-                                              const RealParams& P, SegShared<NW, V, SEG>& S,
-                                              Eval&& eval, Add&& add, const NbList<VL>& store) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t warp_s0 = s - uint32_t(lane);
-    uint32_t cnt = 0, done = 0;
-    auto flush = [&]() {
-        uint32_t total;
-        const uint32_t off = warp_exclusive_scan(cnt, &total);
-        check(cnt <= uint32_t(SEG) && total <= uint32_t(SEG) * 32u, kChkSegment);
-        S.off[warp][lane] = off;
-        S.base[warp][lane] = done;
-        for (uint32_t k = 0; k < cnt; ++k) S.owner[warp][off + k] = uint8_t(lane);
-        __syncwarp();
-        for (uint32_t e = uint32_t(lane); e < total; e += 32) {
-            const uint32_t o = S.owner[warp][e];
-            const uint32_t k = e - S.off[warp][o];
-            const uint32_t j = S.j[warp][k][o];
-            VL keep;
-            S.v[warp][e] = eval(warp_s0 + o, j, keep);
-            if (store.cap > 0) {
-                const uint32_t slot = S.base[warp][o] + k;
-                if (slot < uint32_t(store.cap)) {
-                    const int64_t at = int64_t(slot) * stride + (warp_s0 + o);
-                    store.j[at] = j;
-                    store.k[at] = keep;
-                }
-            }
-        }
-        __syncwarp();
-        for (uint32_t k = 0; k < cnt; ++k) add(S.v[warp][off + k]);
-        done += cnt;
-        cnt = 0;
-        __syncwarp();
-    };
-
-    const Grid& g = P.g;
-    const PairParams& pp = P.pp;
-    const float4 me = valid ? rec[s] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    int c[3] = {0, 0, 0};
-    if (valid) cell_coords_rec<DIM>(cell_arg<DIM>(cell, s), me, P, c);
-    const int R = g.reach;
-    const int xlo = max(c[0] - R, 0);
-    const int xhi = min(c[0] + R, g.n[0] - 1);
-    const float eps = pp.trim_eps;
-    const float wx = g.wf[0];
-    // rows in a fixed order for the whole warp; a lane whose row is outside
-    // the grid or beyond the cutoff (see for_each_row) gets an empty window
-#pragma unroll 1
-    for (int dz = (DIM == 3 ? -R : 0); dz <= (DIM == 3 ? R : 0); ++dz) {
-#pragma unroll 1
-        for (int dy = (DIM >= 2 ? -R : 0); dy <= (DIM >= 2 ? R : 0); ++dy) {
-            const float sy = DIM >= 2 ? float(dy) * g.wf[1] : 0.0f;
-            const float sz = DIM == 3 ? float(dz) * g.wf[2] : 0.0f;
-            uint32_t j = 0, j3 = 0;
-            float rx = 0.0f;
-            const bool in_grid = valid && (DIM < 2 || (c[1] + dy >= 0 && c[1] + dy < g.n[1])) &&
-                                 (DIM < 3 || (c[2] + dz >= 0 && c[2] + dz < g.n[2]));
-            if (in_grid) {
-                const float gy = DIM >= 2 ? row_gap(dy, me.y, g.wf[1], eps) : 0.0f;
-                const float gz = DIM == 3 ? row_gap(dz, me.z, g.wf[2], eps) : 0.0f;
-                const float r2 = __fsub_rn(pp.reach2, __fmaf_rn(gy, gy, __fmul_rn(gz, gz)));
-                if (r2 >= 0.0f) {
-                    rx = __fadd_rn(sqrt_approx(r2), eps);
-                    const uint32_t rowc = P.cell_base + (uint32_t(c[2] + dz) * uint32_t(g.n[1]) +
-                                                         uint32_t(c[1] + dy)) * uint32_t(g.n[0]);
-                    const bool row_ok = check(
-                        rowc + uint32_t(xhi) + 1u - P.cell_base <=
-                            uint32_t(g.n[0]) * uint32_t(g.n[1]) * uint32_t(g.n[2]), kChkRow);
-                    uint32_t lo = row_ok ? __ldg(start + rowc + xlo) : 0u;
-                    uint32_t hi = row_ok ? __ldg(start + rowc + xhi + 1) : 0u;
-                    j3 = hi;
-                    while (lo < hi) {
-                        const uint32_t mid = (lo + hi) >> 1;
-                        if (dx_f32(me, __ldg(rec + mid), wx) < -rx) lo = mid + 1;
-                        else hi = mid;
-                    }
-                    j = lo;
-                }
-            }
-            do {
-                while (j < j3 && cnt < uint32_t(SEG)) {
-                    const float4 o = __ldg(rec + j);
-                    const float dx = dx_f32(me, o, wx);
-                    if (dx > rx) {
-                        j = j3;
-                        break;
-                    }
-                    const float d2f = d2_f32<DIM>(dx, me, o, sy, sz);
-                    bool accept = d2f < pp.band_lo;
-                    if (d2f >= pp.band_lo && d2f <= pp.band_hi)
-                        accept = exact_within<DIM>(pos, stride, s, j, pp.psi2);
-                    if (accept && j != s) {
-                        S.j[warp][cnt][lane] = j;
-                        ++cnt;
-                    }
-                    ++j;
-                }
-                if (__any_sync(0xffffffffu, cnt == uint32_t(SEG))) flush();
-            } while (__any_sync(0xffffffffu, j < j3));
-        }
+// The adjoint's (K, dK): the e-th neighbour of a warp (lane-major) at
+// first + e, for warps with at most 32 * cap neighbours.
+struct AdjValues {
+    double2* v;
+    int cap;
+    __device__ __forceinline__ double2* of_warp(uint32_t warp_s0, uint32_t total) const {
+        return total <= 32u * uint32_t(cap) ? v + size_t(warp_s0) * size_t(cap) : nullptr;
     }
-    if (__any_sync(0xffffffffu, cnt > 0)) flush();
-    return done;
-}
+};
 
-// Phases B-C over stored lists (the warp's lanes all fit their lists):
-// eval(owner_s, j, stored value) returns the pair term, add(term) as above.
-template <int NW, class V, int SEG, class VL, class Eval, class Add>
-__device__ __forceinline__ void dense_listed(bool valid, uint32_t s, int64_t stride,
-                                             uint32_t cnt, const NbList<VL>& nb,
-                                             SegShared<NW, V, SEG>& S, Eval&& eval,
-                                             Add&& add) {
-    constexpr uint32_t kChunk = SEG * 32;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+// A particle's neighbours from its mask words (without padding), in order; the
+// word after the current one is loaded ahead.
+struct WordStream {
+    const uint2* e;
+    int64_t stride;
+    uint32_t left;               // words after `ahead`
+    uint2 cur, ahead;
+    __device__ __forceinline__ WordStream(const uint2* first, int64_t st, uint32_t words)
+        : e(first), stride(st), left(words > 0u ? words - 1u : 0u), cur(make_uint2(0u, 0u)),
+          ahead(words > 0u ? *first : make_uint2(0u, 0u)) {}
+    __device__ __forceinline__ uint32_t next() {
+        if (cur.y == 0u) {
+            cur = ahead;
+            if (left > 0u) {
+                ahead = *(e += stride);
+                --left;
+            }
+        }
+        check(cur.y != 0u, kChkSegment);
+        const uint32_t j = cur.x + uint32_t(__ffs(int(cur.y)) - 1);
+        cur.y &= cur.y - 1u;
+        return j;
+    }
+};
+
+// The dense part for the calling warp (all its lanes): listed is the lane's
+// list word (0 for a lane without a particle, kMaskOver for one that searches
+// on its own: both add nothing here).  eval(e, owner_s, j) returns the pair
+// term of the warp's neighbour e, add(term) is called by each lane for its
+// own, in order; begin(total) comes first.
+template <class V, class Begin, class Eval, class Add>
+__device__ __forceinline__ void dense_words(uint32_t s, uint32_t listed, int64_t stride,
+                                            const uint2* e, ChunkShared<V>& S, Begin&& begin,
+                                            Eval&& eval, Add&& add) {
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, warp_s0 = s - lane;
+    if (listed == kMaskOver) listed = 0;
+    const uint32_t cnt = listed >> 8, words = listed & 255u;
     uint32_t total;
-    const uint32_t off = warp_exclusive_scan(valid ? cnt : 0u, &total);
-    S.off[warp][lane] = off;
-    const uint32_t warp_s0 = s - uint32_t(lane);
-    for (uint32_t chunk = 0; chunk < total; chunk += kChunk) {
-        const uint32_t chunk_end = chunk + kChunk;
-        if (valid) {
-            const uint32_t q0 = max(off, chunk), q1 = min(off + cnt, chunk_end);
-            for (uint32_t q = q0; q < q1; ++q) S.owner[warp][q - chunk] = uint8_t(lane);
+    const uint32_t off = warp_exclusive_scan(cnt, &total), end = off + cnt;
+    begin(total);
+    WordStream stream(e + s, stride, words);
+    uint32_t pos = off;
+    for (uint32_t c0 = 0; c0 < total; c0 += kChunk) {
+        const uint32_t m = min(total - c0, uint32_t(kChunk)), stop = min(end, c0 + m);
+        for (; pos < stop; ++pos) {
+            S.j[warp][pos - c0] = stream.next();
+            S.owner[warp][pos - c0] = uint8_t(lane);
         }
         __syncwarp();
-        const uint32_t m = min(total - chunk, kChunk);
-        for (uint32_t e = uint32_t(lane); e < m; e += 32) {
-            const uint32_t o = S.owner[warp][e];
-            const uint32_t so = warp_s0 + o;
-            const int64_t at = int64_t(chunk + e - S.off[warp][o]) * stride + so;
-            S.v[warp][e] = eval(so, __ldg(nb.j + at), __ldg(nb.k + at));
-        }
+        for (uint32_t k = lane; k < m; k += 32)
+            S.v[warp][k] = eval(c0 + k, warp_s0 + S.owner[warp][k], S.j[warp][k]);
         __syncwarp();
-        if (valid) {
-            const uint32_t q0 = max(off, chunk), q1 = min(off + cnt, chunk_end);
-            for (uint32_t q = q0; q < q1; ++q) add(S.v[warp][q - chunk]);
-        }
+        for (uint32_t q = max(off, c0); q < stop; ++q) add(S.v[warp][q - c0]);
         __syncwarp();
     }
+}
+
+// Search of one particle of a binary64 pass: its list word (kMaskOver also when
+// nothing can be kept), neighbour count in cnt.
+template <int DIM, class View>
+__device__ __forceinline__ uint32_t search_listed(uint32_t s, int64_t stride,
+                                                  const double* __restrict__ pos,
+                                                  const float4* __restrict__ rec,
+                                                  const uint32_t* __restrict__ cell,
+                                                  const uint32_t* __restrict__ start, const View& v,
+                                                  const RealParams& P, const NbPlanes& nb,
+                                                  uint32_t& cnt) {
+    bool band;
+    const uint32_t c = cell_arg<DIM>(cell, s);
+    uint32_t nw = search_words<DIM>(s, c, rec[s], stride, rec, start, P, nb, cnt, band,
+                                    [](float, bool) {});
+    if (band) {
+        const float4 b = band_words<DIM, false>(s, cell, stride, pos, rec, start, v, nb, 0.0f, 0.0f);
+        nw = __float_as_uint(b.z);
+        cnt = __float_as_uint(b.w);
+    }
+    return mask_word(nw, cnt, nb.cap);
+}
+
+// Pass 1 of one particle whose neighbours the words do not hold.
+template <int DIM, class View>
+__device__ __noinline__ double search_rowsum(uint32_t s, int64_t stride,
+                                             const double* __restrict__ pos,
+                                             const uint64_t* __restrict__ image,
+                                             const float4* __restrict__ rec,
+                                             const uint32_t* __restrict__ cell,
+                                             const uint32_t* __restrict__ start,
+                                             const double* table, const View& v) {
+    const RealParams& P = v.of_sorted(s);
+    RowSum r;
+    visit_neighbours<DIM>(s, cell_arg<DIM>(cell, s), stride, rec, pos, start, P,
+                          [&](uint32_t j, float, const float4&) {
+                              if (j != s)
+                                  r.add(unit_of(pair_kernel<DIM>(image, stride, s, j, table, P.pp.kc)));
+                          });
+    return r.value();
 }
 
 // Pass 1, binary64 form: r_s = 1 + sum_{j != s} exp(-a d2_sj) (the kernel
@@ -1325,36 +1412,80 @@ __device__ __forceinline__ void dense_listed(bool valid, uint32_t s, int64_t str
 // the ordered pair count.  The kernel values and their sum are fixed-point
 // (expneg.cuh): no binary64 instruction, and the sum is exact whatever its
 // order.  With binary64 operations the pass was bound by that unit (86 % busy):
-// 732 us at 4e6 particles in 2-d with 5.7 neighbours each, 420 now.
+// 732 us at 4e6 particles in 2-d with 5.7 neighbours each, 381 now, bound by
+// instruction issue (72 %).  Two neighbours at a time (their loads and integer
+// chains overlap); 40 registers, 48 in 3-d (four more blocks an SM do not help
+// there: 54 instead of 52 us at 250,007).
 template <int DIM, class View>
-__global__ void __launch_bounds__(kBlock)
+__global__ void __launch_bounds__(kBlock, DIM == 3 ? 5 : 6)
 k_rowsum_f64(int n, int64_t stride, const double* __restrict__ pos,
              const uint64_t* __restrict__ image, const float4* __restrict__ rec,
              const uint32_t* __restrict__ cell, const uint32_t* __restrict__ start,
-             const uint64_t* __restrict__ exp_table, const __grid_constant__ View v,
-             double* __restrict__ r_out, unsigned long long* __restrict__ pair_counter,
-             NbList64 nb, const uint32_t* __restrict__ ghost_id) {
-    __shared__ uint64_t table[kExpTable];
-    __shared__ SegShared<kWarpsPerBlock, uint64_t> seg;
+             const double* __restrict__ exp_table, const __grid_constant__ View v,
+             const double* __restrict__ mass, double2* __restrict__ rm,
+             unsigned long long* __restrict__ pair_counter, const __grid_constant__ NbPlanes nb,
+             uint32_t* __restrict__ listed_out, PairValues kv,
+             const uint32_t* __restrict__ ghost_id) {
+    __shared__ double table[kExpTable];
     for (int t = threadIdx.x; t < kExpTable; t += blockDim.x) table[t] = exp_table[t];
     __syncthreads();
+    const uint32_t s = blockIdx.x * blockDim.x + threadIdx.x;
+    uint32_t cnt = 0;
+    if (s < uint32_t(n)) {
+        const RealParams& P = v.of_sorted(s);
+        uint32_t listed = 0;
+        double r = 1.0;
+        if (P.transfer) {
+            listed = search_listed<DIM>(s, stride, pos, rec, cell, start, v, P, nb, cnt);
+            if (listed == kMaskOver) {
+                r = search_rowsum<DIM>(s, stride, pos, image, rec, cell, start, table, v);
+            } else {
+                uint64_t xs[DIM];
+#pragma unroll
+                for (int a = 0; a < DIM; ++a) xs[a] = image[a * stride + s];
+                RowSum sum;
+                WordStream stream(nb.e + s, stride, listed & 255u);
+                auto kernel = [&](uint32_t j) {
+                    uint64_t d2h = 0;
+#pragma unroll
+                    for (int a = 0; a < DIM; ++a) d2h += axis_square(xs[a], __ldg(image + a * stride + j));
+                    return gauss_fixed(d2h, table, P.pp.kc);
+                };
+                double* keep = kv.v + s;
+                uint32_t k = 0;
+                for (; k + 2 <= cnt; k += 2) {
+                    const uint32_t j0 = stream.next(), j1 = stream.next();
+                    const double K0 = kernel(j0), K1 = kernel(j1);
+                    if (k + 1u < uint32_t(kv.cap)) {
+                        keep[0] = K0;
+                        keep[stride] = K1;
+                        keep += 2 * stride;
+                    }
+                    sum.add(unit_of(K0));
+                    sum.add(unit_of(K1));
+                }
+                if (k < cnt) {
+                    const double K = kernel(stream.next());
+                    if (k + 1u < uint32_t(kv.cap)) *keep = K;
+                    sum.add(unit_of(K));
+                }
+                r = sum.value();
+            }
+        }
+        rm[s] = make_double2(r, mass[s]);
+        if (listed_out) listed_out[s] = listed;
+        // with ghost_id (a tile), pairs are counted for the tile's own particles only
+        if (ghost_id && (ghost_id[s] & kGhostBit)) cnt = 0;
+    }
+    add_pair_count(cnt, pair_counter);
+}
+
+// Species B of a binary64 reaction run: its masses in place of A's in the
+// records {r, m} that pass 2 reads.
+__global__ void __launch_bounds__(kBlock)
+k_record_mass(int n, const double* __restrict__ mass_b, double2* __restrict__ rm) {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    const RealParams& P = v.of_sorted(uint32_t(s < n ? s : 0));
-    const bool valid = s < n && P.transfer;
-    RowSum r;
-    const uint32_t cnt = seg_pairs<DIM>(
-        valid, uint32_t(s), stride, rec, pos, cell, start, P, seg,
-        [&](uint32_t so, uint32_t j, double& K) {
-            const FixedK f = pair_kernel<DIM>(image, stride, so, j, table, v.of_sorted(so).pp.kc);
-            K = f.value();
-            return f.unit();
-        },
-        [&](uint64_t unit) { r.add(unit); }, nb);
-    if (s < n) r_out[s] = r.value();
-    if (nb.cap > 0 && s < n) nb.count[s] = valid ? cnt : 0u;
-    // with ghost_id (a tile), pairs are counted for the tile's own particles only
-    const bool counted = valid && !(ghost_id && (ghost_id[s] & kGhostBit));
-    add_pair_count(counted ? cnt : 0u, pair_counter);
+    if (s < n) rm[s].y = mass_b[s];
 }
 
 // The next step's walk done at the end of pass 2 (walk-ahead, for the steps of
@@ -1394,50 +1525,87 @@ __device__ __forceinline__ void walk_ahead(const RealParams& P, int s, int64_t s
 }
 
 // Pass 2, binary64 form: M'_s = M_s + beta sum_j (M_j - M_s) 2 K_sj / (r_s + r_j).
-// The weight is formed in integers (expneg.cuh), which leaves the binary64
-// unit three operations a pair of nine: 543 -> 330 us (4e6 particles, 2-d).
+// Weight, flux and sum are integer arithmetic (expneg.cuh), which leaves the
+// binary64 unit the mass difference, one operation a pair of nine: 543 -> 269 us
+// (4e6 particles, 2-d), 593 -> 322 with the next walk.
+// Pass 2 of one particle whose neighbours the words do not hold.
+template <int DIM, class View>
+__device__ __noinline__ double search_flux_f64(uint32_t s, int64_t stride,
+                                               const double* __restrict__ pos,
+                                               const uint64_t* __restrict__ image,
+                                               const float4* __restrict__ rec,
+                                               const uint32_t* __restrict__ cell,
+                                               const uint32_t* __restrict__ start,
+                                               const double* table, const View& v,
+                                               const double2* __restrict__ rm) {
+    const RealParams& P = v.of_sorted(s);
+    const double2 me = rm[s];
+    FluxSum64 sum;
+    visit_neighbours<DIM>(s, cell_arg<DIM>(cell, s), stride, rec, pos, start, P,
+                          [&](uint32_t j, float, const float4&) {
+                              if (j == s) return;
+                              const double K = pair_kernel<DIM>(image, stride, s, j, table, P.pp.kc);
+                              const double2 q = __ldg(rm + j);
+                              sum.add(__dsub_rn(q.y, me.y), weight_fixed(K, me.x, q.x));
+                          });
+    return sum.value();
+}
+
 template <int DIM, class View, int WALK = 0>
-__global__ void __launch_bounds__(kBlock)
+__global__ void __launch_bounds__(kBlock, 5)
 k_exchange_f64(int n, int64_t stride, const double* __restrict__ pos,
                const uint64_t* __restrict__ image, const float4* __restrict__ rec,
                const uint32_t* __restrict__ cell, const uint32_t* __restrict__ start,
-               const uint64_t* __restrict__ exp_table, const __grid_constant__ View v,
-               const double* __restrict__ r, const double* __restrict__ mass,
-               double* __restrict__ mass_out, NbList64 nb, const WalkAhead wa = WalkAhead{}) {
-    __shared__ uint64_t table[kExpTable];
-    __shared__ SegShared<kWarpsPerBlock, double> seg;
+               const double* __restrict__ exp_table, const __grid_constant__ View v,
+               const double2* __restrict__ rm, double* __restrict__ mass_out, NbPlanes nb,
+               const uint32_t* __restrict__ listed_in, PairValues kv,
+               const WalkAhead wa = WalkAhead{}) {
+    __shared__ double table[kExpTable];   // of use to the particles that search or evaluate again
     for (int t = threadIdx.x; t < kExpTable; t += blockDim.x) table[t] = exp_table[t];
     __syncthreads();
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    const RealParams& P = v.of_sorted(uint32_t(s < n ? s : 0));
-    const bool valid = s < n && P.transfer;
-    double acc = 0.0;
-    auto flux = [&](uint32_t so, uint32_t j, double K) {
-        const double W = weight_fixed(K, __ldg(r + so), __ldg(r + j));
-        return __dmul_rn(__dsub_rn(__ldg(mass + j), __ldg(mass + so)), W);
-    };
-    const uint32_t listed = (nb.cap > 0 && valid) ? nb.count[s] : 0u;
-    const bool fits = nb.cap > 0 && __all_sync(0xffffffffu, listed <= uint32_t(nb.cap));
-    if (fits) {
-        dense_listed(valid, uint32_t(s), stride, listed, nb, seg, flux,
-                     [&](double f) { acc = __dadd_rn(acc, f); });
-    } else {
-        seg_pairs<DIM>(
-            valid, uint32_t(s), stride, rec, pos, cell, start, P, seg,
-            [&](uint32_t so, uint32_t j, double& K) {
-                K = pair_kernel<DIM>(image, stride, so, j, table, v.of_sorted(so).pp.kc).value();
-                return flux(so, j, K);
-            },
-            [&](double f) { acc = __dadd_rn(acc, f); }, NbList64{});
+    const uint32_t s = blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= uint32_t(n)) return;
+    const RealParams& P = v.of_sorted(s);
+    const double2 me = __ldg(rm + s);
+    double m = me.y;
+    if (P.transfer) {
+        const uint32_t listed = listed_in ? listed_in[s] : kMaskOver;
+        double flux;
+        if (listed == kMaskOver) {
+            flux = search_flux_f64<DIM>(s, stride, pos, image, rec, cell, start, table, v, rm);
+        } else {
+            const uint32_t cnt = listed >> 8;
+            // pass 1's kernel values: whole pairs below the capacity
+            const uint32_t kept = kv.cap > 0 ? min(cnt, uint32_t(kv.cap - 1) & ~1u) : 0u;
+            const uint32_t listed_k = cnt < uint32_t(kv.cap) ? cnt : kept;
+            FluxSum64 sum;
+            WordStream stream(nb.e + s, stride, listed & 255u);
+            const double* keep = kv.v + s;
+            uint32_t k = 0;
+            for (; k + 2 <= listed_k; k += 2, keep += 2 * stride) {
+                const uint32_t j0 = stream.next(), j1 = stream.next();
+                const double K0 = __ldg(keep), K1 = __ldg(keep + stride);
+                const double2 q0 = __ldg(rm + j0), q1 = __ldg(rm + j1);
+                sum.add(__dsub_rn(q0.y, me.y), weight_fixed(K0, me.x, q0.x));
+                sum.add(__dsub_rn(q1.y, me.y), weight_fixed(K1, me.x, q1.x));
+            }
+            for (; k < cnt; ++k) {
+                const uint32_t j = stream.next();
+                const double K = k < listed_k ? __ldg(keep)
+                                              : pair_kernel<DIM>(image, stride, s, j, table, P.pp.kc);
+                const double2 q = __ldg(rm + j);
+                sum.add(__dsub_rn(q.y, me.y), weight_fixed(K, me.x, q.x));
+            }
+            flux = sum.value();
+        }
+        m = __dadd_rn(m, __dmul_rn(P.pp.beta, flux));
     }
-    if (s < n) mass_out[s] = valid ? __dadd_rn(mass[s], __dmul_rn(P.pp.beta, acc)) : mass[s];
-    if constexpr (WALK > 0) {
-        if (s < n) walk_ahead<DIM, WALK>(P, s, stride, pos, wa);
-    }
+    mass_out[s] = m;
+    if constexpr (WALK > 0) walk_ahead<DIM, WALK>(P, int(s), stride, pos, wa);
 }
 
 // The particle's record that pass 2 reads per neighbour, written whole by pass
-// 1: m = {m_hi, m_lo, r, list word (bits, see Nb32; of use to the particle
+// 1: m = {m_hi, m_lo, r, list word (bits, see NbPlanes; of use to the particle
 // itself only)}, the mass's binary32 head/tail split and the row sum.  Below
 // 3-d it is preceded by a copy of the particle's rec, so that all of a
 // neighbour's 32 bytes (from which pass 2 also forms K again) are one sector
@@ -1468,59 +1636,10 @@ __device__ __forceinline__ float4 load_ex(const float4* __restrict__ ex, uint32_
     return __ldg(ex + size_t(ExRec<DIM>::kVec) * j + (ExRec<DIM>::kVec - 1));
 }
 
-// Pass 1 of a 1-d or 2-d particle that met candidates inside the narrow band
-// around the cutoff (about 1e-5 of all candidates): walks its windows again,
-// adds those the exact test accepts to the row sum and writes its mask words
-// with them.  Returns {rsum, rc, words (bits), neighbours (bits)}.  A real
-// call, so its registers do not weigh on the candidate loop.
-template <int DIM, class View>
-__device__ __noinline__ float4 band_accepts(uint32_t s, int64_t stride,
-                                            const double* __restrict__ pos,
-                                            const float4* __restrict__ rec,
-                                            const uint32_t* __restrict__ start, const View& v,
-                                            Nb32 nb, float rsum, float rc) {
-    const RealParams& P = v.of_sorted(s);
-    const PairParams& pp = P.pp;
-    const float4 me = rec[s];
-    uint32_t cnt = 0, nw = 0;
-    for_each_row<DIM>(0u, me, rec, start, P,
-                      [&](uint32_t j, uint32_t j3, float rx, float sy, float sz) {
-        // (no padding: pass 2 takes a particle's words as they come)
-        while (j < j3) {
-            const uint32_t base = j, end = min(j3, base + 32u);
-            uint32_t bits = 0;
-            for (; j < end; ++j) {
-                const float4 o = __ldg(rec + j);
-                const float dx = dx_f32(me, o, P.g.wf[0]);
-                if (dx > rx) {
-                    j3 = j;
-                    break;
-                }
-                const float d2f = d2_f32<DIM>(dx, me, o, sy, sz);
-                if (d2f > pp.band_hi) continue;
-                if (d2f >= pp.band_lo) {
-                    if (!exact_within<DIM>(pos, stride, s, j, pp.psi2)) continue;
-                    const float y = __fsub_rn(ex2_approx(-pp.a_log2e * d2f), rc);
-                    const float t = __fadd_rn(rsum, y);
-                    rc = __fsub_rn(__fsub_rn(t, rsum), y);
-                    rsum = t;
-                }
-                if (j != s) bits |= 1u << (j - base);
-            }
-            if (bits) {
-                cnt += uint32_t(__popc(bits));
-                if (nw < uint32_t(nb.cap)) nb.e[int64_t(nw) * stride + s] = make_uint2(base, bits);
-                ++nw;
-            }
-        }
-    });
-    return make_float4(rsum, rc, __uint_as_float(nw), __uint_as_float(cnt));
-}
-
 // Pass 1, precision form: binary32 kernel exp2(-a log2(e) d2f) with the
 // hardware ex2, compensated binary32 row sum, rounded to binary32; written
 // in the particle's record ex (ExRec); with nb.cap > 0 also what pass 2 needs
-// of the search (Nb32).  Bound by instruction issue and the candidate loads'
+// of the search (NbPlanes).  Bound by instruction issue and the candidate loads'
 // latency.  In 1-d and 2-d the accepted neighbours leave as mask words, one
 // 8-byte store a row next to the other lanes' stores: a {j, K} list entry per
 // neighbour was a partly written sector each, and those writes bounded the
@@ -1533,7 +1652,7 @@ k_rowsum_f32(int n, int64_t stride, const double* __restrict__ pos, const float4
              const uint32_t* __restrict__ cell, const uint32_t* __restrict__ start,
              const __grid_constant__ View v, const double* __restrict__ mass,
              float4* __restrict__ ex, unsigned long long* __restrict__ pair_counter,
-             const uint32_t* __restrict__ ghost_id, Nb32 nb) {
+             const uint32_t* __restrict__ ghost_id, const __grid_constant__ NbPlanes nb) {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     uint32_t cnt = 0;
     if (s < n) {
@@ -1566,73 +1685,15 @@ k_rowsum_f32(int n, int64_t stride, const double* __restrict__ pos, const float4
                                  });
             list_word = cnt;
         } else {
-            const PairParams& pp = P.pp;
-            const Grid& g = P.g;
-            const float4 me = rec[s];
-            const float na = -pp.a_log2e, wx = g.wf[0], eps = pp.trim_eps;
-            const int R = g.reach, cx = int(me.w), cy = DIM == 2 ? int(me.z) : 0;
-            const int xlo = max(cx - R, 0), xhi = min(cx + R, g.n[0] - 1);
-            uint2* wp = nb.e + s;          // next mask word
-            uint32_t nw = 0;
-            bool band = false;
-            // rows in a fixed order for the whole warp: an empty window where
-            // the row is outside the grid or beyond the cutoff (for_each_row
-            // has the windows' derivation)
-#pragma unroll 1
-            for (int dy = DIM == 2 ? -R : 0; dy <= (DIM == 2 ? R : 0); ++dy) {
-                const float sy = DIM == 2 ? float(dy) * g.wf[1] : 0.0f;
-                const float gy = DIM == 2 ? row_gap(dy, me.y, g.wf[1], eps) : 0.0f;
-                const float r2 = __fsub_rn(pp.reach2, __fmul_rn(gy, gy));
-                const bool in_grid = DIM == 1 || (cy + dy >= 0 && cy + dy < g.n[1]);
-                uint32_t j = 0, j3 = 0;
-                float rx = 0.0f;
-                if (in_grid && r2 >= 0.0f) {
-                    rx = __fadd_rn(sqrt_approx(r2), eps);
-                    const uint32_t rowc =
-                        P.cell_base + uint32_t(DIM == 2 ? cy + dy : 0) * uint32_t(g.n[0]);
-                    if (check(rowc + uint32_t(xhi) + 1u - P.cell_base <=
-                                  uint32_t(g.n[0]) * uint32_t(g.n[1]) * uint32_t(g.n[2]), kChkRow)) {
-                        j = __ldg(start + rowc + xlo);
-                        j3 = __ldg(start + rowc + xhi + 1);
-                        uint32_t hi = j3;
-                        while (j < hi) {
-                            const uint32_t mid = (j + hi) >> 1;
-                            if (dx_f32(me, __ldg(rec + mid), wx) < -rx) j = mid + 1;
-                            else hi = mid;
-                        }
-                    }
-                }
-                const uint32_t padded = nw + uint32_t(nb.pad);
-                while (j < j3) {
-                    const uint32_t base = j, end = min(j3, base + 32u);
-                    uint32_t bits = 0, bit = 1;
-                    for (; j < end; ++j, bit <<= 1) {
-                        const float4 o = __ldg(rec + j);
-                        const float dx = dx_f32(me, o, wx);
-                        if (dx > rx) {
-                            j3 = j;
-                            break;
-                        }
-                        const float d2f = d2_f32<DIM>(dx, me, o, sy, 0.0f);
-                        band |= (d2f >= pp.band_lo) & (d2f <= pp.band_hi);
-                        const bool accept = d2f < pp.band_lo;
-                        add(ex2_approx(na * d2f), accept);
-                        bits |= accept ? bit : 0u;
-                    }
-                    // the self pair gives the row sum's self term only
-                    if (uint32_t(s) - base < 32u) bits &= ~(1u << (uint32_t(s) - base));
-                    if (bits) {
-                        cnt += uint32_t(__popc(bits));
-                        if (nw < uint32_t(nb.cap)) *wp = make_uint2(base, bits);
-                        wp += stride;
-                        ++nw;
-                    }
-                }
-                for (; nw < padded; ++nw, wp += stride)
-                    if (nw < uint32_t(nb.cap)) *wp = make_uint2(0u, 0u);
-            }
+            const float na = -P.pp.a_log2e;
+            bool band;
+            uint32_t nw = search_words<DIM>(uint32_t(s), 0u, rec[s], stride, rec, start, P, nb, cnt,
+                                            band, [&](float d2f, bool accept) {
+                                                add(ex2_approx(na * d2f), accept);
+                                            });
             if (band) {
-                const float4 b = band_accepts<DIM>(uint32_t(s), stride, pos, rec, start, v, nb, rsum, rc);
+                const float4 b = band_words<DIM, true>(uint32_t(s), cell, stride, pos, rec, start, v,
+                                                       nb, rsum, rc);
                 rsum = b.x;
                 rc = b.y;
                 nw = __float_as_uint(b.z);
@@ -1875,7 +1936,7 @@ __global__ void __launch_bounds__(kBlock, (TWO || View::kBatch ? 1536 : 2048) / 
 k_exchange_f32(int n, int64_t stride, const double* __restrict__ pos, const float4* __restrict__ rec,
                const uint32_t* __restrict__ cell, const uint32_t* __restrict__ start,
                const __grid_constant__ View v, const float4* __restrict__ ex,
-               const double* __restrict__ mass, double* __restrict__ mass_out, Nb32 nb,
+               const double* __restrict__ mass, double* __restrict__ mass_out, NbPlanes nb,
                const float2* __restrict__ exb = nullptr, const double* __restrict__ mass_b = nullptr,
                double* __restrict__ mass_b_out = nullptr, double kp = 0.0, double dt = 0.0,
                float kpdt_f = 0.0f, const WalkAhead wa = WalkAhead{}) {
@@ -1897,7 +1958,7 @@ k_exchange_f32(int n, int64_t stride, const double* __restrict__ pos, const floa
     const float4 xs = load_ex<DIM>(ex, uint32_t(s));
     FluxSum f{xs.z, float(2.0 * P.pp.beta), make_float2(xs.x, xs.y)};   // beta folded into W
     FluxSum g{xs.z, f.two_beta, TWO ? __ldg(exb + s) : make_float2(0.0f, 0.0f)};
-    const uint32_t listed = __float_as_uint(xs.w);   // see Nb32
+    const uint32_t listed = __float_as_uint(xs.w);   // see NbPlanes
     if (nb.cap > 0 && (DIM == 3 ? listed <= uint32_t(nb.cap) : listed != kMaskOver)) {
         if constexpr (DIM < 3) {
             const PairFlux<DIM, TWO, true> pf{ex, exb, __ldg(ex + 2 * size_t(s)), -P.pp.a_log2e,
@@ -2042,7 +2103,7 @@ __device__ __forceinline__ void pair_terms(const double* __restrict__ pos,
                                            const uint64_t* __restrict__ image,
                                            const double* __restrict__ tan, int64_t stride,
                                            uint32_t s, uint32_t j, const RealParams& P,
-                                           const uint64_t* table, double* K, double* dK) {
+                                           const double* table, double* K, double* dK) {
     double d2 = 0.0, dot = 0.0;
 #pragma unroll
     for (int a = 0; a < DIM; ++a) {
@@ -2051,13 +2112,73 @@ __device__ __forceinline__ void pair_terms(const double* __restrict__ pos,
         d2 = (a == 0) ? __dmul_rn(d, d) : __fma_rn(d, d, d2);
         dot = __fma_rn(d, dt, dot);
     }
-    *K = pair_kernel<DIM>(image, stride, s, j, table, P.pp.kc).value();
+    *K = pair_kernel<DIM>(image, stride, s, j, table, P.pp.kc);
     *dK = __dmul_rn(*K, __dmul_rn(__fma_rn(d2, P.inv_2D, -dot), P.inv_h2));
 }
 
-// The adjoint passes run on the segment engine with two binary64 terms per
-// pair (smaller segments: two values per entry).
-constexpr int kAdjSeg = 8;
+// The two passes of one particle whose neighbours the words do not hold.
+template <int DIM, class View>
+__device__ __noinline__ double2 adj_search_rowsum(uint32_t s, int64_t stride,
+                                                  const double* __restrict__ pos,
+                                                  const uint64_t* __restrict__ image,
+                                                  const double* __restrict__ tan,
+                                                  const float4* __restrict__ rec,
+                                                  const uint32_t* __restrict__ cell,
+                                                  const uint32_t* __restrict__ start,
+                                                  const double* table, const View& v) {
+    const RealParams& P = v.of_sorted(s);
+    double2 r = make_double2(1.0, 0.0);
+    visit_neighbours<DIM>(s, cell_arg<DIM>(cell, s), stride, rec, pos, start, P,
+                          [&](uint32_t j, float, const float4&) {
+                              if (j == s) return;
+                              double K, dK;
+                              pair_terms<DIM>(pos, image, tan, stride, s, j, P, table, &K, &dK);
+                              r.x = __dadd_rn(r.x, K);
+                              r.y = __dadd_rn(r.y, dK);
+                          });
+    return r;
+}
+
+// One pair's terms of pass B: {W (lambda_j - lambda_s), dW (M_j - M_s)}.
+__device__ __forceinline__ double2 adj_flux(double2 kd, const double* __restrict__ r,
+                                            const double* __restrict__ dr,
+                                            const double* __restrict__ mass,
+                                            const double* __restrict__ lam, uint32_t s, uint32_t j) {
+    const double inv = quot_pos(1.0, __dadd_rn(__ldg(r + s), __ldg(r + j)));
+    const double W = __dmul_rn(__dmul_rn(2.0, kd.x), inv);
+    const double dW = __dmul_rn(
+        __dmul_rn(2.0, inv),
+        __fma_rn(-__dmul_rn(kd.x, inv), __dadd_rn(__ldg(dr + s), __ldg(dr + j)), kd.y));
+    return make_double2(__dmul_rn(W, __dsub_rn(__ldg(lam + j), __ldg(lam + s))),
+                        __dmul_rn(dW, __dsub_rn(__ldg(mass + j), __ldg(mass + s))));
+}
+
+template <int DIM, class View>
+__device__ __noinline__ double2 adj_search_flux(uint32_t s, int64_t stride,
+                                                const double* __restrict__ pos,
+                                                const uint64_t* __restrict__ image,
+                                                const double* __restrict__ tan,
+                                                const float4* __restrict__ rec,
+                                                const uint32_t* __restrict__ cell,
+                                                const uint32_t* __restrict__ start,
+                                                const double* table, const View& v,
+                                                const double* __restrict__ r,
+                                                const double* __restrict__ dr,
+                                                const double* __restrict__ mass,
+                                                const double* __restrict__ lam) {
+    const RealParams& P = v.of_sorted(s);
+    double2 acc = make_double2(0.0, 0.0);
+    visit_neighbours<DIM>(s, cell_arg<DIM>(cell, s), stride, rec, pos, start, P,
+                          [&](uint32_t j, float, const float4&) {
+                              if (j == s) return;
+                              double2 kd;
+                              pair_terms<DIM>(pos, image, tan, stride, s, j, P, table, &kd.x, &kd.y);
+                              const double2 t = adj_flux(kd, r, dr, mass, lam, s, j);
+                              acc.x = __dadd_rn(acc.x, t.x);
+                              acc.y = __dadd_rn(acc.y, t.y);
+                          });
+    return acc;
+}
 
 // Pass A: r_s = sum_j K_sj (self included) and dr_s = sum_j dK_sj / dD.
 template <int DIM, class View>
@@ -2065,31 +2186,40 @@ __global__ void __launch_bounds__(kBlock)
 k_adj_rowsum(int n, int64_t stride, const double* __restrict__ pos,
              const uint64_t* __restrict__ image, const double* __restrict__ tan,
              const float4* __restrict__ rec, const uint32_t* __restrict__ cell,
-             const uint32_t* __restrict__ start, const uint64_t* __restrict__ exp_table,
+             const uint32_t* __restrict__ start, const double* __restrict__ exp_table,
              const __grid_constant__ View v, double* __restrict__ r_out,
-             double* __restrict__ dr_out, NbList<double2> nb) {
-    __shared__ uint64_t table[kExpTable];
-    __shared__ SegShared<kWarpsPerBlock, double2, kAdjSeg> seg;
+             double* __restrict__ dr_out, NbPlanes nb, uint32_t* __restrict__ listed_out,
+             AdjValues kv) {
+    __shared__ double table[kExpTable];
+    __shared__ ChunkShared<double2> chunk;
     for (int t = threadIdx.x; t < kExpTable; t += blockDim.x) table[t] = exp_table[t];
     __syncthreads();
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    const RealParams& P = v.of_sorted(uint32_t(s < n ? s : 0));
-    const bool valid = s < n && P.transfer;
-    double r = 1.0, dr = 0.0;
-    const uint32_t cnt = seg_pairs<DIM>(
-        valid, uint32_t(s), stride, rec, pos, cell, start, P, seg,
-        [&](uint32_t so, uint32_t j, double2& keep) {
-            pair_terms<DIM>(pos, image, tan, stride, so, j, v.of_sorted(so), table, &keep.x, &keep.y);
-            return keep;
+    const uint32_t s = blockIdx.x * blockDim.x + threadIdx.x;
+    const RealParams& P = v.of_sorted(s < uint32_t(n) ? s : 0u);
+    const bool valid = s < uint32_t(n) && P.transfer;
+    uint32_t listed = 0, cnt = 0;
+    if (valid) listed = search_listed<DIM>(s, stride, pos, rec, cell, start, v, P, nb, cnt);
+    double2 sum = make_double2(1.0, 0.0);
+    double2* keep = nullptr;
+    dense_words(
+        s, listed, stride, nb.e, chunk,
+        [&](uint32_t total) { keep = kv.of_warp(s - (threadIdx.x & 31u), total); },
+        [&](uint32_t e, uint32_t so, uint32_t j) {
+            double2 kd;
+            pair_terms<DIM>(pos, image, tan, stride, so, j, v.of_sorted(so), table, &kd.x, &kd.y);
+            if (keep) keep[e] = kd;
+            return kd;
         },
         [&](double2 t) {
-            r = __dadd_rn(r, t.x);
-            dr = __dadd_rn(dr, t.y);
-        }, nb);
-    if (s < n) {
-        r_out[s] = r;
-        dr_out[s] = dr;
-        if (nb.cap > 0) nb.count[s] = valid ? cnt : 0u;
+            sum.x = __dadd_rn(sum.x, t.x);
+            sum.y = __dadd_rn(sum.y, t.y);
+        });
+    if (s < uint32_t(n)) {
+        if (listed == kMaskOver)
+            sum = adj_search_rowsum<DIM>(s, stride, pos, image, tan, rec, cell, start, table, v);
+        r_out[s] = sum.x;
+        dr_out[s] = sum.y;
+        listed_out[s] = listed;
     }
 }
 
@@ -2099,53 +2229,44 @@ k_adj_rowsum(int n, int64_t stride, const double* __restrict__ pos,
 template <int DIM, class View>
 __global__ void __launch_bounds__(kBlock)
 k_adj_exchange(int n, int64_t stride, const double* __restrict__ pos,
-               const uint64_t* __restrict__ image, const double* __restrict__ tan, const float4* __restrict__ rec,
-               const uint32_t* __restrict__ cell, const uint32_t* __restrict__ start,
-               const uint64_t* __restrict__ exp_table, const __grid_constant__ View v,
-               const double* __restrict__ r, const double* __restrict__ dr,
-               const double* __restrict__ mass, const double* __restrict__ lam,
-               double* __restrict__ lam_out, double* __restrict__ gD, NbList<double2> nb) {
-    __shared__ uint64_t table[kExpTable];
-    __shared__ SegShared<kWarpsPerBlock, double2, kAdjSeg> seg;
+               const uint64_t* __restrict__ image, const double* __restrict__ tan,
+               const float4* __restrict__ rec, const uint32_t* __restrict__ cell,
+               const uint32_t* __restrict__ start, const double* __restrict__ exp_table,
+               const __grid_constant__ View v, const double* __restrict__ r,
+               const double* __restrict__ dr, const double* __restrict__ mass,
+               const double* __restrict__ lam, double* __restrict__ lam_out,
+               double* __restrict__ gD, NbPlanes nb, const uint32_t* __restrict__ listed_in,
+               AdjValues kv) {
+    __shared__ double table[kExpTable];
+    __shared__ ChunkShared<double2> chunk;
     for (int t = threadIdx.x; t < kExpTable; t += blockDim.x) table[t] = exp_table[t];
     __syncthreads();
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    const RealParams& P = v.of_sorted(uint32_t(s < n ? s : 0));
-    const bool valid = s < n && P.transfer;
-    double lacc = 0.0, gacc = 0.0;
-    auto terms = [&](uint32_t so, uint32_t j, double K, double dK) {
-        const double inv = quot_pos(1.0, __dadd_rn(__ldg(r + so), __ldg(r + j)));
-        const double W = __dmul_rn(__dmul_rn(2.0, K), inv);
-        const double dW = __dmul_rn(
-            __dmul_rn(2.0, inv),
-            __fma_rn(-__dmul_rn(K, inv), __dadd_rn(__ldg(dr + so), __ldg(dr + j)), dK));
-        return make_double2(__dmul_rn(W, __dsub_rn(__ldg(lam + j), __ldg(lam + so))),
-                            __dmul_rn(dW, __dsub_rn(__ldg(mass + j), __ldg(mass + so))));
-    };
-    auto add = [&](double2 t) {
-        lacc = __dadd_rn(lacc, t.x);
-        gacc = __dadd_rn(gacc, t.y);
-    };
-    const uint32_t listed = (nb.cap > 0 && valid) ? nb.count[s] : 0u;
-    const bool fits = nb.cap > 0 && __all_sync(0xffffffffu, listed <= uint32_t(nb.cap));
-    if (fits) {
-        dense_listed(valid, uint32_t(s), stride, listed, nb, seg,
-                     [&](uint32_t so, uint32_t j, double2 kd) { return terms(so, j, kd.x, kd.y); },
-                     add);
-    } else {
-        seg_pairs<DIM>(
-            valid, uint32_t(s), stride, rec, pos, cell, start, P, seg,
-            [&](uint32_t so, uint32_t j, double2& keep) {
-                pair_terms<DIM>(pos, image, tan, stride, so, j, v.of_sorted(so), table, &keep.x,
-                                &keep.y);
-                return terms(so, j, keep.x, keep.y);
-            },
-            add, NbList<double2>{});
-    }
-    if (s < n) {
+    const uint32_t s = blockIdx.x * blockDim.x + threadIdx.x;
+    const RealParams& P = v.of_sorted(s < uint32_t(n) ? s : 0u);
+    const bool valid = s < uint32_t(n) && P.transfer;
+    const uint32_t listed = valid ? listed_in[s] : 0u;
+    double2 acc = make_double2(0.0, 0.0);
+    const double2* keep = nullptr;
+    dense_words(
+        s, listed, stride, nb.e, chunk,
+        [&](uint32_t total) { keep = kv.of_warp(s - (threadIdx.x & 31u), total); },
+        [&](uint32_t e, uint32_t so, uint32_t j) {
+            double2 kd;
+            if (keep) kd = __ldg(keep + e);
+            else pair_terms<DIM>(pos, image, tan, stride, so, j, v.of_sorted(so), table, &kd.x, &kd.y);
+            return adj_flux(kd, r, dr, mass, lam, so, j);
+        },
+        [&](double2 t) {
+            acc.x = __dadd_rn(acc.x, t.x);
+            acc.y = __dadd_rn(acc.y, t.y);
+        });
+    if (s < uint32_t(n)) {
+        if (listed == kMaskOver)
+            acc = adj_search_flux<DIM>(s, stride, pos, image, tan, rec, cell, start, table, v, r, dr,
+                                       mass, lam);
         const double ls = lam[s];
-        lam_out[s] = valid ? __fma_rn(P.pp.beta, lacc, ls) : ls;
-        gD[s] = valid ? __dmul_rn(__dmul_rn(P.pp.beta, ls), gacc) : 0.0;
+        lam_out[s] = valid ? __fma_rn(P.pp.beta, acc.x, ls) : ls;
+        gD[s] = valid ? __dmul_rn(__dmul_rn(P.pp.beta, ls), acc.y) : 0.0;
     }
 }
 

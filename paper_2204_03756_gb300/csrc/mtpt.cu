@@ -215,7 +215,7 @@ struct mtpt_handle {
     // per-step scratch
     DevBuf<uint32_t> key, perm, cell, count, start;
     DevBuf<unsigned long long> scan_state;   // scan tiles' words + the ticket
-    DevBuf<double2> sortkey;          // (x, id | cell << 32) per slot (k_scatter)
+    DevBuf<double2> sortkey;          // (x, id | cell << 32) per slot (k_scatter); then record_buf
     DevBuf<double2> sortrec;          // payload records per slot (k_scatter_rec)
     bool fresh = false;               // state loaded in input order, not yet sorted
     // bimolecular reaction A + B -> 0: species B's masses (cell order, double
@@ -229,21 +229,25 @@ struct mtpt_handle {
     DevBuf<int> corner_first;
     DevBuf<uint32_t> id_first;
     DevBuf<RealParams> params_dev;
-    DevBuf<double> r64;
+    DevBuf<double> r64;               // the adjoint's row sums
     DevBuf<float4> ex;                // precision form: {m_hi, m_lo, r, list length} per particle
-    DevBuf<uint32_t> nb_j, nb_count;      // binary64 form neighbour lists
+    // what pass 1's search leaves for pass 2 (NbPlanes): the planes, their number
+    // and the words every row is filled up to; in the binary64 form also the
+    // list words and the kernel values (nb_kcap a particle)
+    DevBuf<uint2> nb_e;
+    DevBuf<uint32_t> nb_listed;
     DevBuf<double> nb_k;
-    int nb_cap = 0;
-    DevBuf<uint2> nb32_e;                 // precision form: what pass 2 reads of pass 1's search (Nb32)
-    int nb32_cap = 0, nb32_pad = 0;       // its planes; mask words every row is filled up to
-    DevBuf<uint32_t> adj_nb_j, adj_nb_count;     // adjoint (K, dK) lists
+    int nb_cap = 0, nb_pad = 0, nb_kcap = 0;
+    // the same of the adjoint's passes, its values (K, dK)
+    DevBuf<uint2> adj_nb_e;
+    DevBuf<uint32_t> adj_nb_listed;
     DevBuf<double2> adj_nb_k;
-    int adj_cap = 0;
+    int adj_cap = 0, adj_kcap = 0;
     DevBuf<double> out_tmp;
     // staging copy of host-loaded input and its check tables
     DevBuf<double> stage, chk_box;
     DevBuf<uint32_t> chk_first, chk_flag;
-    DevBuf<uint64_t> exp_table;
+    DevBuf<double> exp_table;
     DevBuf<uint64_t> image;           // fixed-point images of the positions (expneg.cuh), cell order
     // pipelined host I/O: two staging slots each way, per-slot check flags,
     // copy streams and the events that order them against `stream`
@@ -578,10 +582,9 @@ int setup_grids(mtpt_handle* h) {
         h->any_advect |= h->params[k].advect != 0;
     }
     if (cell_base > int64_t(0xffffffffLL) - kScanTile) return MTPT_ERR_INVALID_ARG;
-    // neighbour-list slots: the expected neighbour count of the densest
-    // realisation (density x volume of the cutoff ball) plus four standard
-    // deviations of its Poisson spread plus 4, within [8, 64]; `window`: the
-    // expected candidates of one neighbour row (density x 2 psi x row height)
+    // `expect`: the expected neighbours of the densest realisation (density x
+    // volume of the cutoff ball); `window`: the expected candidates of one
+    // neighbour row (density x 2 psi x the row's cross-section)
     double expect = 0.0, window = 0.0;
     for (int k = 0; k < h->nreal; ++k) {
         const mtpt_params& p = h->reals[k].prm;
@@ -591,36 +594,39 @@ int setup_grids(mtpt_handle* h) {
         const double nk = double(h->reals[k].tiled ? h->reals[k].n_global : h->reals[k].n);
         expect = std::max(expect, nk / vol * ball * std::pow(h->reals[k].psi, double(p.dim)));
         window = std::max(window, nk / vol * 2.0 * h->reals[k].psi *
-                                      (p.dim == 2 ? h->params[k].g.w[1] : 1.0));
+                                      (p.dim >= 2 ? h->params[k].g.w[1] : 1.0) *
+                                      (p.dim == 3 ? h->params[k].g.w[2] : 1.0));
     }
-    const int list_cap =
-        int(std::min(64.0, std::max(8.0, std::ceil(expect + 4.0 * std::sqrt(expect) + 4.0))));
-    h->nb_cap = h->precision == MTPT_FP64 ? list_cap : 0;
-    // the precision form keeps lists in 3-d and mask words per row below it
-    // (32 candidates a word; five standard deviations, at most 8 words); rows
-    // that often need a second word are padded to the same number of words
+    // mask words: 32 candidates each, as many a row as five standard deviations
+    // above the expected window need (at most 8); rows that often need a second
+    // word are padded to the same number of words in the precision form
     // (pass 2 at density 10: 1.6 instead of 2.2 ms for 1e7 particles; at
     // windows that seldom do, the padding only lengthens pass 2: 1.46 instead
     // of 1.20 ms for the 512-realisation ensemble)
-    h->nb32_cap = h->nb32_pad = 0;
-    if (h->precision == MTPT_FP32W && h->dim == 3) {
-        h->nb32_cap = list_cap;
-    } else if (h->precision == MTPT_FP32W) {
-        const double longest = window + 5.0 * std::sqrt(window) + 4.0;
-        const int rows = h->dim == 2 ? 2 * h->params[0].g.reach + 1 : 1;
-        h->nb32_cap = rows * int(std::min(8.0, std::ceil(longest / 32.0)));
-        const double usual = window + 2.0 * std::sqrt(window);
-        if (rows > 1 && usual > 32.0) h->nb32_pad = int(std::min(8.0, std::ceil(usual / 32.0)));
-    }
-    h->adj_cap = list_cap;
+    const int rows = int(std::pow(2.0 * h->params[0].g.reach + 1.0, h->dim - 1.0) + 0.5);
+    const double longest = window + 5.0 * std::sqrt(window) + 4.0;
+    const int words = std::min(255, rows * int(std::min(8.0, std::ceil(longest / 32.0))));
+    const double usual = window + 2.0 * std::sqrt(window);
+    // the precision form's lists in 3-d: four standard deviations of a
+    // particle's Poisson spread plus 4, within [8, 64]
+    const int list_cap =
+        int(std::min(64.0, std::max(8.0, std::ceil(expect + 4.0 * std::sqrt(expect) + 4.0))));
+    const bool f32 = h->precision == MTPT_FP32W;
+    h->nb_cap = f32 && h->dim == 3 ? list_cap : words;
+    h->nb_pad = f32 && h->dim == 2 && usual > 32.0 ? int(std::min(8.0, std::ceil(usual / 32.0))) : 0;
+    // kernel values of the binary64 form, per particle; the adjoint's, where 32
+    // particles share their space, so one standard deviation is six of theirs
+    h->nb_kcap = f32 ? 0 : int(std::min(128.0, std::ceil(expect + 4.0 * std::sqrt(expect) + 4.0)));
+    h->adj_kcap = int(std::min(128.0, std::ceil(expect + std::sqrt(expect) + 4.0)));
+    h->adj_cap = words;
     h->n_cells = cell_base;
     h->n_corners = corner_base;
     h->n_cells_pad = ((h->n_cells + 1 + kScanTile - 1) / kScanTile) * kScanTile;
     return MTPT_OK;
 }
 
-uint64_t* exp_table_host() {
-    static uint64_t table[kExpTable];
+double* exp_table_host() {
+    static double table[kExpTable];
     static std::once_flag once;
     std::call_once(once, []() { fill_exp_table(table); });
     return table;
@@ -674,12 +680,8 @@ int ensure_capacity(mtpt_handle* h, int64_t n, int64_t keep = 0) {
         g.want(h->sortkey, size_t(cap));
         g.want(h->cell, size_t(cap));
         g.want(h->rec, size_t(cap));
-        if (h->precision == MTPT_FP64) {
-            g.want(h->r64, size_t(cap));
-            g.want(h->image, size_t(d) * size_t(cap));
-        } else {
-            g.want(h->ex, size_t(ex_vec(d)) * size_t(cap));
-        }
+        if (h->precision == MTPT_FP64) g.want(h->image, size_t(d) * size_t(cap));
+        else g.want(h->ex, size_t(ex_vec(d)) * size_t(cap));
     }
     if (!h->batch) g.want(h->sortrec, size_t(sort_rec_chunks(d)) * size_t(std::max(cap, h->cap)));
     g.want(h->status, 1);
@@ -745,13 +747,11 @@ int ensure_cells(mtpt_handle* h) {
     g.want(h->start, padded);
     g.want(h->scan_state, padded / kScanTile + 1);   // + the scan's ticket
     g.want(h->corners, size_t(std::max(h->n_corners, 1)));
-    if (h->nb_cap > 0) {
-        const size_t slots = size_t(h->nb_cap) * size_t(h->cap);
-        g.want(h->nb_j, slots);
-        g.want(h->nb_k, slots);
-        g.want(h->nb_count, size_t(h->cap));
+    g.want(h->nb_e, size_t(h->nb_cap) * size_t(h->cap));
+    if (h->nb_kcap > 0) {
+        g.want(h->nb_listed, size_t(h->cap));
+        g.want(h->nb_k, size_t(h->nb_kcap) * size_t(h->cap));
     }
-    if (h->nb32_cap > 0) g.want(h->nb32_e, size_t(h->nb32_cap) * size_t(h->cap));
     if (g.grows()) drop_graph(h);
     MTPT_TRY(g.commit());
     // the scan's words for this grid's tiles
@@ -917,11 +917,22 @@ void reaction_rate(const mtpt_handle* h, double* kp, double* dt) {
     *dt = p.dt;
 }
 
+// The binary64 form's records {row sum, mass}, which pass 2 reads once per
+// neighbour: in the sort keys' array, free once the gather is done.
+double2* record_buf(const mtpt_handle* h) { return h->sortkey.p; }
+
+NbPlanes planes(const mtpt_handle* h) {
+    return {h->nb_e.p, h->nb_e.p ? h->nb_cap : 0, h->nb_pad};
+}
+PairValues kernel_values(const mtpt_handle* h) {
+    return {h->nb_k.p, h->nb_k.p ? h->nb_kcap : 0};
+}
+
 // Pass 2 of the precision form: plain (walk 0), or with the next step's walk
 // into buffer c (1; 2 with advection: see WalkAhead); TWO: both species and
 // the reaction (plain handles only).
 template <int DIM, class View, bool TWO, int WALK>
-int launch_exchange_f32(mtpt_handle* h, const View& vs, int o, int c, const Nb32& nb,
+int launch_exchange_f32(mtpt_handle* h, const View& vs, int o, int c, const NbPlanes& nb,
                         const WalkAhead& wa) {
     double kp = 0.0, dt = 0.0;
     if (TWO) reaction_rate(h, &kp, &dt);
@@ -936,7 +947,7 @@ int launch_exchange_f32(mtpt_handle* h, const View& vs, int o, int c, const Nb32
 }
 
 template <int DIM, class View, bool TWO>
-int launch_exchange_f32(mtpt_handle* h, const View& vs, int o, int c, const Nb32& nb,
+int launch_exchange_f32(mtpt_handle* h, const View& vs, int o, int c, const NbPlanes& nb,
                         bool walk_ahead) {
     WalkAhead wa{};
     if (!walk_ahead) return launch_exchange_f32<DIM, View, TWO, 0>(h, vs, o, c, nb, wa);
@@ -952,7 +963,7 @@ int launch_exchange_f32(mtpt_handle* h, const View& vs, int o, int c, const Nb32
 template <int DIM, class View>
 int launch_pairs_f32(mtpt_handle* h, const View& vs, int o, int c, bool walk_ahead) {
     const int n = int(h->n), block = h->pair_block;
-    const Nb32 nb{h->nb32_e.p, h->nb32_e.p ? h->nb32_cap : 0, h->nb32_pad};
+    const NbPlanes nb = planes(h);
     {
         MTPT_TIMED(h, "rowsum_f32");
         k_rowsum_f32<DIM, View><<<(n + block - 1) / block, block, 0, h->stream>>>(
@@ -985,9 +996,10 @@ int launch_species_b(mtpt_handle* h, int n, int64_t stride, const double* pos_s,
     cudaStream_t st = h->stream;
     {
         MTPT_TIMED(h, "exchange_f64");
+        k_record_mass<<<blocks, kBlock, 0, st>>>(n, h->massb[o].p, record_buf(h));
         k_exchange_f64<DIM, View><<<blocks, kBlock, 0, st>>>(
-            n, stride, pos_s, h->image.p, h->rec.p, h->cell.p, h->start.p, h->exp_table.p, vs, h->r64.p,
-            h->massb[o].p, h->massb[c].p, NbList64{h->nb_j.p, h->nb_k.p, h->nb_count.p, h->nb_cap});
+            n, stride, pos_s, h->image.p, h->rec.p, h->cell.p, h->start.p, h->exp_table.p, vs,
+            record_buf(h), h->massb[c].p, planes(h), h->nb_listed.p, kernel_values(h));
     }
     MTPT_CUDA_TRY(cudaGetLastError());
     double kp, dt;
@@ -1070,11 +1082,11 @@ int launch_step(mtpt_handle* h, int flags, bool walk_ahead) {
         {
             MTPT_TIMED(h, "rowsum_f64");
             k_rowsum_f64<DIM, View><<<blocks, kBlock, 0, st>>>(
-                n, stride, pos_s, h->image.p, h->rec.p, h->cell.p, h->start.p, h->exp_table.p, vs, h->r64.p,
-                h->pair_counter.p, NbList64{h->nb_j.p, h->nb_k.p, h->nb_count.p, h->nb_cap},
+                n, stride, pos_s, h->image.p, h->rec.p, h->cell.p, h->start.p, h->exp_table.p, vs,
+                h->mass[o].p, record_buf(h), h->pair_counter.p, planes(h), h->nb_listed.p,
+                kernel_values(h),
                 h->ntiles > 0 ? h->id[o].p : nullptr);
         }
-        const NbList64 nb64{h->nb_j.p, h->nb_k.p, h->nb_count.p, h->nb_cap};
         if (walk_ahead) {
             // pass 2 plus the next step's walk into buffer c (see WalkAhead)
             WalkAhead wa{h->id[o].p, h->pos[c].p, h->id[c].p, h->key.p, h->count.p,
@@ -1087,16 +1099,16 @@ int launch_step(mtpt_handle* h, int flags, bool walk_ahead) {
             if (h->any_advect)
                 k_exchange_f64<DIM, View, 2><<<blocks, kBlock, 0, st>>>(
                     n, stride, pos_s, h->image.p, h->rec.p, h->cell.p, h->start.p, h->exp_table.p, vs,
-                    h->r64.p, h->mass[o].p, h->mass[c].p, nb64, wa);
+                    record_buf(h), h->mass[c].p, planes(h), h->nb_listed.p, kernel_values(h), wa);
             else
                 k_exchange_f64<DIM, View, 1><<<blocks, kBlock, 0, st>>>(
                     n, stride, pos_s, h->image.p, h->rec.p, h->cell.p, h->start.p, h->exp_table.p, vs,
-                    h->r64.p, h->mass[o].p, h->mass[c].p, nb64, wa);
+                    record_buf(h), h->mass[c].p, planes(h), h->nb_listed.p, kernel_values(h), wa);
         } else {
             MTPT_TIMED(h, "exchange_f64");
             k_exchange_f64<DIM, View><<<blocks, kBlock, 0, st>>>(
-                n, stride, pos_s, h->image.p, h->rec.p, h->cell.p, h->start.p, h->exp_table.p, vs, h->r64.p,
-                h->mass[o].p, h->mass[c].p, nb64);
+                n, stride, pos_s, h->image.p, h->rec.p, h->cell.p, h->start.p, h->exp_table.p, vs,
+                record_buf(h), h->mass[c].p, planes(h), h->nb_listed.p, kernel_values(h));
         }
     } else {
         MTPT_TRY((launch_pairs_f32<DIM, View>(h, vs, o, c, walk_ahead)));
@@ -1288,7 +1300,7 @@ struct HostSnapshot {
     std::vector<RealHost> reals;
     std::vector<RealParams> params;
     int64_t n = 0, n_cells = 0, n_cells_pad = 0;
-    int n_corners = 0, nb_cap = 0, nb32_cap = 0, nb32_pad = 0, adj_cap = 0, cur = 0;
+    int n_corners = 0, nb_cap = 0, nb_pad = 0, nb_kcap = 0, adj_cap = 0, adj_kcap = 0, cur = 0;
     int pair_block = 256;
     bool any_transfer = false, any_walk = false, any_advect = false, fresh = false;
     bool have_row_sums = false, have_particles = false, adj_ready = false;
@@ -1303,7 +1315,8 @@ struct HostSnapshot {
             return false;
         }
         n = h->n; n_cells = h->n_cells; n_cells_pad = h->n_cells_pad;
-        n_corners = h->n_corners; nb_cap = h->nb_cap; nb32_cap = h->nb32_cap; nb32_pad = h->nb32_pad;
+        n_corners = h->n_corners; nb_cap = h->nb_cap; nb_pad = h->nb_pad; nb_kcap = h->nb_kcap;
+        adj_kcap = h->adj_kcap;
         adj_cap = h->adj_cap; cur = h->cur; pair_block = h->pair_block;
         any_transfer = h->any_transfer; any_walk = h->any_walk; any_advect = h->any_advect;
         fresh = h->fresh; have_row_sums = h->have_row_sums; have_particles = h->have_particles;
@@ -1314,7 +1327,8 @@ struct HostSnapshot {
         std::copy(reals.begin(), reals.end(), h->reals);
         std::copy(params.begin(), params.end(), h->params);
         h->n = n; h->n_cells = n_cells; h->n_cells_pad = n_cells_pad;
-        h->n_corners = n_corners; h->nb_cap = nb_cap; h->nb32_cap = nb32_cap; h->nb32_pad = nb32_pad;
+        h->n_corners = n_corners; h->nb_cap = nb_cap; h->nb_pad = nb_pad; h->nb_kcap = nb_kcap;
+        h->adj_kcap = adj_kcap;
         h->adj_cap = adj_cap; h->cur = cur; h->pair_block = pair_block;
         h->any_transfer = any_transfer; h->any_walk = any_walk; h->any_advect = any_advect;
         h->fresh = fresh; h->have_row_sums = have_row_sums; h->have_particles = have_particles;
@@ -1375,7 +1389,7 @@ int load_particles_body(mtpt_handle* h, const int64_t* counts, const double* pos
     drop_graph(h);
     if (!h->exp_table.p) {
         MTPT_TRY(h->exp_table.ensure(kExpTable));
-        MTPT_CUDA_TRY(cudaMemcpyAsync(h->exp_table.p, exp_table_host(), kExpTable * sizeof(uint64_t),
+        MTPT_CUDA_TRY(cudaMemcpyAsync(h->exp_table.p, exp_table_host(), kExpTable * sizeof(double),
                                       cudaMemcpyHostToDevice, h->stream));
     }
     MTPT_TRY(upload_tables(h));
@@ -1761,14 +1775,15 @@ int launch_adjoint_step(mtpt_handle* h) {
     h->adjoint_sweep = false;
     MTPT_TRY(sorted);
     k_take_by_id<<<blocks, kBlock, 0, st>>>(n, h->id[o].p, h->lam_in.p, h->lam_s.p);
-    const NbList<double2> adj_nb{h->adj_nb_j.p, h->adj_nb_k.p, h->adj_nb_count.p,
-                                 h->adj_nb_k.p ? h->adj_cap : 0};
+    const NbPlanes adj_nb{h->adj_nb_e.p, h->adj_cap, 0};
+    const AdjValues adj_kv{h->adj_nb_k.p, h->adj_kcap};
     k_adj_rowsum<DIM, SingleView><<<blocks, kBlock, 0, st>>>(
         n, stride, h->pos[o].p, h->image.p, h->tan[o].p, h->rec.p, h->cell.p, h->start.p, h->exp_table.p, v,
-        h->r64.p, h->dr64.p, adj_nb);
+        h->r64.p, h->dr64.p, adj_nb, h->adj_nb_listed.p, adj_kv);
     k_adj_exchange<DIM, SingleView><<<blocks, kBlock, 0, st>>>(
         n, stride, h->pos[o].p, h->image.p, h->tan[o].p, h->rec.p, h->cell.p, h->start.p, h->exp_table.p, v,
-        h->r64.p, h->dr64.p, h->mass[o].p, h->lam_s.p, h->lam_new.p, h->gD.p, adj_nb);
+        h->r64.p, h->dr64.p, h->mass[o].p, h->lam_s.p, h->lam_new.p, h->gD.p, adj_nb,
+        h->adj_nb_listed.p, adj_kv);
     k_put_by_id<<<blocks, kBlock, 0, st>>>(n, h->id[o].p, h->lam_new.p, h->lam_in.p);
     const int nparts = (n + kReduceThreads - 1) / kReduceThreads;
     k_block_sums<<<nparts, kReduceThreads, 0, st>>>(n, h->gD.p, h->partial.p);
@@ -1806,11 +1821,9 @@ int mtpt_adjoint_forward(mtpt_handle* h, int64_t nsteps, int64_t checkpoint_ever
         MTPT_TRY(b->ensure(cap));
     MTPT_TRY(h->r64.ensure(cap));
     MTPT_TRY(h->image.ensure(size_t(h->dim) * cap));
-    if (h->adj_cap > 0) {
-        MTPT_TRY(h->adj_nb_j.ensure(size_t(h->adj_cap) * cap));
-        MTPT_TRY(h->adj_nb_k.ensure(size_t(h->adj_cap) * cap));
-        MTPT_TRY(h->adj_nb_count.ensure(cap));
-    }
+    MTPT_TRY(h->adj_nb_e.ensure(size_t(h->adj_cap) * cap));
+    MTPT_TRY(h->adj_nb_listed.ensure(cap));
+    MTPT_TRY(h->adj_nb_k.ensure((cap + 31) / 32 * 32 * size_t(h->adj_kcap)));   // whole warps
     MTPT_TRY(h->partial.ensure(size_t((n + kReduceThreads - 1) / kReduceThreads + 1)));
     MTPT_TRY(h->acc.ensure(1));
     h->tangent_on = true;
@@ -1924,10 +1937,9 @@ int mtpt_destroy(mtpt_handle* h) {
     h->tan[0].release(); h->tan[1].release(); h->snaps.release(); h->dr64.release();
     h->lam_in.release(); h->lam_s.release(); h->lam_new.release(); h->gD.release();
     h->partial.release(); h->acc.release();
-    h->nb_j.release(); h->nb_k.release(); h->nb_count.release();
-    h->nb32_e.release();
+    h->nb_e.release(); h->nb_listed.release(); h->nb_k.release();
     h->massb[0].release(); h->massb[1].release(); h->exb.release();
-    h->adj_nb_j.release(); h->adj_nb_k.release(); h->adj_nb_count.release();
+    h->adj_nb_e.release(); h->adj_nb_listed.release(); h->adj_nb_k.release();
     h->tile_counts.release(); h->tile_base.release(); h->tile_cursor.release();
     h->tile_native.release(); h->tile_flag.release(); h->tile_keep.release();
     h->tile_stage.release(); h->tile_tables_dev.release();
@@ -2092,8 +2104,9 @@ int mtpt_get_row_sums(mtpt_handle* h, double* out) {
     MTPT_TRY(ensure_out_tmp(h));
     if (h->n > 0) {
         if (h->precision == MTPT_FP64) {
-            if (h->batch) MTPT_TRY((launch_row_sums_out<BatchView, double>(h, h->r64.p, 1)));
-            else MTPT_TRY((launch_row_sums_out<SingleView, double>(h, h->r64.p, 1)));
+            const double* r = reinterpret_cast<const double*>(record_buf(h));   // .x
+            if (h->batch) MTPT_TRY((launch_row_sums_out<BatchView, double>(h, r, 2)));
+            else MTPT_TRY((launch_row_sums_out<SingleView, double>(h, r, 2)));
         } else {
             // r: .z of the record's last float4
             const int step = 4 * ex_vec(h->dim);
@@ -2405,7 +2418,7 @@ int tile_install_t(mtpt_handle* h, int64_t n_keep, const double* keep, int64_t n
         if (!h->exp_table.p) {
             MTPT_TRY(h->exp_table.ensure(kExpTable));
             MTPT_CUDA_TRY(cudaMemcpyAsync(h->exp_table.p, exp_table_host(),
-                                          kExpTable * sizeof(uint64_t), cudaMemcpyHostToDevice,
+                                          kExpTable * sizeof(double), cudaMemcpyHostToDevice,
                                           h->stream));
         }
         MTPT_TRY(upload_tables(h));
@@ -2805,7 +2818,7 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[MTPT_NOALLOC_SC
 // exponential's table (written once per device at set-up) and the per-call
 // words that the init kernel writes.
 struct NoallocHead {
-    uint64_t exp_table[kExpTable];
+    double exp_table[kExpTable];
     RealParams params;
     int corner_first[2];
     uint32_t status;
@@ -2815,9 +2828,9 @@ struct NoallocHead {
 constexpr size_t kNoallocHeadBytes = (sizeof(NoallocHead) + 255) & ~size_t(255);
 
 // Worst case of the per-call pieces carved after the head, at n =
-// MTPT_NOALLOC_MAX_PARTICLES: 3-d binary64 form, 124 bytes per particle (mass
+// MTPT_NOALLOC_MAX_PARTICLES: 3-d binary64 form, 116 bytes per particle (mass
 // copy 8, sorted positions 24 and mass 8, two id arrays 8, key 4, permutation
-// 4, sort key 16, cell 4, rec 16, row sum 8, images 24); the
+// 4, sort key 16, cell 4, rec 16, images 24; 2-d binary32 form 116); the
 // cell grid capped at 4 n + 64 cells (setup_grid), so count and start hold at
 // most that many plus one cells padded to a scan tile, and the corner tables
 // at most the sum of the per-axis cell counts (<= their product + 2); each
@@ -2825,7 +2838,7 @@ constexpr size_t kNoallocHeadBytes = (sizeof(NoallocHead) + 255) & ~size_t(255);
 constexpr size_t kNoallocMaxCells = 4 * size_t(MTPT_NOALLOC_MAX_PARTICLES) + 64;
 constexpr size_t kNoallocMaxCellsPad = (kNoallocMaxCells + 1 + kScanTile - 1) / kScanTile * kScanTile;
 constexpr size_t kNoallocWorstBytes =
-    kNoallocHeadBytes + 124 * size_t(MTPT_NOALLOC_MAX_PARTICLES) +
+    kNoallocHeadBytes + 116 * size_t(MTPT_NOALLOC_MAX_PARTICLES) +
     2 * sizeof(uint32_t) * kNoallocMaxCellsPad +
     sizeof(unsigned long long) * (kNoallocMaxCellsPad / kScanTile + 1) +
     sizeof(float2) * (kNoallocMaxCells + 2) + 16 * 256;
@@ -2850,7 +2863,7 @@ int noalloc_scratch(void** out) {
         cudaError_t e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
         if (e == cudaSuccess)
             e = cudaMemcpy(static_cast<NoallocHead*>(p)->exp_table, exp_table_host(),
-                           kExpTable * sizeof(uint64_t), cudaMemcpyHostToDevice);
+                           kExpTable * sizeof(double), cudaMemcpyHostToDevice);
         if (e != cudaSuccess) (void)cudaGetLastError();
         g_noalloc_err[dev] = e;
         g_noalloc_addr[dev] = (e == cudaSuccess) ? p : nullptr;
@@ -2933,7 +2946,6 @@ extern "C" int mtpt_step_noalloc(const mtpt_params* params, int64_t n, uint64_t 
     h.cell.p = cv.take<uint32_t>(size_t(n));
     h.rec.p = cv.take<float4>(size_t(n));
     if (h.precision == MTPT_FP64) {
-        h.r64.p = cv.take<double>(size_t(n));
         h.image.p = cv.take<uint64_t>(size_t(d) * size_t(n));
     } else {
         h.ex.p = cv.take<float4>(size_t(ex_vec(d)) * size_t(n));
@@ -2943,18 +2955,18 @@ extern "C" int mtpt_step_noalloc(const mtpt_params* params, int64_t n, uint64_t 
     h.start.p = cv.take<uint32_t>(cells_pad);
     h.scan_state.p = cv.take<unsigned long long>(cells_pad / kScanTile + 1);   // + the ticket
     if (cv.overflow) return MTPT_ERR_TOO_LARGE;
-    // neighbour lists or masks in what is left, where they fit whole (the same
-    // sums either way: without them pass 2 searches, which took 73 instead of
+    // what pass 1 keeps for pass 2 in what is left, whole or not at all (the same
+    // sums either way: without it pass 2 searches, which took 73 instead of
     // 68 us for the call at 20,011 particles in 2-d, precision form)
-    const size_t list_bytes = size_t(n) * (size_t(h.nb_cap) * 12 + 4 + size_t(h.nb32_cap) * 8);
-    if (cv.used + 4 * 256 + list_bytes > size_t(MTPT_NOALLOC_SCRATCH_BYTES)) {
-        h.nb_cap = h.nb32_cap = h.nb32_pad = 0;
-    } else if (h.nb_cap > 0) {
-        h.nb_k.p = cv.take<double>(size_t(h.nb_cap) * size_t(n));
-        h.nb_j.p = cv.take<uint32_t>(size_t(h.nb_cap) * size_t(n));
-        h.nb_count.p = cv.take<uint32_t>(size_t(n));
-    } else if (h.nb32_cap > 0) {
-        h.nb32_e.p = cv.take<uint2>(size_t(h.nb32_cap) * size_t(n));
+    const bool f64 = h.precision == MTPT_FP64;
+    auto fits = [&](size_t bytes) {
+        return cv.used + 2 * 256 + bytes <= size_t(MTPT_NOALLOC_SCRATCH_BYTES);
+    };
+    if (fits(size_t(n) * (8 * size_t(h.nb_cap) + (f64 ? 4 : 0)))) {
+        h.nb_e.p = cv.take<uint2>(size_t(h.nb_cap) * size_t(n));
+        if (f64) h.nb_listed.p = cv.take<uint32_t>(size_t(n));
+        if (f64 && fits(8 * size_t(n) * size_t(h.nb_kcap)))
+            h.nb_k.p = cv.take<double>(size_t(n) * size_t(h.nb_kcap));
     }
 
     // The handle's buffer pairs: index 0 is the caller's state (positions are

@@ -17,17 +17,25 @@ SRC = """
 using namespace mtpt;
 extern "C" {
 double kernel(int dim, const double* x, const double* y, double a, double psi) {
-    uint64_t table[kExpTable];
+    double table[kExpTable];
     fill_exp_table(table);
     const KernelConsts c = kernel_consts(a, psi);
     uint64_t d2h = 0;
     for (int k = 0; k < dim; ++k) d2h += axis_square(x_image(x[k], c.x_shift), x_image(y[k], c.x_shift));
-    return gauss_fixed(d2h, table, c).value();
+    return gauss_fixed(d2h, table, c);
 }
-double weight(double K, double ra, double rb) { return weight_fixed(K, ra, rb); }
-double row_sum(int n, const unsigned long long* unit) {
+double weight(double K, double ra, double rb) {
+    const FixedWeight w = weight_fixed(K, ra, rb);
+    return std::ldexp(double(w.q), w.x);
+}
+double flux_sum(int n, const double* dm, const double* K, const double* ra, const double* rb) {
+    FluxSum64 f;
+    for (int k = 0; k < n; ++k) f.add(dm[k], weight_fixed(K[k], ra[k], rb[k]));
+    return f.value();
+}
+double row_sum(int n, const double* K) {
     RowSum r;
-    for (int k = 0; k < n; ++k) r.add(unit[k]);
+    for (int k = 0; k < n; ++k) r.add(unit_of(K[k]));
     return r.value();
 }
 }
@@ -45,8 +53,10 @@ def lib(tmp_path_factory):
     dp = ctypes.POINTER(ctypes.c_double)
     so.kernel.argtypes = [ctypes.c_int, dp, dp, ctypes.c_double, ctypes.c_double]
     so.weight.argtypes = [ctypes.c_double] * 3
-    so.row_sum.argtypes = [ctypes.c_int, ctypes.POINTER(ctypes.c_ulonglong)]
-    so.kernel.restype = so.weight.restype = so.row_sum.restype = ctypes.c_double
+    so.row_sum.argtypes = [ctypes.c_int, dp]
+    so.flux_sum.argtypes = [ctypes.c_int, dp, dp, dp, dp]
+    for f in (so.kernel, so.weight, so.row_sum, so.flux_sum):
+        f.restype = ctypes.c_double
     getcontext().prec = 50
     return so
 
@@ -63,8 +73,9 @@ def test_kernel_against_decimal(lib, lam, h2, side, dim):
     psi, a = lam * np.sqrt(2.0 * h2), 1.0 / (2.0 * h2)
     # |T's error| <= 3 + 6 d units of 2^-60 (psi^2) in d2 and the constant's
     # 2^-63: a relative error of K of lam^2 (3 + 6 d) 2^-60 at most, plus the
-    # rounding of T (4 units of at most lam^2 2^-57) and of K itself (2^-53)
-    bound = 2.0 ** -53 + lam ** 2 * ((3 + 6 * dim) * 2.0 ** -60 + 4 * 2.0 ** -57) + 2.0 ** -58
+    # rounding of T (4 units of at most lam^2 2^-57) and of the table, the series
+    # and their product (2^-53 each)
+    bound = 3 * 2.0 ** -53 + lam ** 2 * ((3 + 6 * dim) * 2.0 ** -60 + 4 * 2.0 ** -57) + 2.0 ** -58
     for it in range(300):
         x = rng.uniform(-side, side, dim) * (1e-3 if it % 3 == 0 else 1.0)
         y = x + rng.uniform(-1.0, 1.0, dim) * psi / np.sqrt(dim) * (it % 7 != 0)
@@ -93,11 +104,41 @@ def test_weight_against_decimal(lib):
 
 
 @pytest.mark.parametrize("n", [0, 1, 2, 3, 4, 7, 8, 63, 64, 1000, 5000])
-def test_row_sum_is_exact(lib, n):
+def test_row_sum_against_decimal(lib, n):
+    """1 + sum K: every term to 2^-62, one rounding at the end."""
     rng = np.random.default_rng(n)
-    unit = rng.integers(0, 2 ** 62, n, dtype=np.uint64, endpoint=True)
+    K = np.exp(-rng.uniform(0.0, 9.0, n))
     if n > 2:
-        unit[:2] = 2 ** 62
-    want = Decimal(1) + sum((Decimal(int(u)) for u in unit), Decimal(0)) / Decimal(2) ** 62
-    got = lib.row_sum(n, unit.ctypes.data_as(ctypes.POINTER(ctypes.c_ulonglong)))
-    assert abs(Decimal(got) - want) <= Decimal(2.0 ** -53) * want
+        K[:2] = (1.0, 2.0 ** -70)
+    want = Decimal(1) + sum((Decimal(float(k)) for k in K), Decimal(0))
+    got = lib.row_sum(n, _ptr(K))
+    assert abs(Decimal(got) - want) <= Decimal(2.0 ** -53) * want + n * Decimal(2) ** -62
+
+
+@pytest.mark.parametrize("n", [0, 1, 2, 5, 31, 33, 64, 2000])
+@pytest.mark.parametrize("spread", [0, 40, 1000])
+def test_flux_sum_against_decimal(lib, n, spread):
+    """sum W dm over masses of one size and of sizes 2^+-spread apart: every term
+    to 2^-52 of the largest, and the sum rounded once."""
+    rng = np.random.default_rng(n + spread)
+    dm = rng.uniform(-1.0, 1.0, n) * 2.0 ** rng.integers(-spread, 1, n)
+    if n > 3:
+        dm[:2] = (0.0, -0.0)
+    K, ra, rb = np.exp(-rng.uniform(0.0, 9.0, n)), 1.0 + rng.uniform(0, 9, n), 1.0 + rng.uniform(0, 9, n)
+    terms = [2 * Decimal(float(k)) / (Decimal(float(a)) + Decimal(float(b))) * Decimal(float(m))
+             for k, a, b, m in zip(K, ra, rb, dm)]
+    want = sum(terms, Decimal(0))
+    big = max([abs(t) for t in terms], default=Decimal(0))
+    got = lib.flux_sum(n, _ptr(dm), _ptr(K), _ptr(ra), _ptr(rb))
+    assert abs(Decimal(got) - want) <= Decimal(2.0 ** -52) * n * big + Decimal(2.0 ** -53) * abs(want)
+    assert lib.flux_sum(n, _ptr(-dm), _ptr(K), _ptr(ra), _ptr(rb)) == -got or n > 1
+
+
+def test_flux_sum_of_differences_that_are_not_finite(lib):
+    one = np.ones(3)
+    for dm, want in ((np.array([1.0, np.inf, 2.0]), np.inf), (np.array([-np.inf, 5.0, 1.0]), -np.inf),
+                     (np.array([np.inf, -np.inf, 1.0]), np.nan), (np.array([1.0, np.nan, 1.0]), np.nan)):
+        got = lib.flux_sum(3, _ptr(dm), _ptr(one), _ptr(one), _ptr(one))
+        assert got == want or (np.isnan(want) and np.isnan(got))
+    big = np.array([1.5e308, -1.5e308, 1e300])
+    assert np.isfinite(lib.flux_sum(3, _ptr(big), _ptr(one), _ptr(one), _ptr(one)))
