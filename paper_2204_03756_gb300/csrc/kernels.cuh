@@ -13,10 +13,12 @@
 //   mass[s], id[s]       binary64 mass, uint32 input index (keys the walk)
 //   cell[s]              linear cell index of particle s (written and read in 3-d
 //                        only: below 3-d the record carries the cell coordinates)
-//   rec[s]               float4: binary32 offsets of the particle from its
+//   rec (load_rec)       float4: binary32 offsets of the particle from its
 //                        cell's lower corner (x, y, z), and in .w the cell's
 //                        x index (a small integer, exact in binary32); in
-//                        2-d, .z (no offset there) holds the cell's y index
+//                        2-d, .z (no offset there) holds the cell's y index.
+//                        Stored two particles a 32-byte block, component by
+//                        component: {x0 x1 w0 w1 y0 y1 z0 z1}
 //   start[c]             first particle of cell c (exclusive prefix sum)
 // Cells are row-major (x fastest), so the three cells (cx-1..cx+1) of one
 // neighbour row are one contiguous particle range; inside a cell particles
@@ -147,6 +149,63 @@ struct BatchView {
 __device__ __forceinline__ long long order_key(double x) {
     const long long b = __double_as_longlong(x);
     return b ^ ((b >> 63) & 0x7fffffffffffffffLL);
+}
+
+// A particle's record rec (see the layout above).
+__device__ __forceinline__ size_t rec_at(uint32_t j) { return size_t(j & ~1u) * 4u + (j & 1u); }
+__device__ __forceinline__ float4 load_rec(const float* __restrict__ rec, uint32_t j) {
+    const float* q = rec + rec_at(j);
+    return make_float4(__ldg(q), __ldg(q + 4), __ldg(q + 6), __ldg(q + 2));
+}
+__device__ __forceinline__ void store_rec(float* __restrict__ rec, uint32_t j, const float4& v) {
+    float* q = rec + rec_at(j);
+    q[0] = v.x;
+    q[2] = v.w;
+    q[4] = v.y;
+    q[6] = v.z;
+}
+
+// Two binary32 values in one register pair, one operation on both: each rounds as the scalar one.
+__device__ __forceinline__ uint64_t pack2(float a, float b) {
+    uint64_t v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(a), "f"(b));
+    return v;
+}
+__device__ __forceinline__ float2 unpack2(uint64_t v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+// The records of particles j and j + 1, j even, as one 32-byte load.
+struct RecPair {
+    uint64_t x, w, y, z;
+};
+__device__ __forceinline__ RecPair load_rec_pair(const float* __restrict__ rec, uint32_t j) {
+    RecPair r;
+    asm("ld.global.nc.v4.b64 {%0, %1, %2, %3}, [%4];"
+        : "=l"(r.x), "=l"(r.w), "=l"(r.y), "=l"(r.z)
+        : "l"(rec + size_t(j) * 4u));
+    return r;
 }
 
 // x split as hi + lo with hi = x truncated to binary32 (integer operations
@@ -671,7 +730,7 @@ k_gather(int n, int64_t stride, const uint32_t* __restrict__ perm,
          const double* __restrict__ pos_in, const double* __restrict__ mass_in,
          uint32_t* __restrict__ id_out, double* __restrict__ pos_out,
          double* __restrict__ mass_out, uint32_t* __restrict__ cell_out,
-         float4* __restrict__ rec_out,
+         float* __restrict__ rec_out,
          const float2* __restrict__ corners, uint32_t* __restrict__ rid_out,
          const __grid_constant__ View v, const double* __restrict__ tan_in = nullptr,
          double* __restrict__ tan_out = nullptr, const double* __restrict__ mass_b_in = nullptr,
@@ -724,7 +783,8 @@ k_gather(int n, int64_t stride, const uint32_t* __restrict__ perm,
             off[a] = __fadd_rn(__fsub_rn(xh, cr.x), __fsub_rn(xlo, cr.y));
         }
     }
-    rec_out[dst] = make_float4(off[0], off[1], DIM == 2 ? float(cc[1]) : off[2], float(cc[0]));
+    store_rec(rec_out, dst,
+              make_float4(off[0], off[1], DIM == 2 ? float(cc[1]) : off[2], float(cc[0])));
 }
 
 // Sort of a freshly loaded single run, whose particles arrive in input order
@@ -781,7 +841,7 @@ __global__ void __launch_bounds__(kBlock)
 k_gather_rec(int n, int64_t stride, const double2* __restrict__ recs,
              const uint32_t* __restrict__ start, uint32_t* __restrict__ id_out,
              double* __restrict__ pos_out, double* __restrict__ mass_out,
-             uint32_t* __restrict__ cell_out, float4* __restrict__ rec_out,
+             uint32_t* __restrict__ cell_out, float* __restrict__ rec_out,
              const float2* __restrict__ corners,
              const __grid_constant__ SingleView v, double* __restrict__ tan_out,
              uint64_t* __restrict__ image_out) {
@@ -833,7 +893,8 @@ k_gather_rec(int n, int64_t stride, const double2* __restrict__ recs,
             off[a] = __fadd_rn(__fsub_rn(xh, cr.x), __fsub_rn(xlo, cr.y));
         }
     }
-    rec_out[dst] = make_float4(off[0], off[1], DIM == 2 ? float(cc[1]) : off[2], float(cc[0]));
+    store_rec(rec_out, dst,
+              make_float4(off[0], off[1], DIM == 2 ? float(cc[1]) : off[2], float(cc[0])));
 }
 
 // ---------------------------------------------------------------------------
@@ -896,6 +957,13 @@ __device__ __forceinline__ float dx_f32(const float4& me, const float4& o, float
     return __fmaf_rn(__fsub_rn(o.w, me.w), wx, __fsub_rn(o.x, me.x));
 }
 
+// The same of the candidate with index j.
+__device__ __forceinline__ float dx_of(const float4& me, const float* __restrict__ rec, uint32_t j,
+                                       float wx) {
+    const float* q = rec + rec_at(j);
+    return __fmaf_rn(__fsub_rn(__ldg(q + 2), me.w), wx, __fsub_rn(__ldg(q), me.x));
+}
+
 template <int DIM>
 __device__ __forceinline__ float d2_f32(float dx, const float4& me, const float4& o, float sy,
                                         float sz) {
@@ -936,7 +1004,7 @@ __device__ __forceinline__ float row_gap(int d, float off, float w, float eps) {
 // row(j0, j3, rx, sy, sz) is called for every row that can hold a neighbour.
 template <int DIM, class Row>
 __device__ __forceinline__ void for_each_row(uint32_t cell, const float4 me,
-                                             const float4* __restrict__ rec,
+                                             const float* __restrict__ rec,
                                              const uint32_t* __restrict__ start,
                                              const RealParams& P, Row&& row) {
     const Grid& g = P.g;
@@ -971,7 +1039,7 @@ __device__ __forceinline__ void for_each_row(uint32_t cell, const float4 me,
             const uint32_t j3 = hi;
             while (lo < hi) {
                 const uint32_t mid = (lo + hi) >> 1;
-                if (dx_f32(me, __ldg(rec + mid), wx) < -rx) lo = mid + 1;
+                if (dx_of(me, rec, mid, wx) < -rx) lo = mid + 1;
                 else hi = mid;
             }
             row(lo, j3, rx, sy, sz);
@@ -982,18 +1050,18 @@ __device__ __forceinline__ void for_each_row(uint32_t cell, const float4 me,
 // visit(j, d2f, rec_j) is called for every neighbour j of s (s included).
 template <int DIM, class Visit>
 __device__ __forceinline__ void visit_neighbours(uint32_t s, uint32_t cell, int64_t stride,
-                                                 const float4* __restrict__ rec,
+                                                 const float* __restrict__ rec,
                                                  const double* __restrict__ pos,
                                                  const uint32_t* __restrict__ start,
                                                  const RealParams& P, Visit&& visit) {
     const PairParams& pp = P.pp;
-    const float4 me = rec[s];
+    const float4 me = load_rec(rec, s);
     const float wx = P.g.wf[0];
     for_each_row<DIM>(cell, me, rec, start, P,
                       [&](uint32_t j0, uint32_t j3, float rx, float sy, float sz) {
 #pragma unroll 2
         for (uint32_t j = j0; j < j3; ++j) {
-            const float4 o = __ldg(rec + j);
+            const float4 o = load_rec(rec, j);
             const float dx = dx_f32(me, o, wx);
             if (dx > rx) break;
             const float d2f = d2_f32<DIM>(dx, me, o, sy, sz);
@@ -1012,55 +1080,63 @@ __device__ __noinline__ bool exact_within(const double* __restrict__ pos, int64_
     return exact_d2<DIM>(pos, stride, s, j) <= psi2;
 }
 
+// The candidates inside the narrow band around the cutoff that the exact test
+// accepts: visit(j, d2f) in candidate order.
+template <int DIM, class Visit>
+__device__ __forceinline__ void scan_band(uint32_t s, uint32_t cell, int64_t stride,
+                                          const float* __restrict__ rec,
+                                          const double* __restrict__ pos,
+                                          const uint32_t* __restrict__ start, const RealParams& P,
+                                          Visit&& visit) {
+    const PairParams& pp = P.pp;
+    const float4 me = load_rec(rec, s);
+    const float wx = P.g.wf[0];
+    for_each_row<DIM>(cell, me, rec, start, P,
+                      [&](uint32_t j0, uint32_t j3, float rx, float sy, float sz) {
+        for (uint32_t j = j0; j < j3; ++j) {
+            const float4 o = load_rec(rec, j);
+            const float dx = dx_f32(me, o, wx);
+            if (dx > rx) break;
+            const float d2f = d2_f32<DIM>(dx, me, o, sy, sz);
+            if (d2f >= pp.band_lo && d2f <= pp.band_hi &&
+                exact_within<DIM>(pos, stride, s, j, pp.psi2))
+                visit(j, d2f);
+        }
+    });
+}
+
 // As visit_neighbours, but calls visit(j, d2f, accept) for every candidate of
-// the windows (the pass bodies run without a branch on the cutoff).  A
-// candidate inside the narrow band around the cutoff gets the exact binary64
-// test in place, or, with DEFER_BAND, is first visited as rejected and, if
-// the particle met any, a second walk visits those the exact test accepts
-// (rare: the band holds ~1e-5 of candidates; measured faster for the row
-// sums, not for the exchange).
+// the windows.  A candidate inside the narrow band around the cutoff gets the
+// exact binary64 test in place, or, with DEFER_BAND, is first visited as
+// rejected and, if the particle met any, a second walk visits those the exact
+// test accepts (the order in which 3-d lists hold their neighbours).
 template <int DIM, bool DEFER_BAND, class Visit>
 __device__ __forceinline__ void scan_neighbours(uint32_t s, uint32_t cell, int64_t stride,
-                                                const float4* __restrict__ rec,
+                                                const float* __restrict__ rec,
                                                 const double* __restrict__ pos,
                                                 const uint32_t* __restrict__ start,
                                                 const RealParams& P, Visit&& visit) {
     const PairParams& pp = P.pp;
-    const float4 me = rec[s];
+    const float4 me = load_rec(rec, s);
     const float wx = P.g.wf[0];
     bool band = false;
     for_each_row<DIM>(cell, me, rec, start, P,
                       [&](uint32_t j0, uint32_t j3, float rx, float sy, float sz) {
         for (uint32_t j = j0; j < j3; ++j) {
-            const float4 o = __ldg(rec + j);
+            const float4 o = load_rec(rec, j);
             const float dx = dx_f32(me, o, wx);
             if (dx > rx) break;
             const float d2f = d2_f32<DIM>(dx, me, o, sy, sz);
-            if constexpr (DEFER_BAND) {
-                band |= (d2f >= pp.band_lo) & (d2f <= pp.band_hi);
-                visit(j, d2f, d2f < pp.band_lo);
-            } else {
-                bool accept = d2f < pp.band_lo;
-                if (d2f >= pp.band_lo && d2f <= pp.band_hi)
-                    accept = exact_within<DIM>(pos, stride, s, j, pp.psi2);
-                visit(j, d2f, accept);
-            }
+            const bool inside = d2f >= pp.band_lo && d2f <= pp.band_hi;
+            bool accept = d2f < pp.band_lo;
+            if constexpr (DEFER_BAND) band |= inside;
+            else if (inside) accept = exact_within<DIM>(pos, stride, s, j, pp.psi2);
+            visit(j, d2f, accept);
         }
     });
-    if (DEFER_BAND && band) {
-        for_each_row<DIM>(cell, me, rec, start, P,
-                          [&](uint32_t j0, uint32_t j3, float rx, float sy, float sz) {
-            for (uint32_t j = j0; j < j3; ++j) {
-                const float4 o = __ldg(rec + j);
-                const float dx = dx_f32(me, o, wx);
-                if (dx > rx) break;
-                const float d2f = d2_f32<DIM>(dx, me, o, sy, sz);
-                if (d2f >= pp.band_lo && d2f <= pp.band_hi &&
-                    exact_within<DIM>(pos, stride, s, j, pp.psi2))
-                    visit(j, d2f, true);
-            }
-        });
-    }
+    if (DEFER_BAND && band)
+        scan_band<DIM>(s, cell, stride, rec, pos, start, P,
+                       [&](uint32_t j, float d2f) { visit(j, d2f, true); });
 }
 
 __device__ __forceinline__ float ex2_approx(float x) {
@@ -1109,14 +1185,28 @@ __device__ __forceinline__ uint32_t mask_word(uint32_t words, uint32_t neighbour
     return words <= uint32_t(cap) && neighbours < (1u << 24) - 1u ? neighbours << 8 | words : kMaskOver;
 }
 
-// The search of one particle: its windows row by row, the accepted candidates
+// The search of one particle, its windows row by row, two candidates (one
+// block of records) at a time: one 32-byte load, the distances as packed
+// binary32 operations, the tests on the distances' bits (ordered like the
+// values).  A window starts at an even index and may end at an odd one, so
+// candidates outside it are masked off.  With WORDS, the accepted candidates
 // (those below the narrow band around the cutoff; `band` reports candidates
-// inside it) into mask words at e (its first plane's entry).  cand(d2f,
-// accept) is called for every candidate, the self pair included.  Returns the
-// words written or wanted; cnt receives the accepted neighbours j != s.
-template <int DIM, class Cand>
+// inside it) go into mask words; EACH calls cand(j, d2f, accept) for every
+// candidate, the self pair included.  Returns the words written or wanted;
+// cnt receives the accepted neighbours j != s (WORDS only).
+//
+// Bound by instruction issue: singly, a candidate took about 20 instructions
+// of which the pair shares or packs all but three.  The bisection to a
+// window's first candidate pays only in long rows: of up to kBisectFrom
+// candidates the loop takes those on the left too (never accepted), two at a
+// time.  Pass 1 of the precision form: 175 -> 158 us by pairs and 142 without
+// the bisection (4e6 particles in 2-d, three cells hold 5.4), 191 -> 187 (2e6 in
+// 3-d, 2.6); at density 10 (54 candidates a row) 1.55 -> 1.18 ms by pairs, with
+// the bisection (1.31 without).
+constexpr uint32_t kBisectFrom = 24;
+template <int DIM, bool WORDS, bool EACH, class Cand>
 __device__ __forceinline__ uint32_t search_words(uint32_t s, uint32_t cell, const float4 me,
-                                                 int64_t stride, const float4* __restrict__ rec,
+                                                 int64_t stride, const float* __restrict__ rec,
                                                  const uint32_t* __restrict__ start,
                                                  const RealParams& P, const NbPlanes& nb,
                                                  uint32_t& cnt, bool& band, Cand&& cand) {
@@ -1126,10 +1216,11 @@ __device__ __forceinline__ uint32_t search_words(uint32_t s, uint32_t cell, cons
     cell_coords_rec<DIM>(cell, me, P, c);
     const float wx = g.wf[0], eps = pp.trim_eps;
     const int R = g.reach, xlo = max(c[0] - R, 0), xhi = min(c[0] + R, g.n[0] - 1);
-    uint2* wp = nb.e + s;          // next mask word
+    const uint32_t lo_bits = __float_as_uint(pp.band_lo);
+    uint32_t nearest = 0xffffffffu;    // least (bits of d2f) - lo_bits, unsigned
+    uint2* wp = nb.e + s;              // next mask word
     uint32_t nw = 0;
-    cnt = 0;
-    band = false;
+    if constexpr (WORDS) cnt = 0;
     // one row's window and candidates: an empty window where the row is outside
     // the grid or beyond the cutoff (for_each_row has the windows' derivation)
     auto row = [&](int dy, int dz) {
@@ -1150,41 +1241,78 @@ __device__ __forceinline__ uint32_t search_words(uint32_t s, uint32_t cell, cons
                           uint32_t(g.n[0]) * uint32_t(g.n[1]) * uint32_t(g.n[2]), kChkRow)) {
                 j = __ldg(start + rowc + xlo);
                 j3 = __ldg(start + rowc + xhi + 1);
-                uint32_t hi = j3;
-                while (j < hi) {
-                    const uint32_t mid = (j + hi) >> 1;
-                    if (dx_f32(me, __ldg(rec + mid), wx) < -rx) j = mid + 1;
-                    else hi = mid;
+                if (j3 - j > kBisectFrom) {
+                    uint32_t hi = j3;
+                    while (hi - j > 2u) {
+                        const uint32_t mid = (j + hi) >> 1;
+                        if (dx_of(me, rec, mid, wx) < -rx) j = mid + 1;
+                        else hi = mid;
+                    }
                 }
             }
         }
         const uint32_t padded = nw + uint32_t(nb.pad);
-        while (j < j3) {
-            const uint32_t base = j, end = min(j3, base + 32u);
-            uint32_t bits = 0, bit = 1;
-            for (; j < end; ++j, bit <<= 1) {
-                const float4 o = __ldg(rec + j);
-                const float dx = dx_f32(me, o, wx);
-                if (dx > rx) {
-                    j3 = j;
-                    break;
+        const uint32_t first = j;
+        uint32_t b = j & ~1u;
+        // one block of two candidates; false past the window's right end: in x
+        // order, every later candidate lies farther right still (a second
+        // candidate outside the window is the row's last)
+        uint32_t bits = 0;                 // accepted, latest candidate lowest
+        auto block = [&]() {
+            const RecPair o = load_rec_pair(rec, b);
+            const uint64_t dx = fma2(sub2(o.w, pack2(me.w, me.w)), pack2(wx, wx),
+                                     sub2(o.x, pack2(me.x, me.x)));
+            uint64_t d2 = mul2(dx, dx);
+            if constexpr (DIM >= 2) {
+                const uint64_t ey = add2(sub2(o.y, pack2(me.y, me.y)), pack2(sy, sy));
+                if constexpr (DIM == 2) {
+                    d2 = fma2(dx, dx, mul2(ey, ey));
+                } else {
+                    const uint64_t ez = add2(sub2(o.z, pack2(me.z, me.z)), pack2(sz, sz));
+                    d2 = fma2(dx, dx, fma2(ey, ey, mul2(ez, ez)));
                 }
-                const float d2f = d2_f32<DIM>(dx, me, o, sy, sz);
-                band |= (d2f >= pp.band_lo) & (d2f <= pp.band_hi);
-                const bool accept = d2f < pp.band_lo;
-                cand(d2f, accept);
-                bits |= accept ? bit : 0u;
             }
-            if (s - base < 32u) bits &= ~(1u << (s - base));   // the self pair is no neighbour
-            if (bits) {
-                cnt += uint32_t(__popc(bits));
-                if (nw < uint32_t(nb.cap)) *wp = make_uint2(base, bits);
-                wp += stride;
-                ++nw;
+            const float2 d = unpack2(d2);
+            const uint32_t t0 = __float_as_uint(d.x) - lo_bits, t1 = __float_as_uint(d.y) - lo_bits;
+            nearest = min(nearest, min(t0, t1));
+            if constexpr (WORDS) {
+                bits = __funnelshift_l(t0, bits, 1);   // the sign: below the band
+                bits = __funnelshift_l(t1, bits, 1);
+            }
+            if constexpr (EACH) {
+                cand(b, d.x, int32_t(t0) < 0 && b >= first);
+                cand(b + 1u, d.y, int32_t(t1) < 0 && b + 1u < j3);
+            }
+            b += 2u;
+            return !(unpack2(dx).y > rx);
+        };
+        if constexpr (!WORDS) {
+            while (b < j3 && block()) {}
+        } else {
+            while (b < j3) {
+                const uint32_t base = b, end = min(j3, base + 32u);
+                bits = 0;
+                bool more = true;
+                do {
+                    more = block();
+                } while (more && b < end);
+                bits = __brev(bits) >> (32u - (b - base));
+                if (base < first) bits &= ~1u;
+                if (j3 - base < 32u) bits &= (1u << (j3 - base)) - 1u;
+                if (s - base < 32u) bits &= ~(1u << (s - base));   // the self pair is no neighbour
+                if (bits) {
+                    cnt += uint32_t(__popc(bits));
+                    if (nw < uint32_t(nb.cap)) *wp = make_uint2(base, bits);
+                    wp += stride;
+                    ++nw;
+                }
+                if (!more) break;
             }
         }
-        for (; nw < padded; ++nw, wp += stride)
-            if (nw < uint32_t(nb.cap)) *wp = make_uint2(0u, 0u);
+        if constexpr (WORDS) {
+            for (; nw < padded; ++nw, wp += stride)
+                if (nw < uint32_t(nb.cap)) *wp = make_uint2(0u, 0u);
+        }
     };
     // rows in a fixed order for the whole warp
     if constexpr (DIM == 1) {
@@ -1198,6 +1326,7 @@ __device__ __forceinline__ uint32_t search_words(uint32_t s, uint32_t cell, cons
 #pragma unroll 1
             for (int dy = -R; dy <= R; ++dy) row(dy, dz);
     }
+    band = nearest <= __float_as_uint(pp.band_hi) - lo_bits;
     return nw;
 }
 
@@ -1210,12 +1339,12 @@ __device__ __forceinline__ uint32_t search_words(uint32_t s, uint32_t cell, cons
 template <int DIM, bool SUM, class View>
 __device__ __noinline__ float4 band_words(uint32_t s, const uint32_t* __restrict__ cell, int64_t stride,
                                           const double* __restrict__ pos,
-                                          const float4* __restrict__ rec,
+                                          const float* __restrict__ rec,
                                           const uint32_t* __restrict__ start, const View& v,
                                           const NbPlanes& nb, float rsum, float rc) {
     const RealParams& P = v.of_sorted(s);
     const PairParams& pp = P.pp;
-    const float4 me = rec[s];
+    const float4 me = load_rec(rec, s);
     uint32_t cnt = 0, nw = 0;
     for_each_row<DIM>(cell_arg<DIM>(cell, s), me, rec, start, P,
                       [&](uint32_t j, uint32_t j3, float rx, float sy, float sz) {
@@ -1223,7 +1352,7 @@ __device__ __noinline__ float4 band_words(uint32_t s, const uint32_t* __restrict
             const uint32_t base = j, end = min(j3, base + 32u);
             uint32_t bits = 0;
             for (; j < end; ++j) {
-                const float4 o = __ldg(rec + j);
+                const float4 o = load_rec(rec, j);
                 const float dx = dx_f32(me, o, P.g.wf[0]);
                 if (dx > rx) {
                     j3 = j;
@@ -1371,15 +1500,15 @@ __device__ __forceinline__ void dense_words(uint32_t s, uint32_t listed, int64_t
 template <int DIM, class View>
 __device__ __forceinline__ uint32_t search_listed(uint32_t s, int64_t stride,
                                                   const double* __restrict__ pos,
-                                                  const float4* __restrict__ rec,
+                                                  const float* __restrict__ rec,
                                                   const uint32_t* __restrict__ cell,
                                                   const uint32_t* __restrict__ start, const View& v,
                                                   const RealParams& P, const NbPlanes& nb,
                                                   uint32_t& cnt) {
     bool band;
     const uint32_t c = cell_arg<DIM>(cell, s);
-    uint32_t nw = search_words<DIM>(s, c, rec[s], stride, rec, start, P, nb, cnt, band,
-                                    [](float, bool) {});
+    uint32_t nw = search_words<DIM, true, false>(s, c, load_rec(rec, s), stride, rec, start, P, nb,
+                                                 cnt, band, [](uint32_t, float, bool) {});
     if (band) {
         const float4 b = band_words<DIM, false>(s, cell, stride, pos, rec, start, v, nb, 0.0f, 0.0f);
         nw = __float_as_uint(b.z);
@@ -1393,7 +1522,7 @@ template <int DIM, class View>
 __device__ __noinline__ double search_rowsum(uint32_t s, int64_t stride,
                                              const double* __restrict__ pos,
                                              const uint64_t* __restrict__ image,
-                                             const float4* __restrict__ rec,
+                                             const float* __restrict__ rec,
                                              const uint32_t* __restrict__ cell,
                                              const uint32_t* __restrict__ start,
                                              const double* table, const View& v) {
@@ -1419,7 +1548,7 @@ __device__ __noinline__ double search_rowsum(uint32_t s, int64_t stride,
 template <int DIM, class View>
 __global__ void __launch_bounds__(kBlock, DIM == 3 ? 5 : 6)
 k_rowsum_f64(int n, int64_t stride, const double* __restrict__ pos,
-             const uint64_t* __restrict__ image, const float4* __restrict__ rec,
+             const uint64_t* __restrict__ image, const float* __restrict__ rec,
              const uint32_t* __restrict__ cell, const uint32_t* __restrict__ start,
              const double* __restrict__ exp_table, const __grid_constant__ View v,
              const double* __restrict__ mass, double2* __restrict__ rm,
@@ -1533,7 +1662,7 @@ template <int DIM, class View>
 __device__ __noinline__ double search_flux_f64(uint32_t s, int64_t stride,
                                                const double* __restrict__ pos,
                                                const uint64_t* __restrict__ image,
-                                               const float4* __restrict__ rec,
+                                               const float* __restrict__ rec,
                                                const uint32_t* __restrict__ cell,
                                                const uint32_t* __restrict__ start,
                                                const double* table, const View& v,
@@ -1554,7 +1683,7 @@ __device__ __noinline__ double search_flux_f64(uint32_t s, int64_t stride,
 template <int DIM, class View, int WALK = 0>
 __global__ void __launch_bounds__(kBlock, 5)
 k_exchange_f64(int n, int64_t stride, const double* __restrict__ pos,
-               const uint64_t* __restrict__ image, const float4* __restrict__ rec,
+               const uint64_t* __restrict__ image, const float* __restrict__ rec,
                const uint32_t* __restrict__ cell, const uint32_t* __restrict__ start,
                const double* __restrict__ exp_table, const __grid_constant__ View v,
                const double2* __restrict__ rm, double* __restrict__ mass_out, NbPlanes nb,
@@ -1647,8 +1776,8 @@ __device__ __forceinline__ float4 load_ex(const float4* __restrict__ ex, uint32_
 // with masks; 1e7 with 57 each: 6.5 and 1.5 ms).  In 3-d (3.6 neighbours over
 // nine rows) the list is the shorter of the two.
 template <int DIM, class View>
-__global__ void __launch_bounds__(kBlock, (DIM == 3 ? 1536 : 2048) / kBlock)
-k_rowsum_f32(int n, int64_t stride, const double* __restrict__ pos, const float4* __restrict__ rec,
+__global__ void __launch_bounds__(kBlock, (DIM == 3 || View::kBatch ? 1536 : 2048) / kBlock)
+k_rowsum_f32(int n, int64_t stride, const double* __restrict__ pos, const float* __restrict__ rec,
              const uint32_t* __restrict__ cell, const uint32_t* __restrict__ start,
              const __grid_constant__ View v, const double* __restrict__ mass,
              float4* __restrict__ ex, unsigned long long* __restrict__ pair_counter,
@@ -1674,23 +1803,29 @@ k_rowsum_f32(int n, int64_t stride, const double* __restrict__ pos, const float4
             const float na = -P.pp.a_log2e;
             const uint32_t cap = uint32_t(nb.cap);
             uint2* lp = nb.e + s;          // slot `cnt` of s
-            scan_neighbours<DIM, true>(uint32_t(s), cell[s], stride, rec, pos, start, P,
-                                 [&](uint32_t j, float d2f, bool accept) {
-                                     const float K = ex2_approx(na * d2f);
-                                     add(K, accept);
-                                     const bool keep = accept && j != uint32_t(s);
-                                     if (keep && cnt < cap) *lp = make_uint2(j, __float_as_uint(K));
-                                     if (keep) lp += stride;
-                                     cnt += keep ? 1u : 0u;
-                                 });
+            bool band;
+            auto visit = [&](uint32_t j, float d2f, bool accept) {
+                const float K = ex2_approx(na * d2f);
+                add(K, accept);
+                const bool keep = accept && j != uint32_t(s);
+                if (keep && cnt < cap) *lp = make_uint2(j, __float_as_uint(K));
+                if (keep) lp += stride;
+                cnt += keep ? 1u : 0u;
+            };
+            uint32_t unused;
+            search_words<DIM, false, true>(uint32_t(s), cell[s], load_rec(rec, uint32_t(s)), stride, rec,
+                                           start, P, nb, unused, band, visit);
+            // the band's exact accepts come last
+            if (band)
+                scan_band<DIM>(uint32_t(s), cell[s], stride, rec, pos, start, P,
+                               [&](uint32_t j, float d2f) { visit(j, d2f, true); });
             list_word = cnt;
         } else {
             const float na = -P.pp.a_log2e;
             bool band;
-            uint32_t nw = search_words<DIM>(uint32_t(s), 0u, rec[s], stride, rec, start, P, nb, cnt,
-                                            band, [&](float d2f, bool accept) {
-                                                add(ex2_approx(na * d2f), accept);
-                                            });
+            uint32_t nw = search_words<DIM, true, true>(
+                uint32_t(s), 0u, load_rec(rec, uint32_t(s)), stride, rec, start, P, nb, cnt, band,
+                [&](uint32_t, float d2f, bool accept) { add(ex2_approx(na * d2f), accept); });
             if (band) {
                 const float4 b = band_words<DIM, true>(uint32_t(s), cell, stride, pos, rec, start, v,
                                                        nb, rsum, rc);
@@ -1705,7 +1840,7 @@ k_rowsum_f32(int n, int64_t stride, const double* __restrict__ pos, const float4
         split_double(mass[s], &mhi, &mlo);
         const float4 m = make_float4(mhi, mlo, __fsub_rn(rsum, rc), __uint_as_float(list_word));
         if constexpr (DIM == 3) ex[s] = m;
-        else store_pair_rec(ex, uint32_t(s), rec[s], m);
+        else store_pair_rec(ex, uint32_t(s), load_rec(rec, uint32_t(s)), m);
         // with ghost_id (a tile), pairs are counted for the tile's own particles only
         if (ghost_id && (ghost_id[s] & kGhostBit)) cnt = 0;
     }
@@ -1747,7 +1882,7 @@ struct FluxSum {
 template <int DIM, class View>
 __device__ __noinline__ float2 search_flux(uint32_t s, int64_t stride,
                                            const double* __restrict__ pos,
-                                           const float4* __restrict__ rec,
+                                           const float* __restrict__ rec,
                                            const uint32_t* __restrict__ cell,
                                            const uint32_t* __restrict__ start, const View& v,
                                            const float4* __restrict__ ex, float rs, float2 ms,
@@ -1837,7 +1972,7 @@ k_react(int n, double* __restrict__ ma, double* __restrict__ mb, double kp, doub
 template <int DIM, class View>
 __device__ __noinline__ float4 search_flux2(uint32_t s, int64_t stride,
                                             const double* __restrict__ pos,
-                                            const float4* __restrict__ rec,
+                                            const float* __restrict__ rec,
                                             const uint32_t* __restrict__ cell,
                                             const uint32_t* __restrict__ start, const View& v,
                                             const float4* __restrict__ ex,
@@ -1933,7 +2068,7 @@ __device__ __noinline__ float4 words_flux(const uint2* __restrict__ e, int64_t s
 // The bounds hold for blocks of 128 too (the tuning's other block size).
 template <int DIM, class View, bool TWO = false, int WALK = 0>
 __global__ void __launch_bounds__(kBlock, (TWO || View::kBatch ? 1536 : 2048) / kBlock)
-k_exchange_f32(int n, int64_t stride, const double* __restrict__ pos, const float4* __restrict__ rec,
+k_exchange_f32(int n, int64_t stride, const double* __restrict__ pos, const float* __restrict__ rec,
                const uint32_t* __restrict__ cell, const uint32_t* __restrict__ start,
                const __grid_constant__ View v, const float4* __restrict__ ex,
                const double* __restrict__ mass, double* __restrict__ mass_out, NbPlanes nb,
@@ -2065,7 +2200,7 @@ k_exchange_f32(int n, int64_t stride, const double* __restrict__ pos, const floa
 // Test support: every accepted ordered pair j != s as (id_s, id_j).
 template <int DIM, class View>
 __global__ void __launch_bounds__(kBlock)
-k_emit_pairs(int n, int64_t stride, const double* __restrict__ pos, const float4* __restrict__ rec,
+k_emit_pairs(int n, int64_t stride, const double* __restrict__ pos, const float* __restrict__ rec,
              const uint32_t* __restrict__ cell, const uint32_t* __restrict__ start,
              const uint32_t* __restrict__ id, const __grid_constant__ View v,
              unsigned long long cap, unsigned long long* __restrict__ counter,
@@ -2122,7 +2257,7 @@ __device__ __noinline__ double2 adj_search_rowsum(uint32_t s, int64_t stride,
                                                   const double* __restrict__ pos,
                                                   const uint64_t* __restrict__ image,
                                                   const double* __restrict__ tan,
-                                                  const float4* __restrict__ rec,
+                                                  const float* __restrict__ rec,
                                                   const uint32_t* __restrict__ cell,
                                                   const uint32_t* __restrict__ start,
                                                   const double* table, const View& v) {
@@ -2158,7 +2293,7 @@ __device__ __noinline__ double2 adj_search_flux(uint32_t s, int64_t stride,
                                                 const double* __restrict__ pos,
                                                 const uint64_t* __restrict__ image,
                                                 const double* __restrict__ tan,
-                                                const float4* __restrict__ rec,
+                                                const float* __restrict__ rec,
                                                 const uint32_t* __restrict__ cell,
                                                 const uint32_t* __restrict__ start,
                                                 const double* table, const View& v,
@@ -2185,7 +2320,7 @@ template <int DIM, class View>
 __global__ void __launch_bounds__(kBlock)
 k_adj_rowsum(int n, int64_t stride, const double* __restrict__ pos,
              const uint64_t* __restrict__ image, const double* __restrict__ tan,
-             const float4* __restrict__ rec, const uint32_t* __restrict__ cell,
+             const float* __restrict__ rec, const uint32_t* __restrict__ cell,
              const uint32_t* __restrict__ start, const double* __restrict__ exp_table,
              const __grid_constant__ View v, double* __restrict__ r_out,
              double* __restrict__ dr_out, NbPlanes nb, uint32_t* __restrict__ listed_out,
@@ -2230,7 +2365,7 @@ template <int DIM, class View>
 __global__ void __launch_bounds__(kBlock)
 k_adj_exchange(int n, int64_t stride, const double* __restrict__ pos,
                const uint64_t* __restrict__ image, const double* __restrict__ tan,
-               const float4* __restrict__ rec, const uint32_t* __restrict__ cell,
+               const float* __restrict__ rec, const uint32_t* __restrict__ cell,
                const uint32_t* __restrict__ start, const double* __restrict__ exp_table,
                const __grid_constant__ View v, const double* __restrict__ r,
                const double* __restrict__ dr, const double* __restrict__ mass,

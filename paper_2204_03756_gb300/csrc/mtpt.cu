@@ -224,7 +224,7 @@ struct mtpt_handle {
     double react_k = 0.0;
     DevBuf<double> massb[2];
     DevBuf<float2> exb;               // precision form: species B's mass split for pass 2
-    DevBuf<float4> rec;
+    DevBuf<float> rec;                // two particles a block (kernels.cuh)
     DevBuf<float2> corners;
     DevBuf<int> corner_first;
     DevBuf<uint32_t> id_first;
@@ -646,6 +646,9 @@ int build_corners(mtpt_handle* h, const RealParams* params_dev, const int* first
 // (the adjoint's), so one allocation serves every record sort.
 int64_t sort_rec_chunks(int dim) { return (2 + 2 * dim + 1) / 2; }
 
+// Floats of n particles' records: whole blocks of two.
+size_t rec_floats(int64_t n) { return size_t((n + 1) / 2) * 8; }
+
 // float4 per particle of the precision form's pair records (ExRec).
 int ex_vec(int dim) { return dim == 3 ? ExRec<3>::kVec : ExRec<2>::kVec; }
 
@@ -679,7 +682,7 @@ int ensure_capacity(mtpt_handle* h, int64_t n, int64_t keep = 0) {
         g.want(h->perm, size_t(cap));
         g.want(h->sortkey, size_t(cap));
         g.want(h->cell, size_t(cap));
-        g.want(h->rec, size_t(cap));
+        g.want(h->rec, rec_floats(cap));
         if (h->precision == MTPT_FP64) g.want(h->image, size_t(d) * size_t(cap));
         else g.want(h->ex, size_t(ex_vec(d)) * size_t(cap));
     }
@@ -2944,7 +2947,7 @@ extern "C" int mtpt_step_noalloc(const mtpt_params* params, int64_t n, uint64_t 
     h.perm.p = cv.take<uint32_t>(size_t(n));
     h.sortkey.p = cv.take<double2>(size_t(n));
     h.cell.p = cv.take<uint32_t>(size_t(n));
-    h.rec.p = cv.take<float4>(size_t(n));
+    h.rec.p = cv.take<float>(rec_floats(n));
     if (h.precision == MTPT_FP64) {
         h.image.p = cv.take<uint64_t>(size_t(d) * size_t(n));
     } else {
