@@ -92,6 +92,12 @@ MTPT_HD double from_mantissa(uint64_t w, int e) {
     return double_of((uint64_t(e + 1022) << 52) + (w >> 11) + ((w >> 10) & 1u));
 }
 
+// v 2^e for a normal result, 0 for v = 0.
+MTPT_HD double scaled(uint64_t v, int e) {
+    const int z = clz64(v | 1u);
+    return v == 0u ? 0.0 : from_mantissa(v << z, e + 63 - z);
+}
+
 // X = round(x 2^S) mod 2^64 (0 for subnormals, infinities and NaN, which no
 // accepted pair has beyond its own zero).
 MTPT_HD uint64_t x_image(double x, int shift) {
@@ -106,11 +112,13 @@ MTPT_HD uint64_t x_image(double x, int shift) {
     return (b >> 63) ? 0u - v : v;
 }
 
-// |dx|^2 of one axis, in units of 2^(64 - 2 S).
-MTPT_HD uint64_t axis_square(uint64_t xi, uint64_t xj) {
+// |x_i - x_j| of one axis in units of 2^-S, and its square in units of
+// 2^(64 - 2 S).
+MTPT_HD uint64_t axis_distance(uint64_t xi, uint64_t xj) {
     const uint64_t d = xi - xj;
-    return square_hi((d >> 63) ? 0u - d : d);
+    return (d >> 63) ? 0u - d : d;
 }
+MTPT_HD uint64_t axis_square(uint64_t xi, uint64_t xj) { return square_hi(axis_distance(xi, xj)); }
 
 // exp(-a d2) from d2h = d2 2^(2 S - 64).
 MTPT_HD double gauss_fixed(uint64_t d2h, const double* __restrict__ table, const KernelConsts& c) {
@@ -146,43 +154,59 @@ MTPT_HD uint64_t unit_of(double K) {
 struct FixedWeight {
     uint64_t q;
     int x;
+    MTPT_HD double value() const { return scaled(q, x); }
+};
+struct Reciprocal {
+    uint32_t y;                  // 2^93 / d, d = (ra + rb) 2^(1085 - e) in [2^62, 2^64)
+    int64_t e1;                  // 2^61 (1 - d y / 2^93)
+    int e;
+    MTPT_HD Reciprocal(double ra, double rb) {
+        const uint64_t ab = bits_of(ra), bb = bits_of(rb);
+        const uint64_t frac = 0xfffffffffffffull, one = 0x10000000000000ull;
+        const int ea = int(ab >> 52), eb = int(bb >> 52);
+        e = ea > eb ? ea : eb;
+        const uint64_t d = ((((ab & frac) | one) << 10) >> (e - ea)) +
+                           ((((bb & frac) | one) << 10) >> (e - eb));
+        const uint32_t dh = uint32_t(d >> 32), dl = uint32_t(d);
+#if defined(__CUDA_ARCH__)
+        float s;
+        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(s) : "f"(__uint2float_rn(dh)));
+        y = __float2uint_rz(s * 2305843009213693952.0f);                // 2^61; [2^29, 2^31]
+#else
+        y = uint32_t(2305843009213693952.0f / float(dh));
+#endif
+        const int64_t e0 = int64_t((1ull << 61) - mul_wide(dh, y));     // |e0| < 2^40
+        y += uint32_t((int64_t(int32_t(e0 >> 19)) * int64_t(y)) >> 42);
+        e1 = int64_t((1ull << 61) - mul_wide(dh, y) - (mul_wide(dl, y) >> 32));   // < 2^34
+    }
+    // m / (ra + rb) for m = mk 2^(ek - 1085), mk in [2^62, 2^63), as q 2^x
+    MTPT_HD FixedWeight times(uint64_t mk, int ek) const {
+        const uint64_t q0 = mul_wide(uint32_t(mk >> 32), y) + (mul_wide(uint32_t(mk), y) >> 32);
+        return {q0 + uint64_t((int64_t(int32_t(e1 >> 3)) * int64_t(q0 >> 31)) >> 27), ek - e - 61};
+    }
+    // 2 K / (ra + rb) and 1 / (ra + rb)
+    MTPT_HD FixedWeight weight(double K) const {
+        const uint64_t kb = bits_of(K);
+        return times(((kb & 0xfffffffffffffull) | 0x10000000000000ull) << 10, int(kb >> 52) + 1);
+    }
+    MTPT_HD FixedWeight inverse() const { return times(1ull << 62, 1023); }
 };
 MTPT_HD FixedWeight weight_fixed(double K, double ra, double rb) {
-    const uint64_t kb = bits_of(K), ab = bits_of(ra), bb = bits_of(rb);
-    const uint64_t frac = 0xfffffffffffffull, one = 0x10000000000000ull;
-    const int ek = int(kb >> 52), ea = int(ab >> 52), eb = int(bb >> 52);
-    const int e = ea > eb ? ea : eb;
-    const uint64_t mk = ((kb & frac) | one) << 10;                      // [2^62, 2^63)
-    const uint64_t d = ((((ab & frac) | one) << 10) >> (e - ea)) +
-                       ((((bb & frac) | one) << 10) >> (e - eb));       // [2^62, 2^64)
-    const uint32_t dh = uint32_t(d >> 32), dl = uint32_t(d);
-    // y = 2^93 / d, in [2^29, 2^31]
-#if defined(__CUDA_ARCH__)
-    float s;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(s) : "f"(__uint2float_rn(dh)));
-    uint32_t y = __float2uint_rz(s * 2305843009213693952.0f);           // 2^61
-#else
-    uint32_t y = uint32_t(2305843009213693952.0f / float(dh));
-#endif
-    const int64_t e0 = int64_t((1ull << 61) - mul_wide(dh, y));         // |e0| < 2^40
-    y += uint32_t((int64_t(int32_t(e0 >> 19)) * int64_t(y)) >> 42);
-    const int64_t e1 = int64_t((1ull << 61) - mul_wide(dh, y) - (mul_wide(dl, y) >> 32));   // < 2^34
-    const uint64_t q0 = mul_wide(uint32_t(mk >> 32), y) + (mul_wide(uint32_t(mk), y) >> 32);
-    const uint64_t q = q0 + uint64_t((int64_t(int32_t(e1 >> 3)) * int64_t(q0 >> 31)) >> 27);
-    // q = mk / d 2^61; K = mk 2^(ek - 1085), ra + rb = d 2^(e - 1085)
-    return {q, ek - e - 60};
+    return Reciprocal(ra, rb).weight(K);
 }
 
 // A particle's flux sum, sum W dm over its neighbours with dm a difference of
-// masses: 64-bit integers against the largest exponent so far (each term keeps
-// 54 bits or more, and the sum five bits above the terms, or more when it
-// needs them).  A term changes sign exactly when dm does.  Differences that
-// are not finite make the sum what binary64 additions would.
+// masses, or the sum of plain binary64 terms: 64-bit integers against the
+// largest exponent so far (each term keeps 54 bits or more, and the sum five
+// bits above the terms, or more when it needs them).  A term changes sign
+// exactly when dm does.  Terms that are not finite make the sum what binary64
+// additions would.
 struct FluxSum64 {
     int64_t acc = 0;
     int x = -100000;             // the sum is acc 2^x
     double special = 0.0;
-    MTPT_HD void add(double dm, const FixedWeight& w) {
+    // W dm (or, without w, dm itself)
+    MTPT_HD void add(double dm, const FixedWeight* w) {
         const uint64_t b = bits_of(dm);
         const int e = int(b >> 52) & 0x7ff;
         if (e == 0x7ff) {
@@ -190,9 +214,9 @@ struct FluxSum64 {
             return;
         }
         const uint64_t m = (b & 0xfffffffffffffull) | (e ? 0x10000000000000ull : 0u);
-        // dm = m 2^(e - 1075), subnormals with e = 1
-        int64_t g = int64_t(mul_hi(m << 10, w.q) >> 3);                 // below 2^58
-        int y = (e ? e : 1) - 1075 - 10 + 64 + 3 + w.x;
+        // dm = m 2^(e - 1075), subnormals with e = 1; the term is g 2^y, g < 2^58
+        int64_t g = int64_t(w ? mul_hi(m << 10, w->q) >> 3 : m << 5);
+        const int y = (e ? e : 1) - 1075 + (w ? -10 + 64 + 3 + w->x : -5);
         g = (b >> 63) ? -g : g;
         const int up = y - x;
         if (up > 0) {
@@ -207,6 +231,20 @@ struct FluxSum64 {
             x += 4;
         }
     }
+    MTPT_HD void add(double dm, const FixedWeight& w) { add(dm, &w); }
+    // a product of two binary64 values, the first one normal or zero
+    MTPT_HD void add_product(double a, double b) {
+        const uint64_t ab = bits_of(a);
+        const int e = int(ab >> 52) & 0x7ff;
+        if (e == 0x7ff) {
+            special += a * b;
+            return;
+        }
+        const FixedWeight w{e ? ((ab & 0xfffffffffffffull) | 0x10000000000000ull) << 9 : 0u,
+                            e - 1075 - 9};
+        add((ab >> 63) ? -b : b, &w);
+    }
+    MTPT_HD void add(double term) { add(term, nullptr); }
     MTPT_HD double value() const {
         if (!(special == 0.0)) return special;
         if (acc == 0) return 0.0;

@@ -243,31 +243,6 @@ __device__ __forceinline__ double f32_to_f64(float f) {
     return __hiloint2double(int(sign | ((e + 896u) << 20) | (m >> 3)), int(m << 29));
 }
 
-// Head of a binary64 x >= 0 with x < 2^128 as binary32, truncated (integer
-// operations only); 0 below 2^-126.
-__device__ __forceinline__ float head_f32(double x) {
-    const uint32_t whi = uint32_t(__double2hiint(x));
-    const uint32_t wlo = uint32_t(__double2loint(x));
-    const int e = int(whi >> 20);
-    const uint32_t bits = (uint32_t(e - 896) << 23) | ((whi & 0xfffffu) << 3) | (wlo >> 29);
-    return e < 897 ? 0.0f : __uint_as_float(bits);
-}
-
-// num / den for num >= 0 and 1 <= den < 2^127 with binary64 fma only: a
-// binary32 reciprocal seed (relative error below 2^-21 after the head
-// truncation), one Newton-Raphson step for 1/den (error below 2^-41), then
-// the quotient and one residual correction q + (num - den q) / den (P.
-// Markstein, "IA-64 and Elementary Functions", 2000, ch. 8), which leaves an
-// error below one unit in the last place.  Five binary64 operations.
-__device__ __forceinline__ double quot_pos(double num, double den) {
-    float y0;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y0) : "f"(head_f32(den)));
-    double y = f32_to_f64(y0);
-    y = __fma_rn(y, __fma_rn(-den, y, 1.0), y);
-    const double q = __dmul_rn(num, y);
-    return __fma_rn(__fma_rn(-den, q, num), y, q);
-}
-
 // True when x is an infinity or a NaN (integer test on the exponent field).
 __device__ __forceinline__ bool not_finite(double x) {
     return (uint32_t(__double2hiint(x)) & 0x7ff00000u) == 0x7ff00000u;
@@ -1390,8 +1365,9 @@ __device__ __noinline__ float4 band_words(uint32_t s, const uint32_t* __restrict
 // spends as many instructions on handing them out: pass 1 took 405 us that way
 // instead of 381, pass 2 with the walk 389 instead of 322, 4e6 particles in
 // 2-d.)
-// The adjoint's pair terms are mostly binary64 operations, which cost the same
-// however many lanes are active, so there a warp works in two parts: each lane
+// The adjoint's pair terms keep seven or eight binary64 operations, which cost the
+// same however many lanes are active (a thread per particle took 45 and 51 us a
+// pass where this takes 36 and 40), so there a warp works in two parts: each lane
 // searches its particle and leaves mask words; then the warp takes the words'
 // neighbours in lane-major order, kChunk at a time: the lanes write out their
 // neighbours' indexes (shared memory), all 32 evaluate one each until the chunk
@@ -2233,24 +2209,43 @@ k_emit_pairs(int n, int64_t stride, const double* __restrict__ pos, const float*
 // and step t adds beta sum_i lambda_{t+1,i} sum_j dW_ij (M_j - M_i) to dL/dD.
 // Pair-set and bin changes contribute zero almost everywhere.
 // ---------------------------------------------------------------------------
+// The positions enter through their fixed-point images: distances, d2 and K are
+// integer work, and the binary64 unit keeps seven operations a pair (the
+// tangents' differences and products, K's last product, dK).  Returns K and
+// h^2 dK/dD: the passes carry dK and dr times h^2, and pass B divides its sum.
 template <int DIM>
-__device__ __forceinline__ void pair_terms(const double* __restrict__ pos,
-                                           const uint64_t* __restrict__ image,
-                                           const double* __restrict__ tan, int64_t stride,
-                                           uint32_t s, uint32_t j, const RealParams& P,
-                                           const double* table, double* K, double* dK) {
-    double d2 = 0.0, dot = 0.0;
+__device__ __forceinline__ double2 pair_terms(const uint64_t* __restrict__ image,
+                                              const double* __restrict__ tan, int64_t stride,
+                                              uint32_t s, uint32_t j, const RealParams& P,
+                                              const double* table) {
+    const KernelConsts& kc = P.pp.kc;
+    uint64_t d2h = 0;
+    double dot = 0.0;
 #pragma unroll
     for (int a = 0; a < DIM; ++a) {
-        const double d = __dsub_rn(__ldg(pos + a * stride + s), __ldg(pos + a * stride + j));
+        const uint64_t xi = __ldg(image + a * stride + s), xj = __ldg(image + a * stride + j);
+        const uint64_t d = axis_distance(xi, xj);
+        d2h += square_hi(d);
+        const double sign_d = double_of(bits_of(scaled(d, -kc.x_shift)) |
+                                        ((xi - xj) & 0x8000000000000000ull));
         const double dt = __dsub_rn(__ldg(tan + a * stride + s), __ldg(tan + a * stride + j));
-        d2 = (a == 0) ? __dmul_rn(d, d) : __fma_rn(d, d, d2);
-        dot = __fma_rn(d, dt, dot);
+        dot = a == 0 ? __dmul_rn(sign_d, dt) : __fma_rn(sign_d, dt, dot);
     }
-    *K = pair_kernel<DIM>(image, stride, s, j, table, P.pp.kc);
-    *dK = __dmul_rn(*K, __dmul_rn(__fma_rn(d2, P.inv_2D, -dot), P.inv_h2));
+    const double K = gauss_fixed(d2h, table, kc);
+    const double d2 = scaled(d2h, 64 - 2 * kc.x_shift);
+    return make_double2(K, __dmul_rn(K, __fma_rn(d2, P.inv_2D, -dot)));
 }
 
+// The sums of pass A: the row sum exactly, its derivative in 64-bit integers.
+struct AdjRowSum {
+    RowSum r;
+    FluxSum64 dr;
+    __device__ __forceinline__ void add(double2 kd) {
+        r.add(unit_of(kd.x));
+        dr.add(kd.y);
+    }
+    __device__ __forceinline__ double2 value() const { return make_double2(r.value(), dr.value()); }
+};
 // The two passes of one particle whose neighbours the words do not hold.
 template <int DIM, class View>
 __device__ __noinline__ double2 adj_search_rowsum(uint32_t s, int64_t stride,
@@ -2262,31 +2257,58 @@ __device__ __noinline__ double2 adj_search_rowsum(uint32_t s, int64_t stride,
                                                   const uint32_t* __restrict__ start,
                                                   const double* table, const View& v) {
     const RealParams& P = v.of_sorted(s);
-    double2 r = make_double2(1.0, 0.0);
+    AdjRowSum sum;
     visit_neighbours<DIM>(s, cell_arg<DIM>(cell, s), stride, rec, pos, start, P,
                           [&](uint32_t j, float, const float4&) {
-                              if (j == s) return;
-                              double K, dK;
-                              pair_terms<DIM>(pos, image, tan, stride, s, j, P, table, &K, &dK);
-                              r.x = __dadd_rn(r.x, K);
-                              r.y = __dadd_rn(r.y, dK);
+                              if (j != s)
+                                  sum.add(pair_terms<DIM>(image, tan, stride, s, j, P, table));
                           });
-    return r;
+    return sum.value();
 }
 
-// One pair's terms of pass B: {W (lambda_j - lambda_s), dW (M_j - M_s)}.
-__device__ __forceinline__ double2 adj_flux(double2 kd, const double* __restrict__ r,
-                                            const double* __restrict__ dr,
-                                            const double* __restrict__ mass,
-                                            const double* __restrict__ lam, uint32_t s, uint32_t j) {
-    const double inv = quot_pos(1.0, __dadd_rn(__ldg(r + s), __ldg(r + j)));
-    const double W = __dmul_rn(__dmul_rn(2.0, kd.x), inv);
-    const double dW = __dmul_rn(
-        __dmul_rn(2.0, inv),
-        __fma_rn(-__dmul_rn(kd.x, inv), __dadd_rn(__ldg(dr + s), __ldg(dr + j)), kd.y));
-    return make_double2(__dmul_rn(W, __dsub_rn(__ldg(lam + j), __ldg(lam + s))),
-                        __dmul_rn(dW, __dsub_rn(__ldg(mass + j), __ldg(mass + s))));
+// What pass B reads of a particle: {r, h^2 dr, M, lambda} as one 32-byte record.
+struct AdjRec {
+    double r, dr, mass, lam;
+};
+__device__ __forceinline__ AdjRec load_adj_rec(const double* __restrict__ rec4, uint32_t j) {
+    AdjRec q;
+    asm("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];"
+        : "=d"(q.r), "=d"(q.dr), "=d"(q.mass), "=d"(q.lam)
+        : "l"(rec4 + 4 * size_t(j)));
+    return q;
 }
+__global__ void __launch_bounds__(kBlock)
+k_adj_records(int n, const double* __restrict__ r, const double* __restrict__ dr,
+              const double* __restrict__ mass, const uint32_t* __restrict__ id,
+              const double* __restrict__ lam_in, double* __restrict__ rec4) {
+    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= n) return;
+    asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(rec4 + 4 * size_t(s)), "d"(r[s]),
+                 "d"(dr[s]), "d"(mass[s]), "d"(lam_in[id[s]])
+                 : "memory");
+}
+
+// Half of one pair's terms of pass B, {W (lambda_j - lambda_s), h^2 dW (M_j - M_s)} / 2:
+// with h = K / (r_s + r_j), W = 2 h and dW = 2 (dK - h (dr_s + dr_j)) / (r_s + r_j).
+// The reciprocal is integer work, which leaves eight binary64 operations of
+// nineteen.
+__device__ __forceinline__ double2 adj_flux(double2 kd, const AdjRec& me, const AdjRec& o) {
+    const double inv = Reciprocal(me.r, o.r).inverse().value();
+    const double h = __dmul_rn(kd.x, inv);
+    const double dh = __dmul_rn(inv, __fma_rn(-h, __dadd_rn(me.dr, o.dr), kd.y));
+    return make_double2(__dmul_rn(h, __dsub_rn(o.lam, me.lam)),
+                        __dmul_rn(dh, __dsub_rn(o.mass, me.mass)));
+}
+struct AdjFluxSum {
+    FluxSum64 lam, gD;
+    __device__ __forceinline__ void add(double2 t) {
+        lam.add(t.x);
+        gD.add(t.y);
+    }
+    __device__ __forceinline__ double2 value() const {
+        return make_double2(lam.value(), gD.value());
+    }
+};
 
 template <int DIM, class View>
 __device__ __noinline__ double2 adj_search_flux(uint32_t s, int64_t stride,
@@ -2297,34 +2319,43 @@ __device__ __noinline__ double2 adj_search_flux(uint32_t s, int64_t stride,
                                                 const uint32_t* __restrict__ cell,
                                                 const uint32_t* __restrict__ start,
                                                 const double* table, const View& v,
-                                                const double* __restrict__ r,
-                                                const double* __restrict__ dr,
-                                                const double* __restrict__ mass,
-                                                const double* __restrict__ lam) {
+                                                const double* __restrict__ rec4) {
     const RealParams& P = v.of_sorted(s);
-    double2 acc = make_double2(0.0, 0.0);
+    const double* mine = rec4 + 4 * size_t(s);
+    const AdjRec me{mine[0], mine[1], mine[2], mine[3]};
+    AdjFluxSum sum;
     visit_neighbours<DIM>(s, cell_arg<DIM>(cell, s), stride, rec, pos, start, P,
                           [&](uint32_t j, float, const float4&) {
                               if (j == s) return;
-                              double2 kd;
-                              pair_terms<DIM>(pos, image, tan, stride, s, j, P, table, &kd.x, &kd.y);
-                              const double2 t = adj_flux(kd, r, dr, mass, lam, s, j);
-                              acc.x = __dadd_rn(acc.x, t.x);
-                              acc.y = __dadd_rn(acc.y, t.y);
+                              const double* q = rec4 + 4 * size_t(j);
+                              sum.add(adj_flux(pair_terms<DIM>(image, tan, stride, s, j, P, table), me,
+                                               AdjRec{q[0], q[1], q[2], q[3]}));
                           });
-    return acc;
+    return sum.value();
 }
 
-// Pass A: r_s = sum_j K_sj (self included) and dr_s = sum_j dK_sj / dD.
+// What one step leaves on the adjoint's tape beside its mask words and (K, dK)
+// (see mtpt_adjoint_backward): with these, and none of the step's positions,
+// cells or tangents, pass B runs.
+struct TapeOut {
+    const double* mass;          // masses entering the step, ids: cell order
+    const uint32_t* id;
+    double* mass_out;
+    uint32_t* id_out;
+    uint32_t* incomplete;        // set when a particle's words or a warp's values did not fit
+};
+
+// Pass A: r_s = sum_j K_sj (self included) and h^2 sum_j dK_sj / dD; with
+// tape.mass_out also the rest of the step's tape.
 template <int DIM, class View>
-__global__ void __launch_bounds__(kBlock)
+__global__ void __launch_bounds__(kBlock, 4)
 k_adj_rowsum(int n, int64_t stride, const double* __restrict__ pos,
              const uint64_t* __restrict__ image, const double* __restrict__ tan,
              const float* __restrict__ rec, const uint32_t* __restrict__ cell,
              const uint32_t* __restrict__ start, const double* __restrict__ exp_table,
              const __grid_constant__ View v, double* __restrict__ r_out,
              double* __restrict__ dr_out, NbPlanes nb, uint32_t* __restrict__ listed_out,
-             AdjValues kv) {
+             AdjValues kv, TapeOut tape) {
     __shared__ double table[kExpTable];
     __shared__ ChunkShared<double2> chunk;
     for (int t = threadIdx.x; t < kExpTable; t += blockDim.x) table[t] = exp_table[t];
@@ -2334,44 +2365,51 @@ k_adj_rowsum(int n, int64_t stride, const double* __restrict__ pos,
     const bool valid = s < uint32_t(n) && P.transfer;
     uint32_t listed = 0, cnt = 0;
     if (valid) listed = search_listed<DIM>(s, stride, pos, rec, cell, start, v, P, nb, cnt);
-    double2 sum = make_double2(1.0, 0.0);
+    AdjRowSum rows;
     double2* keep = nullptr;
     dense_words(
         s, listed, stride, nb.e, chunk,
         [&](uint32_t total) { keep = kv.of_warp(s - (threadIdx.x & 31u), total); },
         [&](uint32_t e, uint32_t so, uint32_t j) {
-            double2 kd;
-            pair_terms<DIM>(pos, image, tan, stride, so, j, v.of_sorted(so), table, &kd.x, &kd.y);
+            const double2 kd = pair_terms<DIM>(image, tan, stride, so, j, v.of_sorted(so), table);
             if (keep) keep[e] = kd;
             return kd;
         },
-        [&](double2 t) {
-            sum.x = __dadd_rn(sum.x, t.x);
-            sum.y = __dadd_rn(sum.y, t.y);
-        });
+        [&](double2 kd) { rows.add(kd); });
     if (s < uint32_t(n)) {
+        double2 sum = rows.value();
         if (listed == kMaskOver)
             sum = adj_search_rowsum<DIM>(s, stride, pos, image, tan, rec, cell, start, table, v);
         r_out[s] = sum.x;
         dr_out[s] = sum.y;
         listed_out[s] = listed;
+        if (tape.mass_out) {
+            tape.mass_out[s] = tape.mass[s];
+            tape.id_out[s] = tape.id[s];
+            if (listed == kMaskOver || !keep) atomicOr(tape.incomplete, 1u);
+        }
     }
 }
 
 // Pass B: lambda_t,s = lambda_s + beta sum_j W_sj (lambda_j - lambda_s) and the
-// step's D-gradient term g_s = beta lambda_s sum_j dW_sj (M_j - M_s), with M the
-// masses entering the step.
+// step's D-gradient terms g_s = beta lambda_s sum_j dW_sj (M_j - M_s), with M the
+// masses entering the step, summed over the block in a fixed tree.
+// Lambda goes back to input order at once.
+//
+// Both passes are bound by the binary64 unit and its latency together: 44 -> 36 us
+// (A) and 54 -> 40 us (B) at 250,000 particles with 2.8 neighbours each when K,
+// reciprocals and sums became integer work and the neighbour's four values one
+// load; four blocks an SM (three and six: 7 and 4 % slower sweeps).
 template <int DIM, class View>
-__global__ void __launch_bounds__(kBlock)
+__global__ void __launch_bounds__(kBlock, 4)
 k_adj_exchange(int n, int64_t stride, const double* __restrict__ pos,
                const uint64_t* __restrict__ image, const double* __restrict__ tan,
                const float* __restrict__ rec, const uint32_t* __restrict__ cell,
                const uint32_t* __restrict__ start, const double* __restrict__ exp_table,
-               const __grid_constant__ View v, const double* __restrict__ r,
-               const double* __restrict__ dr, const double* __restrict__ mass,
-               const double* __restrict__ lam, double* __restrict__ lam_out,
-               double* __restrict__ gD, NbPlanes nb, const uint32_t* __restrict__ listed_in,
-               AdjValues kv) {
+               const __grid_constant__ View v, const double* __restrict__ rec4,
+               const uint32_t* __restrict__ id, double* __restrict__ lam_out,
+               double* __restrict__ gD_block, NbPlanes nb,
+               const uint32_t* __restrict__ listed_in, AdjValues kv) {
     __shared__ double table[kExpTable];
     __shared__ ChunkShared<double2> chunk;
     for (int t = threadIdx.x; t < kExpTable; t += blockDim.x) table[t] = exp_table[t];
@@ -2380,48 +2418,41 @@ k_adj_exchange(int n, int64_t stride, const double* __restrict__ pos,
     const RealParams& P = v.of_sorted(s < uint32_t(n) ? s : 0u);
     const bool valid = s < uint32_t(n) && P.transfer;
     const uint32_t listed = valid ? listed_in[s] : 0u;
-    double2 acc = make_double2(0.0, 0.0);
+    AdjFluxSum sums;
+    double g = 0.0;
     const double2* keep = nullptr;
     dense_words(
         s, listed, stride, nb.e, chunk,
         [&](uint32_t total) { keep = kv.of_warp(s - (threadIdx.x & 31u), total); },
         [&](uint32_t e, uint32_t so, uint32_t j) {
-            double2 kd;
-            if (keep) kd = __ldg(keep + e);
-            else pair_terms<DIM>(pos, image, tan, stride, so, j, v.of_sorted(so), table, &kd.x, &kd.y);
-            return adj_flux(kd, r, dr, mass, lam, so, j);
+            const AdjRec me = load_adj_rec(rec4, so), o = load_adj_rec(rec4, j);
+            const double2 kd = keep ? __ldg(keep + e)
+                                    : pair_terms<DIM>(image, tan, stride, so, j, v.of_sorted(so), table);
+            return adj_flux(kd, me, o);
         },
-        [&](double2 t) {
-            acc.x = __dadd_rn(acc.x, t.x);
-            acc.y = __dadd_rn(acc.y, t.y);
-        });
+        [&](double2 t) { sums.add(t); });
     if (s < uint32_t(n)) {
+        double2 acc = sums.value();      // halves of the sums
         if (listed == kMaskOver)
-            acc = adj_search_flux<DIM>(s, stride, pos, image, tan, rec, cell, start, table, v, r, dr,
-                                       mass, lam);
-        const double ls = lam[s];
-        lam_out[s] = valid ? __fma_rn(P.pp.beta, acc.x, ls) : ls;
-        gD[s] = valid ? __dmul_rn(__dmul_rn(P.pp.beta, ls), acc.y) : 0.0;
+            acc = adj_search_flux<DIM>(s, stride, pos, image, tan, rec, cell, start, table, v, rec4);
+        const double ls = rec4[4 * size_t(s) + 3], two_beta = 2.0 * P.pp.beta;
+        lam_out[id[s]] = valid ? __fma_rn(two_beta, acc.x, ls) : ls;
+        if (valid) g = __dmul_rn(__dmul_rn(__dmul_rn(two_beta, P.inv_h2), ls), acc.y);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) g = __dadd_rn(g, __shfl_xor_sync(0xffffffffu, g, o));
+    __shared__ double warp_g[kWarpsPerBlock];
+    if ((threadIdx.x & 31) == 0) warp_g[threadIdx.x >> 5] = g;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < kWarpsPerBlock; ++w) g = __dadd_rn(g, warp_g[w]);
+        gD_block[blockIdx.x] = g;
     }
 }
 
-// Deterministic sum of x[0..n): fixed-size blocks reduce their slice in a fixed
-// tree, then one block adds the block sums in index order to *acc.
 constexpr int kReduceThreads = 512;
 
-__global__ void __launch_bounds__(kReduceThreads)
-k_block_sums(int n, const double* __restrict__ x, double* __restrict__ partial) {
-    __shared__ double buf[kReduceThreads];
-    const int i = blockIdx.x * kReduceThreads + threadIdx.x;
-    buf[threadIdx.x] = i < n ? x[i] : 0.0;
-    __syncthreads();
-    for (int w = kReduceThreads / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) buf[threadIdx.x] = __dadd_rn(buf[threadIdx.x], buf[threadIdx.x + w]);
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) partial[blockIdx.x] = buf[0];
-}
-
+// Deterministic sum of a step's (or a segment's) block sums.
 // One block: thread t adds partial[t], partial[t + T], ... in order, then a
 // fixed tree over the threads; the result is added to *acc.
 __global__ void __launch_bounds__(kReduceThreads)
@@ -2438,16 +2469,11 @@ k_sum_into(int nparts, const double* __restrict__ partial, double* __restrict__ 
     if (threadIdx.x == 0) *acc = __dadd_rn(*acc, buf[0]);
 }
 
-// Input-order <-> cell-order moves of a per-particle binary64 array.
+// A per-particle binary64 array from input order into cell order.
 __global__ void k_take_by_id(int n, const uint32_t* __restrict__ id, const double* __restrict__ src,
                              double* __restrict__ dst) {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s < n) dst[s] = src[id[s]];
-}
-__global__ void k_put_by_id(int n, const uint32_t* __restrict__ id, const double* __restrict__ src,
-                            double* __restrict__ dst) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s < n) dst[id[s]] = src[s];
 }
 
 // Row sums in input order and in the paper's units:

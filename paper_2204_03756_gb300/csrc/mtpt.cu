@@ -71,10 +71,12 @@ bool injected_alloc_failure() {
     return false;
 }
 
-// Every device allocation of the library goes through here.
-int device_alloc(void** out, size_t bytes) {
+// Every device allocation of the library goes through here (`optional`: the
+// caller does without it when there is no memory; not counted by the
+// injection, which is to surface).
+int device_alloc(void** out, size_t bytes, bool optional = false) {
     *out = nullptr;
-    if (injected_alloc_failure()) return MTPT_ERR_NO_MEMORY;
+    if (!optional && injected_alloc_failure()) return MTPT_ERR_NO_MEMORY;
     if (cudaMalloc(out, bytes) != cudaSuccess) {
         (void)cudaGetLastError();
         *out = nullptr;
@@ -89,10 +91,10 @@ template <typename T>
 struct DevBuf {
     T* p = nullptr;
     size_t count = 0;
-    int ensure(size_t n) {
+    int ensure(size_t n, bool optional = false) {
         if (n == 0 || (n <= count && p)) return MTPT_OK;
         void* q = nullptr;
-        MTPT_TRY(device_alloc(&q, n * sizeof(T)));
+        MTPT_TRY(device_alloc(&q, n * sizeof(T), optional));
         release();
         p = static_cast<T*>(q);
         count = n;
@@ -272,7 +274,10 @@ struct mtpt_handle {
     uint64_t adj_step0 = 0;
     bool adj_ready = false;
     bool adjoint_sweep = false;       // the sorts feed the adjoint's pair passes
-    DevBuf<double> dr64, lam_in, lam_s, lam_new, gD, partial, acc;
+    DevBuf<double> dr64, lam_in, adj_rec, partial, acc;
+    DevBuf<unsigned char> tape;       // one segment's steps (TapeSlot), when it fits
+    int64_t tape_steps = 0;
+    DevBuf<uint32_t> tape_flag;       // TapeOut::incomplete
     // captured two-step graph (valid for `graph_cur`, `graph_flags` and the
     // mass buffer pair as it was: every step swaps the pair, so between loads
     // its order follows `cur`, but a pipelined load moves `cur` alone)
@@ -615,9 +620,9 @@ int setup_grids(mtpt_handle* h) {
     h->nb_cap = f32 && h->dim == 3 ? list_cap : words;
     h->nb_pad = f32 && h->dim == 2 && usual > 32.0 ? int(std::min(8.0, std::ceil(usual / 32.0))) : 0;
     // kernel values of the binary64 form, per particle; the adjoint's, where 32
-    // particles share their space, so one standard deviation is six of theirs
+    // particles share their space (1.2 deviations of one are seven of theirs)
     h->nb_kcap = f32 ? 0 : int(std::min(128.0, std::ceil(expect + 4.0 * std::sqrt(expect) + 4.0)));
-    h->adj_kcap = int(std::min(128.0, std::ceil(expect + std::sqrt(expect) + 4.0)));
+    h->adj_kcap = int(std::min(128.0, std::ceil(expect + 1.2 * std::sqrt(expect) + 2.0)));
     h->adj_cap = words;
     h->n_cells = cell_base;
     h->n_corners = corner_base;
@@ -1754,53 +1759,179 @@ int snapshot(mtpt_handle* h, int64_t k, bool save) {
     return MTPT_OK;
 }
 
-// One backward step: walk (with tangents) and sort exactly as forward step t
-// did, then the adjoint passes, lambda kept in input order between steps.
+// One step's place on the tape of a segment: what pass B reads (the mask words
+// and values of pass A, its row sums, the masses entering the step, the ids),
+// so that the backward sweep neither walks nor sorts nor searches again.
+struct TapeSlot {
+    uint2* words;
+    double2* kd;
+    double *r, *dr, *mass;
+    uint32_t *id, *listed;
+};
+// (K, dK) values of whole warps.
+size_t adj_values(const mtpt_handle* h) {
+    return size_t(std::max<int64_t>(h->cap, 1) + 31) / 32 * 32 * size_t(h->adj_kcap);
+}
+size_t tape_step_bytes(const mtpt_handle* h) {
+    return size_t(h->cap) * (8 * size_t(h->adj_cap) + 3 * 8 + 2 * 4) + 16 * adj_values(h) + 7 * 256;
+}
+int ensure_adjoint_rows(mtpt_handle* h) {
+    const size_t cap = size_t(std::max<int64_t>(h->cap, 1));
+    MTPT_TRY(h->adj_nb_e.ensure(size_t(h->adj_cap) * cap));
+    MTPT_TRY(h->adj_nb_listed.ensure(cap));
+    return h->adj_nb_k.ensure(adj_values(h));
+}
+TapeSlot tape_slot(const mtpt_handle* h, int64_t k) {
+    const size_t cap = size_t(h->cap);
+    unsigned char* p = h->tape.p + size_t(k) * tape_step_bytes(h);
+    auto take = [&p](size_t bytes) {
+        p = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(p) + 255) & ~uintptr_t(255));
+        unsigned char* q = p;
+        p += bytes;
+        return q;
+    };
+    TapeSlot t;
+    t.kd = reinterpret_cast<double2*>(take(16 * adj_values(h)));
+    t.words = reinterpret_cast<uint2*>(take(cap * 8 * size_t(h->adj_cap)));
+    t.r = reinterpret_cast<double*>(take(cap * 8));
+    t.dr = reinterpret_cast<double*>(take(cap * 8));
+    t.mass = reinterpret_cast<double*>(take(cap * 8));
+    t.id = reinterpret_cast<uint32_t*>(take(cap * 4));
+    t.listed = reinterpret_cast<uint32_t*>(take(cap * 4));
+    return t;
+}
+// The handle's own pass A outputs, for steps that are not on the tape.
+TapeSlot own_slot(const mtpt_handle* h, int o) {
+    return {h->adj_nb_e.p, h->adj_nb_k.p, h->r64.p, h->dr64.p, h->mass[o].p, h->id[o].p,
+            h->adj_nb_listed.p};
+}
+constexpr size_t kTapeBytesMax = size_t(16) << 30;   // longer tapes take the steps one by one
+
+// The walk (with tangents) and sort of the step that follows buffer cur's
+// state, as forward step t did them, into the other buffer.
 template <int DIM>
-int launch_adjoint_step(mtpt_handle* h) {
+int launch_adjoint_sort(mtpt_handle* h) {
     const int n = int(h->n);
-    const int64_t stride = h->cap;
-    const int blocks = grid_for(n);
-    cudaStream_t st = h->stream;
     const int c = h->cur, o = 1 - h->cur;
+    cudaStream_t st = h->stream;
     const SingleView v = make_view<SingleView>(h, c, c);
     if (h->any_advect)
-        k_walk_key<DIM, SingleView, true, true><<<blocks, kBlock, 0, st>>>(
-            n, stride, h->pos[c].p, h->id[c].p, h->step_dev.p, h->any_walk ? 1 : 0, 1, v,
+        k_walk_key<DIM, SingleView, true, true><<<grid_for(n), kBlock, 0, st>>>(
+            n, h->cap, h->pos[c].p, h->id[c].p, h->step_dev.p, h->any_walk ? 1 : 0, 1, v,
             h->key.p, h->count.p, h->status.p, h->tan[c].p);
     else
-        k_walk_key<DIM, SingleView, true><<<blocks, kBlock, 0, st>>>(
-            n, stride, h->pos[c].p, h->id[c].p, h->step_dev.p, h->any_walk ? 1 : 0, 1, v,
+        k_walk_key<DIM, SingleView, true><<<grid_for(n), kBlock, 0, st>>>(
+            n, h->cap, h->pos[c].p, h->id[c].p, h->step_dev.p, h->any_walk ? 1 : 0, 1, v,
             h->key.p, h->count.p, h->status.p, h->tan[c].p);
-    MTPT_TRY(launch_scan(h, st, true));
-    h->adjoint_sweep = true;
-    const int sorted = launch_sort<DIM, SingleView>(h, c, o, v);
-    h->adjoint_sweep = false;
-    MTPT_TRY(sorted);
-    k_take_by_id<<<blocks, kBlock, 0, st>>>(n, h->id[o].p, h->lam_in.p, h->lam_s.p);
-    const NbPlanes adj_nb{h->adj_nb_e.p, h->adj_cap, 0};
-    const AdjValues adj_kv{h->adj_nb_k.p, h->adj_kcap};
-    k_adj_rowsum<DIM, SingleView><<<blocks, kBlock, 0, st>>>(
-        n, stride, h->pos[o].p, h->image.p, h->tan[o].p, h->rec.p, h->cell.p, h->start.p, h->exp_table.p, v,
-        h->r64.p, h->dr64.p, adj_nb, h->adj_nb_listed.p, adj_kv);
-    k_adj_exchange<DIM, SingleView><<<blocks, kBlock, 0, st>>>(
-        n, stride, h->pos[o].p, h->image.p, h->tan[o].p, h->rec.p, h->cell.p, h->start.p, h->exp_table.p, v,
-        h->r64.p, h->dr64.p, h->mass[o].p, h->lam_s.p, h->lam_new.p, h->gD.p, adj_nb,
-        h->adj_nb_listed.p, adj_kv);
-    k_put_by_id<<<blocks, kBlock, 0, st>>>(n, h->id[o].p, h->lam_new.p, h->lam_in.p);
-    const int nparts = (n + kReduceThreads - 1) / kReduceThreads;
-    k_block_sums<<<nparts, kReduceThreads, 0, st>>>(n, h->gD.p, h->partial.p);
-    k_sum_into<<<1, kReduceThreads, 0, st>>>(nparts, h->partial.p, h->acc.p);
     MTPT_CUDA_TRY(cudaGetLastError());
-    h->cur = o;
+    MTPT_TRY(launch_scan(h, st, true));
+    return launch_sort<DIM, SingleView>(h, c, o, v);
+}
+
+// Pass A on buffer o's sorted state, the masses entering the step in `mass`.
+template <int DIM>
+int launch_adjoint_rows(mtpt_handle* h, int o, const double* mass, const TapeSlot& t, bool taped) {
+    const SingleView v = make_view<SingleView>(h, o, o);
+    const TapeOut out = taped ? TapeOut{mass, h->id[o].p, t.mass, t.id, h->tape_flag.p} : TapeOut{};
+    k_adj_rowsum<DIM, SingleView><<<grid_for(h->n), kBlock, 0, h->stream>>>(
+        int(h->n), h->cap, h->pos[o].p, h->image.p, h->tan[o].p, h->rec.p, h->cell.p, h->start.p,
+        h->exp_table.p, v, t.r, t.dr, NbPlanes{t.words, h->adj_cap, 0}, t.listed,
+        AdjValues{t.kd, h->adj_kcap}, out);
+    MTPT_CUDA_TRY(cudaGetLastError());
     return MTPT_OK;
 }
 
-int dispatch_adjoint_step(mtpt_handle* h) {
+// Pass B, lambda kept in input order between steps; the step's block sums go
+// to gD_block.  (Buffer o's positions, tangents and cells are read only for
+// particles whose words or values are not there: never on the tape.)
+template <int DIM>
+int launch_adjoint_pass(mtpt_handle* h, int o, const TapeSlot& t, double* gD_block) {
+    const int n = int(h->n), blocks = grid_for(n);
+    cudaStream_t st = h->stream;
+    const SingleView v = make_view<SingleView>(h, o, o);
+    k_adj_records<<<blocks, kBlock, 0, st>>>(n, t.r, t.dr, t.mass, t.id, h->lam_in.p, h->adj_rec.p);
+    k_adj_exchange<DIM, SingleView><<<blocks, kBlock, 0, st>>>(
+        n, h->cap, h->pos[o].p, h->image.p, h->tan[o].p, h->rec.p, h->cell.p, h->start.p,
+        h->exp_table.p, v, h->adj_rec.p, t.id, h->lam_in.p, gD_block,
+        NbPlanes{t.words, h->adj_cap, 0}, t.listed, AdjValues{t.kd, h->adj_kcap});
+    MTPT_CUDA_TRY(cudaGetLastError());
+    return MTPT_OK;
+}
+
+int sum_blocks(mtpt_handle* h, int64_t parts) {
+    k_sum_into<<<1, kReduceThreads, 0, h->stream>>>(int(parts), h->partial.p, h->acc.p);
+    MTPT_CUDA_TRY(cudaGetLastError());
+    return MTPT_OK;
+}
+
+// Steps t0..t1-1 forward from the checkpoint in the current buffer, each with
+// pass A on the tape.
+template <int DIM>
+int record_segment(mtpt_handle* h, int64_t t0, int64_t t1) {
+    MTPT_CUDA_TRY(cudaMemsetAsync(h->tape_flag.p, 0, sizeof(uint32_t), h->stream));
+    for (int64_t t = t0; t < t1; ++t) {
+        const TapeSlot slot = tape_slot(h, t - t0);
+        if (t + 1 < t1) {
+            // (the step swaps the mass pair: those entering it are in the other buffer)
+            MTPT_TRY(dispatch_step(h, MTPT_DO_WALK | MTPT_DO_TRANSFER));
+            MTPT_TRY(launch_adjoint_rows<DIM>(h, h->cur, h->mass[1 - h->cur].p, slot, true));
+        } else {
+            MTPT_TRY(launch_adjoint_sort<DIM>(h));
+            h->cur = 1 - h->cur;
+            MTPT_TRY(launch_adjoint_rows<DIM>(h, h->cur, h->mass[h->cur].p, slot, true));
+        }
+    }
+    return MTPT_OK;
+}
+
+// One segment of the backward sweep from its checkpoint (slot k of the
+// snapshots), steps t1-1 down to t0.
+template <int DIM>
+int backward_segment(mtpt_handle* h, int64_t k, int64_t t0, int64_t t1) {
+    const int64_t blocks = grid_for(h->n);
+    MTPT_TRY(snapshot(h, k, false));
+    MTPT_TRY(set_step_dev(h, h->adj_step0 + uint64_t(t0)));
+    if (t1 - t0 <= h->tape_steps && size_t(t1 - t0) * tape_step_bytes(h) <= h->tape.count) {
+        MTPT_TRY(record_segment<DIM>(h, t0, t1));
+        uint32_t incomplete = 0;
+        MTPT_CUDA_TRY(cudaMemcpyAsync(&incomplete, h->tape_flag.p, sizeof(incomplete),
+                                      cudaMemcpyDeviceToHost, h->stream));
+        MTPT_CUDA_TRY(cudaStreamSynchronize(h->stream));
+        if (!incomplete) {
+            for (int64_t t = t1 - 1; t >= t0; --t)
+                MTPT_TRY(launch_adjoint_pass<DIM>(h, h->cur, tape_slot(h, t - t0),
+                                                  h->partial.p + (t - t0) * blocks));
+            return sum_blocks(h, (t1 - t0) * blocks);
+        }
+        MTPT_TRY(snapshot(h, k, false));
+        MTPT_TRY(set_step_dev(h, h->adj_step0 + uint64_t(t0)));
+    }
+    // no room for the tape, or particles that it cannot hold: the state before
+    // every step on the snapshots, and each step's walk, sort and pass A again
+    const int64_t first = h->adj_nck;
+    for (int64_t t = t0; t < t1; ++t) {
+        MTPT_TRY(snapshot(h, first + (t - t0), true));
+        if (t + 1 < t1) MTPT_TRY(dispatch_step(h, MTPT_DO_WALK | MTPT_DO_TRANSFER));
+    }
+    for (int64_t t = t1 - 1; t >= t0; --t) {
+        MTPT_TRY(snapshot(h, first + (t - t0), false));
+        MTPT_TRY(set_step_dev(h, h->adj_step0 + uint64_t(t)));
+        MTPT_TRY(launch_adjoint_sort<DIM>(h));
+        const int o = 1 - h->cur;
+        const TapeSlot slot = own_slot(h, o);
+        MTPT_TRY(launch_adjoint_rows<DIM>(h, o, h->mass[o].p, slot, false));
+        MTPT_TRY(launch_adjoint_pass<DIM>(h, o, slot, h->partial.p));
+        MTPT_TRY(sum_blocks(h, blocks));
+        h->cur = o;
+    }
+    return MTPT_OK;
+}
+
+int dispatch_backward_segment(mtpt_handle* h, int64_t k, int64_t t0, int64_t t1) {
     switch (h->dim) {
-        case 1: return launch_adjoint_step<1>(h);
-        case 2: return launch_adjoint_step<2>(h);
-        default: return launch_adjoint_step<3>(h);
+        case 1: return backward_segment<1>(h, k, t0, t1);
+        case 2: return backward_segment<2>(h, k, t0, t1);
+        default: return backward_segment<3>(h, k, t0, t1);
     }
 }
 
@@ -1820,15 +1951,19 @@ int mtpt_adjoint_forward(mtpt_handle* h, int64_t nsteps, int64_t checkpoint_ever
     const int64_t seg = std::min(checkpoint_every, nsteps);
     h->snap_bytes = (snap_size(h) + 255) & ~size_t(255);
     MTPT_TRY(h->snaps.ensure(size_t(nck + seg + 1) * h->snap_bytes));
-    for (auto* b : {&h->dr64, &h->lam_in, &h->lam_s, &h->lam_new, &h->gD})
-        MTPT_TRY(b->ensure(cap));
+    for (auto* b : {&h->dr64, &h->lam_in}) MTPT_TRY(b->ensure(cap));
+    MTPT_TRY(h->adj_rec.ensure(4 * cap));
     MTPT_TRY(h->r64.ensure(cap));
     MTPT_TRY(h->image.ensure(size_t(h->dim) * cap));
-    MTPT_TRY(h->adj_nb_e.ensure(size_t(h->adj_cap) * cap));
-    MTPT_TRY(h->adj_nb_listed.ensure(cap));
-    MTPT_TRY(h->adj_nb_k.ensure((cap + 31) / 32 * 32 * size_t(h->adj_kcap)));   // whole warps
-    MTPT_TRY(h->partial.ensure(size_t((n + kReduceThreads - 1) / kReduceThreads + 1)));
+    MTPT_TRY(ensure_adjoint_rows(h));
+    MTPT_TRY(h->partial.ensure(size_t(seg) * size_t(grid_for(n) + 1)));
     MTPT_TRY(h->acc.ensure(1));
+    MTPT_TRY(h->tape_flag.ensure(1));
+    // the tape is room for speed: without it the sweep takes its steps one by one
+    h->tape_steps = 0;
+    const size_t tape_bytes = size_t(seg) * tape_step_bytes(h);
+    if (n > 0 && tape_bytes <= kTapeBytesMax && h->tape.ensure(tape_bytes, true) == MTPT_OK)
+        h->tape_steps = seg;
     h->tangent_on = true;
     h->adj_step0 = h->step;
     int rc = MTPT_OK;
@@ -1855,29 +1990,20 @@ int mtpt_adjoint_backward(mtpt_handle* h, const double* gmass_dev, double* gmass
     const int64_t n = h->n, K = h->adj_every, T = h->adj_steps, nck = h->adj_nck;
     const int64_t seg = std::min(K, T);
     const int64_t final_slot = nck + seg;
+    // (a retuning since the recording may have given the grid more rows)
+    MTPT_TRY(ensure_adjoint_rows(h));
     MTPT_CUDA_TRY(cudaMemcpyAsync(h->lam_in.p, gmass_dev, size_t(n) * sizeof(double),
                                   cudaMemcpyDeviceToDevice, h->stream));
     MTPT_CUDA_TRY(cudaMemsetAsync(h->acc.p, 0, sizeof(double), h->stream));
     drop_graph(h);
     h->tangent_on = true;
+    h->adjoint_sweep = true;          // the sorts write the images of pass A
     int rc = MTPT_OK;
     for (int64_t k = nck - 1; k >= 0 && rc == MTPT_OK; --k) {
         const int64_t t0 = k * K, t1 = std::min(t0 + K, T);
-        // forward over the segment from its checkpoint, recording the state
-        // before every step on the tape
-        rc = snapshot(h, k, false);
-        if (rc == MTPT_OK) rc = set_step_dev(h, h->adj_step0 + uint64_t(t0));
-        for (int64_t t = t0; t < t1 && rc == MTPT_OK; ++t) {
-            rc = snapshot(h, nck + (t - t0), true);
-            if (rc == MTPT_OK && t + 1 < t1) rc = dispatch_step(h, MTPT_DO_WALK | MTPT_DO_TRANSFER);
-        }
-        // backward through the tape
-        for (int64_t t = t1 - 1; t >= t0 && rc == MTPT_OK; --t) {
-            rc = snapshot(h, nck + (t - t0), false);
-            if (rc == MTPT_OK) rc = set_step_dev(h, h->adj_step0 + uint64_t(t));
-            if (rc == MTPT_OK) rc = dispatch_adjoint_step(h);
-        }
+        rc = dispatch_backward_segment(h, k, t0, t1);
     }
+    h->adjoint_sweep = false;
     h->tangent_on = false;
     // leave the handle in its final forward state
     if (rc == MTPT_OK) rc = snapshot(h, final_slot, false);
@@ -1938,7 +2064,8 @@ int mtpt_destroy(mtpt_handle* h) {
     h->status.release(); h->pair_counter.release(); h->step_dev.release();
     h->emit_counter.release(); h->emit_i.release(); h->emit_j.release();
     h->tan[0].release(); h->tan[1].release(); h->snaps.release(); h->dr64.release();
-    h->lam_in.release(); h->lam_s.release(); h->lam_new.release(); h->gD.release();
+    h->lam_in.release(); h->adj_rec.release();
+    h->tape.release(); h->tape_flag.release();
     h->partial.release(); h->acc.release();
     h->nb_e.release(); h->nb_listed.release(); h->nb_k.release();
     h->massb[0].release(); h->massb[1].release(); h->exb.release();
