@@ -3,11 +3,11 @@
 // A handle owns the particle state of one realisation -- or of a batch of
 // independent realisations -- on one device, in cell order, and runs one time
 // step of Sec. 3 as a fixed sequence of kernels on the handle's stream:
-//   walk_key -> scan (3 launches) -> scatter -> gather -> rowsum -> exchange
+//   walk_key -> scan -> scatter -> gather -> rowsum -> exchange
 // A batch concatenates its realisations' particles and gives each
 // realisation its own block of cells in one global cell list, so every phase
 // is one launch over all particles of all realisations.  Multi-step calls
-// replay a captured CUDA graph of two steps.  No step goes through the host:
+// replay a captured CUDA graph of several steps.  No step goes through the host:
 // the only host<->device traffic is in mtpt_set_particles* / mtpt_get_*
 // (the *_async pair copies on two streams of its own, ordered by events).
 #include <cuda_runtime.h>
@@ -33,7 +33,10 @@ using namespace mtpt;
 namespace {
 
 constexpr int kMaxDim = 3;
-constexpr int64_t kGraphMinSteps = 4;   // multi-step calls from this size replay a graph
+// Steps of one captured graph (even: the buffer pairs then return to where they
+// were).  2, 8 and 32 replay alike (32.2 us a step at 1e4 particles, 33.6 without
+// graphs); the other steps of a call are launched one by one.
+constexpr int64_t kGraphSteps = 8;
 constexpr int kSettleBlocks = 152;      // grid-stride blocks of k_load_settle (one per SM)
 
 // With MTPT_DEBUG set in the environment, a failing runtime call is named on
@@ -155,6 +158,22 @@ struct GrowAll {
 };
 
 int grid_for(int64_t n) { return int((n + kBlock - 1) / kBlock); }
+
+// Launches a kernel that starts with after_previous() or ordered_index(), with
+// programmatic stream serialisation (an error is left for cudaGetLastError).
+template <typename... P, typename... A>
+void launch(void (*kernel)(P...), int blocks, int threads, cudaStream_t stream, A&&... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(unsigned(blocks));
+    cfg.blockDim = dim3(unsigned(threads));
+    cfg.stream = stream;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    (void)cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
 
 // Host-side data of one realisation.
 struct RealHost {
@@ -278,7 +297,7 @@ struct mtpt_handle {
     DevBuf<unsigned char> tape;       // one segment's steps (TapeSlot), when it fits
     int64_t tape_steps = 0;
     DevBuf<uint32_t> tape_flag;       // TapeOut::incomplete
-    // captured two-step graph (valid for `graph_cur`, `graph_flags` and the
+    // captured graph of plain steps (valid for `graph_cur`, `graph_flags` and the
     // mass buffer pair as it was: every step swaps the pair, so between loads
     // its order follows `cur`, but a pipelined load moves `cur` alone)
     cudaGraphExec_t graph = nullptr;
@@ -739,7 +758,7 @@ std::atomic<int> g_scan_hold{-1};
 // Exclusive prefix sum of the cell counts into start (one launch).
 int launch_scan(mtpt_handle* h, cudaStream_t st, bool advance) {
     const int ntiles = int(h->n_cells_pad / kScanTile);
-    k_scan<<<ntiles, kScanThreads, 0, st>>>(reinterpret_cast<const uint4*>(h->count.p),
+    launch(k_scan, ntiles, kScanThreads, st, reinterpret_cast<const uint4*>(h->count.p),
                                             reinterpret_cast<uint4*>(h->start.p),
                                             h->scan_state.p, ntiles, h->step_dev.p,
                                             advance ? 1 : 0, g_scan_hold.load());
@@ -859,13 +878,13 @@ int launch_sort_t(mtpt_handle* h, int c, int o, const View& vin) {
     double* tan_out = TANGENT ? h->tan[o].p : nullptr;
     {
         MTPT_TIMED(h, "scatter");
-        k_scatter<<<blocks, kBlock, 0, h->stream>>>(n, h->key.p, h->start.p, h->count.p,
+        launch(k_scatter, blocks, kBlock, h->stream, n, h->key.p, h->start.p, h->count.p,
                                                     h->pos[c].p, h->id[c].p, h->perm.p,
                                                     h->sortkey.p);
         MTPT_CUDA_TRY(cudaGetLastError());
     }
     MTPT_TIMED(h, "gather");
-    k_gather<DIM, View, TANGENT><<<blocks, kBlock, 0, h->stream>>>(
+    launch(k_gather<DIM, View, TANGENT>, blocks, kBlock, h->stream, 
         n, stride, h->perm.p, h->sortkey.p, h->start.p, h->pos[c].p, h->mass[c].p, h->id[o].p,
         h->pos[o].p, h->mass[o].p, h->cell.p, h->rec.p, h->corners.p, rid_out, vin, tan_in,
         tan_out, h->reactive ? h->massb[c].p : nullptr, h->reactive ? h->massb[o].p : nullptr,
@@ -884,14 +903,14 @@ int launch_sort_rec(mtpt_handle* h, int c, int o, const SingleView& vin) {
     MTPT_TRY(h->sortrec.ensure(size_t(SortRec<DIM, TANGENT>::kChunks) * size_t(h->cap)));
     {
         MTPT_TIMED(h, "scatter");
-        k_scatter_rec<DIM, TANGENT><<<blocks, kBlock, 0, h->stream>>>(
+        launch(k_scatter_rec<DIM, TANGENT>, blocks, kBlock, h->stream, 
             n, stride, h->key.p, h->start.p, h->count.p, h->pos[c].p, h->mass[c].p, h->id[c].p,
             TANGENT ? h->tan[c].p : nullptr, h->sortrec.p);
         MTPT_CUDA_TRY(cudaGetLastError());
     }
     MTPT_TIMED(h, "gather");
     double* tan_out = TANGENT ? h->tan[o].p : nullptr;
-    k_gather_rec<DIM, TANGENT><<<blocks, kBlock, 0, h->stream>>>(
+    launch(k_gather_rec<DIM, TANGENT>, blocks, kBlock, h->stream, 
         n, stride, h->sortrec.p, h->start.p, h->id[o].p, h->pos[o].p, h->mass[o].p, h->cell.p,
         h->rec.p, h->corners.p, vin, tan_out, image_buf(h));
     MTPT_CUDA_TRY(cudaGetLastError());
@@ -946,7 +965,7 @@ int launch_exchange_f32(mtpt_handle* h, const View& vs, int o, int c, const NbPl
     if (TWO) reaction_rate(h, &kp, &dt);
     MTPT_TIMED(h, WALK ? "exchange_walk_f32" : "exchange_f32");
     const int n = int(h->n), block = h->pair_block;
-    k_exchange_f32<DIM, View, TWO, WALK><<<(n + block - 1) / block, block, 0, h->stream>>>(
+    launch(k_exchange_f32<DIM, View, TWO, WALK>, (n + block - 1) / block, block, h->stream, 
         n, h->cap, h->pos[o].p, h->rec.p, h->cell.p, h->start.p, vs, h->ex.p, h->mass[o].p,
         h->mass[c].p, nb, TWO ? h->exb.p : nullptr, TWO ? h->massb[o].p : nullptr,
         TWO ? h->massb[c].p : nullptr, kp, dt, float(kp * dt), wa);
@@ -974,7 +993,7 @@ int launch_pairs_f32(mtpt_handle* h, const View& vs, int o, int c, bool walk_ahe
     const NbPlanes nb = planes(h);
     {
         MTPT_TIMED(h, "rowsum_f32");
-        k_rowsum_f32<DIM, View><<<(n + block - 1) / block, block, 0, h->stream>>>(
+        launch(k_rowsum_f32<DIM, View>, (n + block - 1) / block, block, h->stream, 
             n, h->cap, h->pos[o].p, h->rec.p, h->cell.p, h->start.p, vs, h->mass[o].p, h->ex.p,
             h->pair_counter.p, h->ntiles > 0 ? h->id[o].p : nullptr, nb);
         MTPT_CUDA_TRY(cudaGetLastError());
@@ -983,7 +1002,7 @@ int launch_pairs_f32(mtpt_handle* h, const View& vs, int o, int c, bool walk_ahe
         if (h->reactive) {
             // species B's split, then one pass 2 for both species and the
             // reaction (batches refuse it)
-            k_split_mass<<<grid_for(n), kBlock, 0, h->stream>>>(n, h->massb[o].p, h->exb.p);
+            launch(k_split_mass, grid_for(n), kBlock, h->stream, n, h->massb[o].p, h->exb.p);
             MTPT_CUDA_TRY(cudaGetLastError());
             return launch_exchange_f32<DIM, View, true>(h, vs, o, c, nb, walk_ahead);
         }
@@ -1004,17 +1023,17 @@ int launch_species_b(mtpt_handle* h, int n, int64_t stride, const double* pos_s,
     cudaStream_t st = h->stream;
     {
         MTPT_TIMED(h, "exchange_f64");
-        k_record_mass<<<blocks, kBlock, 0, st>>>(n, h->massb[o].p, record_buf(h));
-        k_exchange_f64<DIM, View><<<blocks, kBlock, 0, st>>>(
+        launch(k_record_mass, blocks, kBlock, st, n, h->massb[o].p, record_buf(h));
+        launch(k_exchange_f64<DIM, View>, blocks, kBlock, st, 
             n, stride, pos_s, h->image.p, h->rec.p, h->cell.p, h->start.p, h->exp_table.p, vs,
-            record_buf(h), h->massb[c].p, planes(h), h->nb_listed.p, kernel_values(h));
+            record_buf(h), h->massb[c].p, planes(h), h->nb_listed.p, kernel_values(h), WalkAhead{});
     }
     MTPT_CUDA_TRY(cudaGetLastError());
     double kp, dt;
     reaction_rate(h, &kp, &dt);
     {
         MTPT_TIMED(h, "react");
-        k_react<true><<<blocks, kBlock, 0, st>>>(n, h->mass[c].p, h->massb[c].p, kp, dt,
+        launch(k_react<true>, blocks, kBlock, st, n, h->mass[c].p, h->massb[c].p, kp, dt,
                                                  float(kp * dt));
     }
     MTPT_CUDA_TRY(cudaGetLastError());
@@ -1034,7 +1053,7 @@ int launch_step(mtpt_handle* h, int flags, bool walk_ahead) {
         // an empty handle (e.g. a tile without particles) keeps its walk's
         // step counter in line with the host mirror
         if ((flags & MTPT_DO_WALK) && h->step_dev.p) {
-            k_advance_step<<<1, 1, 0, h->stream>>>(h->step_dev.p);
+            launch(k_advance_step, 1, 1, h->stream, h->step_dev.p);
             MTPT_CUDA_TRY(cudaGetLastError());
         }
         return MTPT_OK;
@@ -1050,28 +1069,28 @@ int launch_step(mtpt_handle* h, int flags, bool walk_ahead) {
         MTPT_TIMED(h, "walk_key");
         if (h->tangent_on) {
             if (h->any_advect)
-                k_walk_key<DIM, View, true, true><<<blocks, kBlock, 0, st>>>(
+                launch(k_walk_key<DIM, View, true, true>, blocks, kBlock, st, 
                     n, stride, h->pos[c].p, h->id[c].p, h->step_dev.p, walk ? 1 : 0,
                     transfer ? 1 : 0, vin, h->key.p, h->count.p, h->status.p, h->tan[c].p);
             else
-                k_walk_key<DIM, View, true><<<blocks, kBlock, 0, st>>>(
+                launch(k_walk_key<DIM, View, true>, blocks, kBlock, st, 
                     n, stride, h->pos[c].p, h->id[c].p, h->step_dev.p, walk ? 1 : 0,
                     transfer ? 1 : 0, vin, h->key.p, h->count.p, h->status.p, h->tan[c].p);
         } else if (h->any_advect) {
-            k_walk_key<DIM, View, false, true><<<blocks, kBlock, 0, st>>>(
+            launch(k_walk_key<DIM, View, false, true>, blocks, kBlock, st, 
                 n, stride, h->pos[c].p, h->id[c].p, h->step_dev.p, walk ? 1 : 0,
-                transfer ? 1 : 0, vin, h->key.p, h->count.p, h->status.p);
+                transfer ? 1 : 0, vin, h->key.p, h->count.p, h->status.p, nullptr);
         } else {
-            k_walk_key<DIM, View><<<blocks, kBlock, 0, st>>>(
+            launch(k_walk_key<DIM, View>, blocks, kBlock, st, 
                 n, stride, h->pos[c].p, h->id[c].p, h->step_dev.p, walk ? 1 : 0,
-                transfer ? 1 : 0, vin, h->key.p, h->count.p, h->status.p);
+                transfer ? 1 : 0, vin, h->key.p, h->count.p, h->status.p, nullptr);
         }
         MTPT_CUDA_TRY(cudaGetLastError());
     }
     const bool advance = (flags & MTPT_DO_WALK) != 0;
     if (!transfer) {
         if (advance) {
-            k_advance_step<<<1, 1, 0, st>>>(h->step_dev.p);
+            launch(k_advance_step, 1, 1, st, h->step_dev.p);
             MTPT_CUDA_TRY(cudaGetLastError());
         }
         return MTPT_OK;
@@ -1089,7 +1108,7 @@ int launch_step(mtpt_handle* h, int flags, bool walk_ahead) {
     if (!split) {
         {
             MTPT_TIMED(h, "rowsum_f64");
-            k_rowsum_f64<DIM, View><<<blocks, kBlock, 0, st>>>(
+            launch(k_rowsum_f64<DIM, View>, blocks, kBlock, st, 
                 n, stride, pos_s, h->image.p, h->rec.p, h->cell.p, h->start.p, h->exp_table.p, vs,
                 h->mass[o].p, record_buf(h), h->pair_counter.p, planes(h), h->nb_listed.p,
                 kernel_values(h),
@@ -1105,18 +1124,18 @@ int launch_step(mtpt_handle* h, int flags, bool walk_ahead) {
             }
             MTPT_TIMED(h, "exchange_walk_f64");
             if (h->any_advect)
-                k_exchange_f64<DIM, View, 2><<<blocks, kBlock, 0, st>>>(
+                launch(k_exchange_f64<DIM, View, 2>, blocks, kBlock, st, 
                     n, stride, pos_s, h->image.p, h->rec.p, h->cell.p, h->start.p, h->exp_table.p, vs,
                     record_buf(h), h->mass[c].p, planes(h), h->nb_listed.p, kernel_values(h), wa);
             else
-                k_exchange_f64<DIM, View, 1><<<blocks, kBlock, 0, st>>>(
+                launch(k_exchange_f64<DIM, View, 1>, blocks, kBlock, st, 
                     n, stride, pos_s, h->image.p, h->rec.p, h->cell.p, h->start.p, h->exp_table.p, vs,
                     record_buf(h), h->mass[c].p, planes(h), h->nb_listed.p, kernel_values(h), wa);
         } else {
             MTPT_TIMED(h, "exchange_f64");
-            k_exchange_f64<DIM, View><<<blocks, kBlock, 0, st>>>(
+            launch(k_exchange_f64<DIM, View>, blocks, kBlock, st, 
                 n, stride, pos_s, h->image.p, h->rec.p, h->cell.p, h->start.p, h->exp_table.p, vs,
-                record_buf(h), h->mass[c].p, planes(h), h->nb_listed.p, kernel_values(h));
+                record_buf(h), h->mass[c].p, planes(h), h->nb_listed.p, kernel_values(h), WalkAhead{});
         }
     } else {
         MTPT_TRY((launch_pairs_f32<DIM, View>(h, vs, o, c, walk_ahead)));
@@ -1154,9 +1173,9 @@ int dispatch_step(mtpt_handle* h, int flags, bool walk_ahead = false) {
     }
 }
 
-// Captures steps into an executable graph: two consecutive plain steps (the
-// buffer pairs swap every step, so two steps return them to the starting
-// arrangement), or, with walk_ahead, one middle step of a walk-ahead run
+// Captures kGraphSteps steps into an executable graph: consecutive plain steps
+// (the buffer pairs swap every step, so an even number returns them to the
+// starting arrangement), or, with walk_ahead, middle steps of a walk-ahead run
 // (entered with the walk done, it leaves it done for the next step and swaps
 // nothing).
 int capture_steps(mtpt_handle* h, int flags, bool walk_ahead) {
@@ -1177,8 +1196,8 @@ int capture_steps(mtpt_handle* h, int flags, bool walk_ahead) {
     DevBuf<double> massb0 = h->massb[0], massb1 = h->massb[1];
     h->stream = h->capture_stream;
     MTPT_CUDA_TRY(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
-    int rc = dispatch_step(h, flags, walk_ahead);
-    if (rc == MTPT_OK && !walk_ahead) rc = dispatch_step(h, flags);
+    int rc = MTPT_OK;
+    for (int64_t k = 0; k < kGraphSteps && rc == MTPT_OK; ++k) rc = dispatch_step(h, flags, walk_ahead);
     cudaGraph_t graph = nullptr;
     const cudaError_t ec = cudaStreamEndCapture(h->stream, &graph);
     // capture only recorded the launches: restore the host bookkeeping
@@ -1226,18 +1245,19 @@ bool walk_ahead_ok(const mtpt_handle* h, int flags) {
 }
 
 int run_steps(mtpt_handle* h, int64_t nsteps, int flags) {
-    const bool use_graph = nsteps >= kGraphMinSteps && !h->timing && !h->tangent_on && h->n > 0;
+    const bool use_graph = nsteps >= kGraphSteps && !h->timing && !h->tangent_on && h->n > 0;
     if (nsteps >= 2 && walk_ahead_ok(h, flags)) {
         // first step (walk, and the record sort after a host load), the middle
-        // steps (replayed from a one-step graph), a last step without walk-ahead
+        // steps (replayed from a graph), a last step without walk-ahead
         MTPT_TRY(dispatch_step(h, flags, true));
         int64_t middle = nsteps - 2;
-        if (use_graph && middle > 0) {
+        if (use_graph && middle >= kGraphSteps) {
             // (walk-ahead runs only with both flags, so the flags need no key)
             const int k = h->cur;
             if (!h->graph_mid[k] || h->graph_mid_mass0[k] != h->mass[0].p)
                 MTPT_TRY(capture_steps(h, flags, true));
-            for (; middle > 0; --middle) MTPT_CUDA_TRY(cudaGraphLaunch(h->graph_mid[k], h->stream));
+            for (; middle >= kGraphSteps; middle -= kGraphSteps)
+                MTPT_CUDA_TRY(cudaGraphLaunch(h->graph_mid[k], h->stream));
         }
         for (; middle > 0; --middle) MTPT_TRY(dispatch_step(h, flags, true));
         MTPT_TRY(dispatch_step(h, flags, false));
@@ -1249,11 +1269,12 @@ int run_steps(mtpt_handle* h, int64_t nsteps, int flags) {
         MTPT_TRY(dispatch_step(h, flags));
         done = 1;
     }
-    if (use_graph) {
+    if (use_graph && nsteps - done >= kGraphSteps) {
         if (!h->graph || h->graph_cur != h->cur || h->graph_flags != flags ||
             h->graph_mass0 != h->mass[0].p)
             MTPT_TRY(capture_steps(h, flags, false));
-        for (; done + 2 <= nsteps; done += 2) MTPT_CUDA_TRY(cudaGraphLaunch(h->graph, h->stream));
+        for (; done + kGraphSteps <= nsteps; done += kGraphSteps)
+            MTPT_CUDA_TRY(cudaGraphLaunch(h->graph, h->stream));
         // an even number of steps leaves the buffers where they started; a
         // transfer step leaves row sums behind
         const bool transfer = (flags & MTPT_DO_TRANSFER) && h->any_transfer;
@@ -1279,7 +1300,7 @@ int unpermute_to(mtpt_handle* h, const double* src, int naxes, double* out_dev) 
                                         cudaMemcpyDeviceToDevice, h->stream));
         return MTPT_OK;
     }
-    k_unpermute<double><<<grid_for(h->n), kBlock, 0, h->stream>>>(
+    launch(k_unpermute<double>, grid_for(h->n), kBlock, h->stream, 
         int(h->n), h->cap, naxes, h->id[h->cur].p, src, 1, 1.0, out_dev);
     MTPT_CUDA_TRY(cudaGetLastError());
     return MTPT_OK;
@@ -1295,7 +1316,7 @@ int copy_out_host(mtpt_handle* h, int naxes, double* out) {
 }
 
 int set_step_dev(mtpt_handle* h, uint64_t step) {
-    k_set_step<<<1, 1, 0, h->stream>>>(h->step_dev.p, (unsigned long long)step);
+    launch(k_set_step, 1, 1, h->stream, h->step_dev.p, (unsigned long long)step);
     MTPT_CUDA_TRY(cudaGetLastError());
     h->step = step;
     return MTPT_OK;
@@ -1673,9 +1694,9 @@ int launch_emit(mtpt_handle* h, int64_t cap) {
     const int64_t stride = h->cap;
     const int c = h->cur, o = 1 - h->cur;
     const View vin = make_view<View>(h, c, c);
-    k_walk_key<DIM, View><<<blocks, kBlock, 0, h->stream>>>(n, stride, h->pos[c].p, h->id[c].p,
+    launch(k_walk_key<DIM, View>, blocks, kBlock, h->stream, n, stride, h->pos[c].p, h->id[c].p,
                                                             h->step_dev.p, 0, 1, vin, h->key.p,
-                                                            h->count.p, h->status.p);
+                                                            h->count.p, h->status.p, nullptr);
     MTPT_TRY(launch_scan(h, h->stream, false));
     MTPT_TRY((launch_sort<DIM, View>(h, c, o, vin)));
     const View vs = make_view<View>(h, o, o);
@@ -1816,11 +1837,11 @@ int launch_adjoint_sort(mtpt_handle* h) {
     cudaStream_t st = h->stream;
     const SingleView v = make_view<SingleView>(h, c, c);
     if (h->any_advect)
-        k_walk_key<DIM, SingleView, true, true><<<grid_for(n), kBlock, 0, st>>>(
+        launch(k_walk_key<DIM, SingleView, true, true>, grid_for(n), kBlock, st, 
             n, h->cap, h->pos[c].p, h->id[c].p, h->step_dev.p, h->any_walk ? 1 : 0, 1, v,
             h->key.p, h->count.p, h->status.p, h->tan[c].p);
     else
-        k_walk_key<DIM, SingleView, true><<<grid_for(n), kBlock, 0, st>>>(
+        launch(k_walk_key<DIM, SingleView, true>, grid_for(n), kBlock, st, 
             n, h->cap, h->pos[c].p, h->id[c].p, h->step_dev.p, h->any_walk ? 1 : 0, 1, v,
             h->key.p, h->count.p, h->status.p, h->tan[c].p);
     MTPT_CUDA_TRY(cudaGetLastError());
@@ -1833,7 +1854,7 @@ template <int DIM>
 int launch_adjoint_rows(mtpt_handle* h, int o, const double* mass, const TapeSlot& t, bool taped) {
     const SingleView v = make_view<SingleView>(h, o, o);
     const TapeOut out = taped ? TapeOut{mass, h->id[o].p, t.mass, t.id, h->tape_flag.p} : TapeOut{};
-    k_adj_rowsum<DIM, SingleView><<<grid_for(h->n), kBlock, 0, h->stream>>>(
+    launch(k_adj_rowsum<DIM, SingleView>, grid_for(h->n), kBlock, h->stream, 
         int(h->n), h->cap, h->pos[o].p, h->image.p, h->tan[o].p, h->rec.p, h->cell.p, h->start.p,
         h->exp_table.p, v, t.r, t.dr, NbPlanes{t.words, h->adj_cap, 0}, t.listed,
         AdjValues{t.kd, h->adj_kcap}, out);
@@ -1849,8 +1870,8 @@ int launch_adjoint_pass(mtpt_handle* h, int o, const TapeSlot& t, double* gD_blo
     const int n = int(h->n), blocks = grid_for(n);
     cudaStream_t st = h->stream;
     const SingleView v = make_view<SingleView>(h, o, o);
-    k_adj_records<<<blocks, kBlock, 0, st>>>(n, t.r, t.dr, t.mass, t.id, h->lam_in.p, h->adj_rec.p);
-    k_adj_exchange<DIM, SingleView><<<blocks, kBlock, 0, st>>>(
+    launch(k_adj_records, blocks, kBlock, st, n, t.r, t.dr, t.mass, t.id, h->lam_in.p, h->adj_rec.p);
+    launch(k_adj_exchange<DIM, SingleView>, blocks, kBlock, st, 
         n, h->cap, h->pos[o].p, h->image.p, h->tan[o].p, h->rec.p, h->cell.p, h->start.p,
         h->exp_table.p, v, h->adj_rec.p, t.id, h->lam_in.p, gD_block,
         NbPlanes{t.words, h->adj_cap, 0}, t.listed, AdjValues{t.kd, h->adj_kcap});
@@ -1859,7 +1880,7 @@ int launch_adjoint_pass(mtpt_handle* h, int o, const TapeSlot& t, double* gD_blo
 }
 
 int sum_blocks(mtpt_handle* h, int64_t parts) {
-    k_sum_into<<<1, kReduceThreads, 0, h->stream>>>(int(parts), h->partial.p, h->acc.p);
+    launch(k_sum_into, 1, kReduceThreads, h->stream, int(parts), h->partial.p, h->acc.p);
     MTPT_CUDA_TRY(cudaGetLastError());
     return MTPT_OK;
 }
@@ -3127,7 +3148,7 @@ extern "C" int mtpt_step_noalloc(const mtpt_params* params, int64_t n, uint64_t 
     MTPT_TRY(build_corners(&h, &head->params, head->corner_first));
     MTPT_TRY(dispatch_step(&h, MTPT_DO_WALK | MTPT_DO_TRANSFER));
     // masses back to the caller's order; positions are already there
-    k_unpermute<double><<<grid_for(n), kBlock, 0, st>>>(int(n), h.cap, 1, h.id[h.cur].p,
+    launch(k_unpermute<double>, grid_for(n), kBlock, st, int(n), h.cap, 1, h.id[h.cur].p,
                                                         h.mass[h.cur].p, 1, 1.0, mass_dev);
     MTPT_CUDA_TRY(cudaGetLastError());
     return MTPT_OK;
