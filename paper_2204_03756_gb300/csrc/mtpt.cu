@@ -639,9 +639,10 @@ int setup_grids(mtpt_handle* h) {
     h->nb_cap = f32 && h->dim == 3 ? list_cap : words;
     h->nb_pad = f32 && h->dim == 2 && usual > 32.0 ? int(std::min(8.0, std::ceil(usual / 32.0))) : 0;
     // kernel values of the binary64 form, per particle; the adjoint's, where 32
-    // particles share their space (1.2 deviations of one are seven of theirs)
+    // particles share their space (neighbours in space, so their mean spreads up
+    // to half as wide as one's count: 3.4 deviations of one among 3e5 particles)
     h->nb_kcap = f32 ? 0 : int(std::min(128.0, std::ceil(expect + 4.0 * std::sqrt(expect) + 4.0)));
-    h->adj_kcap = int(std::min(128.0, std::ceil(expect + 1.2 * std::sqrt(expect) + 2.0)));
+    h->adj_kcap = int(std::min(128.0, std::ceil(expect + 4.0 * std::sqrt(expect) + 2.0)));
     h->adj_cap = words;
     h->n_cells = cell_base;
     h->n_corners = corner_base;
