@@ -2030,17 +2030,11 @@ struct PairFlux {
     }
 };
 
-// Pass 2 of a particle with more than three mask words (long windows), word
-// by word, the next word loaded ahead: {acc_A, comp_A, acc_B, comp_B}.  A
-// real call, so its registers do not weigh on the short particles' loop.
-template <int DIM, bool TWO>
-__device__ __noinline__ float4 words_flux(const uint2* __restrict__ e, int64_t stride,
-                                          uint32_t words, const float4* __restrict__ ex,
-                                          const float2* __restrict__ exb, float4 me, float na,
-                                          float wx, float wy, float rs, float two_beta, float2 ms,
-                                          float2 msb) {
-    const PairFlux<DIM, TWO, false> pf{ex, exb, me, na, wx, wy};
-    FluxSum f{rs, two_beta, ms}, g{rs, two_beta, msb};
+// Pass 2 of a particle's mask words (padding included) word by word, the next
+// word loaded ahead.
+template <int DIM, bool TWO, bool WIDE>
+__device__ __forceinline__ void add_words(const uint2* __restrict__ e, int64_t stride, uint32_t words,
+                                          const PairFlux<DIM, TWO, WIDE>& pf, FluxSum& f, FluxSum& g) {
     uint2 ahead = __ldg(e);
     for (uint32_t w = 1; w <= words; ++w) {
         const uint32_t base = ahead.x;
@@ -2055,6 +2049,20 @@ __device__ __noinline__ float4 words_flux(const uint2* __restrict__ e, int64_t s
             pf.add(f, g, j0, j1, two);
         }
     }
+}
+
+// The same as a real call, for the few particles with more than three words of
+// a run whose windows are short: its registers do not weigh on their loop.
+// {acc_A, comp_A, acc_B, comp_B}.
+template <int DIM, bool TWO>
+__device__ __noinline__ float4 words_flux(const uint2* __restrict__ e, int64_t stride,
+                                          uint32_t words, const float4* __restrict__ ex,
+                                          const float2* __restrict__ exb, float4 me, float na,
+                                          float wx, float wy, float rs, float two_beta, float2 ms,
+                                          float2 msb) {
+    const PairFlux<DIM, TWO, false> pf{ex, exb, me, na, wx, wy};
+    FluxSum f{rs, two_beta, ms}, g{rs, two_beta, msb};
+    add_words<DIM, TWO>(e, stride, words, pf, f, g);
     return make_float4(f.acc, f.comp, g.acc, g.comp);
 }
 
@@ -2066,11 +2074,15 @@ __device__ __noinline__ float4 words_flux(const uint2* __restrict__ e, int64_t s
 // latency.  Masks in place of lists move 24 instead of 45 bytes a particle for
 // eight more operations a neighbour: 104 us at 4e6 particles in 2-d (100 with
 // lists), 1.5 ms at 1e7 with 57 neighbours (2.0).  Registers: 32 keep all 2048
-// threads of an SM (four more would cost 4 us); both species, or a batch's
-// view, need 40 (62 and 58 us at 32 and 40 for the reaction at 1e6).
+// threads of an SM (four more would cost 4 us); both species need 40 (62 and 58
+// us at 32 and 40 for the reaction at 1e6), a batch's view 36 (1.23, 1.15 and 1.19
+// ms at 32, 36 and 40 for the 512-member ensemble).
 // The bounds hold for blocks of 128 too (the tuning's other block size).
-template <int DIM, class View, bool TWO = false, int WALK = 0>
-__global__ void __launch_bounds__(kBlock, (TWO || View::kBatch ? 1536 : 2048) / kBlock)
+// LONG: for runs with long windows (padded words), whose particles all go word
+// by word, inline and with 32-byte loads (1.59 -> 1.39 ms at 1e7 particles with
+// 57 neighbours, the next walk included).
+template <int DIM, class View, bool TWO = false, int WALK = 0, bool LONG = false>
+__global__ void __launch_bounds__(kBlock, (TWO ? 1536 : (View::kBatch || LONG ? 1792 : 2048)) / kBlock)
 k_exchange_f32(int n, int64_t stride, const double* __restrict__ pos, const float* __restrict__ rec,
                const uint32_t* __restrict__ cell, const uint32_t* __restrict__ start,
                const __grid_constant__ View v, const float4* __restrict__ ex,
@@ -2103,7 +2115,9 @@ k_exchange_f32(int n, int64_t stride, const double* __restrict__ pos, const floa
                                               P.g.wf[0], P.g.wf[1]};
             const uint2* e = nb.e + s;
             const uint32_t words = listed & 255u;
-            if (words <= 3u) {
+            if constexpr (LONG) {
+                if (words) add_words<DIM, TWO>(e, stride, words, pf, f, g);
+            } else if (words <= 3u) {
                 // up to three words (a row each, at the densities where a row's
                 // window stays below 32 candidates): one stream of neighbours
                 // over them, so a warp runs as long as its longest particle's

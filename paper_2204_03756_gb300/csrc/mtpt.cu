@@ -885,7 +885,7 @@ int launch_sort_t(mtpt_handle* h, int c, int o, const View& vin) {
         MTPT_CUDA_TRY(cudaGetLastError());
     }
     MTPT_TIMED(h, "gather");
-    launch(k_gather<DIM, View, TANGENT>, blocks, kBlock, h->stream, 
+    launch(k_gather<DIM, View, TANGENT>, blocks, kBlock, h->stream,
         n, stride, h->perm.p, h->sortkey.p, h->start.p, h->pos[c].p, h->mass[c].p, h->id[o].p,
         h->pos[o].p, h->mass[o].p, h->cell.p, h->rec.p, h->corners.p, rid_out, vin, tan_in,
         tan_out, h->reactive ? h->massb[c].p : nullptr, h->reactive ? h->massb[o].p : nullptr,
@@ -904,14 +904,14 @@ int launch_sort_rec(mtpt_handle* h, int c, int o, const SingleView& vin) {
     MTPT_TRY(h->sortrec.ensure(size_t(SortRec<DIM, TANGENT>::kChunks) * size_t(h->cap)));
     {
         MTPT_TIMED(h, "scatter");
-        launch(k_scatter_rec<DIM, TANGENT>, blocks, kBlock, h->stream, 
+        launch(k_scatter_rec<DIM, TANGENT>, blocks, kBlock, h->stream,
             n, stride, h->key.p, h->start.p, h->count.p, h->pos[c].p, h->mass[c].p, h->id[c].p,
             TANGENT ? h->tan[c].p : nullptr, h->sortrec.p);
         MTPT_CUDA_TRY(cudaGetLastError());
     }
     MTPT_TIMED(h, "gather");
     double* tan_out = TANGENT ? h->tan[o].p : nullptr;
-    launch(k_gather_rec<DIM, TANGENT>, blocks, kBlock, h->stream, 
+    launch(k_gather_rec<DIM, TANGENT>, blocks, kBlock, h->stream,
         n, stride, h->sortrec.p, h->start.p, h->id[o].p, h->pos[o].p, h->mass[o].p, h->cell.p,
         h->rec.p, h->corners.p, vin, tan_out, image_buf(h));
     MTPT_CUDA_TRY(cudaGetLastError());
@@ -966,10 +966,15 @@ int launch_exchange_f32(mtpt_handle* h, const View& vs, int o, int c, const NbPl
     if (TWO) reaction_rate(h, &kp, &dt);
     MTPT_TIMED(h, WALK ? "exchange_walk_f32" : "exchange_f32");
     const int n = int(h->n), block = h->pair_block;
-    launch(k_exchange_f32<DIM, View, TWO, WALK>, (n + block - 1) / block, block, h->stream, 
-        n, h->cap, h->pos[o].p, h->rec.p, h->cell.p, h->start.p, vs, h->ex.p, h->mass[o].p,
-        h->mass[c].p, nb, TWO ? h->exb.p : nullptr, TWO ? h->massb[o].p : nullptr,
-        TWO ? h->massb[c].p : nullptr, kp, dt, float(kp * dt), wa);
+    auto go = [&](auto longs) {
+        launch(k_exchange_f32<DIM, View, TWO, WALK, decltype(longs)::value>, (n + block - 1) / block,
+               block, h->stream, n, h->cap, h->pos[o].p, h->rec.p, h->cell.p, h->start.p, vs, h->ex.p,
+               h->mass[o].p, h->mass[c].p, nb, TWO ? h->exb.p : nullptr, TWO ? h->massb[o].p : nullptr,
+               TWO ? h->massb[c].p : nullptr, kp, dt, float(kp * dt), wa);
+    };
+    // (padded words: rows whose windows often pass 32 candidates, 2-d only)
+    if (DIM == 2 && nb.pad > 0) go(std::integral_constant<bool, DIM == 2>{});
+    else go(std::false_type{});
     MTPT_CUDA_TRY(cudaGetLastError());
     return MTPT_OK;
 }
@@ -994,7 +999,7 @@ int launch_pairs_f32(mtpt_handle* h, const View& vs, int o, int c, bool walk_ahe
     const NbPlanes nb = planes(h);
     {
         MTPT_TIMED(h, "rowsum_f32");
-        launch(k_rowsum_f32<DIM, View>, (n + block - 1) / block, block, h->stream, 
+        launch(k_rowsum_f32<DIM, View>, (n + block - 1) / block, block, h->stream,
             n, h->cap, h->pos[o].p, h->rec.p, h->cell.p, h->start.p, vs, h->mass[o].p, h->ex.p,
             h->pair_counter.p, h->ntiles > 0 ? h->id[o].p : nullptr, nb);
         MTPT_CUDA_TRY(cudaGetLastError());
@@ -1025,7 +1030,7 @@ int launch_species_b(mtpt_handle* h, int n, int64_t stride, const double* pos_s,
     {
         MTPT_TIMED(h, "exchange_f64");
         launch(k_record_mass, blocks, kBlock, st, n, h->massb[o].p, record_buf(h));
-        launch(k_exchange_f64<DIM, View>, blocks, kBlock, st, 
+        launch(k_exchange_f64<DIM, View>, blocks, kBlock, st,
             n, stride, pos_s, h->image.p, h->rec.p, h->cell.p, h->start.p, h->exp_table.p, vs,
             record_buf(h), h->massb[c].p, planes(h), h->nb_listed.p, kernel_values(h), WalkAhead{});
     }
@@ -1070,19 +1075,19 @@ int launch_step(mtpt_handle* h, int flags, bool walk_ahead) {
         MTPT_TIMED(h, "walk_key");
         if (h->tangent_on) {
             if (h->any_advect)
-                launch(k_walk_key<DIM, View, true, true>, blocks, kBlock, st, 
+                launch(k_walk_key<DIM, View, true, true>, blocks, kBlock, st,
                     n, stride, h->pos[c].p, h->id[c].p, h->step_dev.p, walk ? 1 : 0,
                     transfer ? 1 : 0, vin, h->key.p, h->count.p, h->status.p, h->tan[c].p);
             else
-                launch(k_walk_key<DIM, View, true>, blocks, kBlock, st, 
+                launch(k_walk_key<DIM, View, true>, blocks, kBlock, st,
                     n, stride, h->pos[c].p, h->id[c].p, h->step_dev.p, walk ? 1 : 0,
                     transfer ? 1 : 0, vin, h->key.p, h->count.p, h->status.p, h->tan[c].p);
         } else if (h->any_advect) {
-            launch(k_walk_key<DIM, View, false, true>, blocks, kBlock, st, 
+            launch(k_walk_key<DIM, View, false, true>, blocks, kBlock, st,
                 n, stride, h->pos[c].p, h->id[c].p, h->step_dev.p, walk ? 1 : 0,
                 transfer ? 1 : 0, vin, h->key.p, h->count.p, h->status.p, nullptr);
         } else {
-            launch(k_walk_key<DIM, View>, blocks, kBlock, st, 
+            launch(k_walk_key<DIM, View>, blocks, kBlock, st,
                 n, stride, h->pos[c].p, h->id[c].p, h->step_dev.p, walk ? 1 : 0,
                 transfer ? 1 : 0, vin, h->key.p, h->count.p, h->status.p, nullptr);
         }
@@ -1109,7 +1114,7 @@ int launch_step(mtpt_handle* h, int flags, bool walk_ahead) {
     if (!split) {
         {
             MTPT_TIMED(h, "rowsum_f64");
-            launch(k_rowsum_f64<DIM, View>, blocks, kBlock, st, 
+            launch(k_rowsum_f64<DIM, View>, blocks, kBlock, st,
                 n, stride, pos_s, h->image.p, h->rec.p, h->cell.p, h->start.p, h->exp_table.p, vs,
                 h->mass[o].p, record_buf(h), h->pair_counter.p, planes(h), h->nb_listed.p,
                 kernel_values(h),
@@ -1125,16 +1130,16 @@ int launch_step(mtpt_handle* h, int flags, bool walk_ahead) {
             }
             MTPT_TIMED(h, "exchange_walk_f64");
             if (h->any_advect)
-                launch(k_exchange_f64<DIM, View, 2>, blocks, kBlock, st, 
+                launch(k_exchange_f64<DIM, View, 2>, blocks, kBlock, st,
                     n, stride, pos_s, h->image.p, h->rec.p, h->cell.p, h->start.p, h->exp_table.p, vs,
                     record_buf(h), h->mass[c].p, planes(h), h->nb_listed.p, kernel_values(h), wa);
             else
-                launch(k_exchange_f64<DIM, View, 1>, blocks, kBlock, st, 
+                launch(k_exchange_f64<DIM, View, 1>, blocks, kBlock, st,
                     n, stride, pos_s, h->image.p, h->rec.p, h->cell.p, h->start.p, h->exp_table.p, vs,
                     record_buf(h), h->mass[c].p, planes(h), h->nb_listed.p, kernel_values(h), wa);
         } else {
             MTPT_TIMED(h, "exchange_f64");
-            launch(k_exchange_f64<DIM, View>, blocks, kBlock, st, 
+            launch(k_exchange_f64<DIM, View>, blocks, kBlock, st,
                 n, stride, pos_s, h->image.p, h->rec.p, h->cell.p, h->start.p, h->exp_table.p, vs,
                 record_buf(h), h->mass[c].p, planes(h), h->nb_listed.p, kernel_values(h), WalkAhead{});
         }
@@ -1301,7 +1306,7 @@ int unpermute_to(mtpt_handle* h, const double* src, int naxes, double* out_dev) 
                                         cudaMemcpyDeviceToDevice, h->stream));
         return MTPT_OK;
     }
-    launch(k_unpermute<double>, grid_for(h->n), kBlock, h->stream, 
+    launch(k_unpermute<double>, grid_for(h->n), kBlock, h->stream,
         int(h->n), h->cap, naxes, h->id[h->cur].p, src, 1, 1.0, out_dev);
     MTPT_CUDA_TRY(cudaGetLastError());
     return MTPT_OK;
@@ -1838,11 +1843,11 @@ int launch_adjoint_sort(mtpt_handle* h) {
     cudaStream_t st = h->stream;
     const SingleView v = make_view<SingleView>(h, c, c);
     if (h->any_advect)
-        launch(k_walk_key<DIM, SingleView, true, true>, grid_for(n), kBlock, st, 
+        launch(k_walk_key<DIM, SingleView, true, true>, grid_for(n), kBlock, st,
             n, h->cap, h->pos[c].p, h->id[c].p, h->step_dev.p, h->any_walk ? 1 : 0, 1, v,
             h->key.p, h->count.p, h->status.p, h->tan[c].p);
     else
-        launch(k_walk_key<DIM, SingleView, true>, grid_for(n), kBlock, st, 
+        launch(k_walk_key<DIM, SingleView, true>, grid_for(n), kBlock, st,
             n, h->cap, h->pos[c].p, h->id[c].p, h->step_dev.p, h->any_walk ? 1 : 0, 1, v,
             h->key.p, h->count.p, h->status.p, h->tan[c].p);
     MTPT_CUDA_TRY(cudaGetLastError());
@@ -1855,7 +1860,7 @@ template <int DIM>
 int launch_adjoint_rows(mtpt_handle* h, int o, const double* mass, const TapeSlot& t, bool taped) {
     const SingleView v = make_view<SingleView>(h, o, o);
     const TapeOut out = taped ? TapeOut{mass, h->id[o].p, t.mass, t.id, h->tape_flag.p} : TapeOut{};
-    launch(k_adj_rowsum<DIM, SingleView>, grid_for(h->n), kBlock, h->stream, 
+    launch(k_adj_rowsum<DIM, SingleView>, grid_for(h->n), kBlock, h->stream,
         int(h->n), h->cap, h->pos[o].p, h->image.p, h->tan[o].p, h->rec.p, h->cell.p, h->start.p,
         h->exp_table.p, v, t.r, t.dr, NbPlanes{t.words, h->adj_cap, 0}, t.listed,
         AdjValues{t.kd, h->adj_kcap}, out);
@@ -1872,7 +1877,7 @@ int launch_adjoint_pass(mtpt_handle* h, int o, const TapeSlot& t, double* gD_blo
     cudaStream_t st = h->stream;
     const SingleView v = make_view<SingleView>(h, o, o);
     launch(k_adj_records, blocks, kBlock, st, n, t.r, t.dr, t.mass, t.id, h->lam_in.p, h->adj_rec.p);
-    launch(k_adj_exchange<DIM, SingleView>, blocks, kBlock, st, 
+    launch(k_adj_exchange<DIM, SingleView>, blocks, kBlock, st,
         n, h->cap, h->pos[o].p, h->image.p, h->tan[o].p, h->rec.p, h->cell.p, h->start.p,
         h->exp_table.p, v, h->adj_rec.p, t.id, h->lam_in.p, gD_block,
         NbPlanes{t.words, h->adj_cap, 0}, t.listed, AdjValues{t.kd, h->adj_kcap});
