@@ -577,15 +577,17 @@ k_scan(const uint4* __restrict__ count4, uint4* __restrict__ start4,
     __shared__ uint32_t s_tile;
     __shared__ unsigned long long s_tag;
     after_previous();
-    if (threadIdx.x == 0) {
+    // (a grid of one tile, the small runs', has no tile to wait for or to tell)
+    const bool single = ntiles == 1;
+    if (threadIdx.x == 0 && !single) {
         // tiles in ticket order: a block only ever waits on blocks that started
         const unsigned long long t = atomicAdd(state + ntiles, 1ull);
         s_tile = uint32_t(t % unsigned(ntiles));
         s_tag = (t / unsigned(ntiles)) % kScanTagMod + 1ull;
     }
-    __syncthreads();
-    const uint32_t tile = s_tile;
-    const unsigned long long tag = s_tag;
+    if (!single) __syncthreads();
+    const uint32_t tile = single ? 0u : s_tile;
+    const unsigned long long tag = single ? 0ull : s_tag;
     // this thread's 16 consecutive cells
     const size_t base = (size_t(tile) * kScanThreads + threadIdx.x) * kVec;
     uint4 c[kVec];
@@ -597,7 +599,7 @@ k_scan(const uint4* __restrict__ count4, uint4* __restrict__ start4,
     }
     uint32_t total;
     const uint32_t excl = block_exclusive_scan(own, &total);
-    if (threadIdx.x == 0 && int(tile) != hold) st_relaxed_u64(state + tile, (tag << 32) | total);
+    if (threadIdx.x == 0 && !single && int(tile) != hold) st_relaxed_u64(state + tile, (tag << 32) | total);
     // the totals of every earlier tile, one word per thread at a time
     uint32_t part = 0;
     bool gave_up = false;
@@ -616,8 +618,8 @@ k_scan(const uint4* __restrict__ count4, uint4* __restrict__ start4,
         }
     }
     if (gave_up) atomicAdd(&g_scan_waits_given_up, 1ull);
-    uint32_t prefix;
-    block_exclusive_scan(part, &prefix);
+    uint32_t prefix = 0;
+    if (!single) block_exclusive_scan(part, &prefix);
     if (advance && threadIdx.x == 0 && tile == uint32_t(ntiles - 1)) *step_dev += 1ull;
     uint32_t e = prefix + excl;
 #pragma unroll
