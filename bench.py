@@ -69,27 +69,30 @@ def _algo_bytes_per_particle(kernel: str, dim: int, form: str) -> float:
         "rowsum_f64": x + r, "rowsum_f32": x + r,          # positions in, r out
         "exchange_f64": x + 8 + r + 8, "exchange_f32": x + 8 + r + 8,  # X, M, r in; M out
         # pass 2 and the next step's walk (walk-ahead): both kernels' bytes
-        "exchange_walk_f32": x + 8 + r + 8 + 2 * x,
+        "exchange_walk_f32": x + 8 + r + 8 + 2 * x, "exchange_walk_f64": x + 8 + r + 8 + 2 * x,
         "gather": 2 * (x + 8 + 4),         # state copied into cell order
         "scatter": 8, "scan": 0,
     }
     return float(table.get(kernel, 0))
 
 
-# DRAM bytes per particle of each kernel from one-kernel ncu captures of the
-# bench's own launch (profiles/step_kernels_gaussian_2d_4M.md: gaussian_2d,
-# 4e6 particles, precision form, one launch per capture after three steps).
+# DRAM bytes per particle of each kernel from ncu captures of the step at the
+# bench's size (profiles/step_kernels_gaussian_2d_4M.md: 4e6 particles uniform
+# at density 1, both forms, in the steady state of a run).
 # Valid only for the library source it was measured on: a different hash of
 # the CUDA sources and the header reports traffic as null.
 TRAFFIC_DIM = 2
-TRAFFIC_SOURCE_SHA1 = "fd2803d8f07e"
+TRAFFIC_SOURCE_SHA1 = "ba807a185991"
 TRAFFIC_BYTES_PER_PARTICLE = {
-    "walk_key": (88933632 + 31892736) / 4e6,
-    "scatter": (81824512 + 34699776) / 4e6,
-    "gather": (152929792 + 124269312) / 4e6,
-    "rowsum_f32": (238171904 + 292427776) / 4e6,
-    "exchange_f32": (389639424 + 26841344) / 4e6,
-    "exchange_walk_f32": (478508544 + 117244416) / 4e6,
+    "walk_key": (88931840 + 26869760) / 4e6,
+    "scatter": (81750016 + 31522560) / 4e6,
+    "gather": (152978688 + 121016320) / 4e6,
+    "rowsum_f32": (129983232 + 160186368) / 4e6,
+    "exchange_f32": (255971584 + 23240960) / 4e6,
+    "exchange_walk_f32": (344909056 + 114266624) / 4e6,
+    "rowsum_f64": (301616896 + 357873664) / 4e6,
+    "exchange_f64": (468413184 + 25653248) / 4e6,
+    "exchange_walk_f64": (557378560 + 118183424) / 4e6,
 }
 
 
@@ -98,12 +101,15 @@ TRAFFIC_BYTES_PER_PARTICLE = {
 # issue rate, against the issue peak of 4 warp instructions per clock per SM
 # (one per scheduler).
 INSTR_PER_PARTICLE = {
-    "walk_key": 43906125 / 4e6,
-    "scatter": 4125000 / 4e6,
-    "gather": 38024198 / 4e6,
-    "rowsum_f32": 178884629 / 4e6,
-    "exchange_f32": 49384081 / 4e6,
-    "exchange_walk_f32": 93525743 / 4e6,
+    "walk_key": 44144207 / 4e6,
+    "scatter": 4375000 / 4e6,
+    "gather": 40648040 / 4e6,
+    "rowsum_f32": 139910274 / 4e6,
+    "exchange_f32": 77449564 / 4e6,
+    "exchange_walk_f32": 121358548 / 4e6,
+    "rowsum_f64": 307013436 / 4e6,
+    "exchange_f64": 221882905 / 4e6,
+    "exchange_walk_f64": 266126674 / 4e6,
 }
 SMS, SCHEDULERS_PER_SM = 152, 4
 
@@ -112,15 +118,16 @@ SMS, SCHEDULERS_PER_SM = 152, 4
 # profiles/step_kernels_gaussian_2d_4M.md), reported beside the roofline
 # while the kernel source hash matches.
 BINDING = {
-    "exchange_f32": ("DRAM 58 % with long-scoreboard stalls on the list reads and the "
-                     "neighbour-record gathers; issue 46 % at 21 of 32 active lanes"),
-    "exchange_walk_f32": ("DRAM 59 % and binary64 pipe 52 % (pass 2's update and the next "
-                          "step's x + sigma xi); issue 61 % at 26 of 32 active lanes"),
-    "rowsum_f32": "instruction issue: 72 % of issue slots at 18 of 32 active lanes; DRAM 32 %",
-    "rowsum_f64": "binary64 pipe 86 % busy",
-    "exchange_f64": "binary64 pipe 86 % busy",
-    "gather": "DRAM 62 % (payload reads through the permutation, cell-ordered writes)",
-    "scatter": "DRAM 42 % at 10 % issue (slot atomics, permutation and sort-key stores)",
+    "exchange_f32": ("instruction issue 62 % at 18 of 32 active lanes, waiting on the "
+                     "neighbour-record gathers; DRAM 35 %"),
+    "exchange_walk_f32": ("instruction issue 72 % at 23 of 32 active lanes and binary64 pipe 49 % "
+                          "(the next step's x + sigma xi); DRAM 43 %"),
+    "rowsum_f32": "instruction issue: 80 % of issue slots at 24 of 32 active lanes; DRAM 26 %",
+    "rowsum_f64": "instruction issue 72 % at 20 of 32 active lanes (integer kernel values)",
+    "exchange_f64": "instruction issue 66 % at 18 of 32 active lanes and binary64 pipe 59 %",
+    "exchange_walk_f64": "instruction issue 66 % at 20 of 32 active lanes and binary64 pipe 61 %",
+    "gather": "DRAM 59 % (payload reads through the permutation, cell-ordered writes), issue 56 %",
+    "scatter": "DRAM 41 % at 10 % issue (slot atomics, permutation and sort-key stores)",
     "walk_key": "binary64 pipe 80 % busy (x + sigma xi)",
 }
 
@@ -511,22 +518,6 @@ def time_adjoint(rank, nbins=(100, 100), checkpoint_every=20):
             "precision": "forward fp32w, adjoint passes f64"}
 
 
-# binary64 instructions per accepted ordered pair of the binary64 pair passes:
-# rowsum -- squared distance 2d (a difference and a multiply or fma per axis),
-# the kernel exponential 7 (2 fma reduction, 4 fma polynomial, 1 table
-# multiply; the reduction index and the 2^-q scaling are integer/binary32),
-# the row-sum add 1; exchange (kernel values read back from the neighbour
-# lists) -- r_i + r_j 1, the quotient 5 (Newton step 2, product 1,
-# correction 2), the mass difference, the product and the flux add 3.
-def _f64_ops_per_pair(kernel: str, dim: int) -> float:
-    return {"rowsum_f64": 2 * dim + 7 + 1, "exchange_f64": 1 + 5 + 3}[kernel]
-
-
-# GB300 binary64 issue rate: 2 binary64 operations per clock per SM (recipe's
-# 1.25 TFLOP/s counts an fma as two) x 152 SMs x 2.07 GHz
-F64_PEAK_OPS = 2 * 152 * 2.07e9
-
-
 def issue_rate(name, w, per_launch_s, clocks):
     """Warp instructions issued per second by one launch of `name` (from the
     captured count per particle) against the issue peak at the SM clock the
@@ -549,16 +540,6 @@ def roofline(w, res, peaks):
     share = total_ms / sum(v[1] for v in kst.values())
     current = w.dim == TRAFFIC_DIM and _kernel_source_sha1() == TRAFFIC_SOURCE_SHA1
     binding = BINDING.get(name) if current else None
-    if name in ("rowsum_f64", "exchange_f64"):
-        pairs = res["pairs_per_particle_step"] * w.n
-        ops = _f64_ops_per_pair(name, w.dim) * pairs
-        achieved = ops / per_launch_s / 1e9
-        return {"bound": "alu", "kernel": name, "achieved": achieved,
-                "peak": F64_PEAK_OPS / 1e9, "unit": "G binary64 op/s",
-                "frac": achieved / (F64_PEAK_OPS / 1e9), "traffic": None,
-                "algorithmic_ops_per_launch": ops, "launch_ms": per_launch_s * 1e3,
-                "share_of_step": share, "binding_ncu": binding,
-                "peak_source": "derived: 2 binary64 ops/clk/SM x 152 SMs x 2.07 GHz"}
     algo = _algo_bytes_per_particle(name, w.dim, res["form"]) * w.n
     achieved = algo / per_launch_s / 1e9
     traffic = None

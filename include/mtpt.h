@@ -386,8 +386,10 @@ int mtpt_step_noalloc(const mtpt_params* params, int64_t n, uint64_t step, doubl
  * loaded state, as mtpt_step does, while
  * recording a checkpoint of the state every `checkpoint_every` steps and the
  * position tangents dX/dD.  Memory: (nsteps / checkpoint_every +
- * checkpoint_every + 1) snapshots of (4 dim + 12) bytes per particle.
- * Synchronises. */
+ * checkpoint_every + 1) snapshots of (16 dim + 12) bytes per particle, and, when
+ * it can be had and is at most 16 GiB, a tape of checkpoint_every steps (some
+ * 250 bytes per particle and step at 3 neighbours) that spares the reverse
+ * sweep each step's second walk, sort and search.  Synchronises. */
 int mtpt_adjoint_forward(mtpt_handle* h, int64_t nsteps, int64_t checkpoint_every);
 
 /* Adjoint (no counterpart in the paper).  Reverse sweep of the run recorded

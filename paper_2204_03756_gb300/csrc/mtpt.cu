@@ -303,7 +303,7 @@ struct mtpt_handle {
     cudaGraphExec_t graph = nullptr;
     int graph_cur = -1, graph_flags = -1;
     const double* graph_mass0 = nullptr;
-    // one walk-ahead middle step, per current buffer (a call's last step
+    // walk-ahead middle steps, per current buffer (a call's last step
     // swaps the pairs, so consecutive calls alternate between the two)
     cudaGraphExec_t graph_mid[2] = {nullptr, nullptr};
     const double* graph_mid_mass0[2] = {nullptr, nullptr};
@@ -1017,7 +1017,7 @@ int launch_pairs_f32(mtpt_handle* h, const View& vs, int o, int c, bool walk_ahe
 }
 
 // Species B of a binary64 reaction run: its transfer with the weights of
-// this step (the row sums and neighbour lists of species A's passes), then
+// this step (the row sums, mask words and kernel values of species A's passes), then
 // the reaction on every particle (k_react).  B's masses move from buffer o
 // to c like A's.  (The precision form does both species and the reaction in
 // one pass 2: launch_pairs_f32.)
