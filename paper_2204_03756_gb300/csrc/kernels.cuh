@@ -1786,7 +1786,8 @@ k_rowsum_f32(int n, int64_t stride, const double* __restrict__ pos, const float*
              const uint32_t* __restrict__ cell, const uint32_t* __restrict__ start,
              const __grid_constant__ View v, const double* __restrict__ mass,
              float4* __restrict__ ex, unsigned long long* __restrict__ pair_counter,
-             const uint32_t* __restrict__ ghost_id, const __grid_constant__ NbPlanes nb) {
+             const uint32_t* __restrict__ ghost_id, const __grid_constant__ NbPlanes nb,
+             const double* __restrict__ mass_b, float2* __restrict__ exb) {
     const int s = int(ordered_index());
     uint32_t cnt = 0;
     if (s < n) {
@@ -1846,6 +1847,10 @@ k_rowsum_f32(int n, int64_t stride, const double* __restrict__ pos, const float*
         const float4 m = make_float4(mhi, mlo, __fsub_rn(rsum, rc), __uint_as_float(list_word));
         if constexpr (DIM == 3) ex[s] = m;
         else store_pair_rec(ex, uint32_t(s), load_rec(rec, uint32_t(s)), m);
+        if (mass_b) {                      // a reaction: species B's split for pass 2
+            split_double(mass_b[s], &mhi, &mlo);
+            exb[s] = make_float2(mhi, mlo);
+        }
         // with ghost_id (a tile), pairs are counted for the tile's own particles only
         if (ghost_id && (ghost_id[s] & kGhostBit)) cnt = 0;
     }
@@ -1915,17 +1920,6 @@ __device__ __noinline__ float2 search_flux(uint32_t s, int64_t stride,
 // that neither D -> 0 nor the species in deficit loses digits).  A particle
 // with a negative mass of either species (sign bit set) does not react.
 // ---------------------------------------------------------------------------
-
-// The precision form's mass split of species B for its pass 2: the binary32
-// head/tail of mass_b[s] (species A's is in the particle record ex).
-__global__ void __launch_bounds__(kBlock)
-k_split_mass(int n, const double* __restrict__ mass_b, float2* __restrict__ exb) {
-    const int s = int(ordered_index());
-    if (s >= n) return;
-    float hi, lo;
-    split_double(mass_b[s], &hi, &lo);
-    exb[s] = make_float2(hi, lo);
-}
 
 // F64: binary64 throughout (exp, expm1 and IEEE division).  Otherwise (the
 // precision form) the two factors 1/q and e^-x / q in binary32 from the

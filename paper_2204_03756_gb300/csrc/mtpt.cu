@@ -1001,15 +1001,13 @@ int launch_pairs_f32(mtpt_handle* h, const View& vs, int o, int c, bool walk_ahe
         MTPT_TIMED(h, "rowsum_f32");
         launch(k_rowsum_f32<DIM, View>, (n + block - 1) / block, block, h->stream,
             n, h->cap, h->pos[o].p, h->rec.p, h->cell.p, h->start.p, vs, h->mass[o].p, h->ex.p,
-            h->pair_counter.p, h->ntiles > 0 ? h->id[o].p : nullptr, nb);
+            h->pair_counter.p, h->ntiles > 0 ? h->id[o].p : nullptr, nb,
+            h->reactive ? h->massb[o].p : nullptr, h->exb.p);
         MTPT_CUDA_TRY(cudaGetLastError());
     }
     if constexpr (!View::kBatch) {
         if (h->reactive) {
-            // species B's split, then one pass 2 for both species and the
-            // reaction (batches refuse it)
-            launch(k_split_mass, grid_for(n), kBlock, h->stream, n, h->massb[o].p, h->exb.p);
-            MTPT_CUDA_TRY(cudaGetLastError());
+            // one pass 2 for both species and the reaction (batches refuse it)
             return launch_exchange_f32<DIM, View, true>(h, vs, o, c, nb, walk_ahead);
         }
     }
