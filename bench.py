@@ -82,17 +82,17 @@ def _algo_bytes_per_particle(kernel: str, dim: int, form: str) -> float:
 # Valid only for the library source it was measured on: a different hash of
 # the CUDA sources and the header reports traffic as null.
 TRAFFIC_DIM = 2
-TRAFFIC_SOURCE_SHA1 = "ba807a185991"
+TRAFFIC_SOURCE_SHA1 = "017bf38ccff2"
 TRAFFIC_BYTES_PER_PARTICLE = {
-    "walk_key": (88931840 + 26869760) / 4e6,
-    "scatter": (81750016 + 31522560) / 4e6,
-    "gather": (152978688 + 121016320) / 4e6,
-    "rowsum_f32": (129983232 + 160186368) / 4e6,
-    "exchange_f32": (255971584 + 23240960) / 4e6,
-    "exchange_walk_f32": (344909056 + 114266624) / 4e6,
-    "rowsum_f64": (301616896 + 357873664) / 4e6,
-    "exchange_f64": (468413184 + 25653248) / 4e6,
-    "exchange_walk_f64": (557378560 + 118183424) / 4e6,
+    "walk_key": (88930048 + 26795264) / 4e6,
+    "scatter": (81750272 + 31210752) / 4e6,
+    "gather": (152943872 + 120843520) / 4e6,
+    "rowsum_f32": (129801216 + 160057088) / 4e6,
+    "exchange_f32": (256001024 + 22994944) / 4e6,
+    "exchange_walk_f32": (344891392 + 114317312) / 4e6,
+    "rowsum_f64": (301448704 + 358059776) / 4e6,
+    "exchange_f64": (468410624 + 25627136) / 4e6,
+    "exchange_walk_f64": (557393152 + 118498048) / 4e6,
 }
 
 
@@ -103,7 +103,7 @@ TRAFFIC_BYTES_PER_PARTICLE = {
 INSTR_PER_PARTICLE = {
     "walk_key": 44144207 / 4e6,
     "scatter": 4375000 / 4e6,
-    "gather": 40648040 / 4e6,
+    "gather": 40648032 / 4e6,
     "rowsum_f32": 139910274 / 4e6,
     "exchange_f32": 77449564 / 4e6,
     "exchange_walk_f32": 121358548 / 4e6,
@@ -120,13 +120,13 @@ SMS, SCHEDULERS_PER_SM = 152, 4
 BINDING = {
     "exchange_f32": ("instruction issue 62 % at 18 of 32 active lanes, waiting on the "
                      "neighbour-record gathers; DRAM 35 %"),
-    "exchange_walk_f32": ("instruction issue 72 % at 23 of 32 active lanes and binary64 pipe 49 % "
+    "exchange_walk_f32": ("instruction issue 72 % at 23 of 32 active lanes and binary64 pipe 50 % "
                           "(the next step's x + sigma xi); DRAM 43 %"),
-    "rowsum_f32": "instruction issue: 80 % of issue slots at 24 of 32 active lanes; DRAM 26 %",
+    "rowsum_f32": "instruction issue: 79 % of issue slots at 24 of 32 active lanes; DRAM 26 %",
     "rowsum_f64": "instruction issue 72 % at 20 of 32 active lanes (integer kernel values)",
-    "exchange_f64": "instruction issue 66 % at 18 of 32 active lanes and binary64 pipe 59 %",
-    "exchange_walk_f64": "instruction issue 66 % at 20 of 32 active lanes and binary64 pipe 61 %",
-    "gather": "DRAM 59 % (payload reads through the permutation, cell-ordered writes), issue 56 %",
+    "exchange_f64": "instruction issue 67 % at 18 of 32 active lanes and binary64 pipe 60 %",
+    "exchange_walk_f64": "instruction issue 66 % at 20 of 32 active lanes and binary64 pipe 62 %",
+    "gather": "DRAM 60 % (payload reads through the permutation, cell-ordered writes), issue 57 %",
     "scatter": "DRAM 41 % at 10 % issue (slot atomics, permutation and sort-key stores)",
     "walk_key": "binary64 pipe 80 % busy (x + sigma xi)",
 }
