@@ -1561,8 +1561,12 @@ k_rowsum_f64(int n, int64_t stride, const double* __restrict__ pos,
              uint32_t* __restrict__ listed_out, PairValues kv,
              const uint32_t* __restrict__ ghost_id) {
     __shared__ double table[kExpTable];
-    const uint32_t s = ordered_index();
+    // Ahead of the wait, here and in pass 2: a copy from the host wrote the table,
+    // never a kernel, and it overlaps the kernel before (100 steps of 1e4
+    // particles: 3.15 -> 3.06 ms; nothing at 4e6).  Without the table in shared
+    // memory pass 2's dense runs took 1 % longer.
     for (int t = threadIdx.x; t < kExpTable; t += blockDim.x) table[t] = exp_table[t];
+    const uint32_t s = ordered_index();
     __syncthreads();
     uint32_t cnt = 0;
     if (s < uint32_t(n)) {
@@ -1695,8 +1699,8 @@ k_exchange_f64(int n, int64_t stride, const double* __restrict__ pos,
                const uint32_t* __restrict__ listed_in, PairValues kv,
                const WalkAhead wa = WalkAhead{}) {
     __shared__ double table[kExpTable];   // of use to the particles that search or evaluate again
-    const uint32_t s = ordered_index();
     for (int t = threadIdx.x; t < kExpTable; t += blockDim.x) table[t] = exp_table[t];
+    const uint32_t s = ordered_index();   // (the table ahead of the wait, as in pass 1)
     __syncthreads();
     if (s >= uint32_t(n)) return;
     const RealParams& P = v.of_sorted(s);
