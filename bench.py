@@ -82,17 +82,17 @@ def _algo_bytes_per_particle(kernel: str, dim: int, form: str) -> float:
 # Valid only for the library source it was measured on: a different hash of
 # the CUDA sources and the header reports traffic as null.
 TRAFFIC_DIM = 2
-TRAFFIC_SOURCE_SHA1 = "017bf38ccff2"
+TRAFFIC_SOURCE_SHA1 = "fbf8b19fbc7c"
 TRAFFIC_BYTES_PER_PARTICLE = {
-    "walk_key": (88930048 + 26795264) / 4e6,
-    "scatter": (81750272 + 31210752) / 4e6,
-    "gather": (152943872 + 120843520) / 4e6,
-    "rowsum_f32": (129801216 + 160057088) / 4e6,
-    "exchange_f32": (256001024 + 22994944) / 4e6,
-    "exchange_walk_f32": (344891392 + 114317312) / 4e6,
-    "rowsum_f64": (301448704 + 358059776) / 4e6,
-    "exchange_f64": (468410624 + 25627136) / 4e6,
-    "exchange_walk_f64": (557393152 + 118498048) / 4e6,
+    "walk_key": (88931328 + 26738432) / 4e6,
+    "scatter": (81750016 + 31188224) / 4e6,
+    "gather": (152983296 + 121382656) / 4e6,
+    "rowsum_f32": (129977088 + 159955712) / 4e6,
+    "exchange_f32": (256063488 + 23515392) / 4e6,
+    "exchange_walk_f32": (344992512 + 114313216) / 4e6,
+    "rowsum_f64": (301554176 + 358192640) / 4e6,
+    "exchange_f64": (468451584 + 25626368) / 4e6,
+    "exchange_walk_f64": (557374464 + 118109952) / 4e6,
 }
 
 
@@ -103,13 +103,13 @@ TRAFFIC_BYTES_PER_PARTICLE = {
 INSTR_PER_PARTICLE = {
     "walk_key": 44144207 / 4e6,
     "scatter": 4375000 / 4e6,
-    "gather": 40648032 / 4e6,
+    "gather": 40648031 / 4e6,
     "rowsum_f32": 139910274 / 4e6,
     "exchange_f32": 77449564 / 4e6,
     "exchange_walk_f32": 121358548 / 4e6,
-    "rowsum_f64": 307013436 / 4e6,
-    "exchange_f64": 221882905 / 4e6,
-    "exchange_walk_f64": 266126674 / 4e6,
+    "rowsum_f64": 307388436 / 4e6,
+    "exchange_f64": 222132905 / 4e6,
+    "exchange_walk_f64": 266376106 / 4e6,
 }
 SMS, SCHEDULERS_PER_SM = 152, 4
 
@@ -120,13 +120,13 @@ SMS, SCHEDULERS_PER_SM = 152, 4
 BINDING = {
     "exchange_f32": ("instruction issue 62 % at 18 of 32 active lanes, waiting on the "
                      "neighbour-record gathers; DRAM 35 %"),
-    "exchange_walk_f32": ("instruction issue 72 % at 23 of 32 active lanes and binary64 pipe 50 % "
+    "exchange_walk_f32": ("instruction issue 72 % at 23 of 32 active lanes and binary64 pipe 49 % "
                           "(the next step's x + sigma xi); DRAM 43 %"),
     "rowsum_f32": "instruction issue: 79 % of issue slots at 24 of 32 active lanes; DRAM 26 %",
     "rowsum_f64": "instruction issue 72 % at 20 of 32 active lanes (integer kernel values)",
-    "exchange_f64": "instruction issue 67 % at 18 of 32 active lanes and binary64 pipe 60 %",
-    "exchange_walk_f64": "instruction issue 66 % at 20 of 32 active lanes and binary64 pipe 62 %",
-    "gather": "DRAM 60 % (payload reads through the permutation, cell-ordered writes), issue 57 %",
+    "exchange_f64": "instruction issue 66 % at 18 of 32 active lanes and binary64 pipe 59 %",
+    "exchange_walk_f64": "instruction issue 66 % at 20 of 32 active lanes and binary64 pipe 61 %",
+    "gather": "DRAM 60 % (payload reads through the permutation, cell-ordered writes), issue 56 %",
     "scatter": "DRAM 41 % at 10 % issue (slot atomics, permutation and sort-key stores)",
     "walk_key": "binary64 pipe 80 % busy (x + sigma xi)",
 }
