@@ -73,6 +73,8 @@ constexpr int kScanTile = kScanPerThread * kScanThreads;  // cells per scan bloc
 // takes the set-up of each launch out of the chain: one step of 1e4 particles and
 // its two reads 55.7 -> 39.0 us (eight kernels), the adjoint's 200 steps of 250,000
 // 44.5 -> 38.5 ms.
+// (For kernels that only update a word in place: what is read through a pointer
+// to const goes through ordered_index.)
 __device__ __forceinline__ void after_previous() {
     asm volatile("griddepcontrol.launch_dependents;");
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -576,10 +578,11 @@ k_scan(const uint4* __restrict__ count4, uint4* __restrict__ start4,
     constexpr int kVec = kScanPerThread / 4;
     __shared__ uint32_t s_tile;
     __shared__ unsigned long long s_tag;
-    after_previous();
+    // (one block a tile: its threads' indexes, behind the wait)
+    const uint32_t thread = ordered_index() % uint32_t(kScanThreads);
     // (a grid of one tile, the small runs', has no tile to wait for or to tell)
     const bool single = ntiles == 1;
-    if (threadIdx.x == 0 && !single) {
+    if (thread == 0 && !single) {
         // tiles in ticket order: a block only ever waits on blocks that started
         const unsigned long long t = atomicAdd(state + ntiles, 1ull);
         s_tile = uint32_t(t % unsigned(ntiles));
@@ -589,7 +592,7 @@ k_scan(const uint4* __restrict__ count4, uint4* __restrict__ start4,
     const uint32_t tile = single ? 0u : s_tile;
     const unsigned long long tag = single ? 0ull : s_tag;
     // this thread's 16 consecutive cells
-    const size_t base = (size_t(tile) * kScanThreads + threadIdx.x) * kVec;
+    const size_t base = (size_t(tile) * kScanThreads + thread) * kVec;
     uint4 c[kVec];
     uint32_t own = 0;
 #pragma unroll
@@ -599,11 +602,11 @@ k_scan(const uint4* __restrict__ count4, uint4* __restrict__ start4,
     }
     uint32_t total;
     const uint32_t excl = block_exclusive_scan(own, &total);
-    if (threadIdx.x == 0 && !single && int(tile) != hold) st_relaxed_u64(state + tile, (tag << 32) | total);
+    if (thread == 0 && !single && int(tile) != hold) st_relaxed_u64(state + tile, (tag << 32) | total);
     // the totals of every earlier tile, one word per thread at a time
     uint32_t part = 0;
     bool gave_up = false;
-    for (uint32_t p = threadIdx.x; p < tile; p += kScanThreads) {
+    for (uint32_t p = thread; p < tile; p += kScanThreads) {
         unsigned long long w = ld_relaxed_u64(state + p);
         for (int polls = 0; (w >> 32) != tag && polls < kScanWaitLimit; ++polls) {
             __nanosleep(64);
@@ -620,7 +623,7 @@ k_scan(const uint4* __restrict__ count4, uint4* __restrict__ start4,
     if (gave_up) atomicAdd(&g_scan_waits_given_up, 1ull);
     uint32_t prefix = 0;
     if (!single) block_exclusive_scan(part, &prefix);
-    if (advance && threadIdx.x == 0 && tile == uint32_t(ntiles - 1)) *step_dev += 1ull;
+    if (advance && thread == 0 && tile == uint32_t(ntiles - 1)) *step_dev += 1ull;
     uint32_t e = prefix + excl;
 #pragma unroll
     for (int k = 0; k < kVec; ++k) {

@@ -1,0 +1,48 @@
+"""The kernels launched to overlap the one before (mtpt.cu `launch`), by their
+source: each waits for that kernel before it reads what a kernel may have
+written."""
+import os
+import re
+
+import pytest
+
+from paper_2204_03756_gb300 import build
+
+
+def _source(name):
+    with open(os.path.join(build.SRC_DIR, name)) as f:
+        return re.sub(r"//[^\n]*", "", f.read())
+
+
+def _kernel(src, name):
+    """(parameter list, body) of the kernel's definition."""
+    m = re.search(r"\b%s\s*\(" % name, src)
+    end = m.end()
+    depth = 1
+    while depth:
+        depth += {"(": 1, ")": -1}.get(src[end], 0)
+        end += 1
+    body = src.index("{", end)
+    stop, depth = body + 1, 1
+    while depth:
+        depth += {"{": 1, "}": -1}.get(src[stop], 0)
+        stop += 1
+    return src[m.end():end - 1], src[body:stop]
+
+
+KERNELS = sorted(set(re.findall(r"\blaunch\((k_\w+)", _source("mtpt.cu"))))
+
+
+def test_the_step_kernels_are_found():
+    assert {"k_scan", "k_gather", "k_rowsum_f32", "k_exchange_f64", "k_adj_exchange"} <= set(KERNELS)
+
+
+@pytest.mark.parametrize("name", KERNELS)
+def test_indexes_pass_through_the_wait(name):
+    """A read-only load whose address does not come out of the wait may be moved
+    ahead of it: a kernel that reads through pointers to const takes its index
+    from ordered_index()."""
+    params, body = _kernel(_source("kernels.cuh"), name)
+    if "ordered_index()" not in body:
+        assert "after_previous()" in body
+        assert not re.search(r"\bconst\b[^,]*\*", params)
