@@ -74,19 +74,67 @@ constexpr int kScanTile = kScanPerThread * kScanThreads;  // cells per scan bloc
 // its two reads 55.7 -> 39.0 us (eight kernels), the adjoint's 200 steps of 250,000
 // 44.5 -> 38.5 ms.
 // (For kernels that only update a word in place: what is read through a pointer
-// to const goes through ordered_index.)
+// to const takes its index from ordered_index.)
 __device__ __forceinline__ void after_previous() {
     asm volatile("griddepcontrol.launch_dependents;");
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 // The thread's global index, after after_previous(): passing through the asm, it
-// keeps every access that depends on it (read-only loads too, which a memory
-// clobber alone need not hold back) behind the wait.
+// keeps every access that depends on it (loads without a memory clobber of their
+// own too) behind the wait.
 __device__ __forceinline__ uint32_t ordered_index() {
     uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     asm volatile("griddepcontrol.launch_dependents;");
     asm volatile("griddepcontrol.wait;\n\tmov.b32 %0, %0;" : "+r"(i)::"memory");
     return i;
+}
+
+// Loads of what the kernels of a step write.  Such a kernel's lifetime overlaps
+// the writer's, so the read-only path (ld.global.nc, __ldg, pointers to const
+// declared __restrict__), which wants memory that stays the same for as long as
+// the kernel lives, is for the constants of a run alone: the corner tables and the
+// exponential's table.  These are ordinary loads, after the wait by their address.
+__device__ __forceinline__ float ld_global(const float* p) {
+    float v;
+    asm("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float2 ld_global(const float2* p) {
+    float2 v;
+    asm("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float4 ld_global(const float4* p) {
+    float4 v;
+    asm("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];"
+        : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+        : "l"(p));
+    return v;
+}
+__device__ __forceinline__ double ld_global(const double* p) {
+    double v;
+    asm("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ double2 ld_global(const double2* p) {
+    double2 v;
+    asm("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint32_t ld_global(const uint32_t* p) {
+    uint32_t v;
+    asm("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint2 ld_global(const uint2* p) {
+    uint2 v;
+    asm("ld.global.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint64_t ld_global(const uint64_t* p) {
+    uint64_t v;
+    asm("ld.global.u64 %0, [%1];" : "=l"(v) : "l"(p));
+    return v;
 }
 
 __device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long long* p) {
@@ -166,10 +214,10 @@ struct BatchView {
     const uint32_t* rid_input;    // realisation of each particle before the sort
     const uint32_t* rid_sorted;   // realisation of each particle in cell order
     __device__ __forceinline__ const RealParams& of_input(uint32_t i) const {
-        return tbl[__ldg(rid_input + i)];
+        return tbl[ld_global(rid_input + i)];
     }
     __device__ __forceinline__ const RealParams& of_sorted(uint32_t s) const {
-        return tbl[__ldg(rid_sorted + s)];
+        return tbl[ld_global(rid_sorted + s)];
     }
 };
 
@@ -186,9 +234,9 @@ __device__ __forceinline__ long long order_key(double x) {
 
 // A particle's record rec (see the layout above).
 __device__ __forceinline__ size_t rec_at(uint32_t j) { return size_t(j & ~1u) * 4u + (j & 1u); }
-__device__ __forceinline__ float4 load_rec(const float* __restrict__ rec, uint32_t j) {
+__device__ __forceinline__ float4 load_rec(const float* rec, uint32_t j) {
     const float* q = rec + rec_at(j);
-    return make_float4(__ldg(q), __ldg(q + 4), __ldg(q + 6), __ldg(q + 2));
+    return make_float4(ld_global(q), ld_global(q + 4), ld_global(q + 6), ld_global(q + 2));
 }
 __device__ __forceinline__ void store_rec(float* __restrict__ rec, uint32_t j, const float4& v) {
     float* q = rec + rec_at(j);
@@ -233,9 +281,9 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
 struct RecPair {
     uint64_t x, w, y, z;
 };
-__device__ __forceinline__ RecPair load_rec_pair(const float* __restrict__ rec, uint32_t j) {
+__device__ __forceinline__ RecPair load_rec_pair(const float* rec, uint32_t j) {
     RecPair r;
-    asm("ld.global.nc.v4.b64 {%0, %1, %2, %3}, [%4];"
+    asm("ld.global.v4.b64 {%0, %1, %2, %3}, [%4];"
         : "=l"(r.x), "=l"(r.w), "=l"(r.y), "=l"(r.z)
         : "l"(rec + size_t(j) * 4u));
     return r;
@@ -404,8 +452,8 @@ __device__ __forceinline__ void key_particle(const RealParams& P, const double* 
 // cell keys and counts of the counting sort (with do_key).
 template <int DIM, class View, bool TANGENT = false, bool ADVECT = false>
 __global__ void __launch_bounds__(kBlock)
-k_walk_key(int n, int64_t stride, double* __restrict__ pos, const uint32_t* __restrict__ id,
-           const unsigned long long* __restrict__ step_dev, int do_walk, int do_key,
+k_walk_key(int n, int64_t stride, double* __restrict__ pos, const uint32_t* id,
+           const unsigned long long* step_dev, int do_walk, int do_key,
            const __grid_constant__ View v, uint32_t* __restrict__ key,
            uint32_t* __restrict__ count, uint32_t* __restrict__ status,
            double* __restrict__ tan = nullptr) {
@@ -572,7 +620,7 @@ __device__ unsigned long long g_scan_waits_given_up;
 // of the step that reads it has completed.  A tile equal to `hold` never
 // publishes (a test hook: the tiles after it then run out of polls).
 __global__ void __launch_bounds__(kScanThreads)
-k_scan(const uint4* __restrict__ count4, uint4* __restrict__ start4,
+k_scan(const uint4* count4, uint4* __restrict__ start4,
        unsigned long long* __restrict__ state, int ntiles,
        unsigned long long* __restrict__ step_dev, int advance, int hold) {
     constexpr int kVec = kScanPerThread / 4;
@@ -663,9 +711,9 @@ __global__ void k_fill_rid(int n, int nreal, const uint32_t* __restrict__ first,
 // that the in-cell ranking of the gather reads.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kBlock)
-k_scatter(int n, const uint32_t* __restrict__ key, const uint32_t* __restrict__ start,
-          uint32_t* __restrict__ count, const double* __restrict__ x,
-          const uint32_t* __restrict__ id, uint32_t* __restrict__ perm,
+k_scatter(int n, const uint32_t* key, const uint32_t* start,
+          uint32_t* __restrict__ count, const double* x,
+          const uint32_t* id, uint32_t* __restrict__ perm,
           double2* __restrict__ sortkey) {
     const int i = int(ordered_index());
     if (i >= n) return;
@@ -716,7 +764,7 @@ __device__ __forceinline__ void cell_coords_rec(uint32_t cell, const float4& me,
 
 // cell[s] where the pair searches need it (3-d), else nothing is read.
 template <int DIM>
-__device__ __forceinline__ uint32_t cell_arg(const uint32_t* __restrict__ cell, uint32_t s) {
+__device__ __forceinline__ uint32_t cell_arg(const uint32_t* cell, uint32_t s) {
     return DIM == 3 ? cell[s] : 0u;
 }
 
@@ -732,15 +780,15 @@ __device__ __forceinline__ uint32_t cell_arg(const uint32_t* __restrict__ cell, 
 // 2^-23 w, no binary64 instruction).
 template <int DIM, class View, bool TANGENT = false>
 __global__ void __launch_bounds__(kBlock)
-k_gather(int n, int64_t stride, const uint32_t* __restrict__ perm,
-         const double2* __restrict__ sortkey, const uint32_t* __restrict__ start,
-         const double* __restrict__ pos_in, const double* __restrict__ mass_in,
+k_gather(int n, int64_t stride, const uint32_t* perm,
+         const double2* sortkey, const uint32_t* start,
+         const double* pos_in, const double* mass_in,
          uint32_t* __restrict__ id_out, double* __restrict__ pos_out,
          double* __restrict__ mass_out, uint32_t* __restrict__ cell_out,
          float* __restrict__ rec_out,
          const float2* __restrict__ corners, uint32_t* __restrict__ rid_out,
-         const __grid_constant__ View v, const double* __restrict__ tan_in = nullptr,
-         double* __restrict__ tan_out = nullptr, const double* __restrict__ mass_b_in = nullptr,
+         const __grid_constant__ View v, const double* tan_in = nullptr,
+         double* __restrict__ tan_out = nullptr, const double* mass_b_in = nullptr,
          double* __restrict__ mass_b_out = nullptr, uint64_t* __restrict__ image_out = nullptr) {
     const int s = int(ordered_index());
     if (s >= n) return;
@@ -769,7 +817,7 @@ k_gather(int n, int64_t stride, const uint32_t* __restrict__ perm,
     if (!check(dst < e, kChkGather)) return;
     id_out[dst] = my_id;
     if constexpr (DIM == 3) cell_out[dst] = c;   // only the 3-d searches read it
-    if constexpr (View::kBatch) rid_out[dst] = __ldg(v.rid_input + src);
+    if constexpr (View::kBatch) rid_out[dst] = ld_global(v.rid_input + src);
     if (mass_b_out) mass_b_out[dst] = mass_b_in[src];   // second species (reactions)
     const RealParams& P = v.of_input(src);
     mass_out[dst] = m;
@@ -813,10 +861,10 @@ struct SortRec {
 
 template <int DIM, bool TANGENT>
 __global__ void __launch_bounds__(kBlock)
-k_scatter_rec(int n, int64_t stride, const uint32_t* __restrict__ key,
-              const uint32_t* __restrict__ start, uint32_t* __restrict__ count,
-              const double* __restrict__ pos, const double* __restrict__ mass,
-              const uint32_t* __restrict__ id, const double* __restrict__ tan,
+k_scatter_rec(int n, int64_t stride, const uint32_t* key,
+              const uint32_t* start, uint32_t* __restrict__ count,
+              const double* pos, const double* mass,
+              const uint32_t* id, const double* tan,
               double2* __restrict__ recs) {
     using R = SortRec<DIM, TANGENT>;
     const int i = int(ordered_index());
@@ -845,8 +893,8 @@ k_scatter_rec(int n, int64_t stride, const uint32_t* __restrict__ key,
 // reads chunk 0 of the cell's records; outputs as k_gather's.
 template <int DIM, bool TANGENT>
 __global__ void __launch_bounds__(kBlock)
-k_gather_rec(int n, int64_t stride, const double2* __restrict__ recs,
-             const uint32_t* __restrict__ start, uint32_t* __restrict__ id_out,
+k_gather_rec(int n, int64_t stride, const double2* recs,
+             const uint32_t* start, uint32_t* __restrict__ id_out,
              double* __restrict__ pos_out, double* __restrict__ mass_out,
              uint32_t* __restrict__ cell_out, float* __restrict__ rec_out,
              const float2* __restrict__ corners,
@@ -922,12 +970,12 @@ k_gather_rec(int n, int64_t stride, const double2* __restrict__ recs,
 // flux, so no candidate is skipped.
 // ---------------------------------------------------------------------------
 template <int DIM>
-__device__ __forceinline__ double exact_d2(const double* __restrict__ pos, int64_t stride,
+__device__ __forceinline__ double exact_d2(const double* pos, int64_t stride,
                                            uint32_t i, uint32_t j) {
     double d2 = 0.0;
 #pragma unroll
     for (int a = 0; a < DIM; ++a) {
-        const double d = __dsub_rn(__ldg(pos + a * stride + i), __ldg(pos + a * stride + j));
+        const double d = __dsub_rn(ld_global(pos + a * stride + i), ld_global(pos + a * stride + j));
         const double sq = __dmul_rn(d, d);
         d2 = (a == 0) ? sq : __dadd_rn(d2, sq);
     }
@@ -937,13 +985,13 @@ __device__ __forceinline__ double exact_d2(const double* __restrict__ pos, int64
 // Kernel value of an accepted pair from the particles' fixed-point images (see
 // expneg.cuh).  Symmetric in (i, j) bit for bit.
 template <int DIM>
-__device__ __forceinline__ double pair_kernel(const uint64_t* __restrict__ image, int64_t stride,
+__device__ __forceinline__ double pair_kernel(const uint64_t* image, int64_t stride,
                                               uint32_t i, uint32_t j, const double* table,
                                               const KernelConsts& kc) {
     uint64_t d2h = 0;
 #pragma unroll
     for (int a = 0; a < DIM; ++a)
-        d2h += axis_square(__ldg(image + a * stride + i), __ldg(image + a * stride + j));
+        d2h += axis_square(ld_global(image + a * stride + i), ld_global(image + a * stride + j));
     return gauss_fixed(d2h, table, kc);
 }
 
@@ -965,10 +1013,10 @@ __device__ __forceinline__ float dx_f32(const float4& me, const float4& o, float
 }
 
 // The same of the candidate with index j.
-__device__ __forceinline__ float dx_of(const float4& me, const float* __restrict__ rec, uint32_t j,
+__device__ __forceinline__ float dx_of(const float4& me, const float* rec, uint32_t j,
                                        float wx) {
     const float* q = rec + rec_at(j);
-    return __fmaf_rn(__fsub_rn(__ldg(q + 2), me.w), wx, __fsub_rn(__ldg(q), me.x));
+    return __fmaf_rn(__fsub_rn(ld_global(q + 2), me.w), wx, __fsub_rn(ld_global(q), me.x));
 }
 
 template <int DIM>
@@ -1011,8 +1059,8 @@ __device__ __forceinline__ float row_gap(int d, float off, float w, float eps) {
 // row(j0, j3, rx, sy, sz) is called for every row that can hold a neighbour.
 template <int DIM, class Row>
 __device__ __forceinline__ void for_each_row(uint32_t cell, const float4 me,
-                                             const float* __restrict__ rec,
-                                             const uint32_t* __restrict__ start,
+                                             const float* rec,
+                                             const uint32_t* start,
                                              const RealParams& P, Row&& row) {
     const Grid& g = P.g;
     const PairParams& pp = P.pp;
@@ -1041,8 +1089,8 @@ __device__ __forceinline__ void for_each_row(uint32_t cell, const float4 me,
             if (!check(rowc + uint32_t(xhi) + 1u - P.cell_base <=
                            uint32_t(g.n[0]) * uint32_t(g.n[1]) * uint32_t(g.n[2]), kChkRow))
                 continue;
-            uint32_t lo = __ldg(start + rowc + xlo);
-            uint32_t hi = __ldg(start + rowc + xhi + 1);
+            uint32_t lo = ld_global(start + rowc + xlo);
+            uint32_t hi = ld_global(start + rowc + xhi + 1);
             const uint32_t j3 = hi;
             while (lo < hi) {
                 const uint32_t mid = (lo + hi) >> 1;
@@ -1057,9 +1105,9 @@ __device__ __forceinline__ void for_each_row(uint32_t cell, const float4 me,
 // visit(j, d2f, rec_j) is called for every neighbour j of s (s included).
 template <int DIM, class Visit>
 __device__ __forceinline__ void visit_neighbours(uint32_t s, uint32_t cell, int64_t stride,
-                                                 const float* __restrict__ rec,
-                                                 const double* __restrict__ pos,
-                                                 const uint32_t* __restrict__ start,
+                                                 const float* rec,
+                                                 const double* pos,
+                                                 const uint32_t* start,
                                                  const RealParams& P, Visit&& visit) {
     const PairParams& pp = P.pp;
     const float4 me = load_rec(rec, s);
@@ -1082,7 +1130,7 @@ __device__ __forceinline__ void visit_neighbours(uint32_t s, uint32_t cell, int6
 // The exact binary64 test as a real call, so the compiler cannot if-convert
 // it into every candidate's path (it runs only inside the narrow band).
 template <int DIM>
-__device__ __noinline__ bool exact_within(const double* __restrict__ pos, int64_t stride,
+__device__ __noinline__ bool exact_within(const double* pos, int64_t stride,
                                           uint32_t s, uint32_t j, double psi2) {
     return exact_d2<DIM>(pos, stride, s, j) <= psi2;
 }
@@ -1091,9 +1139,9 @@ __device__ __noinline__ bool exact_within(const double* __restrict__ pos, int64_
 // accepts: visit(j, d2f) in candidate order.
 template <int DIM, class Visit>
 __device__ __forceinline__ void scan_band(uint32_t s, uint32_t cell, int64_t stride,
-                                          const float* __restrict__ rec,
-                                          const double* __restrict__ pos,
-                                          const uint32_t* __restrict__ start, const RealParams& P,
+                                          const float* rec,
+                                          const double* pos,
+                                          const uint32_t* start, const RealParams& P,
                                           Visit&& visit) {
     const PairParams& pp = P.pp;
     const float4 me = load_rec(rec, s);
@@ -1119,9 +1167,9 @@ __device__ __forceinline__ void scan_band(uint32_t s, uint32_t cell, int64_t str
 // test accepts (the order in which 3-d lists hold their neighbours).
 template <int DIM, bool DEFER_BAND, class Visit>
 __device__ __forceinline__ void scan_neighbours(uint32_t s, uint32_t cell, int64_t stride,
-                                                const float* __restrict__ rec,
-                                                const double* __restrict__ pos,
-                                                const uint32_t* __restrict__ start,
+                                                const float* rec,
+                                                const double* pos,
+                                                const uint32_t* start,
                                                 const RealParams& P, Visit&& visit) {
     const PairParams& pp = P.pp;
     const float4 me = load_rec(rec, s);
@@ -1213,8 +1261,8 @@ __device__ __forceinline__ uint32_t mask_word(uint32_t words, uint32_t neighbour
 constexpr uint32_t kBisectFrom = 24;
 template <int DIM, bool WORDS, bool EACH, class Cand>
 __device__ __forceinline__ uint32_t search_words(uint32_t s, uint32_t cell, const float4 me,
-                                                 int64_t stride, const float* __restrict__ rec,
-                                                 const uint32_t* __restrict__ start,
+                                                 int64_t stride, const float* rec,
+                                                 const uint32_t* start,
                                                  const RealParams& P, const NbPlanes& nb,
                                                  uint32_t& cnt, bool& band, Cand&& cand) {
     const PairParams& pp = P.pp;
@@ -1246,8 +1294,8 @@ __device__ __forceinline__ uint32_t search_words(uint32_t s, uint32_t cell, cons
                                                  uint32_t(c[1] + dy)) * uint32_t(g.n[0]);
             if (check(rowc + uint32_t(xhi) + 1u - P.cell_base <=
                           uint32_t(g.n[0]) * uint32_t(g.n[1]) * uint32_t(g.n[2]), kChkRow)) {
-                j = __ldg(start + rowc + xlo);
-                j3 = __ldg(start + rowc + xhi + 1);
+                j = ld_global(start + rowc + xlo);
+                j3 = ld_global(start + rowc + xhi + 1);
                 if (j3 - j > kBisectFrom) {
                     uint32_t hi = j3;
                     while (hi - j > 2u) {
@@ -1344,10 +1392,10 @@ __device__ __forceinline__ uint32_t search_words(uint32_t s, uint32_t cell, cons
 // Returns {rsum, rc, words (bits), neighbours (bits)}.  A real call, so its
 // registers do not weigh on the candidate loop.
 template <int DIM, bool SUM, class View>
-__device__ __noinline__ float4 band_words(uint32_t s, const uint32_t* __restrict__ cell, int64_t stride,
-                                          const double* __restrict__ pos,
-                                          const float* __restrict__ rec,
-                                          const uint32_t* __restrict__ start, const View& v,
+__device__ __noinline__ float4 band_words(uint32_t s, const uint32_t* cell, int64_t stride,
+                                          const double* pos,
+                                          const float* rec,
+                                          const uint32_t* start, const View& v,
                                           const NbPlanes& nb, float rsum, float rc) {
     const RealParams& P = v.of_sorted(s);
     const PairParams& pp = P.pp;
@@ -1507,10 +1555,10 @@ __device__ __forceinline__ void dense_words(uint32_t s, uint32_t listed, int64_t
 // nothing can be kept), neighbour count in cnt.
 template <int DIM, class View>
 __device__ __forceinline__ uint32_t search_listed(uint32_t s, int64_t stride,
-                                                  const double* __restrict__ pos,
-                                                  const float* __restrict__ rec,
-                                                  const uint32_t* __restrict__ cell,
-                                                  const uint32_t* __restrict__ start, const View& v,
+                                                  const double* pos,
+                                                  const float* rec,
+                                                  const uint32_t* cell,
+                                                  const uint32_t* start, const View& v,
                                                   const RealParams& P, const NbPlanes& nb,
                                                   uint32_t& cnt) {
     bool band;
@@ -1528,11 +1576,11 @@ __device__ __forceinline__ uint32_t search_listed(uint32_t s, int64_t stride,
 // Pass 1 of one particle whose neighbours the words do not hold.
 template <int DIM, class View>
 __device__ __noinline__ double search_rowsum(uint32_t s, int64_t stride,
-                                             const double* __restrict__ pos,
-                                             const uint64_t* __restrict__ image,
-                                             const float* __restrict__ rec,
-                                             const uint32_t* __restrict__ cell,
-                                             const uint32_t* __restrict__ start,
+                                             const double* pos,
+                                             const uint64_t* image,
+                                             const float* rec,
+                                             const uint32_t* cell,
+                                             const uint32_t* start,
                                              const double* table, const View& v) {
     const RealParams& P = v.of_sorted(s);
     RowSum r;
@@ -1555,14 +1603,14 @@ __device__ __noinline__ double search_rowsum(uint32_t s, int64_t stride,
 // there: 54 instead of 52 us at 250,007).
 template <int DIM, class View>
 __global__ void __launch_bounds__(kBlock, DIM == 3 ? 5 : 6)
-k_rowsum_f64(int n, int64_t stride, const double* __restrict__ pos,
-             const uint64_t* __restrict__ image, const float* __restrict__ rec,
-             const uint32_t* __restrict__ cell, const uint32_t* __restrict__ start,
+k_rowsum_f64(int n, int64_t stride, const double* pos,
+             const uint64_t* image, const float* rec,
+             const uint32_t* cell, const uint32_t* start,
              const double* __restrict__ exp_table, const __grid_constant__ View v,
-             const double* __restrict__ mass, double2* __restrict__ rm,
+             const double* mass, double2* __restrict__ rm,
              unsigned long long* __restrict__ pair_counter, const __grid_constant__ NbPlanes nb,
              uint32_t* __restrict__ listed_out, PairValues kv,
-             const uint32_t* __restrict__ ghost_id) {
+             const uint32_t* ghost_id) {
     __shared__ double table[kExpTable];
     // Ahead of the wait, here and in pass 2: a copy from the host wrote the table,
     // never a kernel, and it overlaps the kernel before (100 steps of 1e4
@@ -1589,7 +1637,7 @@ k_rowsum_f64(int n, int64_t stride, const double* __restrict__ pos,
                 auto kernel = [&](uint32_t j) {
                     uint64_t d2h = 0;
 #pragma unroll
-                    for (int a = 0; a < DIM; ++a) d2h += axis_square(xs[a], __ldg(image + a * stride + j));
+                    for (int a = 0; a < DIM; ++a) d2h += axis_square(xs[a], ld_global(image + a * stride + j));
                     return gauss_fixed(d2h, table, P.pp.kc);
                 };
                 double* keep = kv.v + s;
@@ -1624,7 +1672,7 @@ k_rowsum_f64(int n, int64_t stride, const double* __restrict__ pos,
 // Species B of a binary64 reaction run: its masses in place of A's in the
 // records {r, m} that pass 2 reads.
 __global__ void __launch_bounds__(kBlock)
-k_record_mass(int n, const double* __restrict__ mass_b, double2* __restrict__ rm) {
+k_record_mass(int n, const double* mass_b, double2* __restrict__ rm) {
     const int s = int(ordered_index());
     if (s < n) rm[s].y = mass_b[s];
 }
@@ -1651,7 +1699,7 @@ struct WalkAhead {
 // walk, 2 the walk with the advection term.
 template <int DIM, int WALK>
 __device__ __forceinline__ void walk_ahead(const RealParams& P, int s, int64_t stride,
-                                           const double* __restrict__ pos, const WalkAhead& wa) {
+                                           const double* pos, const WalkAhead& wa) {
     double x[DIM];
 #pragma unroll
     for (int a = 0; a < DIM; ++a) x[a] = pos[a * stride + s];
@@ -1672,13 +1720,13 @@ __device__ __forceinline__ void walk_ahead(const RealParams& P, int s, int64_t s
 // Pass 2 of one particle whose neighbours the words do not hold.
 template <int DIM, class View>
 __device__ __noinline__ double search_flux_f64(uint32_t s, int64_t stride,
-                                               const double* __restrict__ pos,
-                                               const uint64_t* __restrict__ image,
-                                               const float* __restrict__ rec,
-                                               const uint32_t* __restrict__ cell,
-                                               const uint32_t* __restrict__ start,
+                                               const double* pos,
+                                               const uint64_t* image,
+                                               const float* rec,
+                                               const uint32_t* cell,
+                                               const uint32_t* start,
                                                const double* table, const View& v,
-                                               const double2* __restrict__ rm) {
+                                               const double2* rm) {
     const RealParams& P = v.of_sorted(s);
     const double2 me = rm[s];
     FluxSum64 sum;
@@ -1686,7 +1734,7 @@ __device__ __noinline__ double search_flux_f64(uint32_t s, int64_t stride,
                           [&](uint32_t j, float, const float4&) {
                               if (j == s) return;
                               const double K = pair_kernel<DIM>(image, stride, s, j, table, P.pp.kc);
-                              const double2 q = __ldg(rm + j);
+                              const double2 q = ld_global(rm + j);
                               sum.add(__dsub_rn(q.y, me.y), weight_fixed(K, me.x, q.x));
                           });
     return sum.value();
@@ -1694,12 +1742,12 @@ __device__ __noinline__ double search_flux_f64(uint32_t s, int64_t stride,
 
 template <int DIM, class View, int WALK = 0>
 __global__ void __launch_bounds__(kBlock, 5)
-k_exchange_f64(int n, int64_t stride, const double* __restrict__ pos,
-               const uint64_t* __restrict__ image, const float* __restrict__ rec,
-               const uint32_t* __restrict__ cell, const uint32_t* __restrict__ start,
+k_exchange_f64(int n, int64_t stride, const double* pos,
+               const uint64_t* image, const float* rec,
+               const uint32_t* cell, const uint32_t* start,
                const double* __restrict__ exp_table, const __grid_constant__ View v,
-               const double2* __restrict__ rm, double* __restrict__ mass_out, NbPlanes nb,
-               const uint32_t* __restrict__ listed_in, PairValues kv,
+               const double2* rm, double* __restrict__ mass_out, NbPlanes nb,
+               const uint32_t* listed_in, PairValues kv,
                const WalkAhead wa = WalkAhead{}) {
     __shared__ double table[kExpTable];   // of use to the particles that search or evaluate again
     for (int t = threadIdx.x; t < kExpTable; t += blockDim.x) table[t] = exp_table[t];
@@ -1707,7 +1755,7 @@ k_exchange_f64(int n, int64_t stride, const double* __restrict__ pos,
     __syncthreads();
     if (s >= uint32_t(n)) return;
     const RealParams& P = v.of_sorted(s);
-    const double2 me = __ldg(rm + s);
+    const double2 me = ld_global(rm + s);
     double m = me.y;
     if (P.transfer) {
         const uint32_t listed = listed_in ? listed_in[s] : kMaskOver;
@@ -1725,16 +1773,16 @@ k_exchange_f64(int n, int64_t stride, const double* __restrict__ pos,
             uint32_t k = 0;
             for (; k + 2 <= listed_k; k += 2, keep += 2 * stride) {
                 const uint32_t j0 = stream.next(), j1 = stream.next();
-                const double K0 = __ldg(keep), K1 = __ldg(keep + stride);
-                const double2 q0 = __ldg(rm + j0), q1 = __ldg(rm + j1);
+                const double K0 = ld_global(keep), K1 = ld_global(keep + stride);
+                const double2 q0 = ld_global(rm + j0), q1 = ld_global(rm + j1);
                 sum.add(__dsub_rn(q0.y, me.y), weight_fixed(K0, me.x, q0.x));
                 sum.add(__dsub_rn(q1.y, me.y), weight_fixed(K1, me.x, q1.x));
             }
             for (; k < cnt; ++k) {
                 const uint32_t j = stream.next();
-                const double K = k < listed_k ? __ldg(keep)
+                const double K = k < listed_k ? ld_global(keep)
                                               : pair_kernel<DIM>(image, stride, s, j, table, P.pp.kc);
-                const double2 q = __ldg(rm + j);
+                const double2 q = ld_global(rm + j);
                 sum.add(__dsub_rn(q.y, me.y), weight_fixed(K, me.x, q.x));
             }
             flux = sum.value();
@@ -1758,9 +1806,9 @@ struct ExRec {
 struct PairRec {
     float4 rec, m;
 };
-__device__ __forceinline__ PairRec load_pair_rec(const float4* __restrict__ ex, uint32_t j) {
+__device__ __forceinline__ PairRec load_pair_rec(const float4* ex, uint32_t j) {
     PairRec q;
-    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+    asm("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
         : "=f"(q.rec.x), "=f"(q.rec.y), "=f"(q.rec.z), "=f"(q.rec.w), "=f"(q.m.x), "=f"(q.m.y),
           "=f"(q.m.z), "=f"(q.m.w)
         : "l"(ex + 2 * size_t(j)));
@@ -1773,8 +1821,8 @@ __device__ __forceinline__ void store_pair_rec(float4* __restrict__ ex, uint32_t
                  : "memory");
 }
 template <int DIM>
-__device__ __forceinline__ float4 load_ex(const float4* __restrict__ ex, uint32_t j) {
-    return __ldg(ex + size_t(ExRec<DIM>::kVec) * j + (ExRec<DIM>::kVec - 1));
+__device__ __forceinline__ float4 load_ex(const float4* ex, uint32_t j) {
+    return ld_global(ex + size_t(ExRec<DIM>::kVec) * j + (ExRec<DIM>::kVec - 1));
 }
 
 // Pass 1, precision form: binary32 kernel exp2(-a log2(e) d2f) with the
@@ -1789,12 +1837,12 @@ __device__ __forceinline__ float4 load_ex(const float4* __restrict__ ex, uint32_
 // nine rows) the list is the shorter of the two.
 template <int DIM, class View>
 __global__ void __launch_bounds__(kBlock, (DIM == 3 || View::kBatch ? 1536 : 2048) / kBlock)
-k_rowsum_f32(int n, int64_t stride, const double* __restrict__ pos, const float* __restrict__ rec,
-             const uint32_t* __restrict__ cell, const uint32_t* __restrict__ start,
-             const __grid_constant__ View v, const double* __restrict__ mass,
+k_rowsum_f32(int n, int64_t stride, const double* pos, const float* rec,
+             const uint32_t* cell, const uint32_t* start,
+             const __grid_constant__ View v, const double* mass,
              float4* __restrict__ ex, unsigned long long* __restrict__ pair_counter,
-             const uint32_t* __restrict__ ghost_id, const __grid_constant__ NbPlanes nb,
-             const double* __restrict__ mass_b, float2* __restrict__ exb) {
+             const uint32_t* ghost_id, const __grid_constant__ NbPlanes nb,
+             const double* mass_b, float2* __restrict__ exb) {
     const int s = int(ordered_index());
     uint32_t cnt = 0;
     if (s < n) {
@@ -1898,11 +1946,11 @@ struct FluxSum {
 // not weigh on the list loop.
 template <int DIM, class View>
 __device__ __noinline__ float2 search_flux(uint32_t s, int64_t stride,
-                                           const double* __restrict__ pos,
-                                           const float* __restrict__ rec,
-                                           const uint32_t* __restrict__ cell,
-                                           const uint32_t* __restrict__ start, const View& v,
-                                           const float4* __restrict__ ex, float rs, float2 ms,
+                                           const double* pos,
+                                           const float* rec,
+                                           const uint32_t* cell,
+                                           const uint32_t* start, const View& v,
+                                           const float4* ex, float rs, float2 ms,
                                            float two_beta) {
     const RealParams& P = v.of_sorted(s);
     const float na = -P.pp.a_log2e;
@@ -1977,12 +2025,12 @@ k_react(int n, double* __restrict__ ma, double* __restrict__ mb, double kp, doub
 // in exb): {acc_A, comp_A, acc_B, comp_B}.
 template <int DIM, class View>
 __device__ __noinline__ float4 search_flux2(uint32_t s, int64_t stride,
-                                            const double* __restrict__ pos,
-                                            const float* __restrict__ rec,
-                                            const uint32_t* __restrict__ cell,
-                                            const uint32_t* __restrict__ start, const View& v,
-                                            const float4* __restrict__ ex,
-                                            const float2* __restrict__ exb, float rs, float2 ms,
+                                            const double* pos,
+                                            const float* rec,
+                                            const uint32_t* cell,
+                                            const uint32_t* start, const View& v,
+                                            const float4* ex,
+                                            const float2* exb, float rs, float2 ms,
                                             float2 msb, float two_beta) {
     const RealParams& P = v.of_sorted(s);
     const float na = -P.pp.a_log2e;
@@ -1992,7 +2040,7 @@ __device__ __noinline__ float4 search_flux2(uint32_t s, int64_t stride,
                              const float4 xj = load_ex<DIM>(ex, j);
                              const float W = a.weight(xj, ex2_approx(na * d2f));
                              a.add_w(make_float2(xj.x, xj.y), W, accept);
-                             b.add_w(__ldg(exb + j), W, accept);
+                             b.add_w(ld_global(exb + j), W, accept);
                          });
     return make_float4(a.acc, a.comp, b.acc, b.comp);
 }
@@ -2014,13 +2062,13 @@ struct PairFlux {
     }
     __device__ __forceinline__ PairRec load(uint32_t j) const {
         if constexpr (WIDE) return load_pair_rec(ex, j);
-        else return PairRec{__ldg(ex + 2 * size_t(j)), __ldg(ex + 2 * size_t(j) + 1)};
+        else return PairRec{ld_global(ex + 2 * size_t(j)), ld_global(ex + 2 * size_t(j) + 1)};
     }
     __device__ __forceinline__ void add(FluxSum& f, FluxSum& g, uint32_t j0, uint32_t j1,
                                         bool two) const {
         const PairRec q0 = load(j0), q1 = load(j1);
         if constexpr (TWO) {
-            const float2 b0 = __ldg(exb + j0), b1 = __ldg(exb + j1);
+            const float2 b0 = ld_global(exb + j0), b1 = ld_global(exb + j1);
             const float w0 = f.weight(q0.m, kernel(q0.rec)), w1 = f.weight(q1.m, kernel(q1.rec));
             f.add_w(make_float2(q0.m.x, q0.m.y), w0);
             g.add_w(b0, w0);
@@ -2036,13 +2084,13 @@ struct PairFlux {
 // Pass 2 of a particle's mask words (padding included) word by word, the next
 // word loaded ahead.
 template <int DIM, bool TWO, bool WIDE>
-__device__ __forceinline__ void add_words(const uint2* __restrict__ e, int64_t stride, uint32_t words,
+__device__ __forceinline__ void add_words(const uint2* e, int64_t stride, uint32_t words,
                                           const PairFlux<DIM, TWO, WIDE>& pf, FluxSum& f, FluxSum& g) {
-    uint2 ahead = __ldg(e);
+    uint2 ahead = ld_global(e);
     for (uint32_t w = 1; w <= words; ++w) {
         const uint32_t base = ahead.x;
         uint32_t bits = ahead.y;
-        if (w < words) ahead = __ldg(e += stride);
+        if (w < words) ahead = ld_global(e += stride);
         while (bits) {
             const uint32_t j0 = base + uint32_t(__ffs(int(bits)) - 1);
             bits &= bits - 1u;
@@ -2058,9 +2106,9 @@ __device__ __forceinline__ void add_words(const uint2* __restrict__ e, int64_t s
 // a run whose windows are short: its registers do not weigh on their loop.
 // {acc_A, comp_A, acc_B, comp_B}.
 template <int DIM, bool TWO>
-__device__ __noinline__ float4 words_flux(const uint2* __restrict__ e, int64_t stride,
-                                          uint32_t words, const float4* __restrict__ ex,
-                                          const float2* __restrict__ exb, float4 me, float na,
+__device__ __noinline__ float4 words_flux(const uint2* e, int64_t stride,
+                                          uint32_t words, const float4* ex,
+                                          const float2* exb, float4 me, float na,
                                           float wx, float wy, float rs, float two_beta, float2 ms,
                                           float2 msb) {
     const PairFlux<DIM, TWO, false> pf{ex, exb, me, na, wx, wy};
@@ -2086,11 +2134,11 @@ __device__ __noinline__ float4 words_flux(const uint2* __restrict__ e, int64_t s
 // 57 neighbours, the next walk included).
 template <int DIM, class View, bool TWO = false, int WALK = 0, bool LONG = false>
 __global__ void __launch_bounds__(kBlock, (TWO ? 1536 : (View::kBatch || LONG ? 1792 : 2048)) / kBlock)
-k_exchange_f32(int n, int64_t stride, const double* __restrict__ pos, const float* __restrict__ rec,
-               const uint32_t* __restrict__ cell, const uint32_t* __restrict__ start,
-               const __grid_constant__ View v, const float4* __restrict__ ex,
-               const double* __restrict__ mass, double* __restrict__ mass_out, NbPlanes nb,
-               const float2* __restrict__ exb = nullptr, const double* __restrict__ mass_b = nullptr,
+k_exchange_f32(int n, int64_t stride, const double* pos, const float* rec,
+               const uint32_t* cell, const uint32_t* start,
+               const __grid_constant__ View v, const float4* ex,
+               const double* mass, double* __restrict__ mass_out, NbPlanes nb,
+               const float2* exb = nullptr, const double* mass_b = nullptr,
                double* __restrict__ mass_b_out = nullptr, double kp = 0.0, double dt = 0.0,
                float kpdt_f = 0.0f, const WalkAhead wa = WalkAhead{}) {
     const int s = int(ordered_index());
@@ -2110,11 +2158,11 @@ k_exchange_f32(int n, int64_t stride, const double* __restrict__ pos, const floa
     }
     const float4 xs = load_ex<DIM>(ex, uint32_t(s));
     FluxSum f{xs.z, float(2.0 * P.pp.beta), make_float2(xs.x, xs.y)};   // beta folded into W
-    FluxSum g{xs.z, f.two_beta, TWO ? __ldg(exb + s) : make_float2(0.0f, 0.0f)};
+    FluxSum g{xs.z, f.two_beta, TWO ? ld_global(exb + s) : make_float2(0.0f, 0.0f)};
     const uint32_t listed = __float_as_uint(xs.w);   // see NbPlanes
     if (nb.cap > 0 && (DIM == 3 ? listed <= uint32_t(nb.cap) : listed != kMaskOver)) {
         if constexpr (DIM < 3) {
-            const PairFlux<DIM, TWO, true> pf{ex, exb, __ldg(ex + 2 * size_t(s)), -P.pp.a_log2e,
+            const PairFlux<DIM, TWO, true> pf{ex, exb, ld_global(ex + 2 * size_t(s)), -P.pp.a_log2e,
                                               P.g.wf[0], P.g.wf[1]};
             const uint2* e = nb.e + s;
             const uint32_t words = listed & 255u;
@@ -2126,9 +2174,9 @@ k_exchange_f32(int n, int64_t stride, const double* __restrict__ pos, const floa
                 // over them, so a warp runs as long as its longest particle's
                 // count and not its rows'
                 const uint2 none = make_uint2(0u, 0u);
-                uint2 w0 = words > 0u ? __ldg(e) : none;
-                uint2 w1 = words > 1u ? __ldg(e + stride) : none;
-                const uint2 w2 = words > 2u ? __ldg(e + 2 * stride) : none;
+                uint2 w0 = words > 0u ? ld_global(e) : none;
+                uint2 w1 = words > 1u ? ld_global(e + stride) : none;
+                const uint2 w2 = words > 2u ? ld_global(e + 2 * stride) : none;
                 auto next = [&]() {
                     const bool shift = w0.y == 0u;
                     w0 = shift ? w1 : w0;
@@ -2159,9 +2207,9 @@ k_exchange_f32(int n, int64_t stride, const double* __restrict__ pos, const floa
             uint32_t k = 0;
             if constexpr (TWO) {
                 for (; k + 2 <= listed; k += 2, e += 2 * stride) {
-                    const uint2 q0 = __ldg(e), q1 = __ldg(e + stride);
-                    const float4 x0 = __ldg(ex + q0.x), x1 = __ldg(ex + q1.x);
-                    const float2 b0 = __ldg(exb + q0.x), b1 = __ldg(exb + q1.x);
+                    const uint2 q0 = ld_global(e), q1 = ld_global(e + stride);
+                    const float4 x0 = ld_global(ex + q0.x), x1 = ld_global(ex + q1.x);
+                    const float2 b0 = ld_global(exb + q0.x), b1 = ld_global(exb + q1.x);
                     const float w0 = f.weight(x0, __uint_as_float(q0.y));
                     f.add_w(make_float2(x0.x, x0.y), w0);
                     g.add_w(b0, w0);
@@ -2170,26 +2218,26 @@ k_exchange_f32(int n, int64_t stride, const double* __restrict__ pos, const floa
                     g.add_w(b1, w1);
                 }
                 if (k < listed) {
-                    const uint2 q = __ldg(e);
-                    const float4 x = __ldg(ex + q.x);
+                    const uint2 q = ld_global(e);
+                    const float4 x = ld_global(ex + q.x);
                     const float w = f.weight(x, __uint_as_float(q.y));
                     f.add_w(make_float2(x.x, x.y), w);
-                    g.add_w(__ldg(exb + q.x), w);
+                    g.add_w(ld_global(exb + q.x), w);
                 }
             } else {
                 // two entries per iteration, the next two list entries loaded
                 // while this pair's neighbour records are in flight
-                uint2 p0 = listed > 0u ? __ldg(e) : make_uint2(uint32_t(s), 0u);
-                uint2 p1 = listed > 1u ? __ldg(e + stride) : p0;
+                uint2 p0 = listed > 0u ? ld_global(e) : make_uint2(uint32_t(s), 0u);
+                uint2 p1 = listed > 1u ? ld_global(e + stride) : p0;
                 for (; k + 2 <= listed; k += 2, e += 2 * stride) {
                     const uint2 q0 = p0, q1 = p1;
-                    const float4 x0 = __ldg(ex + q0.x), x1 = __ldg(ex + q1.x);
-                    p0 = k + 2 < listed ? __ldg(e + 2 * stride) : q0;
-                    p1 = k + 3 < listed ? __ldg(e + 3 * stride) : q1;
+                    const float4 x0 = ld_global(ex + q0.x), x1 = ld_global(ex + q1.x);
+                    p0 = k + 2 < listed ? ld_global(e + 2 * stride) : q0;
+                    p1 = k + 3 < listed ? ld_global(e + 3 * stride) : q1;
                     f.add(x0, __uint_as_float(q0.y));
                     f.add(x1, __uint_as_float(q1.y));
                 }
-                if (k < listed) f.add(__ldg(ex + p0.x), __uint_as_float(p0.y));   // p0 = entry k
+                if (k < listed) f.add(ld_global(ex + p0.x), __uint_as_float(p0.y));   // p0 = entry k
             }
         }
     } else if constexpr (TWO) {
@@ -2258,8 +2306,8 @@ k_emit_pairs(int n, int64_t stride, const double* __restrict__ pos, const float*
 // tangents' differences and products, K's last product, dK).  Returns K and
 // h^2 dK/dD: the passes carry dK and dr times h^2, and pass B divides its sum.
 template <int DIM>
-__device__ __forceinline__ double2 pair_terms(const uint64_t* __restrict__ image,
-                                              const double* __restrict__ tan, int64_t stride,
+__device__ __forceinline__ double2 pair_terms(const uint64_t* image,
+                                              const double* tan, int64_t stride,
                                               uint32_t s, uint32_t j, const RealParams& P,
                                               const double* table) {
     const KernelConsts& kc = P.pp.kc;
@@ -2267,12 +2315,12 @@ __device__ __forceinline__ double2 pair_terms(const uint64_t* __restrict__ image
     double dot = 0.0;
 #pragma unroll
     for (int a = 0; a < DIM; ++a) {
-        const uint64_t xi = __ldg(image + a * stride + s), xj = __ldg(image + a * stride + j);
+        const uint64_t xi = ld_global(image + a * stride + s), xj = ld_global(image + a * stride + j);
         const uint64_t d = axis_distance(xi, xj);
         d2h += square_hi(d);
         const double sign_d = double_of(bits_of(scaled(d, -kc.x_shift)) |
                                         ((xi - xj) & 0x8000000000000000ull));
-        const double dt = __dsub_rn(__ldg(tan + a * stride + s), __ldg(tan + a * stride + j));
+        const double dt = __dsub_rn(ld_global(tan + a * stride + s), ld_global(tan + a * stride + j));
         dot = a == 0 ? __dmul_rn(sign_d, dt) : __fma_rn(sign_d, dt, dot);
     }
     const double K = gauss_fixed(d2h, table, kc);
@@ -2293,12 +2341,12 @@ struct AdjRowSum {
 // The two passes of one particle whose neighbours the words do not hold.
 template <int DIM, class View>
 __device__ __noinline__ double2 adj_search_rowsum(uint32_t s, int64_t stride,
-                                                  const double* __restrict__ pos,
-                                                  const uint64_t* __restrict__ image,
-                                                  const double* __restrict__ tan,
-                                                  const float* __restrict__ rec,
-                                                  const uint32_t* __restrict__ cell,
-                                                  const uint32_t* __restrict__ start,
+                                                  const double* pos,
+                                                  const uint64_t* image,
+                                                  const double* tan,
+                                                  const float* rec,
+                                                  const uint32_t* cell,
+                                                  const uint32_t* start,
                                                   const double* table, const View& v) {
     const RealParams& P = v.of_sorted(s);
     AdjRowSum sum;
@@ -2314,17 +2362,17 @@ __device__ __noinline__ double2 adj_search_rowsum(uint32_t s, int64_t stride,
 struct AdjRec {
     double r, dr, mass, lam;
 };
-__device__ __forceinline__ AdjRec load_adj_rec(const double* __restrict__ rec4, uint32_t j) {
+__device__ __forceinline__ AdjRec load_adj_rec(const double* rec4, uint32_t j) {
     AdjRec q;
-    asm("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];"
+    asm("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];"
         : "=d"(q.r), "=d"(q.dr), "=d"(q.mass), "=d"(q.lam)
         : "l"(rec4 + 4 * size_t(j)));
     return q;
 }
 __global__ void __launch_bounds__(kBlock)
-k_adj_records(int n, const double* __restrict__ r, const double* __restrict__ dr,
-              const double* __restrict__ mass, const uint32_t* __restrict__ id,
-              const double* __restrict__ lam_in, double* __restrict__ rec4) {
+k_adj_records(int n, const double* r, const double* dr,
+              const double* mass, const uint32_t* id,
+              const double* lam_in, double* __restrict__ rec4) {
     const int s = int(ordered_index());
     if (s >= n) return;
     asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(rec4 + 4 * size_t(s)), "d"(r[s]),
@@ -2356,14 +2404,14 @@ struct AdjFluxSum {
 
 template <int DIM, class View>
 __device__ __noinline__ double2 adj_search_flux(uint32_t s, int64_t stride,
-                                                const double* __restrict__ pos,
-                                                const uint64_t* __restrict__ image,
-                                                const double* __restrict__ tan,
-                                                const float* __restrict__ rec,
-                                                const uint32_t* __restrict__ cell,
-                                                const uint32_t* __restrict__ start,
+                                                const double* pos,
+                                                const uint64_t* image,
+                                                const double* tan,
+                                                const float* rec,
+                                                const uint32_t* cell,
+                                                const uint32_t* start,
                                                 const double* table, const View& v,
-                                                const double* __restrict__ rec4) {
+                                                const double* rec4) {
     const RealParams& P = v.of_sorted(s);
     const double* mine = rec4 + 4 * size_t(s);
     const AdjRec me{mine[0], mine[1], mine[2], mine[3]};
@@ -2393,10 +2441,10 @@ struct TapeOut {
 // tape.mass_out also the rest of the step's tape.
 template <int DIM, class View>
 __global__ void __launch_bounds__(kBlock, 4)
-k_adj_rowsum(int n, int64_t stride, const double* __restrict__ pos,
-             const uint64_t* __restrict__ image, const double* __restrict__ tan,
-             const float* __restrict__ rec, const uint32_t* __restrict__ cell,
-             const uint32_t* __restrict__ start, const double* __restrict__ exp_table,
+k_adj_rowsum(int n, int64_t stride, const double* pos,
+             const uint64_t* image, const double* tan,
+             const float* rec, const uint32_t* cell,
+             const uint32_t* start, const double* __restrict__ exp_table,
              const __grid_constant__ View v, double* __restrict__ r_out,
              double* __restrict__ dr_out, NbPlanes nb, uint32_t* __restrict__ listed_out,
              AdjValues kv, TapeOut tape) {
@@ -2446,14 +2494,14 @@ k_adj_rowsum(int n, int64_t stride, const double* __restrict__ pos,
 // load; four blocks an SM (three and six: 7 and 4 % slower sweeps).
 template <int DIM, class View>
 __global__ void __launch_bounds__(kBlock, 4)
-k_adj_exchange(int n, int64_t stride, const double* __restrict__ pos,
-               const uint64_t* __restrict__ image, const double* __restrict__ tan,
-               const float* __restrict__ rec, const uint32_t* __restrict__ cell,
-               const uint32_t* __restrict__ start, const double* __restrict__ exp_table,
-               const __grid_constant__ View v, const double* __restrict__ rec4,
-               const uint32_t* __restrict__ id, double* __restrict__ lam_out,
+k_adj_exchange(int n, int64_t stride, const double* pos,
+               const uint64_t* image, const double* tan,
+               const float* rec, const uint32_t* cell,
+               const uint32_t* start, const double* __restrict__ exp_table,
+               const __grid_constant__ View v, const double* rec4,
+               const uint32_t* id, double* __restrict__ lam_out,
                double* __restrict__ gD_block, NbPlanes nb,
-               const uint32_t* __restrict__ listed_in, AdjValues kv) {
+               const uint32_t* listed_in, AdjValues kv) {
     __shared__ double table[kExpTable];
     __shared__ ChunkShared<double2> chunk;
     const uint32_t s = ordered_index();
@@ -2470,7 +2518,7 @@ k_adj_exchange(int n, int64_t stride, const double* __restrict__ pos,
         [&](uint32_t total) { keep = kv.of_warp(s - (threadIdx.x & 31u), total); },
         [&](uint32_t e, uint32_t so, uint32_t j) {
             const AdjRec me = load_adj_rec(rec4, so), o = load_adj_rec(rec4, j);
-            const double2 kd = keep ? __ldg(keep + e)
+            const double2 kd = keep ? ld_global(keep + e)
                                     : pair_terms<DIM>(image, tan, stride, so, j, v.of_sorted(so), table);
             return adj_flux(kd, me, o);
         },
@@ -2500,7 +2548,7 @@ constexpr int kReduceThreads = 512;
 // One block: thread t adds partial[t], partial[t + T], ... in order, then a
 // fixed tree over the threads; the result is added to *acc.
 __global__ void __launch_bounds__(kReduceThreads)
-k_sum_into(int nparts, const double* __restrict__ partial, double* __restrict__ acc) {
+k_sum_into(int nparts, const double* partial, double* __restrict__ acc) {
     __shared__ double buf[kReduceThreads];
     double s = 0.0;
     for (int k = int(ordered_index()); k < nparts; k += kReduceThreads) s = __dadd_rn(s, partial[k]);
@@ -2539,8 +2587,8 @@ __device__ __forceinline__ double widen(double x) { return x; }
 __device__ __forceinline__ double widen(float x) { return f32_to_f64(x); }
 
 template <typename T>
-__global__ void k_unpermute(int n, int64_t stride, int naxes, const uint32_t* __restrict__ id,
-                            const T* __restrict__ src, int src_step, double scale,
+__global__ void k_unpermute(int n, int64_t stride, int naxes, const uint32_t* id,
+                            const T* src, int src_step, double scale,
                             double* __restrict__ out) {
     const int s = int(ordered_index());
     if (s >= n) return;

@@ -39,10 +39,31 @@ def test_the_step_kernels_are_found():
 
 @pytest.mark.parametrize("name", KERNELS)
 def test_indexes_pass_through_the_wait(name):
-    """A read-only load whose address does not come out of the wait may be moved
-    ahead of it: a kernel that reads through pointers to const takes its index
-    from ordered_index()."""
+    """A load whose address does not come out of the wait may be moved ahead of
+    it: a kernel that reads through pointers to const takes its index from
+    ordered_index()."""
     params, body = _kernel(_source("kernels.cuh"), name)
     if "ordered_index()" not in body:
         assert "after_previous()" in body
         assert not re.search(r"\bconst\b[^,]*\*", params)
+
+
+CONSTANTS = {"corners", "exp_table"}     # written before the first kernel of a run starts
+
+
+@pytest.mark.parametrize("name", KERNELS)
+def test_read_only_pointers_are_constants(name):
+    """The read-only path wants memory that nothing writes while the kernel
+    lives, and an overlapping kernel is alive while the one before it writes."""
+    params, _ = _kernel(_source("kernels.cuh"), name)
+    assert set(re.findall(r"\bconst\b[^,]*\*\s*__restrict__\s+(\w+)", params)) <= CONSTANTS
+
+
+def test_read_only_loads_are_of_constants():
+    src = _source("kernels.cuh")
+    assert set(re.findall(r"__ldg\((\w+)", src)) <= CONSTANTS
+    assert not re.search(r"\bld\.[\w.]*\.nc\b", src)
+    # nor in the device functions that the kernels share
+    for params in re.findall(r"__device__[^;{]*?\(([^;{]*)\)\s*\{", src):
+        names = set(re.findall(r"\bconst\b[^,]*\*\s*__restrict__\s+(\w+)", params))
+        assert names <= CONSTANTS | {"table"}, names      # (table: in shared memory)
