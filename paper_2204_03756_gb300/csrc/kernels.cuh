@@ -169,7 +169,7 @@ struct Grid {
 
 struct PairParams {
     double psi2;       // cutoff squared: the exact binary64 test d2 <= psi2
-    float band_lo;     // binary32 d2 below this: certainly a neighbour
+    float band_lo;     // binary32 d2 below this: certainly a neighbour; >= +0 (pair_band)
     float band_hi;     // binary32 d2 above this: certainly not a neighbour
     float reach2;      // band_hi (1 + 2^-16): bounds dx^2 + dy^2 (+ dz^2) of a neighbour
     float trim_eps;    // slack of the per-row candidate windows (see for_each_row)
@@ -1243,12 +1243,13 @@ __device__ __forceinline__ uint32_t mask_word(uint32_t words, uint32_t neighbour
 // The search of one particle, its windows row by row, two candidates (one
 // block of records) at a time: one 32-byte load, the distances as packed
 // binary32 operations, the tests on the distances' bits (ordered like the
-// values).  A window starts at an even index and may end at an odd one, so
-// candidates outside it are masked off.  With WORDS, the accepted candidates
-// (those below the narrow band around the cutoff; `band` reports candidates
-// inside it) go into mask words; EACH calls cand(j, d2f, accept) for every
-// candidate, the self pair included.  Returns the words written or wanted;
-// cnt receives the accepted neighbours j != s (WORDS only).
+// values, as neither a distance nor band_lo has a sign bit).  A window starts
+// at an even index and may end at an odd one, so candidates outside it are
+// masked off.  With WORDS, the accepted candidates (those below the narrow
+// band around the cutoff; `band` reports candidates inside it) go into mask
+// words; EACH calls cand(j, d2f, accept) for every candidate, the self pair
+// included.  Returns the words written or wanted; cnt receives the accepted
+// neighbours j != s (WORDS only).
 //
 // Bound by instruction issue: singly, a candidate took about 20 instructions
 // of which the pair shares or packs all but three.  The bisection to a

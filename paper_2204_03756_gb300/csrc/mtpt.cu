@@ -24,6 +24,7 @@
 #include <vector>
 
 #include "../../include/mtpt.h"
+#include "band.cuh"
 #include "kernels.cuh"
 #include "hostio.cuh"
 #include "tiles.cuh"
@@ -561,8 +562,10 @@ int setup_grid(RealHost& R, RealParams& P, int64_t cell_base, int corner_base, d
     const double eta = 2.0 * (u * (3.0 + kdx * (1.0 + dc) * sum_w) + std::ldexp(sum_b, -43)) + 1e-14;
     R.band_eta = eta;
     pp.psi2 = R.psi2;
-    pp.band_lo = std::nextafter(float(R.psi2 * (1.0 - eta)), 0.0f);
-    pp.band_hi = std::nextafter(float(R.psi2 * (1.0 + eta)), INFINITY);
+    const PairBand band = pair_band(R.psi2, eta);
+    pp.band_lo = band.lo;
+    pp.band_hi = band.hi;
+    pp.reach2 = band.reach2;
     // Candidate windows: reach2 bounds dx^2 + g^2 of every accepted candidate
     // with the binary32 roundings of d2f and of the window arithmetic
     // (2^-16 relative is far above them).  trim_eps covers the sqrt rounding,
@@ -570,7 +573,6 @@ int setup_grid(RealHost& R, RealParams& P, int64_t cell_base, int corner_base, d
     // from x order (a particle sits within dc cells of its cell, dc as above
     // for binary32 cell indices and 2^-29 of it for binary64 ones), with a
     // factor 2 to spare.
-    pp.reach2 = std::nextafter(float(double(pp.band_hi) * (1.0 + std::ldexp(1.0, -16))), INFINITY);
     {
         const double dc_cells = g.cell_f32 ? dc : std::ldexp(dc, -29);
         double eps = 0.0;
