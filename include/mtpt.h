@@ -386,10 +386,8 @@ int mtpt_step_noalloc(const mtpt_params* params, int64_t n, uint64_t step, doubl
  * loaded state, as mtpt_step does, while
  * recording a checkpoint of the state every `checkpoint_every` steps and the
  * position tangents dX/dD.  Memory: (nsteps / checkpoint_every +
- * checkpoint_every + 1) snapshots of (16 dim + 12) bytes per particle, and, when
- * it can be had and is at most 16 GiB, a tape of checkpoint_every steps (some
- * 250 bytes per particle and step at 3 neighbours) that spares the reverse
- * sweep each step's second walk, sort and search.  Synchronises. */
+ * checkpoint_every + 1) snapshots of (16 dim + 12) bytes per particle.
+ * Synchronises. */
 int mtpt_adjoint_forward(mtpt_handle* h, int64_t nsteps, int64_t checkpoint_every);
 
 /* Adjoint (no counterpart in the paper).  Reverse sweep of the run recorded
@@ -397,6 +395,9 @@ int mtpt_adjoint_forward(mtpt_handle* h, int64_t nsteps, int64_t checkpoint_ever
  * dL/dM_T (n doubles, DEVICE, input order); gmass0_dev receives dL/dM_0 (n
  * doubles, DEVICE, input order); *dldD receives dL/dD (HOST).  Recomputes
  * each segment forward from its checkpoint, then steps back through it.
+ * While it runs it holds, when it can be had and is at most 16 GiB, a tape of
+ * checkpoint_every steps (some 250 bytes per particle and step at 3 neighbours)
+ * that spares each step's second walk, sort and search.
  * Leaves the handle in the final state of the forward run.  Deterministic
  * (fixed summation orders).  Synchronises.  MTPT_ERR_STATE without a recorded
  * run. */

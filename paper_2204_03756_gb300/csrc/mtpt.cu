@@ -295,7 +295,7 @@ struct mtpt_handle {
     bool adj_ready = false;
     bool adjoint_sweep = false;       // the sorts feed the adjoint's pair passes
     DevBuf<double> dr64, lam_in, adj_rec, partial, acc;
-    DevBuf<unsigned char> tape;       // one segment's steps (TapeSlot), when it fits
+    DevBuf<unsigned char> tape;       // one segment's steps (TapeSlot) during a sweep, when it fits
     int64_t tape_steps = 0;
     DevBuf<uint32_t> tape_flag;       // TapeOut::incomplete
     // captured graph of plain steps (valid for `graph_cur`, `graph_flags` and the
@@ -1918,7 +1918,7 @@ int backward_segment(mtpt_handle* h, int64_t k, int64_t t0, int64_t t1) {
     const int64_t blocks = grid_for(h->n);
     MTPT_TRY(snapshot(h, k, false));
     MTPT_TRY(set_step_dev(h, h->adj_step0 + uint64_t(t0)));
-    if (t1 - t0 <= h->tape_steps && size_t(t1 - t0) * tape_step_bytes(h) <= h->tape.count) {
+    if (t1 - t0 <= h->tape_steps) {
         MTPT_TRY(record_segment<DIM>(h, t0, t1));
         uint32_t incomplete = 0;
         MTPT_CUDA_TRY(cudaMemcpyAsync(&incomplete, h->tape_flag.p, sizeof(incomplete),
@@ -1986,11 +1986,6 @@ int mtpt_adjoint_forward(mtpt_handle* h, int64_t nsteps, int64_t checkpoint_ever
     MTPT_TRY(h->partial.ensure(size_t(seg) * size_t(grid_for(n) + 1)));
     MTPT_TRY(h->acc.ensure(1));
     MTPT_TRY(h->tape_flag.ensure(1));
-    // the tape is room for speed: without it the sweep takes its steps one by one
-    h->tape_steps = 0;
-    const size_t tape_bytes = size_t(seg) * tape_step_bytes(h);
-    if (n > 0 && tape_bytes <= kTapeBytesMax && h->tape.ensure(tape_bytes, true) == MTPT_OK)
-        h->tape_steps = seg;
     h->tangent_on = true;
     h->adj_step0 = h->step;
     int rc = MTPT_OK;
@@ -2023,6 +2018,11 @@ int mtpt_adjoint_backward(mtpt_handle* h, const double* gmass_dev, double* gmass
                                   cudaMemcpyDeviceToDevice, h->stream));
     MTPT_CUDA_TRY(cudaMemsetAsync(h->acc.p, 0, sizeof(double), h->stream));
     drop_graph(h);
+    // the tape is room for speed, held for the sweep alone: without it the sweep
+    // takes its steps one by one
+    const size_t tape_bytes = size_t(seg) * tape_step_bytes(h);
+    const bool taped = n > 0 && tape_bytes <= kTapeBytesMax && h->tape.ensure(tape_bytes, true) == MTPT_OK;
+    h->tape_steps = taped ? seg : 0;
     h->tangent_on = true;
     h->adjoint_sweep = true;          // the sorts write the images of pass A
     int rc = MTPT_OK;
@@ -2032,6 +2032,7 @@ int mtpt_adjoint_backward(mtpt_handle* h, const double* gmass_dev, double* gmass
     }
     h->adjoint_sweep = false;
     h->tangent_on = false;
+    h->tape.release();                // (waits for the sweep)
     // leave the handle in its final forward state
     if (rc == MTPT_OK) rc = snapshot(h, final_slot, false);
     if (rc == MTPT_OK) rc = set_step_dev(h, h->adj_step0 + uint64_t(T));

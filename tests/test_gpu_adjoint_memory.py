@@ -1,0 +1,55 @@
+"""Device memory around the adjoint: what a recorded run holds, what the sweep
+holds, and that it is given back."""
+import numpy as np
+import pytest
+
+from paper_2204_03756_gb300 import mtpt
+
+pytestmark = pytest.mark.gpu
+
+MB = 1 << 20
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_2204_03756_gb300 import build
+    build.build()
+    mtpt.load()
+
+
+def _free():
+    import torch
+    torch.cuda.synchronize()
+    return torch.cuda.mem_get_info()[0]
+
+
+def _recorded(n=20000, steps=40, every=40):
+    rng = np.random.default_rng(1)
+    L = float(np.sqrt(n))
+    p = mtpt.Params(dim=2, D=0.5, kappa=0.5, dt=0.1, lo=(0.0, 0.0), hi=(L, L), seed=4)
+    h = mtpt.mtpt_create(p)
+    mtpt.mtpt_set_particles(h, 2, rng.uniform(0.0, L, size=(2, n)), rng.uniform(0.0, 1.0, n))
+    before = _free()
+    mtpt.mtpt_adjoint_forward(h, steps, every)
+    return h, before
+
+
+def test_the_tape_is_held_for_the_sweep_alone():
+    """A recording holds its snapshots, (steps / every + every + 1) of
+    16 dim + 12 bytes per particle, tangents and per-particle scratch; the tape
+    (some 250 bytes per particle and step) is the sweep's and goes with it."""
+    import torch
+    n, steps = 20000, 40
+    g = torch.ones(n, dtype=torch.float64, device="cuda")
+    g0 = torch.empty_like(g)
+    h, before = _recorded(n, steps, steps)
+    try:
+        recorded = _free()
+        snapshots = (1 + steps + 1) * 44 * n
+        assert before - recorded < snapshots + 60 * MB
+        mtpt.mtpt_adjoint_backward(h, g, g0)
+        assert _free() >= recorded - 4 * MB
+        mtpt.mtpt_adjoint_backward(h, g, g0)
+        assert _free() >= recorded - 4 * MB
+    finally:
+        mtpt.mtpt_destroy(h)
