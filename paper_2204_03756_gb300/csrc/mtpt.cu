@@ -64,23 +64,24 @@ void report_cuda_error(cudaError_t err, const char* expr, int line) {
         if (rc_ != MTPT_OK) return rc_; \
     } while (0)
 
-// Failure injection for the tests (mtpt_debug_fail_alloc): when positive,
-// the countdown's allocation fails as if the device were out of memory.
+// Failure injection for the tests (mtpt_debug_fail_alloc): when positive, the
+// countdown's allocation fails as if the device were out of memory; when
+// negative, the same of the allocations that the library can do without.
 std::atomic<int64_t> g_fail_alloc{0};
 
-bool injected_alloc_failure() {
+bool injected_alloc_failure(bool optional) {
+    const int64_t toward_zero = optional ? 1 : -1;
     int64_t v = g_fail_alloc.load();
-    while (v > 0)
-        if (g_fail_alloc.compare_exchange_weak(v, v - 1)) return v == 1;
+    while (optional ? v < 0 : v > 0)
+        if (g_fail_alloc.compare_exchange_weak(v, v + toward_zero)) return v + toward_zero == 0;
     return false;
 }
 
 // Every device allocation of the library goes through here (`optional`: the
-// caller does without it when there is no memory; not counted by the
-// injection, which is to surface).
+// caller does without it when there is no memory).
 int device_alloc(void** out, size_t bytes, bool optional = false) {
     *out = nullptr;
-    if (!optional && injected_alloc_failure()) return MTPT_ERR_NO_MEMORY;
+    if (injected_alloc_failure(optional)) return MTPT_ERR_NO_MEMORY;
     if (cudaMalloc(out, bytes) != cudaSuccess) {
         (void)cudaGetLastError();
         *out = nullptr;
@@ -1912,7 +1913,8 @@ int record_segment(mtpt_handle* h, int64_t t0, int64_t t1) {
 }
 
 // One segment of the backward sweep from its checkpoint (slot k of the
-// snapshots), steps t1-1 down to t0.
+// snapshots), steps t1-1 down to t0.  On the tape or not, the same terms are added
+// in the same order: the gradient does not depend on how much memory is free.
 template <int DIM>
 int backward_segment(mtpt_handle* h, int64_t k, int64_t t0, int64_t t1) {
     const int64_t blocks = grid_for(h->n);
@@ -1947,11 +1949,10 @@ int backward_segment(mtpt_handle* h, int64_t k, int64_t t0, int64_t t1) {
         const int o = 1 - h->cur;
         const TapeSlot slot = own_slot(h, o);
         MTPT_TRY(launch_adjoint_rows<DIM>(h, o, h->mass[o].p, slot, false));
-        MTPT_TRY(launch_adjoint_pass<DIM>(h, o, slot, h->partial.p));
-        MTPT_TRY(sum_blocks(h, blocks));
+        MTPT_TRY(launch_adjoint_pass<DIM>(h, o, slot, h->partial.p + (t - t0) * blocks));
         h->cur = o;
     }
-    return MTPT_OK;
+    return sum_blocks(h, (t1 - t0) * blocks);
 }
 
 int dispatch_backward_segment(mtpt_handle* h, int64_t k, int64_t t0, int64_t t1) {
@@ -2927,9 +2928,8 @@ int mtpt_get_masses_b(mtpt_handle* h, double* out) {
 }
 
 int mtpt_debug_fail_alloc(int64_t nth, int64_t* remaining) {
-    if (nth < 0) return MTPT_ERR_INVALID_ARG;
     const int64_t before = g_fail_alloc.exchange(nth);
-    if (remaining) *remaining = before;
+    if (remaining) *remaining = before < 0 ? -before : before;
     return MTPT_OK;
 }
 

@@ -542,8 +542,9 @@ def mtpt_get_masses_b(h, n: int) -> np.ndarray:
 
 
 def mtpt_debug_fail_alloc(nth: int) -> int:
-    """Make the nth device allocation from now fail (0: off); returns how many
-    the previous setting still had to go."""
+    """Make the nth device allocation from now fail (0: off; negative: the -nth-th
+    of those that the library can do without); returns how many the previous
+    setting still had to go."""
     left = ctypes.c_int64()
     _check(load().mtpt_debug_fail_alloc(nth, ctypes.byref(left)), "mtpt_debug_fail_alloc")
     return int(left.value)

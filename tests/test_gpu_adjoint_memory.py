@@ -53,3 +53,38 @@ def test_the_tape_is_held_for_the_sweep_alone():
         assert _free() >= recorded - 4 * MB
     finally:
         mtpt.mtpt_destroy(h)
+
+
+def _sweep(p, pos, mass, g, steps, every, without_tape):
+    import torch
+    h = mtpt.mtpt_create(p)
+    try:
+        mtpt.mtpt_set_particles(h, p.dim, pos, mass)
+        mtpt.mtpt_adjoint_forward(h, steps, every)
+        gt = torch.from_numpy(g).cuda()
+        g0 = torch.empty_like(gt)
+        mtpt.mtpt_debug_fail_alloc(-1 if without_tape else 0)
+        dD = mtpt.mtpt_adjoint_backward(h, gt, g0)
+        assert mtpt.mtpt_debug_fail_alloc(0) == 0     # (the injection met the tape)
+        return dD, g0.cpu().numpy(), mtpt.mtpt_get_info(h)
+    finally:
+        mtpt.mtpt_debug_fail_alloc(0)
+        mtpt.mtpt_destroy(h)
+
+
+@pytest.mark.parametrize("form", [mtpt.MTPT_FP64, mtpt.MTPT_FP32W])
+@pytest.mark.parametrize("clump", [0, 150])
+@pytest.mark.parametrize("dim,n,L", [(1, 700, 300.0), (2, 5001, 70.0), (3, 1500, 12.0)])
+def test_gradients_do_not_depend_on_free_memory(form, clump, dim, n, L):
+    """With the tape, without the memory for it, and with a clump that the tape
+    cannot hold: the same bits."""
+    rng = np.random.default_rng(n + clump)
+    pos = rng.uniform(0.0, L, size=(dim, n))
+    pos[:, :clump] = L / 2 + rng.uniform(-0.2, 0.2, size=(dim, clump))
+    mass, g = rng.uniform(0.0, 1.0, n), rng.uniform(-1.0, 1.0, n)
+    p = mtpt.Params(dim=dim, D=0.5, kappa=0.5, dt=0.1, lo=(0.0,) * dim, hi=(L,) * dim, seed=3,
+                    precision=form)
+    for steps, every in ((5, 5), (7, 3)):
+        taped, plain = (_sweep(p, pos, mass, g, steps, every, w) for w in (False, True))
+        assert taped[0] == plain[0]
+        assert np.array_equal(taped[1], plain[1])
