@@ -298,7 +298,7 @@ struct mtpt_handle {
     DevBuf<double> dr64, lam_in, adj_rec, partial, acc;
     DevBuf<unsigned char> tape;       // one segment's steps (TapeSlot) during a sweep, when it fits
     int64_t tape_steps = 0;
-    DevBuf<uint32_t> tape_flag;       // TapeOut::incomplete
+    DevBuf<uint32_t> tape_flag;       // TapeOut::incomplete, pair counter (kTapeWords)
     // captured graph of plain steps (valid for `graph_cur`, `graph_flags` and the
     // mass buffer pair as it was: every step swaps the pair, so between loads
     // its order follows `cur`, but a pipelined load moves `cur` alone)
@@ -1892,11 +1892,27 @@ int sum_blocks(mtpt_handle* h, int64_t parts) {
     return MTPT_OK;
 }
 
+// Words of tape_flag: TapeOut::incomplete, and from kTapePairs the pair counter
+// as it stood before the segment.
+constexpr size_t kTapePairs = 2, kTapeWords = 4;
+
+// Whether the steps recorded so far are whole on the tape (synchronises).
+int tape_whole(mtpt_handle* h, bool* whole) {
+    uint32_t incomplete = 0;
+    MTPT_CUDA_TRY(cudaMemcpyAsync(&incomplete, h->tape_flag.p, sizeof(incomplete),
+                                  cudaMemcpyDeviceToHost, h->stream));
+    MTPT_CUDA_TRY(cudaStreamSynchronize(h->stream));
+    *whole = incomplete == 0;
+    return MTPT_OK;
+}
+
 // Steps t0..t1-1 forward from the checkpoint in the current buffer, each with
-// pass A on the tape.
+// pass A on the tape.  `probe`: the first step tells whether to go on.
 template <int DIM>
-int record_segment(mtpt_handle* h, int64_t t0, int64_t t1) {
+int record_segment(mtpt_handle* h, int64_t t0, int64_t t1, bool probe, bool* whole) {
     MTPT_CUDA_TRY(cudaMemsetAsync(h->tape_flag.p, 0, sizeof(uint32_t), h->stream));
+    MTPT_CUDA_TRY(cudaMemcpyAsync(h->tape_flag.p + kTapePairs, h->pair_counter.p,
+                                  sizeof(unsigned long long), cudaMemcpyDeviceToDevice, h->stream));
     for (int64_t t = t0; t < t1; ++t) {
         const TapeSlot slot = tape_slot(h, t - t0);
         if (t + 1 < t1) {
@@ -1908,30 +1924,39 @@ int record_segment(mtpt_handle* h, int64_t t0, int64_t t1) {
             h->cur = 1 - h->cur;
             MTPT_TRY(launch_adjoint_rows<DIM>(h, h->cur, h->mass[h->cur].p, slot, true));
         }
+        if (probe && t == t0) {
+            MTPT_TRY(tape_whole(h, whole));
+            if (!*whole) return MTPT_OK;
+        }
     }
-    return MTPT_OK;
+    return tape_whole(h, whole);
 }
 
 // One segment of the backward sweep from its checkpoint (slot k of the
 // snapshots), steps t1-1 down to t0.  On the tape or not, the same terms are added
 // in the same order: the gradient does not depend on how much memory is free.
+// Particles that the tape cannot hold (a clump) are mostly there in the other
+// segments too: after one such segment the sweep goes on without the tape, and its
+// first segment looks for them after one step.
 template <int DIM>
 int backward_segment(mtpt_handle* h, int64_t k, int64_t t0, int64_t t1) {
     const int64_t blocks = grid_for(h->n);
     MTPT_TRY(snapshot(h, k, false));
     MTPT_TRY(set_step_dev(h, h->adj_step0 + uint64_t(t0)));
     if (t1 - t0 <= h->tape_steps) {
-        MTPT_TRY(record_segment<DIM>(h, t0, t1));
-        uint32_t incomplete = 0;
-        MTPT_CUDA_TRY(cudaMemcpyAsync(&incomplete, h->tape_flag.p, sizeof(incomplete),
-                                      cudaMemcpyDeviceToHost, h->stream));
-        MTPT_CUDA_TRY(cudaStreamSynchronize(h->stream));
-        if (!incomplete) {
+        bool whole = false;
+        MTPT_TRY(record_segment<DIM>(h, t0, t1, t1 == h->adj_steps, &whole));
+        if (whole) {
             for (int64_t t = t1 - 1; t >= t0; --t)
                 MTPT_TRY(launch_adjoint_pass<DIM>(h, h->cur, tape_slot(h, t - t0),
                                                   h->partial.p + (t - t0) * blocks));
             return sum_blocks(h, (t1 - t0) * blocks);
         }
+        h->tape_steps = 0;
+        // the segment again, its pairs counted once
+        MTPT_CUDA_TRY(cudaMemcpyAsync(h->pair_counter.p, h->tape_flag.p + kTapePairs,
+                                      sizeof(unsigned long long), cudaMemcpyDeviceToDevice,
+                                      h->stream));
         MTPT_TRY(snapshot(h, k, false));
         MTPT_TRY(set_step_dev(h, h->adj_step0 + uint64_t(t0)));
     }
@@ -1986,7 +2011,7 @@ int mtpt_adjoint_forward(mtpt_handle* h, int64_t nsteps, int64_t checkpoint_ever
     MTPT_TRY(ensure_adjoint_rows(h));
     MTPT_TRY(h->partial.ensure(size_t(seg) * size_t(grid_for(n) + 1)));
     MTPT_TRY(h->acc.ensure(1));
-    MTPT_TRY(h->tape_flag.ensure(1));
+    MTPT_TRY(h->tape_flag.ensure(kTapeWords));
     h->tangent_on = true;
     h->adj_step0 = h->step;
     int rc = MTPT_OK;

@@ -88,3 +88,5 @@ def test_gradients_do_not_depend_on_free_memory(form, clump, dim, n, L):
         taped, plain = (_sweep(p, pos, mass, g, steps, every, w) for w in (False, True))
         assert taped[0] == plain[0]
         assert np.array_equal(taped[1], plain[1])
+        # a segment that the tape cannot hold is taken again, its pairs counted once
+        assert taped[2]["pair_count"] == plain[2]["pair_count"]
