@@ -1160,40 +1160,6 @@ __device__ __forceinline__ void scan_band(uint32_t s, uint32_t cell, int64_t str
     });
 }
 
-// As visit_neighbours, but calls visit(j, d2f, accept) for every candidate of
-// the windows.  A candidate inside the narrow band around the cutoff gets the
-// exact binary64 test in place, or, with DEFER_BAND, is first visited as
-// rejected and, if the particle met any, a second walk visits those the exact
-// test accepts (the order in which 3-d lists hold their neighbours).
-template <int DIM, bool DEFER_BAND, class Visit>
-__device__ __forceinline__ void scan_neighbours(uint32_t s, uint32_t cell, int64_t stride,
-                                                const float* rec,
-                                                const double* pos,
-                                                const uint32_t* start,
-                                                const RealParams& P, Visit&& visit) {
-    const PairParams& pp = P.pp;
-    const float4 me = load_rec(rec, s);
-    const float wx = P.g.wf[0];
-    bool band = false;
-    for_each_row<DIM>(cell, me, rec, start, P,
-                      [&](uint32_t j0, uint32_t j3, float rx, float sy, float sz) {
-        for (uint32_t j = j0; j < j3; ++j) {
-            const float4 o = load_rec(rec, j);
-            const float dx = dx_f32(me, o, wx);
-            if (dx > rx) break;
-            const float d2f = d2_f32<DIM>(dx, me, o, sy, sz);
-            const bool inside = d2f >= pp.band_lo && d2f <= pp.band_hi;
-            bool accept = d2f < pp.band_lo;
-            if constexpr (DEFER_BAND) band |= inside;
-            else if (inside) accept = exact_within<DIM>(pos, stride, s, j, pp.psi2);
-            visit(j, d2f, accept);
-        }
-    });
-    if (DEFER_BAND && band)
-        scan_band<DIM>(s, cell, stride, rec, pos, start, P,
-                       [&](uint32_t j, float d2f) { visit(j, d2f, true); });
-}
-
 __device__ __forceinline__ float ex2_approx(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -1245,11 +1211,12 @@ __device__ __forceinline__ uint32_t mask_word(uint32_t words, uint32_t neighbour
 // binary32 operations, the tests on the distances' bits (ordered like the
 // values, as neither a distance nor band_lo has a sign bit).  A window starts
 // at an even index and may end at an odd one, so candidates outside it are
-// masked off.  With WORDS, the accepted candidates (those below the narrow
-// band around the cutoff; `band` reports candidates inside it) go into mask
-// words; EACH calls cand(j, d2f, accept) for every candidate, the self pair
-// included.  Returns the words written or wanted; cnt receives the accepted
-// neighbours j != s (WORDS only).
+// masked off.  With WORDS, the accepted neighbours j != s go to the sink, as mask
+// words {base, bits} in candidate order: those below the narrow band around the
+// cutoff, and, with EXACT, those inside it that the exact test accepts.  EACH
+// calls cand(j, d2, accept, accept1) for every two candidates j and j + 1 (d2 their
+// binary32 distances squared), the self pair included.
+// Without EXACT returns whether any candidate was inside the band.
 //
 // Bound by instruction issue: singly, a candidate took about 20 instructions
 // of which the pair shares or packs all but three.  The bisection to a
@@ -1260,12 +1227,11 @@ __device__ __forceinline__ uint32_t mask_word(uint32_t words, uint32_t neighbour
 // 3-d, 2.6); at density 10 (54 candidates a row) 1.55 -> 1.18 ms by pairs, with
 // the bisection (1.31 without).
 constexpr uint32_t kBisectFrom = 24;
-template <int DIM, bool WORDS, bool EACH, class Cand>
-__device__ __forceinline__ uint32_t search_words(uint32_t s, uint32_t cell, const float4 me,
-                                                 int64_t stride, const float* rec,
-                                                 const uint32_t* start,
-                                                 const RealParams& P, const NbPlanes& nb,
-                                                 uint32_t& cnt, bool& band, Cand&& cand) {
+template <int DIM, bool WORDS, bool EACH, bool EXACT, class Cand, class Sink>
+__device__ __forceinline__ bool search_rows(uint32_t s, uint32_t cell, const float4 me,
+                                            int64_t stride, const double* pos, const float* rec,
+                                            const uint32_t* start, const RealParams& P,
+                                            Cand&& cand, Sink&& sink) {
     const PairParams& pp = P.pp;
     const Grid& g = P.g;
     int c[3];
@@ -1273,10 +1239,8 @@ __device__ __forceinline__ uint32_t search_words(uint32_t s, uint32_t cell, cons
     const float wx = g.wf[0], eps = pp.trim_eps;
     const int R = g.reach, xlo = max(c[0] - R, 0), xhi = min(c[0] + R, g.n[0] - 1);
     const uint32_t lo_bits = __float_as_uint(pp.band_lo);
+    const uint32_t band_span = __float_as_uint(pp.band_hi) - lo_bits;
     uint32_t nearest = 0xffffffffu;    // least (bits of d2f) - lo_bits, unsigned
-    uint2* wp = nb.e + s;              // next mask word
-    uint32_t nw = 0;
-    if constexpr (WORDS) cnt = 0;
     // one row's window and candidates: an empty window where the row is outside
     // the grid or beyond the cutoff (for_each_row has the windows' derivation)
     auto row = [&](int dy, int dz) {
@@ -1307,7 +1271,7 @@ __device__ __forceinline__ uint32_t search_words(uint32_t s, uint32_t cell, cons
                 }
             }
         }
-        const uint32_t padded = nw + uint32_t(nb.pad);
+        if constexpr (WORDS) sink.begin_row();
         const uint32_t first = j;
         uint32_t b = j & ~1u;
         // one block of two candidates; false past the window's right end: in x
@@ -1336,8 +1300,16 @@ __device__ __forceinline__ uint32_t search_words(uint32_t s, uint32_t cell, cons
                 bits = __funnelshift_l(t1, bits, 1);
             }
             if constexpr (EACH) {
-                cand(b, d.x, int32_t(t0) < 0 && b >= first);
-                cand(b + 1u, d.y, int32_t(t1) < 0 && b + 1u < j3);
+                bool a0 = int32_t(t0) < 0 && b >= first, a1 = int32_t(t1) < 0 && b + 1u < j3;
+                if constexpr (EXACT) {
+                    if (min(t0, t1) <= band_span) {
+                        a0 |= t0 <= band_span && b >= first &&
+                              exact_within<DIM>(pos, stride, s, b, pp.psi2);
+                        a1 |= t1 <= band_span && b + 1u < j3 &&
+                              exact_within<DIM>(pos, stride, s, b + 1u, pp.psi2);
+                    }
+                }
+                cand(b, d, a0, a1);
             }
             b += 2u;
             return !(unpack2(dx).y > rx);
@@ -1355,20 +1327,24 @@ __device__ __forceinline__ uint32_t search_words(uint32_t s, uint32_t cell, cons
                 bits = __brev(bits) >> (32u - (b - base));
                 if (base < first) bits &= ~1u;
                 if (j3 - base < 32u) bits &= (1u << (j3 - base)) - 1u;
-                if (s - base < 32u) bits &= ~(1u << (s - base));   // the self pair is no neighbour
-                if (bits) {
-                    cnt += uint32_t(__popc(bits));
-                    if (nw < uint32_t(nb.cap)) *wp = make_uint2(base, bits);
-                    wp += stride;
-                    ++nw;
+                if constexpr (EXACT && !EACH) {
+                    if (nearest <= band_span) {
+                        for (uint32_t k = max(base, first); k < min(b, j3); ++k) {
+                            const float4 o = load_rec(rec, k);
+                            const float d2f = d2_f32<DIM>(dx_f32(me, o, wx), me, o, sy, sz);
+                            if (d2f >= pp.band_lo && d2f <= pp.band_hi &&
+                                exact_within<DIM>(pos, stride, s, k, pp.psi2))
+                                bits |= 1u << (k - base);
+                        }
+                        nearest = 0xffffffffu;
+                    }
                 }
+                if (s - base < 32u) bits &= ~(1u << (s - base));   // the self pair is no neighbour
+                if (bits) sink.word(base, bits);
                 if (!more) break;
             }
         }
-        if constexpr (WORDS) {
-            for (; nw < padded; ++nw, wp += stride)
-                if (nw < uint32_t(nb.cap)) *wp = make_uint2(0u, 0u);
-        }
+        if constexpr (WORDS) sink.end_row();
     };
     // rows in a fixed order for the whole warp
     if constexpr (DIM == 1) {
@@ -1382,8 +1358,68 @@ __device__ __forceinline__ uint32_t search_words(uint32_t s, uint32_t cell, cons
 #pragma unroll 1
             for (int dy = -R; dy <= R; ++dy) row(dy, dz);
     }
-    band = nearest <= __float_as_uint(pp.band_hi) - lo_bits;
-    return nw;
+    return nearest <= band_span;
+}
+
+// Sinks of search_rows: the planes, with their padding ...
+struct PlaneSink {
+    uint2* wp;                         // next mask word
+    int64_t stride;
+    uint32_t cap, pad;
+    uint32_t nw = 0, cnt = 0, padded = 0;   // words written or wanted, neighbours
+    __device__ __forceinline__ PlaneSink(const NbPlanes& nb, uint32_t s, int64_t st)
+        : wp(nb.e + s), stride(st), cap(uint32_t(nb.cap)), pad(uint32_t(nb.pad)) {}
+    __device__ __forceinline__ void begin_row() { padded = nw + pad; }
+    __device__ __forceinline__ void put(uint2 w) {
+        if (nw < cap) *wp = w;
+        wp += stride;
+        ++nw;
+    }
+    __device__ __forceinline__ void word(uint32_t base, uint32_t bits) {
+        cnt += uint32_t(__popc(bits));
+        put(make_uint2(base, bits));
+    }
+    __device__ __forceinline__ void end_row() {
+        while (nw < padded) put(make_uint2(0u, 0u));
+    }
+};
+// ... none ...
+struct NoSink {};
+// ... and a call pair(j0, j1, two) for every two neighbours of a word (j1 = j0
+// and `two` false for the last of an odd number).
+template <class Pair>
+struct PairSink {
+    Pair pair;
+    uint32_t cnt = 0;
+    __device__ __forceinline__ void begin_row() {}
+    __device__ __forceinline__ void word(uint32_t base, uint32_t bits) {
+        cnt += uint32_t(__popc(bits));
+        while (bits) {
+            const uint32_t j0 = base + uint32_t(__ffs(int(bits)) - 1);
+            bits &= bits - 1u;
+            const bool two = bits != 0u;
+            const uint32_t j1 = two ? base + uint32_t(__ffs(int(bits)) - 1) : j0;
+            bits &= bits - 1u;
+            pair(j0, j1, two);
+        }
+    }
+    __device__ __forceinline__ void end_row() {}
+};
+// Every neighbour of s, two at a time, in the order of its mask words, for a
+// particle whose words are not kept, in binary64: returns their number.  The search
+// and the pair terms are apart (a word's candidates, then its neighbours), so the
+// lanes meet again in the expensive terms: the no-allocation step of 65,536
+// particles in 3-d, which has no room for words, took 1072 us at density 8 with each
+// neighbour evaluated where a loop over single records met it, 694 so.
+template <int DIM, class Pair>
+__device__ __forceinline__ uint32_t each_pair(uint32_t s, const uint32_t* cell, int64_t stride,
+                                              const double* pos, const float* rec,
+                                              const uint32_t* start, const RealParams& P,
+                                              Pair&& pair) {
+    PairSink<Pair&> sink{pair};
+    search_rows<DIM, true, false, true>(s, cell_arg<DIM>(cell, s), load_rec(rec, s), stride, pos, rec,
+                                        start, P, [](uint32_t, float2, bool, bool) {}, sink);
+    return sink.cnt;
 }
 
 // The mask words of a particle that met candidates inside the band (about 1e-5
@@ -1552,8 +1588,8 @@ __device__ __forceinline__ void dense_words(uint32_t s, uint32_t listed, int64_t
     }
 }
 
-// Search of one particle of a binary64 pass: its list word (kMaskOver also when
-// nothing can be kept), neighbour count in cnt.
+// Search of one particle of a binary64 pass: its list word, neighbour count in cnt
+// (kMaskOver at once when nothing can be kept: the caller's search counts).
 template <int DIM, class View>
 __device__ __forceinline__ uint32_t search_listed(uint32_t s, int64_t stride,
                                                   const double* pos,
@@ -1562,10 +1598,14 @@ __device__ __forceinline__ uint32_t search_listed(uint32_t s, int64_t stride,
                                                   const uint32_t* start, const View& v,
                                                   const RealParams& P, const NbPlanes& nb,
                                                   uint32_t& cnt) {
-    bool band;
-    const uint32_t c = cell_arg<DIM>(cell, s);
-    uint32_t nw = search_words<DIM, true, false>(s, c, load_rec(rec, s), stride, rec, start, P, nb,
-                                                 cnt, band, [](uint32_t, float, bool) {});
+    cnt = 0;
+    if (nb.cap == 0) return kMaskOver;
+    PlaneSink sink(nb, s, stride);
+    const bool band = search_rows<DIM, true, false, false>(s, cell_arg<DIM>(cell, s), load_rec(rec, s),
+                                                           stride, pos, rec, start, P,
+                                                           [](uint32_t, float2, bool, bool) {}, sink);
+    uint32_t nw = sink.nw;
+    cnt = sink.cnt;
     if (band) {
         const float4 b = band_words<DIM, false>(s, cell, stride, pos, rec, start, v, nb, 0.0f, 0.0f);
         nw = __float_as_uint(b.z);
@@ -1574,23 +1614,23 @@ __device__ __forceinline__ uint32_t search_listed(uint32_t s, int64_t stride,
     return mask_word(nw, cnt, nb.cap);
 }
 
-// Pass 1 of one particle whose neighbours the words do not hold.
+// Pass 1 of one particle whose neighbours the words do not hold: its row sum and,
+// in .y's bits, its neighbours.
 template <int DIM, class View>
-__device__ __noinline__ double search_rowsum(uint32_t s, int64_t stride,
-                                             const double* pos,
-                                             const uint64_t* image,
-                                             const float* rec,
-                                             const uint32_t* cell,
-                                             const uint32_t* start,
-                                             const double* table, const View& v) {
+__device__ __noinline__ double2 search_rowsum(uint32_t s, int64_t stride, const double* pos,
+                                              const uint64_t* image, const float* rec,
+                                              const uint32_t* cell, const uint32_t* start,
+                                              const double* table, const View& v) {
     const RealParams& P = v.of_sorted(s);
     RowSum r;
-    visit_neighbours<DIM>(s, cell_arg<DIM>(cell, s), stride, rec, pos, start, P,
-                          [&](uint32_t j, float, const float4&) {
-                              if (j != s)
-                                  r.add(unit_of(pair_kernel<DIM>(image, stride, s, j, table, P.pp.kc)));
-                          });
-    return r.value();
+    const uint32_t cnt = each_pair<DIM>(
+        s, cell, stride, pos, rec, start, P, [&](uint32_t j0, uint32_t j1, bool two) {
+            const double K0 = pair_kernel<DIM>(image, stride, s, j0, table, P.pp.kc);
+            const double K1 = pair_kernel<DIM>(image, stride, s, j1, table, P.pp.kc);
+            r.add(unit_of(K0));
+            r.add(two ? unit_of(K1) : 0u);
+        });
+    return make_double2(r.value(), __longlong_as_double((long long)cnt));
 }
 
 // Pass 1, binary64 form: r_s = 1 + sum_{j != s} exp(-a d2_sj) (the kernel
@@ -1628,7 +1668,9 @@ k_rowsum_f64(int n, int64_t stride, const double* pos,
         if (P.transfer) {
             listed = search_listed<DIM>(s, stride, pos, rec, cell, start, v, P, nb, cnt);
             if (listed == kMaskOver) {
-                r = search_rowsum<DIM>(s, stride, pos, image, rec, cell, start, table, v);
+                const double2 rc = search_rowsum<DIM>(s, stride, pos, image, rec, cell, start, table, v);
+                r = rc.x;
+                cnt = uint32_t(__double_as_longlong(rc.y));
             } else {
                 uint64_t xs[DIM];
 #pragma unroll
@@ -1731,13 +1773,13 @@ __device__ __noinline__ double search_flux_f64(uint32_t s, int64_t stride,
     const RealParams& P = v.of_sorted(s);
     const double2 me = rm[s];
     FluxSum64 sum;
-    visit_neighbours<DIM>(s, cell_arg<DIM>(cell, s), stride, rec, pos, start, P,
-                          [&](uint32_t j, float, const float4&) {
-                              if (j == s) return;
-                              const double K = pair_kernel<DIM>(image, stride, s, j, table, P.pp.kc);
-                              const double2 q = ld_global(rm + j);
-                              sum.add(__dsub_rn(q.y, me.y), weight_fixed(K, me.x, q.x));
-                          });
+    each_pair<DIM>(s, cell, stride, pos, rec, start, P, [&](uint32_t j0, uint32_t j1, bool two) {
+        const double K0 = pair_kernel<DIM>(image, stride, s, j0, table, P.pp.kc);
+        const double K1 = pair_kernel<DIM>(image, stride, s, j1, table, P.pp.kc);
+        const double2 q0 = ld_global(rm + j0), q1 = ld_global(rm + j1);
+        sum.add(__dsub_rn(q0.y, me.y), weight_fixed(K0, me.x, q0.x));
+        if (two) sum.add(__dsub_rn(q1.y, me.y), weight_fixed(K1, me.x, q1.x));
+    });
     return sum.value();
 }
 
@@ -1874,9 +1916,13 @@ k_rowsum_f32(int n, int64_t stride, const double* pos, const float* rec,
                 if (keep) lp += stride;
                 cnt += keep ? 1u : 0u;
             };
-            uint32_t unused;
-            search_words<DIM, false, true>(uint32_t(s), cell[s], load_rec(rec, uint32_t(s)), stride, rec,
-                                           start, P, nb, unused, band, visit);
+            NoSink none;
+            band = search_rows<DIM, false, true, false>(uint32_t(s), cell[s], load_rec(rec, uint32_t(s)),
+                                                        stride, pos, rec, start, P,
+                                                        [&](uint32_t j, float2 d2, bool a0, bool a1) {
+                                                            visit(j, d2.x, a0);
+                                                            visit(j + 1u, d2.y, a1);
+                                                        }, none);
             // the band's exact accepts come last
             if (band)
                 scan_band<DIM>(uint32_t(s), cell[s], stride, rec, pos, start, P,
@@ -1884,10 +1930,15 @@ k_rowsum_f32(int n, int64_t stride, const double* pos, const float* rec,
             list_word = cnt;
         } else {
             const float na = -P.pp.a_log2e;
-            bool band;
-            uint32_t nw = search_words<DIM, true, true>(
-                uint32_t(s), 0u, load_rec(rec, uint32_t(s)), stride, rec, start, P, nb, cnt, band,
-                [&](uint32_t, float d2f, bool accept) { add(ex2_approx(na * d2f), accept); });
+            PlaneSink sink(nb, uint32_t(s), stride);
+            const bool band = search_rows<DIM, true, true, false>(
+                uint32_t(s), 0u, load_rec(rec, uint32_t(s)), stride, pos, rec, start, P,
+                [&](uint32_t, float2 d2, bool a0, bool a1) {
+                    add(ex2_approx(na * d2.x), a0);
+                    add(ex2_approx(na * d2.y), a1);
+                }, sink);
+            uint32_t nw = sink.nw;
+            cnt = sink.cnt;
             if (band) {
                 const float4 b = band_words<DIM, true>(uint32_t(s), cell, stride, pos, rec, start, v,
                                                        nb, rsum, rc);
@@ -1940,28 +1991,6 @@ struct FluxSum {
         return __dadd_rn(f32_to_f64(acc), f32_to_f64(comp));
     }
 };
-
-// Pass 2 of one particle by search, in the order in which its list or masks
-// hold its neighbours (3-d: the band's exact accepts last), for a particle
-// they do not cover or when there are none.  A real call, so its registers do
-// not weigh on the list loop.
-template <int DIM, class View>
-__device__ __noinline__ float2 search_flux(uint32_t s, int64_t stride,
-                                           const double* pos,
-                                           const float* rec,
-                                           const uint32_t* cell,
-                                           const uint32_t* start, const View& v,
-                                           const float4* ex, float rs, float2 ms,
-                                           float two_beta) {
-    const RealParams& P = v.of_sorted(s);
-    const float na = -P.pp.a_log2e;
-    FluxSum g{rs, two_beta, ms};
-    scan_neighbours<DIM, DIM == 3>(s, cell_arg<DIM>(cell, s), stride, rec, pos, start, P,
-                         [&](uint32_t j, float d2f, bool accept) {
-                             g.add(load_ex<DIM>(ex, j), ex2_approx(na * d2f), accept);
-                         });
-    return make_float2(g.acc, g.comp);
-}
 
 // ---------------------------------------------------------------------------
 // Bimolecular reaction A + B -> 0 (the extension Sec. 8 names; the model is
@@ -2020,30 +2049,6 @@ k_react(int n, double* __restrict__ ma, double* __restrict__ mb, double kp, doub
     react_masses<F64>(a, b, kp, dt, kpdt_f);
     ma[s] = a;
     mb[s] = b;
-}
-
-// As search_flux, for both species of a reaction run (species B's mass split
-// in exb): {acc_A, comp_A, acc_B, comp_B}.
-template <int DIM, class View>
-__device__ __noinline__ float4 search_flux2(uint32_t s, int64_t stride,
-                                            const double* pos,
-                                            const float* rec,
-                                            const uint32_t* cell,
-                                            const uint32_t* start, const View& v,
-                                            const float4* ex,
-                                            const float2* exb, float rs, float2 ms,
-                                            float2 msb, float two_beta) {
-    const RealParams& P = v.of_sorted(s);
-    const float na = -P.pp.a_log2e;
-    FluxSum a{rs, two_beta, ms}, b{rs, two_beta, msb};
-    scan_neighbours<DIM, DIM == 3>(s, cell_arg<DIM>(cell, s), stride, rec, pos, start, P,
-                         [&](uint32_t j, float d2f, bool accept) {
-                             const float4 xj = load_ex<DIM>(ex, j);
-                             const float W = a.weight(xj, ex2_approx(na * d2f));
-                             a.add_w(make_float2(xj.x, xj.y), W, accept);
-                             b.add_w(ld_global(exb + j), W, accept);
-                         });
-    return make_float4(a.acc, a.comp, b.acc, b.comp);
 }
 
 // The 32-byte records of neighbours j0 and, with `two`, j1 (both gathers in
@@ -2115,6 +2120,45 @@ __device__ __noinline__ float4 words_flux(const uint2* e, int64_t stride,
     const PairFlux<DIM, TWO, false> pf{ex, exb, me, na, wx, wy};
     FluxSum f{rs, two_beta, ms}, g{rs, two_beta, msb};
     add_words<DIM, TWO>(e, stride, words, pf, f, g);
+    return make_float4(f.acc, f.comp, g.acc, g.comp);
+}
+
+// Pass 2 of one particle by search, in the order in which its list or masks
+// hold its neighbours (3-d: the band's exact accepts last), for a particle
+// they do not cover or when there are none; TWO: for both species of a reaction
+// run (species B's mass split in exb).  Two candidates at a time, as in pass 1:
+// 3-d, 300,007 particles with some 300 neighbours, beyond their lists: 2001 -> 1564
+// us for two steps.  A real call, with few arguments, so its registers do not weigh
+// on the list loop.  {acc_A, comp_A, acc_B, comp_B}.
+template <int DIM, bool TWO, class View>
+__device__ __noinline__ float4 search_flux(uint32_t s, int64_t stride, const double* pos,
+                                           const float* rec, const uint32_t* cell,
+                                           const uint32_t* start, const View& v, const float4* ex,
+                                           const float2* exb) {
+    const RealParams& P = v.of_sorted(s);
+    const float na = -P.pp.a_log2e;
+    const float4 xs = load_ex<DIM>(ex, s);
+    FluxSum f{xs.z, float(2.0 * P.pp.beta), make_float2(xs.x, xs.y)};
+    FluxSum g{xs.z, f.two_beta, TWO ? ld_global(exb + s) : make_float2(0.0f, 0.0f)};
+    auto add = [&](uint32_t j, const float4& x, float d2f, bool accept) {
+        const float w = f.weight(x, ex2_approx(na * d2f));
+        f.add_w(make_float2(x.x, x.y), w, accept);
+        if constexpr (TWO) g.add_w(ld_global(exb + j), w, accept);
+    };
+    const uint32_t c = cell_arg<DIM>(cell, s);
+    NoSink none;
+    const bool band = search_rows<DIM, false, true, DIM != 3>(
+        s, c, load_rec(rec, s), stride, pos, rec, start, P,
+        [&](uint32_t j, float2 d2, bool a0, bool a1) {
+            if (!a0 && !a1) return;
+            const uint32_t j1 = a1 ? j + 1u : j;       // (j + 1 may lie past the last particle)
+            const float4 x0 = load_ex<DIM>(ex, j), x1 = load_ex<DIM>(ex, j1);
+            add(j, x0, d2.x, a0);
+            add(j1, x1, d2.y, a1);
+        }, none);
+    if (DIM == 3 && band)
+        scan_band<DIM>(s, c, stride, rec, pos, start, P,
+                       [&](uint32_t j, float d2f) { add(j, load_ex<DIM>(ex, j), d2f, true); });
     return make_float4(f.acc, f.comp, g.acc, g.comp);
 }
 
@@ -2241,18 +2285,12 @@ k_exchange_f32(int n, int64_t stride, const double* pos, const float* rec,
                 if (k < listed) f.add(ld_global(ex + p0.x), __uint_as_float(p0.y));   // p0 = entry k
             }
         }
-    } else if constexpr (TWO) {
-        const float4 sum = search_flux2<DIM>(uint32_t(s), stride, pos, rec, cell, start, v, ex, exb,
-                                             f.rs, f.ms, g.ms, f.two_beta);
+    } else {
+        const float4 sum = search_flux<DIM, TWO>(uint32_t(s), stride, pos, rec, cell, start, v, ex, exb);
         f.acc = sum.x;
         f.comp = sum.y;
         g.acc = sum.z;
         g.comp = sum.w;
-    } else {
-        const float2 sum = search_flux<DIM>(uint32_t(s), stride, pos, rec, cell, start, v, ex,
-                                            f.rs, f.ms, f.two_beta);
-        f.acc = sum.x;
-        f.comp = sum.y;
     }
     if constexpr (TWO) {
         // both species' transfer, then the reaction on this particle
@@ -2351,11 +2389,12 @@ __device__ __noinline__ double2 adj_search_rowsum(uint32_t s, int64_t stride,
                                                   const double* table, const View& v) {
     const RealParams& P = v.of_sorted(s);
     AdjRowSum sum;
-    visit_neighbours<DIM>(s, cell_arg<DIM>(cell, s), stride, rec, pos, start, P,
-                          [&](uint32_t j, float, const float4&) {
-                              if (j != s)
-                                  sum.add(pair_terms<DIM>(image, tan, stride, s, j, P, table));
-                          });
+    each_pair<DIM>(s, cell, stride, pos, rec, start, P, [&](uint32_t j0, uint32_t j1, bool) {
+        for (uint32_t j = j0;; j = j1) {
+            sum.add(pair_terms<DIM>(image, tan, stride, s, j, P, table));
+            if (j == j1) break;
+        }
+    });
     return sum.value();
 }
 
@@ -2417,13 +2456,13 @@ __device__ __noinline__ double2 adj_search_flux(uint32_t s, int64_t stride,
     const double* mine = rec4 + 4 * size_t(s);
     const AdjRec me{mine[0], mine[1], mine[2], mine[3]};
     AdjFluxSum sum;
-    visit_neighbours<DIM>(s, cell_arg<DIM>(cell, s), stride, rec, pos, start, P,
-                          [&](uint32_t j, float, const float4&) {
-                              if (j == s) return;
-                              const double* q = rec4 + 4 * size_t(j);
-                              sum.add(adj_flux(pair_terms<DIM>(image, tan, stride, s, j, P, table), me,
-                                               AdjRec{q[0], q[1], q[2], q[3]}));
-                          });
+    each_pair<DIM>(s, cell, stride, pos, rec, start, P, [&](uint32_t j0, uint32_t j1, bool) {
+        for (uint32_t j = j0;; j = j1) {
+            sum.add(adj_flux(pair_terms<DIM>(image, tan, stride, s, j, P, table), me,
+                             load_adj_rec(rec4, j)));
+            if (j == j1) break;
+        }
+    });
     return sum.value();
 }
 
