@@ -67,16 +67,19 @@ constexpr int kScanTile = kScanPerThread * kScanThreads;  // cells per scan bloc
 
 // The kernels of a time step are launched with programmatic stream
 // serialisation (`launch` in mtpt.cu): a kernel may be set up, and its blocks
-// may start, while the kernel before it on the stream still runs.  So each of
-// them first lets the next one start, then waits until the one before is
-// complete and its writes are visible, and only then touches memory.  That
-// takes the set-up of each launch out of the chain: one step of 1e4 particles and
-// its two reads 55.7 -> 39.0 us (eight kernels), the adjoint's 200 steps of 250,000
-// 44.5 -> 38.5 ms.
-// (For kernels that only update a word in place: what is read through a pointer
-// to const takes its index from ordered_index.)
+// may start, once the blocks of the kernel before it on the stream have ended,
+// before that kernel is complete.  So each of them first waits until the one
+// before is complete and its writes are visible, and only then touches memory.
+// That takes the set-up of each launch out of the chain: one step of 1e4 particles
+// and its two reads 55.7 -> 38 us (eight kernels), the adjoint's 200 steps of 250,000
+// 44.5 -> 38.8 ms.
+// (No griddepcontrol.launch_dependents: with the next kernel's blocks resident
+// from the start of this one, a grid of two to six blocks an SM spread unevenly over
+// the SMs: 36.7 instead of 30.7 us a step at 1e5 particles in 2-d, 49.4 instead of 39.9 in
+// 3-d, precision form; the same within 1 % below 2e4 and above 4e5.)
+// (after_previous itself is for kernels that only update a word in place: what is
+// read through a pointer to const takes its index from ordered_index.)
 __device__ __forceinline__ void after_previous() {
-    asm volatile("griddepcontrol.launch_dependents;");
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 // The thread's global index, after after_previous(): passing through the asm, it
@@ -84,7 +87,6 @@ __device__ __forceinline__ void after_previous() {
 // own too) behind the wait.
 __device__ __forceinline__ uint32_t ordered_index() {
     uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    asm volatile("griddepcontrol.launch_dependents;");
     asm volatile("griddepcontrol.wait;\n\tmov.b32 %0, %0;" : "+r"(i)::"memory");
     return i;
 }

@@ -67,3 +67,9 @@ def test_read_only_loads_are_of_constants():
     for params in re.findall(r"__device__[^;{]*?\(([^;{]*)\)\s*\{", src):
         names = set(re.findall(r"\bconst\b[^,]*\*\s*__restrict__\s+(\w+)", params))
         assert names <= CONSTANTS | {"table"}, names      # (table: in shared memory)
+
+
+def test_no_kernel_lets_the_next_one_start_early():
+    """Blocks that wait on the SMs while a kernel of a few blocks an SM still starts
+    spread unevenly: the next kernel may start when this one's blocks have ended."""
+    assert "launch_dependents" not in _source("kernels.cuh")
