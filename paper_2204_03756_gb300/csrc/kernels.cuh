@@ -1218,7 +1218,8 @@ __device__ __forceinline__ uint32_t mask_word(uint32_t words, uint32_t neighbour
 // cutoff, and, with EXACT, those inside it that the exact test accepts.  EACH
 // calls cand(j, d2, accept, accept1) for every two candidates j and j + 1 (d2 their
 // binary32 distances squared), the self pair included.
-// Without EXACT returns whether any candidate was inside the band.
+// Without EXACT returns whether any candidate was inside the band.  A search for
+// words alone ends when the sink is full.
 //
 // Bound by instruction issue: singly, a candidate took about 20 instructions
 // of which the pair shares or packs all but three.  The bisection to a
@@ -1255,7 +1256,9 @@ __device__ __forceinline__ bool search_rows(uint32_t s, uint32_t cell, const flo
                              (DIM < 3 || (c[2] + dz >= 0 && c[2] + dz < g.n[2]));
         uint32_t j = 0, j3 = 0;
         float rx = 0.0f;
-        if (in_grid && r2 >= 0.0f) {
+        bool wanted = in_grid && r2 >= 0.0f;
+        if constexpr (WORDS && !EACH) wanted = wanted && !sink.full();
+        if (wanted) {
             rx = __fadd_rn(sqrt_approx(r2), eps);
             const uint32_t rowc = P.cell_base + (uint32_t(c[2] + dz) * uint32_t(g.n[1]) +
                                                  uint32_t(c[1] + dy)) * uint32_t(g.n[0]);
@@ -1343,6 +1346,7 @@ __device__ __forceinline__ bool search_rows(uint32_t s, uint32_t cell, const flo
                 }
                 if (s - base < 32u) bits &= ~(1u << (s - base));   // the self pair is no neighbour
                 if (bits) sink.word(base, bits);
+                if constexpr (WORDS && !EACH) more = more && !sink.full();
                 if (!more) break;
             }
         }
@@ -1384,6 +1388,7 @@ struct PlaneSink {
     __device__ __forceinline__ void end_row() {
         while (nw < padded) put(make_uint2(0u, 0u));
     }
+    __device__ __forceinline__ bool full() const { return nw > cap; }
 };
 // ... none ...
 struct NoSink {};
@@ -1406,6 +1411,7 @@ struct PairSink {
         }
     }
     __device__ __forceinline__ void end_row() {}
+    __device__ __forceinline__ bool full() const { return false; }
 };
 // Every neighbour of s, two at a time, in the order of its mask words, for a
 // particle whose words are not kept, in binary64: returns their number.  The search
@@ -1591,7 +1597,7 @@ __device__ __forceinline__ void dense_words(uint32_t s, uint32_t listed, int64_t
 }
 
 // Search of one particle of a binary64 pass: its list word, neighbour count in cnt
-// (kMaskOver at once when nothing can be kept: the caller's search counts).
+// (kMaskOver as soon as its words do not fit: the caller's search counts).
 template <int DIM, class View>
 __device__ __forceinline__ uint32_t search_listed(uint32_t s, int64_t stride,
                                                   const double* pos,
@@ -1606,6 +1612,7 @@ __device__ __forceinline__ uint32_t search_listed(uint32_t s, int64_t stride,
     const bool band = search_rows<DIM, true, false, false>(s, cell_arg<DIM>(cell, s), load_rec(rec, s),
                                                            stride, pos, rec, start, P,
                                                            [](uint32_t, float2, bool, bool) {}, sink);
+    if (sink.full()) return kMaskOver;
     uint32_t nw = sink.nw;
     cnt = sink.cnt;
     if (band) {
