@@ -2183,8 +2183,8 @@ __device__ __noinline__ float4 search_flux(uint32_t s, int64_t stride, const dou
 // us at 32 and 40 for the reaction at 1e6), a batch's view 36 (1.23, 1.15 and 1.19
 // ms at 32, 36 and 40 for the 512-member ensemble).
 // The bounds hold for blocks of 128 too (the tuning's other block size).
-// LONG: for runs with long windows (padded words), whose particles all go word
-// by word, inline and with 32-byte loads (1.59 -> 1.39 ms at 1e7 particles with
+// LONG: for runs with long windows (padded words) or half-width cells, whose
+// particles all go word by word, inline and with 32-byte loads (1.59 -> 1.39 ms at 1e7 particles with
 // 57 neighbours, the next walk included).
 template <int DIM, class View, bool TWO = false, int WALK = 0, bool LONG = false>
 __global__ void __launch_bounds__(kBlock, (TWO ? 1536 : (View::kBatch || LONG ? 1792 : 2048)) / kBlock)
