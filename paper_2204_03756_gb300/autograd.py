@@ -17,6 +17,26 @@ import torch
 from . import mtpt
 
 
+class _Recorded:
+    """A recorded run's handle, released by close() or with the last reference: a
+    run that is never differentiated (under no_grad, or whose graph is dropped)
+    holds no device memory after its context."""
+
+    def __init__(self, h):
+        self.h = h
+
+    def close(self):
+        h, self.h = self.h, None
+        if h is not None:
+            mtpt.mtpt_destroy(h)
+
+    def __del__(self):
+        try:
+            self.close()
+        except Exception:
+            pass
+
+
 class _Run(torch.autograd.Function):
     @staticmethod
     def forward(ctx, mass0, D, params, pos0, nsteps, checkpoint_every):
@@ -35,7 +55,7 @@ class _Run(torch.autograd.Function):
         except Exception:
             mtpt.mtpt_destroy(h)
             raise
-        ctx.h = h
+        ctx.recorded = _Recorded(h)
         ctx.D_dtype = D.dtype
         ctx.D_device = D.device
         ctx.mark_non_differentiable(posT)
@@ -43,15 +63,14 @@ class _Run(torch.autograd.Function):
 
     @staticmethod
     def backward(ctx, g_massT, g_posT):
-        h = ctx.h
+        h = ctx.recorded.h
         try:
             g = g_massT.contiguous().to(torch.float64)
             g0 = torch.empty_like(g)
             torch.cuda.current_stream().synchronize()
             dldD = mtpt.mtpt_adjoint_backward(h, g, g0)
         finally:
-            mtpt.mtpt_destroy(h)
-            ctx.h = None
+            ctx.recorded.close()
         gD = torch.tensor(dldD, dtype=ctx.D_dtype, device=ctx.D_device)
         return g0, gD, None, None, None, None
 

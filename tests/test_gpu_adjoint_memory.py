@@ -90,3 +90,35 @@ def test_gradients_do_not_depend_on_free_memory(form, clump, dim, n, L):
         assert np.array_equal(taped[1], plain[1])
         # a segment that the tape cannot hold is taken again, its pairs counted once
         assert taped[2]["pair_count"] == plain[2]["pair_count"]
+
+
+def test_a_run_that_is_not_differentiated_holds_no_memory():
+    """Under no_grad, and with a graph that is dropped before its backward."""
+    import gc
+
+    import torch
+    from paper_2204_03756_gb300 import autograd
+    n, L = 20000, 141.0
+    rng = np.random.default_rng(2)
+    p = mtpt.Params(dim=2, D=0.5, kappa=0.5, dt=0.1, lo=(0.0, 0.0), hi=(L, L), seed=4)
+    pos = torch.from_numpy(rng.uniform(0.0, L, size=(2, n))).cuda()
+    mass = torch.from_numpy(rng.uniform(0.0, 1.0, n)).cuda().requires_grad_()
+    D = torch.tensor(0.5, requires_grad=True)
+
+    def run(grad):
+        with torch.set_grad_enabled(grad):
+            m, _ = autograd.mtpt_run(mass, D, p, pos, 30, 30)
+        del m
+        gc.collect()
+
+    run(False)
+    level = _free()
+    for grad in (False, True) * 3:          # 32 snapshots of 0.9 MB each
+        run(grad)
+        assert _free() >= level - 4 * MB
+    # and a differentiated one
+    m, _ = autograd.mtpt_run(mass, D, p, pos, 30, 30)
+    m.sum().backward()
+    del m
+    gc.collect()
+    assert _free() >= level - 4 * MB
