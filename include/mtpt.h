@@ -565,14 +565,15 @@ int mtpt_get_ids(mtpt_handle* h, uint32_t* out);
 /* Failure injection for tests (no counterpart in the paper): from this call
  * on, the nth device allocation that the library attempts (in this process,
  * on any handle) fails as if the device were out of memory; nth < 0: the same of
- * the -nth-th allocation among those that the library can do without (the
- * adjoint sweep's tape), which the other form does not count; nth = 0 turns the
- * injection off.  *remaining (may be NULL) receives how many allocations the
- * previous setting still had to go (0: it fired or was off).  A call that
- * meets a failure of the first kind returns MTPT_ERR_NO_MEMORY: loads, retuning and the
- * autotuner leave the handle's particles, counters and tuning as they were;
- * the adjoint's recording allocates before it steps; time steps allocate
- * nothing. */
+ * the -nth-th allocation among those that the library can do without (what the
+ * first pair pass keeps for the second, the adjoint sweep's tape), which the
+ * other form does not count; nth = 0 turns the injection off.  *remaining (may be
+ * NULL) receives how many allocations the previous setting still had to go (0: it
+ * fired or was off).  A call that meets a failure of the first kind returns
+ * MTPT_ERR_NO_MEMORY: loads, retuning and the autotuner leave the handle's
+ * particles, counters and tuning as they were; the adjoint's recording allocates
+ * before it steps; time steps allocate nothing.  One that meets a failure of the
+ * second kind gives the same results, more slowly. */
 int mtpt_debug_fail_alloc(int64_t nth, int64_t* remaining);
 
 /* Wait-limit test hook (no counterpart in the paper).  The cell-count scan of

@@ -91,7 +91,9 @@ int device_alloc(void** out, size_t bytes, bool optional = false) {
 }
 
 // A device buffer that only grows.  A growth allocates before it releases,
-// so a failed one leaves the old buffer (and its contents) in place.
+// so a failed one leaves the old buffer (and its contents) in place; one that the
+// library can do without (ensure_optional) releases first, and is empty when there
+// is no memory for it.
 template <typename T>
 struct DevBuf {
     T* p = nullptr;
@@ -104,6 +106,11 @@ struct DevBuf {
         p = static_cast<T*>(q);
         count = n;
         return MTPT_OK;
+    }
+    void ensure_optional(size_t n) {
+        if (n <= count && p) return;
+        release();
+        (void)ensure(n, true);
     }
     void release() {
         if (p) cudaFree(p);
@@ -770,7 +777,9 @@ int launch_scan(mtpt_handle* h, cudaStream_t st, bool advance) {
     return MTPT_OK;
 }
 
-// The cell list's arrays for the current grid, grown all or nothing.
+// The cell list's arrays for the current grid, grown all or nothing, and what pass 1
+// keeps for pass 2 where there is room: without it the passes search again, for the
+// same sums.
 int ensure_cells(mtpt_handle* h) {
     const size_t padded = size_t(h->n_cells_pad);
     GrowAll g;
@@ -778,13 +787,15 @@ int ensure_cells(mtpt_handle* h) {
     g.want(h->start, padded);
     g.want(h->scan_state, padded / kScanTile + 1);   // + the scan's ticket
     g.want(h->corners, size_t(std::max(h->n_corners, 1)));
-    g.want(h->nb_e, size_t(h->nb_cap) * size_t(h->cap));
-    if (h->nb_kcap > 0) {
-        g.want(h->nb_listed, size_t(h->cap));
-        g.want(h->nb_k, size_t(h->nb_kcap) * size_t(h->cap));
-    }
     if (g.grows()) drop_graph(h);
     MTPT_TRY(g.commit());
+    const void *e0 = h->nb_e.p, *listed0 = h->nb_listed.p, *k0 = h->nb_k.p;
+    h->nb_e.ensure_optional(size_t(h->nb_cap) * size_t(h->cap));
+    if (h->nb_kcap > 0) {
+        h->nb_listed.ensure_optional(size_t(h->cap));
+        h->nb_k.ensure_optional(size_t(h->nb_kcap) * size_t(h->cap));
+    }
+    if (h->nb_e.p != e0 || h->nb_listed.p != listed0 || h->nb_k.p != k0) drop_graph(h);
     // the scan's words for this grid's tiles
     MTPT_TRY(reset_scan(h, h->stream));
     // counts start (and, after each scatter, end) at zero
@@ -1807,9 +1818,9 @@ size_t tape_step_bytes(const mtpt_handle* h) {
 }
 int ensure_adjoint_rows(mtpt_handle* h) {
     const size_t cap = size_t(std::max<int64_t>(h->cap, 1));
-    MTPT_TRY(h->adj_nb_e.ensure(size_t(h->adj_cap) * cap));
-    MTPT_TRY(h->adj_nb_listed.ensure(cap));
-    return h->adj_nb_k.ensure(adj_values(h));
+    h->adj_nb_e.ensure_optional(size_t(h->adj_cap) * cap);
+    h->adj_nb_k.ensure_optional(adj_values(h));
+    return h->adj_nb_listed.ensure(cap);
 }
 TapeSlot tape_slot(const mtpt_handle* h, int64_t k) {
     const size_t cap = size_t(h->cap);
@@ -1865,8 +1876,8 @@ int launch_adjoint_rows(mtpt_handle* h, int o, const double* mass, const TapeSlo
     const TapeOut out = taped ? TapeOut{mass, h->id[o].p, t.mass, t.id, h->tape_flag.p} : TapeOut{};
     launch(k_adj_rowsum<DIM, SingleView>, grid_for(h->n), kBlock, h->stream,
         int(h->n), h->cap, h->pos[o].p, h->image.p, h->tan[o].p, h->rec.p, h->cell.p, h->start.p,
-        h->exp_table.p, v, t.r, t.dr, NbPlanes{t.words, h->adj_cap, 0}, t.listed,
-        AdjValues{t.kd, h->adj_kcap}, out);
+        h->exp_table.p, v, t.r, t.dr, NbPlanes{t.words, t.words ? h->adj_cap : 0, 0}, t.listed,
+        AdjValues{t.kd, t.kd ? h->adj_kcap : 0}, out);
     MTPT_CUDA_TRY(cudaGetLastError());
     return MTPT_OK;
 }
@@ -1883,7 +1894,8 @@ int launch_adjoint_pass(mtpt_handle* h, int o, const TapeSlot& t, double* gD_blo
     launch(k_adj_exchange<DIM, SingleView>, blocks, kBlock, st,
         n, h->cap, h->pos[o].p, h->image.p, h->tan[o].p, h->rec.p, h->cell.p, h->start.p,
         h->exp_table.p, v, h->adj_rec.p, t.id, h->lam_in.p, gD_block,
-        NbPlanes{t.words, h->adj_cap, 0}, t.listed, AdjValues{t.kd, h->adj_kcap});
+        NbPlanes{t.words, t.words ? h->adj_cap : 0, 0}, t.listed,
+        AdjValues{t.kd, t.kd ? h->adj_kcap : 0});
     MTPT_CUDA_TRY(cudaGetLastError());
     return MTPT_OK;
 }
