@@ -1539,6 +1539,28 @@ struct AdjValues {
     }
 };
 
+// Neighbour indexes out of kept words and lists.  The checked build takes the
+// particle itself, whose flux is zero, in place of an index that an empty word or
+// one beyond the particles would give.
+struct KeptIndex {
+#ifdef MTPT_CHECKED
+    uint32_t n, self;
+    __device__ __forceinline__ KeptIndex(uint32_t particles, uint32_t s) : n(particles), self(s) {}
+    __device__ __forceinline__ uint32_t of_list(uint32_t j) const {
+        return check(j < n, kChkSegment) ? j : self;
+    }
+    __device__ __forceinline__ uint32_t of_word(uint32_t base, uint32_t bits) const {
+        return check(bits != 0u, kChkSegment) ? of_list(base + uint32_t(__ffs(int(bits)) - 1)) : self;
+    }
+#else
+    __device__ __forceinline__ KeptIndex(uint32_t, uint32_t) {}
+    __device__ __forceinline__ uint32_t of_list(uint32_t j) const { return j; }
+    __device__ __forceinline__ uint32_t of_word(uint32_t base, uint32_t bits) const {
+        return base + uint32_t(__ffs(int(bits)) - 1);
+    }
+#endif
+};
+
 // A particle's neighbours from its mask words (without padding), in order; the
 // word after the current one is loaded ahead.
 struct WordStream {
@@ -1546,9 +1568,11 @@ struct WordStream {
     int64_t stride;
     uint32_t left;               // words after `ahead`
     uint2 cur, ahead;
-    __device__ __forceinline__ WordStream(const uint2* first, int64_t st, uint32_t words)
+    KeptIndex index;
+    __device__ __forceinline__ WordStream(const uint2* first, int64_t st, uint32_t words,
+                                          const KeptIndex& kept)
         : e(first), stride(st), left(words > 0u ? words - 1u : 0u), cur(make_uint2(0u, 0u)),
-          ahead(words > 0u ? *first : make_uint2(0u, 0u)) {}
+          ahead(words > 0u ? *first : make_uint2(0u, 0u)), index(kept) {}
     __device__ __forceinline__ uint32_t next() {
         if (cur.y == 0u) {
             cur = ahead;
@@ -1557,8 +1581,7 @@ struct WordStream {
                 --left;
             }
         }
-        check(cur.y != 0u, kChkSegment);
-        const uint32_t j = cur.x + uint32_t(__ffs(int(cur.y)) - 1);
+        const uint32_t j = index.of_word(cur.x, cur.y);
         cur.y &= cur.y - 1u;
         return j;
     }
@@ -1570,7 +1593,7 @@ struct WordStream {
 // term of the warp's neighbour e, add(term) is called by each lane for its
 // own, in order; begin(total) comes first.
 template <class V, class Begin, class Eval, class Add>
-__device__ __forceinline__ void dense_words(uint32_t s, uint32_t listed, int64_t stride,
+__device__ __forceinline__ void dense_words(uint32_t s, uint32_t n, uint32_t listed, int64_t stride,
                                             const uint2* e, ChunkShared<V>& S, Begin&& begin,
                                             Eval&& eval, Add&& add) {
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, warp_s0 = s - lane;
@@ -1579,7 +1602,7 @@ __device__ __forceinline__ void dense_words(uint32_t s, uint32_t listed, int64_t
     uint32_t total;
     const uint32_t off = warp_exclusive_scan(cnt, &total), end = off + cnt;
     begin(total);
-    WordStream stream(e + s, stride, words);
+    WordStream stream(e + s, stride, words, KeptIndex{n, s});
     uint32_t pos = off;
     for (uint32_t c0 = 0; c0 < total; c0 += kChunk) {
         const uint32_t m = min(total - c0, uint32_t(kChunk)), stop = min(end, c0 + m);
@@ -1685,7 +1708,7 @@ k_rowsum_f64(int n, int64_t stride, const double* pos,
 #pragma unroll
                 for (int a = 0; a < DIM; ++a) xs[a] = image[a * stride + s];
                 RowSum sum;
-                WordStream stream(nb.e + s, stride, listed & 255u);
+                WordStream stream(nb.e + s, stride, listed & 255u, KeptIndex{uint32_t(n), s});
                 auto kernel = [&](uint32_t j) {
                     uint64_t d2h = 0;
 #pragma unroll
@@ -1820,7 +1843,7 @@ k_exchange_f64(int n, int64_t stride, const double* pos,
             const uint32_t kept = kv.cap > 0 ? min(cnt, uint32_t(kv.cap - 1) & ~1u) : 0u;
             const uint32_t listed_k = cnt < uint32_t(kv.cap) ? cnt : kept;
             FluxSum64 sum;
-            WordStream stream(nb.e + s, stride, listed & 255u);
+            WordStream stream(nb.e + s, stride, listed & 255u, KeptIndex{uint32_t(n), s});
             const double* keep = kv.v + s;
             uint32_t k = 0;
             for (; k + 2 <= listed_k; k += 2, keep += 2 * stride) {
@@ -2071,6 +2094,7 @@ struct PairFlux {
     const float2* exb;
     float4 me;
     float na, wx, wy;
+    KeptIndex index;
     __device__ __forceinline__ float kernel(const float4& o) const {
         const float sy = DIM == 2 ? __fmul_rn(__fsub_rn(o.z, me.z), wy) : 0.0f;
         return ex2_approx(na * d2_f32<DIM>(dx_f32(me, o, wx), me, o, sy, 0.0f));
@@ -2107,10 +2131,10 @@ __device__ __forceinline__ void add_words(const uint2* e, int64_t stride, uint32
         uint32_t bits = ahead.y;
         if (w < words) ahead = ld_global(e += stride);
         while (bits) {
-            const uint32_t j0 = base + uint32_t(__ffs(int(bits)) - 1);
+            const uint32_t j0 = pf.index.of_word(base, bits);
             bits &= bits - 1u;
             const bool two = bits != 0u;
-            const uint32_t j1 = two ? base + uint32_t(__ffs(int(bits)) - 1) : j0;
+            const uint32_t j1 = two ? pf.index.of_word(base, bits) : j0;
             bits &= bits - 1u;
             pf.add(f, g, j0, j1, two);
         }
@@ -2125,8 +2149,8 @@ __device__ __noinline__ float4 words_flux(const uint2* e, int64_t stride,
                                           uint32_t words, const float4* ex,
                                           const float2* exb, float4 me, float na,
                                           float wx, float wy, float rs, float two_beta, float2 ms,
-                                          float2 msb) {
-    const PairFlux<DIM, TWO, false> pf{ex, exb, me, na, wx, wy};
+                                          float2 msb, KeptIndex index) {
+    const PairFlux<DIM, TWO, false> pf{ex, exb, me, na, wx, wy, index};
     FluxSum f{rs, two_beta, ms}, g{rs, two_beta, msb};
     add_words<DIM, TWO>(e, stride, words, pf, f, g);
     return make_float4(f.acc, f.comp, g.acc, g.comp);
@@ -2215,9 +2239,10 @@ k_exchange_f32(int n, int64_t stride, const double* pos, const float* rec,
     FluxSum g{xs.z, f.two_beta, TWO ? ld_global(exb + s) : make_float2(0.0f, 0.0f)};
     const uint32_t listed = __float_as_uint(xs.w);   // see NbPlanes
     if (nb.cap > 0 && (DIM == 3 ? listed <= uint32_t(nb.cap) : listed != kMaskOver)) {
+        const KeptIndex index{uint32_t(n), uint32_t(s)};
         if constexpr (DIM < 3) {
             const PairFlux<DIM, TWO, true> pf{ex, exb, ld_global(ex + 2 * size_t(s)), -P.pp.a_log2e,
-                                              P.g.wf[0], P.g.wf[1]};
+                                              P.g.wf[0], P.g.wf[1], index};
             const uint2* e = nb.e + s;
             const uint32_t words = listed & 255u;
             if constexpr (LONG) {
@@ -2235,7 +2260,7 @@ k_exchange_f32(int n, int64_t stride, const double* pos, const float* rec,
                     const bool shift = w0.y == 0u;
                     w0 = shift ? w1 : w0;
                     w1 = shift ? w2 : w1;
-                    const uint32_t j = w0.x + uint32_t(__ffs(int(w0.y)) - 1);
+                    const uint32_t j = index.of_word(w0.x, w0.y);
                     w0.y &= w0.y - 1u;
                     return j;
                 };
@@ -2250,7 +2275,7 @@ k_exchange_f32(int n, int64_t stride, const double* pos, const float* rec,
                 }
             } else {
                 const float4 sum = words_flux<DIM, TWO>(e, stride, words, ex, exb, pf.me, pf.na, pf.wx,
-                                                        pf.wy, f.rs, f.two_beta, f.ms, g.ms);
+                                                        pf.wy, f.rs, f.two_beta, f.ms, g.ms, index);
                 f.acc = sum.x;
                 f.comp = sum.y;
                 g.acc = sum.z;
@@ -2259,9 +2284,13 @@ k_exchange_f32(int n, int64_t stride, const double* pos, const float* rec,
         } else {
             const uint2* e = nb.e + s;
             uint32_t k = 0;
+            auto entry = [&](const uint2* p) {
+                const uint2 q = ld_global(p);
+                return make_uint2(index.of_list(q.x), q.y);
+            };
             if constexpr (TWO) {
                 for (; k + 2 <= listed; k += 2, e += 2 * stride) {
-                    const uint2 q0 = ld_global(e), q1 = ld_global(e + stride);
+                    const uint2 q0 = entry(e), q1 = entry(e + stride);
                     const float4 x0 = ld_global(ex + q0.x), x1 = ld_global(ex + q1.x);
                     const float2 b0 = ld_global(exb + q0.x), b1 = ld_global(exb + q1.x);
                     const float w0 = f.weight(x0, __uint_as_float(q0.y));
@@ -2272,7 +2301,7 @@ k_exchange_f32(int n, int64_t stride, const double* pos, const float* rec,
                     g.add_w(b1, w1);
                 }
                 if (k < listed) {
-                    const uint2 q = ld_global(e);
+                    const uint2 q = entry(e);
                     const float4 x = ld_global(ex + q.x);
                     const float w = f.weight(x, __uint_as_float(q.y));
                     f.add_w(make_float2(x.x, x.y), w);
@@ -2281,13 +2310,13 @@ k_exchange_f32(int n, int64_t stride, const double* pos, const float* rec,
             } else {
                 // two entries per iteration, the next two list entries loaded
                 // while this pair's neighbour records are in flight
-                uint2 p0 = listed > 0u ? ld_global(e) : make_uint2(uint32_t(s), 0u);
-                uint2 p1 = listed > 1u ? ld_global(e + stride) : p0;
+                uint2 p0 = listed > 0u ? entry(e) : make_uint2(uint32_t(s), 0u);
+                uint2 p1 = listed > 1u ? entry(e + stride) : p0;
                 for (; k + 2 <= listed; k += 2, e += 2 * stride) {
                     const uint2 q0 = p0, q1 = p1;
                     const float4 x0 = ld_global(ex + q0.x), x1 = ld_global(ex + q1.x);
-                    p0 = k + 2 < listed ? ld_global(e + 2 * stride) : q0;
-                    p1 = k + 3 < listed ? ld_global(e + 3 * stride) : q1;
+                    p0 = k + 2 < listed ? entry(e + 2 * stride) : q0;
+                    p1 = k + 3 < listed ? entry(e + 3 * stride) : q1;
                     f.add(x0, __uint_as_float(q0.y));
                     f.add(x1, __uint_as_float(q1.y));
                 }
@@ -2509,7 +2538,7 @@ k_adj_rowsum(int n, int64_t stride, const double* pos,
     AdjRowSum rows;
     double2* keep = nullptr;
     dense_words(
-        s, listed, stride, nb.e, chunk,
+        s, uint32_t(n), listed, stride, nb.e, chunk,
         [&](uint32_t total) { keep = kv.of_warp(s - (threadIdx.x & 31u), total); },
         [&](uint32_t e, uint32_t so, uint32_t j) {
             const double2 kd = pair_terms<DIM>(image, tan, stride, so, j, v.of_sorted(so), table);
@@ -2563,7 +2592,7 @@ k_adj_exchange(int n, int64_t stride, const double* pos,
     double g = 0.0;
     const double2* keep = nullptr;
     dense_words(
-        s, listed, stride, nb.e, chunk,
+        s, uint32_t(n), listed, stride, nb.e, chunk,
         [&](uint32_t total) { keep = kv.of_warp(s - (threadIdx.x & 31u), total); },
         [&](uint32_t e, uint32_t so, uint32_t j) {
             const AdjRec me = load_adj_rec(rec4, so), o = load_adj_rec(rec4, j);
