@@ -195,13 +195,19 @@ MTPT_HD FixedWeight weight_fixed(double K, double ra, double rb) {
     return Reciprocal(ra, rb).weight(K);
 }
 
-// A particle's flux sum, sum W dm over its neighbours with dm a difference of
-// masses, or the sum of plain binary64 terms: 64-bit integers against the
-// largest exponent so far (each term keeps 54 bits or more, and the sum five
-// bits above the terms, or more when it needs them).  A term changes sign
-// exactly when dm does.  Terms that are not finite make the sum what binary64
-// additions would.
-struct FluxSum64 {
+// A sum of terms W dm over a particle's neighbours, dm a difference of masses, or of
+// plain binary64 terms: 64-bit integers in units of 2^x, with x from the term of the
+// largest exponent so far, raised when the sum grows past 61 bits.  A unit is at most
+// 2^-54 of the largest term or 2^-57 of the largest partial sum so far, and every
+// term and every change of unit costs less than one (a binary64 addition: 2^-53 of
+// the partial sum).  Terms are cut toward zero.  TOWARD_ZERO cuts the sum so too at a
+// change of unit, and it changes sign exactly when every dm does: what particles
+// give and take is cut alike, and the total mass stays as with binary64 sums (cut
+// downwards it drifted by 1e-19 of itself a step).  That takes 1.5 % of a run's time
+// and 3 % of the adjoint sweep's, whose sums are cut downwards.  Terms that are not
+// finite make the sum what binary64 additions would.
+template <bool TOWARD_ZERO>
+struct IntegerSum {
     int64_t acc = 0;
     int x = -100000;             // the sum is acc 2^x
     double special = 0.0;
@@ -215,35 +221,27 @@ struct FluxSum64 {
         }
         const uint64_t m = (b & 0xfffffffffffffull) | (e ? 0x10000000000000ull : 0u);
         // dm = m 2^(e - 1075), subnormals with e = 1; the term is g 2^y, g < 2^58
-        int64_t g = int64_t(w ? mul_hi(m << 10, w->q) >> 3 : m << 5);
+        uint64_t g = w ? mul_hi(m << 10, w->q) >> 3 : m << 5;
         const int y = (e ? e : 1) - 1075 + (w ? -10 + 64 + 3 + w->x : -5);
-        g = (b >> 63) ? -g : g;
         const int up = y - x;
         if (up > 0) {
-            acc >>= up < 63 ? up : 63;
+            cut(up < 63 ? up : 63);
             x = y;
         } else {
             g >>= up > -63 ? -up : 63;
         }
-        acc += g;
-        if (uint64_t(acc + (1ll << 61)) >> 62) {                        // |acc| >= 2^61
-            acc >>= 4;
+        acc += (b >> 63) ? -int64_t(g) : int64_t(g);
+        if (uint64_t(acc + ((1ll << 61) - 1)) > (1ull << 62) - 2u) {    // |acc| >= 2^61
+            cut(4);
             x += 4;
         }
     }
-    MTPT_HD void add(double dm, const FixedWeight& w) { add(dm, &w); }
-    // a product of two binary64 values, the first one normal or zero
-    MTPT_HD void add_product(double a, double b) {
-        const uint64_t ab = bits_of(a);
-        const int e = int(ab >> 52) & 0x7ff;
-        if (e == 0x7ff) {
-            special += a * b;
-            return;
-        }
-        const FixedWeight w{e ? ((ab & 0xfffffffffffffull) | 0x10000000000000ull) << 9 : 0u,
-                            e - 1075 - 9};
-        add((ab >> 63) ? -b : b, &w);
+    // acc / 2^k, 0 < k < 64
+    MTPT_HD void cut(int k) {
+        if (TOWARD_ZERO) acc += int64_t(uint64_t(acc >> 63) >> (64 - k));
+        acc >>= k;
     }
+    MTPT_HD void add(double dm, const FixedWeight& w) { add(dm, &w); }
     MTPT_HD void add(double term) { add(term, nullptr); }
     MTPT_HD double value() const {
         if (!(special == 0.0)) return special;
@@ -255,6 +253,9 @@ struct FluxSum64 {
         return acc < 0 ? -v : v;
     }
 };
+
+using FluxSum64 = IntegerSum<true>;      // a particle's flux
+using AdjSum64 = IntegerSum<false>;      // the adjoint's sums
 
 // Row sum 1 + sum K in units of 2^-62, exact in 96 bits.
 struct RowSum {

@@ -2408,7 +2408,7 @@ __device__ __forceinline__ double2 pair_terms(const uint64_t* image,
 // The sums of pass A: the row sum exactly, its derivative in 64-bit integers.
 struct AdjRowSum {
     RowSum r;
-    FluxSum64 dr;
+    AdjSum64 dr;
     __device__ __forceinline__ void add(double2 kd) {
         r.add(unit_of(kd.x));
         dr.add(kd.y);
@@ -2470,7 +2470,7 @@ __device__ __forceinline__ double2 adj_flux(double2 kd, const AdjRec& me, const 
                         __dmul_rn(dh, __dsub_rn(o.mass, me.mass)));
 }
 struct AdjFluxSum {
-    FluxSum64 lam, gD;
+    AdjSum64 lam, gD;
     __device__ __forceinline__ void add(double2 t) {
         lam.add(t.x);
         gD.add(t.y);

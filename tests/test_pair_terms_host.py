@@ -28,10 +28,19 @@ double weight(double K, double ra, double rb) {
     const FixedWeight w = weight_fixed(K, ra, rb);
     return std::ldexp(double(w.q), w.x);
 }
-double flux_sum(int n, const double* dm, const double* K, const double* ra, const double* rb) {
-    FluxSum64 f;
+}
+template <class Sum>
+double sum_of(int n, const double* dm, const double* K, const double* ra, const double* rb) {
+    Sum f;
     for (int k = 0; k < n; ++k) f.add(dm[k], weight_fixed(K[k], ra[k], rb[k]));
     return f.value();
+}
+extern "C" {
+double flux_sum(int n, const double* dm, const double* K, const double* ra, const double* rb) {
+    return sum_of<FluxSum64>(n, dm, K, ra, rb);
+}
+double adj_sum(int n, const double* dm, const double* K, const double* ra, const double* rb) {
+    return sum_of<AdjSum64>(n, dm, K, ra, rb);
 }
 double row_sum(int n, const double* K) {
     RowSum r;
@@ -54,8 +63,8 @@ def lib(tmp_path_factory):
     so.kernel.argtypes = [ctypes.c_int, dp, dp, ctypes.c_double, ctypes.c_double]
     so.weight.argtypes = [ctypes.c_double] * 3
     so.row_sum.argtypes = [ctypes.c_int, dp]
-    so.flux_sum.argtypes = [ctypes.c_int, dp, dp, dp, dp]
-    for f in (so.kernel, so.weight, so.row_sum, so.flux_sum):
+    so.flux_sum.argtypes = so.adj_sum.argtypes = [ctypes.c_int, dp, dp, dp, dp]
+    for f in (so.kernel, so.weight, so.row_sum, so.flux_sum, so.adj_sum):
         f.restype = ctypes.c_double
     getcontext().prec = 50
     return so
@@ -119,7 +128,8 @@ def test_row_sum_against_decimal(lib, n):
 @pytest.mark.parametrize("spread", [0, 40, 1000])
 def test_flux_sum_against_decimal(lib, n, spread):
     """sum W dm over masses of one size and of sizes 2^+-spread apart: every term
-    to 2^-52 of the largest, and the sum rounded once."""
+    to 2^-52 of the largest, and the sum rounded once; of the opposite differences,
+    exactly the opposite sum."""
     rng = np.random.default_rng(n + spread)
     dm = rng.uniform(-1.0, 1.0, n) * 2.0 ** rng.integers(-spread, 1, n)
     if n > 3:
@@ -129,9 +139,26 @@ def test_flux_sum_against_decimal(lib, n, spread):
              for k, a, b, m in zip(K, ra, rb, dm)]
     want = sum(terms, Decimal(0))
     big = max([abs(t) for t in terms], default=Decimal(0))
-    got = lib.flux_sum(n, _ptr(dm), _ptr(K), _ptr(ra), _ptr(rb))
-    assert abs(Decimal(got) - want) <= Decimal(2.0 ** -52) * n * big + Decimal(2.0 ** -53) * abs(want)
-    assert lib.flux_sum(n, _ptr(-dm), _ptr(K), _ptr(ra), _ptr(rb)) == -got or n > 1
+    for f in (lib.adj_sum, lib.flux_sum):
+        got = f(n, _ptr(dm), _ptr(K), _ptr(ra), _ptr(rb))
+        assert abs(Decimal(got) - want) <= Decimal(2.0 ** -52) * n * big + Decimal(2.0 ** -53) * abs(want)
+    assert lib.flux_sum(n, _ptr(-dm), _ptr(K), _ptr(ra), _ptr(rb)) == -got
+
+
+@pytest.mark.parametrize("n", [7, 8, 9, 100, 5000])
+@pytest.mark.parametrize("m", [1.0, -1.0, 2.0 - 2.0 ** -52, 1.0 + 2.0 ** -52, 1e-300])
+def test_flux_sum_of_many_like_terms(lib, n, m):
+    """Terms of one sign, which raise the unit as the sum grows: less than two units
+    of 2^-57 of the sum for each, and the sum rounded once."""
+    K, r = np.full(n, 0.7310585786300049), np.full(n, 3.3)
+    dm = np.full(n, m)
+    want = n * Decimal(m) * 2 * Decimal(K[0]) / (2 * Decimal(r[0]))
+    # (the weight and the product are each within 2^-54 too)
+    bound = Decimal(2 * n * 2.0 ** -57 + 3 * 2.0 ** -54 + 2.0 ** -53) * abs(want)
+    for f in (lib.adj_sum, lib.flux_sum):
+        got = f(n, _ptr(dm), _ptr(K), _ptr(r), _ptr(r))
+        assert abs(Decimal(got) - want) <= bound
+    assert lib.flux_sum(n, _ptr(-dm), _ptr(K), _ptr(r), _ptr(r)) == -got
 
 
 def test_flux_sum_of_differences_that_are_not_finite(lib):
