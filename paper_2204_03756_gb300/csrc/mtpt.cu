@@ -499,7 +499,8 @@ int setup_grid(RealHost& R, RealParams& P, int64_t cell_base, int corner_base, d
     for (int a = 0; a < p.dim; ++a) {
         const double L = p.hi[a] - p.lo[a];
         double k = P.transfer ? std::floor(L / psi_eff) : 1.0;
-        ncell[a] = std::max(1.0, std::min(k, double(1 << 30)));
+        // (the records hold the x and, in 2-d, the y index in binary32)
+        ncell[a] = std::max(1.0, std::min(k, double(1 << 24)));
     }
     const double cap = std::max(4.0 * double(R.tiled ? R.n_global : R.n) + 64.0, 64.0);
     double total = ncell[0] * ncell[1] * ncell[2];
