@@ -1242,7 +1242,8 @@ __device__ __forceinline__ bool search_rows(uint32_t s, uint32_t cell, const flo
     const float wx = g.wf[0], eps = pp.trim_eps;
     const int R = g.reach, xlo = max(c[0] - R, 0), xhi = min(c[0] + R, g.n[0] - 1);
     const uint32_t lo_bits = __float_as_uint(pp.band_lo);
-    const uint32_t band_span = __float_as_uint(pp.band_hi) - lo_bits;
+    // (read where it is used: a batch's parameters are in memory)
+    auto band_span = [&]() { return __float_as_uint(pp.band_hi) - lo_bits; };
     uint32_t nearest = 0xffffffffu;    // least (bits of d2f) - lo_bits, unsigned
     // one row's window and candidates: an empty window where the row is outside
     // the grid or beyond the cutoff (for_each_row has the windows' derivation)
@@ -1307,10 +1308,10 @@ __device__ __forceinline__ bool search_rows(uint32_t s, uint32_t cell, const flo
             if constexpr (EACH) {
                 bool a0 = int32_t(t0) < 0 && b >= first, a1 = int32_t(t1) < 0 && b + 1u < j3;
                 if constexpr (EXACT) {
-                    if (min(t0, t1) <= band_span) {
-                        a0 |= t0 <= band_span && b >= first &&
+                    if (min(t0, t1) <= band_span()) {
+                        a0 |= t0 <= band_span() && b >= first &&
                               exact_within<DIM>(pos, stride, s, b, pp.psi2);
-                        a1 |= t1 <= band_span && b + 1u < j3 &&
+                        a1 |= t1 <= band_span() && b + 1u < j3 &&
                               exact_within<DIM>(pos, stride, s, b + 1u, pp.psi2);
                     }
                 }
@@ -1333,7 +1334,7 @@ __device__ __forceinline__ bool search_rows(uint32_t s, uint32_t cell, const flo
                 if (base < first) bits &= ~1u;
                 if (j3 - base < 32u) bits &= (1u << (j3 - base)) - 1u;
                 if constexpr (EXACT && !EACH) {
-                    if (nearest <= band_span) {
+                    if (nearest <= band_span()) {
                         for (uint32_t k = max(base, first); k < min(b, j3); ++k) {
                             const float4 o = load_rec(rec, k);
                             const float d2f = d2_f32<DIM>(dx_f32(me, o, wx), me, o, sy, sz);
@@ -1364,20 +1365,20 @@ __device__ __forceinline__ bool search_rows(uint32_t s, uint32_t cell, const flo
 #pragma unroll 1
             for (int dy = -R; dy <= R; ++dy) row(dy, dz);
     }
-    return nearest <= band_span;
+    return nearest <= band_span();
 }
 
 // Sinks of search_rows: the planes, with their padding ...
 struct PlaneSink {
+    const NbPlanes& nb;
+    const int64_t& stride;
     uint2* wp;                         // next mask word
-    int64_t stride;
-    uint32_t cap, pad;
     uint32_t nw = 0, cnt = 0, padded = 0;   // words written or wanted, neighbours
-    __device__ __forceinline__ PlaneSink(const NbPlanes& nb, uint32_t s, int64_t st)
-        : wp(nb.e + s), stride(st), cap(uint32_t(nb.cap)), pad(uint32_t(nb.pad)) {}
-    __device__ __forceinline__ void begin_row() { padded = nw + pad; }
+    __device__ __forceinline__ PlaneSink(const NbPlanes& planes, uint32_t s, const int64_t& st)
+        : nb(planes), stride(st), wp(planes.e + s) {}
+    __device__ __forceinline__ void begin_row() { padded = nw + uint32_t(nb.pad); }
     __device__ __forceinline__ void put(uint2 w) {
-        if (nw < cap) *wp = w;
+        if (nw < uint32_t(nb.cap)) *wp = w;
         wp += stride;
         ++nw;
     }
@@ -1388,7 +1389,7 @@ struct PlaneSink {
     __device__ __forceinline__ void end_row() {
         while (nw < padded) put(make_uint2(0u, 0u));
     }
-    __device__ __forceinline__ bool full() const { return nw > cap; }
+    __device__ __forceinline__ bool full() const { return nw > uint32_t(nb.cap); }
 };
 // ... none ...
 struct NoSink {};
