@@ -203,11 +203,12 @@ int mtpt_get_realisation_info(mtpt_handle* h, int32_t k, mtpt_info* out);
  * follows Eq. "kernel", the normalisation W_ij = K_ij / (1/2 (column sum +
  * row sum)), and M_i(t + dt) = M_i(t) + delta_i with delta_i of
  * Eq. "changemass", all M_j taken at time t.  Enqueued on the stream;
- * returns the launch status.  Calls of four or more steps replay a CUDA graph
- * captured on first use; in the precision form of a plain handle, the mass
- * transfer of every step of a call but its last also walks the particles for
- * the next step (one kernel instead of two).  Either way the results equal
- * step-by-step launches bit for bit. */
+ * returns the launch status.  On a handle without tiles or a binary64 reaction,
+ * the mass transfer of every step of a call but its last also walks the
+ * particles for the next step (one kernel instead of two).  Calls of ten steps or
+ * more (eight where the steps do not walk ahead) replay a CUDA graph of eight
+ * steps, captured on first use, and launch the others one by one.  Either way the
+ * results equal step-by-step launches bit for bit. */
 int mtpt_step(mtpt_handle* h, int64_t nsteps);
 
 /* As mtpt_step with a subset of the step: flags is a combination of
@@ -352,8 +353,9 @@ int mtpt_timing_reset(mtpt_handle* h);
  * Limits: n <= MTPT_NOALLOC_MAX_PARTICLES (65,536); larger n returns
  * MTPT_ERR_TOO_LARGE before any work is enqueued.  The cell grid is capped
  * at 4 n + 64 cells however sparse the box, so n alone bounds the working
- * memory: the largest layout (3-d, binary32 form, n = 65,536, the cell cap
- * reached) needs about 10.8 MiB of the 12.
+ * memory: the largest layouts (3-d binary64 and 2-d precision form, n = 65,536,
+ * the cell cap reached) need about 11.4 MiB of the 12.  What is left holds what
+ * the first pair pass keeps for the second, as far as it fits (same results).
  *
  * Shared scratch: every call uses the same array, which keeps the last
  * call's contents (each call clears what must start at zero).  Calls whose

@@ -1228,7 +1228,8 @@ __device__ __forceinline__ uint32_t mask_word(uint32_t words, uint32_t neighbour
 // time.  Pass 1 of the precision form: 175 -> 158 us by pairs and 142 without
 // the bisection (4e6 particles in 2-d, three cells hold 5.4), 191 -> 187 (2e6 in
 // 3-d, 2.6); at density 10 (54 candidates a row) 1.55 -> 1.18 ms by pairs, with
-// the bisection (1.31 without).
+// the bisection (1.31 without).  With ordinary loads in place of read-only ones
+// 144 and 186 us and 1.22 ms.
 constexpr uint32_t kBisectFrom = 24;
 template <int DIM, bool WORDS, bool EACH, bool EXACT, class Cand, class Sink>
 __device__ __forceinline__ bool search_rows(uint32_t s, uint32_t cell, const float4 me,
@@ -1488,9 +1489,9 @@ __device__ __noinline__ float4 band_words(uint32_t s, const uint32_t* cell, int6
 // a warp that takes its particles' k-th neighbours together stores and reads
 // their kernel values in whole rows.  (Evaluating the warp's neighbours one a
 // lane, as below, saves the lanes idle in the longest particle's tail but
-// spends as many instructions on handing them out: pass 1 took 405 us that way
-// instead of 381, pass 2 with the walk 389 instead of 322, 4e6 particles in
-// 2-d.)
+// spends as many instructions on handing them out: when both were built, with
+// candidates taken singly, pass 1 took 405 us that way instead of 381, pass 2 with
+// the walk 389 instead of 322, 4e6 particles in 2-d.)
 // The adjoint's pair terms keep seven or eight binary64 operations, which cost the
 // same however many lanes are active (a thread per particle took 45 and 51 us a
 // pass where this takes 36 and 40), so there a warp works in two parts: each lane
@@ -1671,7 +1672,7 @@ __device__ __noinline__ double2 search_rowsum(uint32_t s, int64_t stride, const 
 // the ordered pair count.  The kernel values and their sum are fixed-point
 // (expneg.cuh): no binary64 instruction, and the sum is exact whatever its
 // order.  With binary64 operations the pass was bound by that unit (86 % busy):
-// 732 us at 4e6 particles in 2-d with 5.7 neighbours each, 381 now, bound by
+// 732 us at 4e6 particles in 2-d with 5.7 neighbours each, 341 now, bound by
 // instruction issue (72 %).  Two neighbours at a time (their loads and integer
 // chains overlap); 40 registers, 48 in 3-d (four more blocks an SM do not help
 // there: 54 instead of 52 us at 250,007).
@@ -1791,8 +1792,8 @@ __device__ __forceinline__ void walk_ahead(const RealParams& P, int s, int64_t s
 
 // Pass 2, binary64 form: M'_s = M_s + beta sum_j (M_j - M_s) 2 K_sj / (r_s + r_j).
 // Weight, flux and sum are integer arithmetic (expneg.cuh), which leaves the
-// binary64 unit the mass difference, one operation a pair of nine: 543 -> 269 us
-// (4e6 particles, 2-d), 593 -> 322 with the next walk.
+// binary64 unit the mass difference, one operation a pair of nine: 543 -> 283 us
+// (4e6 particles, 2-d), 593 -> 336 with the next walk.
 // Pass 2 of one particle whose neighbours the words do not hold.
 template <int DIM, class View>
 __device__ __noinline__ double search_flux_f64(uint32_t s, int64_t stride,
@@ -2203,7 +2204,7 @@ __device__ __noinline__ float4 search_flux(uint32_t s, int64_t stride, const dou
 // it.  Both add the same terms in the same order.  Bound by the gathers'
 // latency.  Masks in place of lists move 24 instead of 45 bytes a particle for
 // eight more operations a neighbour: 104 us at 4e6 particles in 2-d (100 with
-// lists), 1.5 ms at 1e7 with 57 neighbours (2.0).  Registers: 32 keep all 2048
+// lists), 1.3 ms at 1e7 with 57 neighbours (2.0).  Registers: 32 keep all 2048
 // threads of an SM (four more would cost 4 us); both species need 40 (62 and 58
 // us at 32 and 40 for the reaction at 1e6), a batch's view 36 (1.23, 1.15 and 1.19
 // ms at 32, 36 and 40 for the 512-member ensemble).
@@ -2570,7 +2571,8 @@ k_adj_rowsum(int n, int64_t stride, const double* pos,
 // Both passes are bound by the binary64 unit and its latency together: 44 -> 36 us
 // (A) and 54 -> 40 us (B) at 250,000 particles with 2.8 neighbours each when K,
 // reciprocals and sums became integer work and the neighbour's four values one
-// load; four blocks an SM (three and six: 7 and 4 % slower sweeps).
+// load (34 and 36 us of kernel time alone now); four blocks an SM (three and six: 7
+// and 4 % slower sweeps).
 template <int DIM, class View>
 __global__ void __launch_bounds__(kBlock, 4)
 k_adj_exchange(int n, int64_t stride, const double* pos,

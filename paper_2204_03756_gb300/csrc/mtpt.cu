@@ -35,8 +35,8 @@ namespace {
 
 constexpr int kMaxDim = 3;
 // Steps of one captured graph (even: the buffer pairs then return to where they
-// were).  2, 8 and 32 replay alike (32.2 us a step at 1e4 particles, 33.6 without
-// graphs); the other steps of a call are launched one by one.
+// were).  Eight: 28.5 us a step at 5,000 particles in 2-d, binary64, calls of 50
+// (29.5 with graphs of two); the other steps of a call are launched one by one.
 constexpr int64_t kGraphSteps = 8;
 constexpr int kSettleBlocks = 152;      // grid-stride blocks of k_load_settle (one per SM)
 
@@ -3153,9 +3153,9 @@ extern "C" int mtpt_step_noalloc(const mtpt_params* params, int64_t n, uint64_t 
     h.start.p = cv.take<uint32_t>(cells_pad);
     h.scan_state.p = cv.take<unsigned long long>(cells_pad / kScanTile + 1);   // + the ticket
     if (cv.overflow) return MTPT_ERR_TOO_LARGE;
-    // what pass 1 keeps for pass 2 in what is left, whole or not at all (the same
-    // sums either way: without it pass 2 searches, which took 73 instead of
-    // 68 us for the call at 20,011 particles in 2-d, precision form)
+    // what pass 1 keeps for pass 2 in what is left (the same sums either way: without
+    // it the passes search again, 53 instead of 49 us for the call at 20,011
+    // particles in 2-d, precision form, and 69 instead of 58 us in binary64)
     const bool f64 = h.precision == MTPT_FP64;
     auto fits = [&](size_t bytes) {
         return cv.used + 2 * 256 + bytes <= size_t(MTPT_NOALLOC_SCRATCH_BYTES);
