@@ -397,9 +397,10 @@ int mtpt_adjoint_forward(mtpt_handle* h, int64_t nsteps, int64_t checkpoint_ever
  * dL/dM_T (n doubles, DEVICE, input order); gmass0_dev receives dL/dM_0 (n
  * doubles, DEVICE, input order); *dldD receives dL/dD (HOST).  Recomputes
  * each segment forward from its checkpoint, then steps back through it.
- * While it runs it holds, when it can be had and is at most 16 GiB, a tape of
- * checkpoint_every steps (some 250 bytes per particle and step at 3 neighbours)
- * that spares each step's second walk, sort and search.
+ * While it runs it holds, when the run has five steps or more and it can be had
+ * and is at most 16 GiB, a tape of checkpoint_every steps (some 250 bytes per
+ * particle and step at 3 neighbours) that spares each step's second walk, sort and
+ * search.
  * Leaves the handle in the final state of the forward run.  Deterministic
  * (fixed summation orders).  Synchronises.  MTPT_ERR_STATE without a recorded
  * run. */

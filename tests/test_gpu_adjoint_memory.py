@@ -55,12 +55,14 @@ def test_the_tape_is_held_for_the_sweep_alone():
         mtpt.mtpt_destroy(h)
 
 
-def _sweep(p, pos, mass, g, steps, every, without_tape):
+def _sweep(p, pos, mass, g, steps, every, without_tape, retune=None):
     import torch
     h = mtpt.mtpt_create(p)
     try:
         mtpt.mtpt_set_particles(h, p.dim, pos, mass)
         mtpt.mtpt_adjoint_forward(h, steps, every)
+        if retune:
+            mtpt.mtpt_set_tuning(h, retune, 128)
         gt = torch.from_numpy(g).cuda()
         g0 = torch.empty_like(gt)
         mtpt.mtpt_debug_fail_alloc(-1 if without_tape else 0)
@@ -122,3 +124,28 @@ def test_a_run_that_is_not_differentiated_holds_no_memory():
     del m
     gc.collect()
     assert _free() >= level - 4 * MB
+
+
+@pytest.mark.parametrize("retune", [0.5, 2.0])
+def test_a_grid_retuned_before_the_sweep_keeps_its_tape(retune):
+    rng = np.random.default_rng(9)
+    n, L = 1800, 42.0
+    pos, mass, g = rng.uniform(0.0, L, size=(2, n)), rng.uniform(0.0, 1.0, n), rng.uniform(-1.0, 1.0, n)
+    p = mtpt.Params(dim=2, D=0.5, kappa=0.5, dt=0.1, lo=(0.0, 0.0), hi=(L, L), seed=4)
+    taped, plain = (_sweep(p, pos, mass, g, 8, 8, w, retune) for w in (False, True))
+    assert taped[0] == plain[0] and np.array_equal(taped[1], plain[1])
+
+
+@pytest.mark.parametrize("steps,met", [(1, False), (4, False), (5, True)])
+def test_short_sweeps_take_no_tape(steps, met):
+    """Below five steps the tape's allocation costs more than it spares."""
+    import torch
+    h, _ = _recorded(2000, steps, 20)
+    try:
+        g = torch.ones(2000, dtype=torch.float64, device="cuda")
+        mtpt.mtpt_debug_fail_alloc(-1)
+        mtpt.mtpt_adjoint_backward(h, g, torch.empty_like(g))
+        assert (mtpt.mtpt_debug_fail_alloc(0) == 0) == met
+    finally:
+        mtpt.mtpt_debug_fail_alloc(0)
+        mtpt.mtpt_destroy(h)
