@@ -82,17 +82,17 @@ def _algo_bytes_per_particle(kernel: str, dim: int, form: str) -> float:
 # Valid only for the library source it was measured on: a different hash of
 # the CUDA sources and the header reports traffic as null.
 TRAFFIC_DIM = 2
-TRAFFIC_SOURCE_SHA1 = "fbf8b19fbc7c"
+TRAFFIC_SOURCE_SHA1 = "b06e5c5e9285"
 TRAFFIC_BYTES_PER_PARTICLE = {
-    "walk_key": (88931328 + 26738432) / 4e6,
-    "scatter": (81750016 + 31188224) / 4e6,
-    "gather": (152983296 + 121382656) / 4e6,
-    "rowsum_f32": (129977088 + 159955712) / 4e6,
-    "exchange_f32": (256063488 + 23515392) / 4e6,
-    "exchange_walk_f32": (344992512 + 114313216) / 4e6,
-    "rowsum_f64": (301554176 + 358192640) / 4e6,
-    "exchange_f64": (468451584 + 25626368) / 4e6,
-    "exchange_walk_f64": (557374464 + 118109952) / 4e6,
+    "walk_key": (88937472 + 26860544) / 4e6,
+    "scatter": (81755904 + 31627776) / 4e6,
+    "gather": (152973056 + 121168128) / 4e6,
+    "rowsum_f32": (129790720 + 159709952) / 4e6,
+    "exchange_f32": (255967232 + 23077376) / 4e6,
+    "exchange_walk_f32": (344989696 + 114353664) / 4e6,
+    "rowsum_f64": (300945408 + 357246208) / 4e6,
+    "exchange_f64": (468420608 + 25666560) / 4e6,
+    "exchange_walk_f64": (557543680 + 118318080) / 4e6,
 }
 
 
@@ -101,15 +101,15 @@ TRAFFIC_BYTES_PER_PARTICLE = {
 # issue rate, against the issue peak of 4 warp instructions per clock per SM
 # (one per scheduler).
 INSTR_PER_PARTICLE = {
-    "walk_key": 44144207 / 4e6,
-    "scatter": 4375000 / 4e6,
-    "gather": 40648031 / 4e6,
-    "rowsum_f32": 139910274 / 4e6,
-    "exchange_f32": 77449564 / 4e6,
-    "exchange_walk_f32": 121358548 / 4e6,
-    "rowsum_f64": 307388436 / 4e6,
-    "exchange_f64": 222132905 / 4e6,
-    "exchange_walk_f64": 266376106 / 4e6,
+    "walk_key": 44019207 / 4e6,
+    "scatter": 4250000 / 4e6,
+    "gather": 40523028 / 4e6,
+    "rowsum_f32": 139784435 / 4e6,
+    "exchange_f32": 77324564 / 4e6,
+    "exchange_walk_f32": 121233548 / 4e6,
+    "rowsum_f64": 307808528 / 4e6,
+    "exchange_f64": 235745231 / 4e6,
+    "exchange_walk_f64": 279989077 / 4e6,
 }
 SMS, SCHEDULERS_PER_SM = 152, 4
 
@@ -120,13 +120,13 @@ SMS, SCHEDULERS_PER_SM = 152, 4
 BINDING = {
     "exchange_f32": ("instruction issue 62 % at 18 of 32 active lanes, waiting on the "
                      "neighbour-record gathers; DRAM 35 %"),
-    "exchange_walk_f32": ("instruction issue 72 % at 23 of 32 active lanes and binary64 pipe 49 % "
-                          "(the next step's x + sigma xi); DRAM 43 %"),
+    "exchange_walk_f32": ("instruction issue 71 % at 23 of 32 active lanes and binary64 pipe 49 % "
+                          "(the next step's x + sigma xi); DRAM 42 %"),
     "rowsum_f32": "instruction issue: 79 % of issue slots at 24 of 32 active lanes; DRAM 26 %",
     "rowsum_f64": "instruction issue 72 % at 20 of 32 active lanes (integer kernel values)",
-    "exchange_f64": "instruction issue 66 % at 18 of 32 active lanes and binary64 pipe 59 %",
-    "exchange_walk_f64": "instruction issue 66 % at 20 of 32 active lanes and binary64 pipe 61 %",
-    "gather": "DRAM 60 % (payload reads through the permutation, cell-ordered writes), issue 56 %",
+    "exchange_f64": "instruction issue 67 % at 17 of 32 active lanes and binary64 pipe 57 %",
+    "exchange_walk_f64": "instruction issue 67 % at 20 of 32 active lanes and binary64 pipe 59 %",
+    "gather": "DRAM 60 % (payload reads through the permutation, cell-ordered writes), issue 57 %",
     "scatter": "DRAM 41 % at 10 % issue (slot atomics, permutation and sort-key stores)",
     "walk_key": "binary64 pipe 80 % busy (x + sigma xi)",
 }
@@ -462,7 +462,7 @@ def time_batched(steps, warmup, rank, world, dist, nreal=512, autotune_steps=4):
             "pairs_per_particle_step": pairs / (total * steps),
             "tuning": tuning, "kernels": kstats,
             "launches_per_step": sum(v[0] for v in kstats.values()) / steps,
-            "graph": "two-step CUDA graph replayed for the timed steps"}
+            "graph": "eight-step CUDA graph replayed for the timed steps"}
 
 
 def time_adjoint(rank, nbins=(100, 100), checkpoint_every=20):
